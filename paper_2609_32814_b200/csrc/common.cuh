@@ -119,6 +119,10 @@ struct ProjArgs {
   int64_t ldx;
   const int *perm;        // output row scatter: bucketed -> original; nullptr = keep bucketed
   const int *in_perm;     // SIMT only: input row gather (nullptr = X already bucketed)
+  // fp32 kernel: the CTAs find the buckets from the row types themselves (types == nullptr: row mod q); offsets, perm
+  // and in_perm are not used then
+  bool count_rows = false;
+  const int32_t *types = nullptr;
   const void *W;
   int64_t ldw;
   const void *bias;
@@ -171,7 +175,10 @@ struct ProjArgs {
   long long wait_limit;   // bound of every device-side wait, in SM clock cycles
 };
 
-cudaError_t launch_proj_simt(const ProjArgs &a, bool in_bf16, cudaStream_t st);
+cudaError_t launch_proj_simt(const ProjArgs &a, bool in_bf16, bool widths4, cudaStream_t st);
+constexpr int kCountRows = 4096;   // largest batch of ProjArgs::count_rows
+// rows of a tile of the SIMT kernels for a batch of M rows and N output columns
+int simt_tile_m(bool in_bf16, int M, int N);
 
 // Large-algebra path: complete-graph law with q equal groups, q up to kBigMaxQ, group widths that
 // need not be multiples of the tile (proj_big.cu).

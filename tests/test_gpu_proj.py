@@ -431,3 +431,42 @@ def test_row_gather_in_the_kernel_matches_the_copy_pass(q, M, dw, fw, kernel):
     assert torch.equal(out[0], out[1])
     assert launches[0] == launches[1] + 1
     assert np.array_equal(H.to_np(out[1]), oracle.proj(wl.X, types, wl.W_up, wl.d_widths, wl.f_widths))
+
+
+# ---- fp32 kernel: buckets counted by the CTAs (small batches, few types) or by the bucketing launch; 64- and 128-row
+# tiles; 16- and 4-byte copies; chunks of 64 k that end inside a group; absent types ----------------------------------
+
+@pytest.mark.parametrize("q,M,s,r", [
+    (2, 1, [64, 64], [64, 64]),
+    (1, 255, [100], [68]),                        # one short chunk behind a full one
+    (3, 257, [4, 132, 60], [72, 8, 136]),         # two rows per thread, unequal widths
+    (3, 300, [5, 66, 63], [7, 65, 130]),          # widths off the 16-byte grid: 4-byte copies
+    (8, 4096, [16] * 8, [64] * 8),                # the largest counted batch, the most types
+    (8, 4097, [16] * 8, [64] * 8),                # one row past it: the bucketing launch
+    (9, 700, [20] * 9, [64] * 9),                 # one type past it
+    (2, 2500, [128, 128], [512, 512]),            # 128-row tiles, ragged
+    (2, 2501, [66, 30], [513, 511]),              # 128-row tiles, 4-byte copies
+])
+@pytest.mark.parametrize("schedule", ["explicit", "cyclic"])
+def test_f32_buckets_tiles_and_copies(q, M, s, r, schedule):
+    types = synth.uniform_types(31 + M, M, q) if schedule == "explicit" else synth.cyclic_types(M, q)
+    if schedule == "explicit" and q == 3:
+        types[types == 1] = 2                     # a type without rows
+    wl = synth.make_workload("f32", config=9, variant=40 + q, dtype="f32", q=q, M=M, D=sum(s), F=sum(r), types=types,
+                             integer=True, with_down=False, d_widths=s, f_widths=r)
+    bias = synth.small_ints(98, (sum(r),))
+    ld = lambda t, n: torch.nn.functional.pad(t, (0, n))[:, :t.shape[1]]
+    X, W, b = H.to_dev(wl.X, "f32"), H.to_dev(wl.W_up, "f32"), H.to_dev(bias, "f32")
+    proj = binding.Proj(s, r, dtype="f32", schedule=schedule)
+    bad = M // 2 if schedule == "explicit" else None
+    if bad is not None:
+        types = types.copy()
+        types[bad] = q                            # outside [0, q): that row of Y is zero
+    Y = torch.full((M, (sum(r) + 7) // 4 * 4), 7.0, device="cuda")[:, :sum(r)]
+    px, pw = (1, 3) if any(w % 4 for w in s + r) else (4, 8)   # leading dimensions off the 16-byte grid as well, or on it
+    proj.forward(ld(X, px), None if schedule == "cyclic" else H.dev_types(types), ld(W, pw), bias=b, out=Y)
+    assert proj.last_status() == (0 if bad is None else 5)
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, s, r, bias=bias)
+    if bad is not None:
+        ref[bad] = 0
+    assert np.array_equal(H.to_np(Y), ref)
