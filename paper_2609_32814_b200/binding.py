@@ -104,13 +104,16 @@ def _check(code: int, where: str):
         raise AlgError(code, where)
 
 
+# (plain integers: the functions' argtypes turn them into pointers, and a call of a few microseconds notices every object made)
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    # what torch.cuda.current_stream().cuda_stream is, without the Stream object (3.3 -> 0.3 us)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _widths(w):
@@ -129,6 +132,7 @@ class _Handle:
     def __init__(self):
         self._h = ctypes.c_void_p()
         self._ws = None
+        self._need = (-1, 0)   # (rows, workspace bytes) of the last call that brought no workspace
 
     def close(self):
         if self._h:
@@ -144,6 +148,14 @@ class _Handle:
     def set_option(self, name: str, value: int):
         """alg_*_set_option: per-handle switches (see OPTIONS and the header)."""
         _check(getattr(lib(), self._set_option)(self._h, OPTIONS[name], int(value)), self._set_option)
+        self._need = (-1, 0)   # (an option may select another kernel)
+
+    def _own_workspace(self, M: int, device) -> torch.Tensor:
+        """The handle's own workspace, grown to what a call with M rows needs."""
+        need = self._need
+        if need[0] != M:
+            need = self._need = (M, self.workspace_bytes(M))
+        return self._workspace(need[1], device)
 
     def _workspace(self, nbytes: int, device) -> torch.Tensor:
         if self._ws is None or self._ws.numel() < nbytes or self._ws.device != device:
@@ -188,7 +200,7 @@ class Proj(_Handle):
         M = X.shape[0]
         if out is None:
             out = torch.empty((M, self.N), dtype=out_dtype or X.dtype, device=X.device)
-        ws = workspace if workspace is not None else self._workspace(self.workspace_bytes(M), X.device)
+        ws = workspace if workspace is not None else self._own_workspace(M, X.device)
         _check(lib().alg_proj_forward(self._h, _ptr(X), X.stride(0) if M else self.K, _ptr(types), M, _ptr(W),
                                       W.stride(0), _ptr(bias), _ACTS[act], _ptr(out),
                                       out.stride(0) if M else self.N, _DTYPES[out.dtype], _ptr(ws), ws.numel(),
@@ -292,7 +304,7 @@ class FFN(_Handle):
             raise ValueError("alg_ffn_forward takes packed row-major tensors")
         if out is None:
             out = torch.empty((M, self.D), dtype=out_dtype or X.dtype, device=X.device)
-        ws = workspace if workspace is not None else self._workspace(self.workspace_bytes(M), X.device)
+        ws = workspace if workspace is not None else self._own_workspace(M, X.device)
         _check(lib().alg_ffn_forward(self._h, _ptr(X), _ptr(types), M, _ptr(W_up), _ptr(b_up), _ptr(W_down),
                                      _ptr(b_down), _ACTS[act], _ptr(out), _DTYPES[out.dtype], _ptr(ws), ws.numel(),
                                      _stream(stream)), "alg_ffn_forward")
@@ -342,7 +354,7 @@ class GatedFFN(FFN):
             raise ValueError("W_gate_up must be D x 2F: [W_gate | W_up]")
         if out is None:
             out = torch.empty((M, self.D), dtype=out_dtype or X.dtype, device=X.device)
-        ws = workspace if workspace is not None else self._workspace(self.workspace_bytes(M), X.device)
+        ws = workspace if workspace is not None else self._own_workspace(M, X.device)
         _check(lib().alg_ffn_gated_forward(self._h, _ptr(X), _ptr(types), M, _ptr(W_gate_up), _ptr(W_down), _ptr(out),
                                            _DTYPES[out.dtype], _ptr(ws), ws.numel(), _stream(stream)),
                "alg_ffn_gated_forward")
@@ -376,7 +388,7 @@ class ProjGrad(_Handle):
         M = G.shape[0]
         if out is None:
             out = torch.empty((M, self.K), dtype=out_dtype or G.dtype, device=G.device)
-        ws = workspace if workspace is not None else self._workspace(self.workspace_bytes(M), G.device)
+        ws = workspace if workspace is not None else self._own_workspace(M, G.device)
         _check(lib().alg_proj_grad_input(self._h, _ptr(G), G.stride(0) if M else self.N, _ptr(types), M, _ptr(W), W.stride(0),
                                          _ptr(out), out.stride(0) if M else self.K, _DTYPES[out.dtype], _ptr(ws), ws.numel(),
                                          _stream(stream)), "alg_proj_grad_input")
@@ -386,7 +398,7 @@ class ProjGrad(_Handle):
         M = X.shape[0]
         if out is None:
             out = torch.empty((self.K, self.N), dtype=out_dtype, device=X.device)
-        ws = workspace if workspace is not None else self._workspace(self.workspace_bytes(M), X.device)
+        ws = workspace if workspace is not None else self._own_workspace(M, X.device)
         _check(lib().alg_proj_grad_weight(self._h, _ptr(X), X.stride(0) if M else self.K, _ptr(G), G.stride(0) if M else self.N,
                                           _ptr(types), M, _ptr(out), out.stride(0), _DTYPES[out.dtype], _ptr(ws), ws.numel(),
                                           _stream(stream)), "alg_proj_grad_weight")

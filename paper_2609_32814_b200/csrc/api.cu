@@ -231,6 +231,12 @@ void plan_big(alg_proj_s &p, int s, int r) {
   p.big.block_k = 64;
 }
 
+// (two attribute queries: cudaGetDeviceProperties asks for everything and takes 2.5 ms a call)
+bool device_facts(int dev, int *major, int *num_sms) {
+  return cudaDeviceGetAttribute(major, cudaDevAttrComputeCapabilityMajor, dev) == cudaSuccess &&
+         cudaDeviceGetAttribute(num_sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+}
+
 // Handle of the large-algebra path only (q > kMaxQ or the interval schedule): no interaction table.
 alg_status_t init_big(alg_proj_s &p, int q, int s, int r, alg_schedule_t sched) {
   p.q = q;
@@ -242,11 +248,10 @@ alg_status_t init_big(alg_proj_s &p, int q, int s, int r, alg_schedule_t sched) 
   p.big.only = true;
   if (q <= kMaxQ)
     for (int g = 0; g < q; ++g) p.s[g] = s, p.r[g] = r;
+  int major = 0;
   if (cudaGetDevice(&p.device) != cudaSuccess) return ALG_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, p.device) != cudaSuccess) return ALG_ERR_CUDA;
-  p.num_sms = prop.multiProcessorCount;
-  if (prop.major != 10) return ALG_ERR_UNSUPPORTED_SHAPE;
+  if (!device_facts(p.device, &major, &p.num_sms)) return ALG_ERR_CUDA;
+  if (major != 10) return ALG_ERR_UNSUPPORTED_SHAPE;
   if (cudaMalloc(&p.d_status, 4 * sizeof(int)) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemset(p.d_status, 0, 4 * sizeof(int)) != cudaSuccess) return ALG_ERR_CUDA;
   if (tc_init() != cudaSuccess) return ALG_ERR_CUDA;
@@ -318,11 +323,10 @@ alg_status_t init_proj(alg_proj_s &p, int q, const int32_t *in_w, const int32_t 
     p.big.on = !p.tc_ok;   // by default only for widths the table-driven tensor path does not take
   }
 
+  int major = 0;
   if (cudaGetDevice(&p.device) != cudaSuccess) return ALG_ERR_CUDA;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, p.device) != cudaSuccess) return ALG_ERR_CUDA;
-  p.num_sms = prop.multiProcessorCount;
-  if (prop.major != 10) return ALG_ERR_UNSUPPORTED_SHAPE;  // sm_100a code only
+  if (!device_facts(p.device, &major, &p.num_sms)) return ALG_ERR_CUDA;
+  if (major != 10) return ALG_ERR_UNSUPPORTED_SHAPE;  // sm_100a code only
   if (cudaMalloc(&p.d_tab, sizeof(DevTable)) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemcpy(p.d_tab, &p.tab, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMalloc(&p.d_tab_tall, sizeof(DevTable)) != cudaSuccess) return ALG_ERR_CUDA;
