@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "exchange.cuh"
 
 using namespace algproj;
 
@@ -90,7 +91,8 @@ struct alg_ffn_s {
   bool fd_ok = false;
   bool rd_ok = false;        // decode step of one row in one launch (row_decode.cu): gated, or plain without fd_ok
   FfnDecodePlan fd = {};
-  unsigned int *d_counters = nullptr;
+  uint8_t *d_exch = nullptr; // the hidden rows of the one-launch decode steps (exchange.cuh)
+  int exch_bytes = 0;        // of one of its two buffers
 };
 
 // Both gradient maps of one forward projection (s[q] -> r[q]).
@@ -1340,6 +1342,14 @@ alg_status_t alg_proj_grad_last_status(alg_proj_grad_t h, void *stream, alg_stat
   return read_status(h->dx.d_status, stream, status);
 }
 
+// The exchange as a handle starts with it: turn 0, both buffers empty.
+static alg_status_t reset_exchange(alg_ffn_s &f) {
+  const size_t buffers = 2 * (size_t)f.exch_bytes;
+  if (!f.d_exch && cudaMalloc(&f.d_exch, kExchHeader + buffers) != cudaSuccess) return ALG_ERR_CUDA;
+  if (cudaMemset(f.d_exch, 0, kExchHeader) != cudaSuccess) return ALG_ERR_CUDA;
+  return cuda_status(cudaMemset(f.d_exch + kExchHeader, 0xFF, buffers));
+}
+
 static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, const int32_t *f_widths,
                                alg_dtype_t dtype, alg_table_t table, const uint8_t *custom_keep,
                                alg_schedule_t schedule, bool gated) {
@@ -1365,16 +1375,20 @@ static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, c
   }
   f->D = f->up.K;
   f->F = f->up.N;
-  if (dtype == ALG_BF16 && !gated && schedule != ALG_SCHED_INTERVAL &&
-      ffn_decode_plan(q, f->up.s, f->down.s, f->D, f->F, f->up.num_sms, &f->fd)) {
-    f->fd_ok = cudaMalloc(&f->d_counters, 2 * sizeof(unsigned int)) == cudaSuccess &&
-               cudaMemset(f->d_counters, 0, 2 * sizeof(unsigned int)) == cudaSuccess;
-  }
-  if (dtype == ALG_BF16 && schedule != ALG_SCHED_INTERVAL && f->up.big.eligible && f->down.big.eligible &&
-      row_decode_fits(q, f->D, f->F)) {
-    // (the two one-launch decode kernels share the exchange counters: both leave them zero)
-    f->rd_ok = f->d_counters != nullptr || (cudaMalloc(&f->d_counters, 2 * sizeof(unsigned int)) == cudaSuccess &&
-                                            cudaMemset(f->d_counters, 0, 2 * sizeof(unsigned int)) == cudaSuccess);
+  f->fd_ok = dtype == ALG_BF16 && !gated && schedule != ALG_SCHED_INTERVAL &&
+             ffn_decode_plan(q, f->up.s, f->down.s, f->D, f->F, f->up.num_sms, &f->fd);
+  f->rd_ok = dtype == ALG_BF16 && schedule != ALG_SCHED_INTERVAL && f->up.big.eligible && f->down.big.eligible &&
+             row_decode_fits(q, f->D, f->F);
+  if (f->fd_ok || f->rd_ok) {   // (the two one-launch decode steps share the exchange)
+    f->exch_bytes = (int)align_up((size_t)(f->rd_ok ? kRowDecodeMaxM : 1) * f->F * 2, 256);
+    s = reset_exchange(*f);
+    if (s != ALG_OK) {
+      if (f->d_exch) cudaFree(f->d_exch);
+      free_proj(f->down);
+      free_proj(f->up);
+      delete f;
+      return s;
+    }
   }
   *out = f;
   return ALG_OK;
@@ -1404,7 +1418,7 @@ alg_status_t alg_ffn_destroy(alg_ffn_t h) {
   if (!h) return ALG_ERR_INVALID_ARG;
   for (int e = 0; e < 5; ++e)
     if (h->ev[e]) cudaEventDestroy(h->ev[e]);
-  if (h->d_counters) cudaFree(h->d_counters);
+  if (h->d_exch) cudaFree(h->d_exch);
   free_proj(h->down);
   free_proj(h->up);
   delete h;
@@ -1448,7 +1462,8 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
     d.Y = Y;
     d.y_bf16 = y_dtype == ALG_BF16;
     d.D = h->D, d.F = h->F, d.q = u.q;
-    d.counters = h->d_counters;
+    d.counters = (unsigned int *)(h->d_exch + kExchCounters);
+    d.exch = h->d_exch, d.exch_bytes = h->exch_bytes;
     d.status = u.d_status;
     d.wait_limit = u.wait_limit;
     d.extra_expect_bytes = u.test_extra_expect;
@@ -1473,14 +1488,13 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
     d.W2 = W_down, d.ldw2 = h->D;
     d.b1 = b_up, d.b2 = b_down;
     d.act = (int)act;
-    d.H = ws + L.h;
     d.Y = Y, d.ldy = h->D;
     d.y_bf16 = y_dtype == ALG_BF16;
     d.D = h->D, d.F = h->F, d.q = h->up.q;
-    d.counters = h->d_counters;
+    d.exch = h->d_exch, d.exch_bytes = h->exch_bytes;
     d.status = h->up.d_status;
     d.wait_limit = h->up.wait_limit;
-    d.extra_arrivals = h->up.test_extra_expect ? 1 : 0;
+    d.test_withhold = h->up.test_extra_expect ? 1 : 0;
     return cuda_status(launch_row_decode(d, h->up.num_sms, st));
   }
   if (use_decode(h->up, M) && use_decode(h->down, M)) {
@@ -1602,9 +1616,7 @@ alg_status_t alg_ffn_macs(alg_ffn_t h, const int64_t *rows_per_type, int64_t *ma
 alg_status_t alg_ffn_last_status(alg_ffn_t h, void *stream, alg_status_t *status) {
   if (!h) return ALG_ERR_INVALID_ARG;
   alg_status_t s = read_status(h->up.d_status, stream, status);
-  // a launch that gave up may have left the exchange counters of the one-launch decode step half way
-  if (s == ALG_OK && *status != ALG_OK && h->d_counters)
-    s = cuda_status(cudaMemset(h->d_counters, 0, 2 * sizeof(unsigned int)));
+  if (s == ALG_OK && *status == ALG_ERR_DEVICE_TIMEOUT && h->d_exch) s = reset_exchange(*h);
   return s;
 }
 

@@ -300,14 +300,16 @@ struct FfnDecodeArgs {
   const void *W_up, *W_down;   // canonical banks, packed: [D][F] and [F][D]
   const void *b_up, *b_down;
   int act;
-  void *H;                // [M][F] bf16 scratch in global memory
+  void *H;                // [M][F] bf16 scratch in global memory (more than one row)
   void *Y;                // [M][D]
   int y_bf16;
   int D, F, q;
   int su, sd, n_up, n_dn;
   int off_wu, off_stage, off_p, off_ctl;   // shared-memory offsets (the W_down slice sits at 0)
   int kc_up, kc_dn, m_pad;                 // K-chunk lengths of the staged activations; staged rows (8 or 16)
-  unsigned int *counters;                  // [0] producers arrived, [1] consumers past the wait; zero between launches
+  uint8_t *exch;                           // one row: its hidden row between the phases (exchange.cuh), buffers of exch_bytes
+  int exch_bytes;
+  unsigned int *counters;                  // more rows: [0] producers arrived, [1] consumers past the wait; zero between launches
   int *status;
   long long wait_limit;
   int extra_expect_bytes;
@@ -334,7 +336,6 @@ struct RowDecodeArgs {
   int64_t ldw2;
   const void *b1, *b2;      // bf16 biases or nullptr (not gated)
   int act;                  // activation of phase 1 (not gated)
-  void *H;                  // [M][F] bf16 scratch in global memory, 16-byte aligned (FFN modes)
   void *Y;                  // [M][ldy]: D columns (projection: F)
   int64_t ldy;
   int y_bf16;
@@ -344,10 +345,11 @@ struct RowDecodeArgs {
   int pc1, pc2;             // columns of a warp's piece (8 or 16)                 (set by the launcher)
   int ks1, ks2;             // warps sharing the weight rows of a piece            (set by the launcher)
   int units1, units2;       // pieces x sharing warps                              (set by the launcher)
-  unsigned int *counters;   // [0] CTAs that finished phase 1, [1] CTAs past the wait; zero between launches (FFN modes)
+  uint8_t *exch;            // FFN modes: hidden rows between the phases (exchange.cuh), buffers of exch_bytes
+  int exch_bytes;
   int *status;
   long long wait_limit;
-  int extra_arrivals;       // test hook: arrivals the wait between the phases expects beyond the grid's (never come)
+  int test_withhold;        // test hook: CTA 0 keeps its hidden values to itself, so that the waits for them run out
 };
 bool row_decode_fits(int q, int D, int F);
 cudaError_t launch_row_decode(const RowDecodeArgs &a, int num_sms, cudaStream_t st);

@@ -22,15 +22,20 @@
 //                     "row b uses block k only if k in B(t_b, j)" is applied by clearing the A
 //                     fragment rows that do not use the block; the 8 partial tiles are summed in a
 //                     fixed order through shared memory; bias, activation, bf16 -> H in global memory.
-//   exchange        : producers publish with fence + one atomic add on a counter; consumers poll it
-//                     (bounded), the last consumer clears the counters for the next launch.
+//   exchange        : one row: H goes through the handle's exchange buffer, whose consumers load again what
+//                     is not there yet (exchange.cuh).  Several rows: producers publish with fence + one
+//                     atomic add on a counter; consumers poll it (bounded), the last consumer clears the
+//                     counters for the next launch (96 CTAs polling 8 rows: 12.1 us a layer against 9.6).
+//                     One row has a kernel of its own: the branch alone cost 0.6 us a layer of both, the
+//                     step is that sensitive to the code it has to fetch.
 //   down phase      : H staged from L2 over the shared memory the W_up slice no longer needs; same
 //                     MMA / reduction; bias; Y stored.
-// Every wait (mbarriers the copies arrive on, one counter) is bounded by the handle's wait limit; on expiry the CTA
+// Every wait (mbarriers the copies arrive on, a counter or the values of H) is bounded by the handle's wait limit; on expiry the CTA
 // raises ALG_ERR_DEVICE_TIMEOUT, skips its arithmetic, gives copies in flight time to land and
 // returns.
 #include <algorithm>
 
+#include "exchange.cuh"
 #include "tc_common.cuh"
 
 namespace algproj {
@@ -134,7 +139,6 @@ struct Phase {
   int act;
   void *out;                  // H (bf16) or Y
   int out_ld, out_bf16;
-  bool first_chunk_staged;    // chunk 0 was requested by the caller already
 };
 struct Shared {
   Ctl *ctl;
@@ -177,6 +181,30 @@ __device__ __forceinline__ void stage_chunk(const Shared &sh, const Phase &ph, i
   cp_async_arrive(sh.bar_x);
 }
 
+// One row, all threads: one K chunk of the hidden row, out of the exchange buffer as its values arrive.  (The other
+// staged rows keep whatever is there: the row rule clears their A fragments.)
+__device__ __forceinline__ void stage_hidden(const Shared &sh, const Phase &ph, int kc0, int len) {
+  const int pieces = len >> 3;
+  const long long t0 = clock64();
+  uint32_t spins = 0;
+  for (int p = threadIdx.x; p < pieces; p += kThreads) {
+    const __nv_bfloat16 *src = ph.src + kc0 + p * 8;
+    uint4 v = exch_load4(src);
+    while (!exch_ready(v)) {
+      if ((++spins & 63u) == 0) {
+        if (sh.ctl->abort_flag) return;
+        if (clock64() - t0 > sh.wait_limit) {
+          sh.ctl->abort_flag = 1;
+          atomicExch(sh.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+          return;
+        }
+      }
+      v = exch_load4(src);
+    }
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ph.stage_base + (uint32_t)(p << 4)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+  }
+}
+
 // One projection phase of a CTA:  out[:, strip] = act(src *_q W[:, strip] + bias).
 // The K range is staged chunk by chunk (one chunk for M <= 8 at the benchmark shape).  Warp w takes
 // the 16-deep K steps w, w+8, ... of every needed input group, in batches of SETS steps: all
@@ -185,12 +213,13 @@ __device__ __forceinline__ void stage_chunk(const Shared &sh, const Phase &ph, i
 // "row b uses block k only if k in B(t_b, j)" is applied by clearing the rows of the A fragment that
 // do not use the block.  The 8 warps' partial tiles are then summed in warp order through shared
 // memory (deterministic), bias and activation applied, rows < M stored.
-// NT = 8-column tiles of the strip.  Returns false when a wait ran out.
-template <int NT>
+// NT = 8-column tiles of the strip.  HIDDEN: the phase reads the hidden state (down); else it writes it (up).  ONE: one
+// row.  Returns false when a wait ran out.
+template <int NT, bool HIDDEN, bool ONE>
 __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, uint32_t &x_parity) {
   constexpr int SETS = NT <= 2 ? 4 : (NT <= 4 ? 2 : 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool HALF = sh.m_pad == 8;
+  const bool HALF = ONE || sh.m_pad == 8;
   const int g = lane >> 2, t4 = lane & 3;
   const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8;
   const int a_row = HALF ? (lane & 7) : frag_row;
@@ -207,12 +236,19 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
   bool ok = true;
   for (int kc0 = 0; kc0 < ph.K && ok; kc0 += ph.kc) {
     const int len = min(ph.kc, ph.K - kc0);
-    if (kc0 || !ph.first_chunk_staged) {
+    if (HIDDEN && ONE) {
       if (kc0) __syncthreads();   // the previous chunk has been consumed
-      stage_chunk(sh, ph, kc0, len);
+      stage_hidden(sh, ph, kc0, len);
+      __syncthreads();
+      ok = !sh.ctl->abort_flag;
+    } else {
+      if (kc0) {   // (the caller has requested the first one)
+        __syncthreads();   // the previous chunk has been consumed
+        stage_chunk(sh, ph, kc0, len);
+      }
+      ok = wait_bar(sh, sh.bar_x, x_parity);
+      x_parity ^= 1u;
     }
-    ok = wait_bar(sh, sh.bar_x, x_parity);
-    x_parity ^= 1u;
     if (!ok) break;
     for (int k = 0; k < sh.q; ++k) {
       if (!((ph.need >> k) & 1u)) continue;
@@ -284,7 +320,10 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
     }
     z0 = act_f(z0, ph.act), z1 = act_f(z1, ph.act);
     if ((sh.ctl->bad_rows >> m) & 1u) z0 = z1 = 0.f;   // out-of-range type: the row's output is defined to be zero
-    if (ph.out_bf16) {
+    if (!HIDDEN && ONE) {
+      __nv_bfloat162 v = __floats2bfloat162_rn(z0, z1);
+      exch_store((__nv_bfloat16 *)ph.out + (int64_t)m * ph.out_ld + col, *(uint32_t *)&v);
+    } else if (ph.out_bf16) {
       __nv_bfloat162 v = __floats2bfloat162_rn(z0, z1);
       *(uint32_t *)((__nv_bfloat16 *)ph.out + (int64_t)m * ph.out_ld + col) = *(uint32_t *)&v;
     } else {
@@ -294,8 +333,8 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
   return true;
 }
 // NTU / NTD: 8-column tiles of the up / down strip (compile-time, so that every kernel gets the
-// registers its own shape needs).
-template <int NTU, int NTD>
+// registers its own shape needs).  ONE: one row, and the hidden row travels through the exchange buffer.
+template <int NTU, int NTD, bool ONE>
 __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecodeArgs a) {
   // the next launch of the stream may start now: it only requests its own weights before it waits
   // (triggering later -- after the up phase or after the exchange -- was measured no faster)
@@ -307,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   uint8_t *st_sm = smem + a.off_stage;          // X stage; the H stage starts at wu_sm and runs through here
   Ctl *ctl = (Ctl *)(smem + a.off_ctl);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c = blockIdx.x, q = a.q, M = a.M;
+  const int c = blockIdx.x, q = a.q, M = ONE ? 1 : a.M;
   const bool has_up = c < a.n_up, has_dn = c < a.n_dn;
   const int col_u = c * a.su, col_d = c * a.sd;
   const int D = a.D, F = a.F;
@@ -386,6 +425,8 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   asm volatile("griddepcontrol.wait;" ::: "memory");
   TR(3);
 
+  ExchTurn turn = {0u, 0};
+  if (ONE) turn = exch_turn(a.exch);   // (on its way while the activations are staged)
   Shared sh;
   sh.ctl = ctl, sh.p_sm = (float *)(smem + a.off_p), sh.bar_x = bar_x;
   sh.M = M, sh.m_pad = a.m_pad, sh.q = q, sh.wait_limit = a.wait_limit, sh.status = a.status;
@@ -393,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   up.src = (const __nv_bfloat16 *)a.X, up.ld = D, up.K = D, up.kc = a.kc_up, up.pitch_bytes = a.kc_up * 2;
   up.stage_base = smem_u32(st_sm), up.w_base = smem_u32(wu_sm), up.cols = a.su, up.col0 = col_u;
   up.so = ctl->so_d, up.rows_k = ctl->rows_up, up.bias = a.b_up, up.act = a.act;
-  up.out = a.H, up.out_ld = F, up.out_bf16 = 1, up.first_chunk_staged = true;
+  up.out_ld = F, up.out_bf16 = 1;
   uint32_t x_parity = 0;
   if (has_up) stage_chunk(sh, up, 0, min(a.kc_up, D));
   // the row types as the previous kernel left them: the ones that count
@@ -423,6 +464,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   }
   TR(4);
   bool ok = true;
+  void *const hidden = ONE ? (void *)(a.exch + kExchHeader + turn.parity * (unsigned)a.exch_bytes) : a.H;
 
   // ---------------- up phase: H[:, strip] = act(X *_q W_up + b_up) ----------------
   if (has_up) {
@@ -430,45 +472,54 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
     if (ok && missed) ok = wait_bar(sh, bar_miss, 0);
     TR(5);
     up.need = ctl->need_up;
-    if (ok) ok = run_phase_t<NTU>(sh, up, x_parity);
+    up.out = hidden;
+    if (ok) ok = run_phase_t<NTU, false, ONE>(sh, up, x_parity);
     TR(6);
-    // publish: every thread's H stores become visible device-wide, then one arrival per CTA
-    __threadfence();
-    __syncthreads();
-    if (tid == 0 && ok) atomicAdd(a.counters, 1u);
-  }
-  if (has_dn) {
-    // ---------------- exchange: all of H must be there ----------------
-    if (tid == 0) {
-      const long long t0 = clock64();
-      int go = ctl->abort_flag ? 0 : 1;
-      while (go && ld_acquire_u32(a.counters) < (unsigned)a.n_up) {
-        if (clock64() - t0 > a.wait_limit) {
-          atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
-          ctl->abort_flag = 1;
-          go = 0;
-        }
-      }
-      ctl->go = go;
+    if (!ONE) {   // publish: every thread's H stores become visible device-wide, then one arrival per CTA
+      __threadfence();
+      __syncthreads();
+      if (tid == 0 && ok) atomicAdd(a.counters, 1u);
     }
-    __syncthreads();   // also: every warp is done with the W_up slice and the partial-sum buffer
-    ok = ctl->go != 0;
-    // the last consumer past the wait clears the counters: the next launch starts from zero
-    if (tid == 0 && ok && atomicAdd(a.counters + 1, 1u) == (unsigned)(a.n_dn - 1)) a.counters[0] = 0u, a.counters[1] = 0u;
+  }
+  if (ONE) exch_clear(a.exch, a.exch_bytes, turn, F * 2, 1);
+  if (has_dn) {
+    if (!ONE) {
+      // ---------------- exchange: all of H must be there ----------------
+      if (tid == 0) {
+        const long long t0 = clock64();
+        int go = ctl->abort_flag ? 0 : 1;
+        while (go && ld_acquire_u32(a.counters) < (unsigned)a.n_up) {
+          if (clock64() - t0 > a.wait_limit) {
+            atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+            ctl->abort_flag = 1;
+            go = 0;
+          }
+        }
+        ctl->go = go;
+      }
+      __syncthreads();   // also: every warp is done with the W_up slice and the partial-sum buffer
+      ok = ctl->go != 0;
+      // the last consumer past the wait clears the counters: the next launch starts from zero
+      if (tid == 0 && ok && atomicAdd(a.counters + 1, 1u) == (unsigned)(a.n_dn - 1)) a.counters[0] = 0u, a.counters[1] = 0u;
+    }
     TR(7);
     // ---------------- down phase: Y[:, strip] = H *_q W_down + b_down ----------------
     if (ok) {
       Phase dn;
-      dn.src = (const __nv_bfloat16 *)a.H, dn.ld = F, dn.K = F, dn.kc = a.kc_dn, dn.pitch_bytes = a.kc_dn * 2;
+      dn.src = (const __nv_bfloat16 *)hidden, dn.ld = F, dn.K = F, dn.kc = a.kc_dn, dn.pitch_bytes = a.kc_dn * 2;
       dn.stage_base = smem_u32(wu_sm), dn.w_base = smem_u32(wd_sm), dn.cols = a.sd, dn.col0 = col_d;
       dn.so = ctl->so_f, dn.rows_k = ctl->rows_dn, dn.need = ctl->need_dn, dn.bias = a.b_down, dn.act = ALG_ACT_NONE;
-      dn.out = a.Y, dn.out_ld = D, dn.out_bf16 = a.y_bf16, dn.first_chunk_staged = true;
-      stage_chunk(sh, dn, 0, min(a.kc_dn, F));   // H travels while the weight barrier is checked
+      dn.out = a.Y, dn.out_ld = D, dn.out_bf16 = a.y_bf16;
+      if (!ONE) stage_chunk(sh, dn, 0, min(a.kc_dn, F));   // H travels while the weight barrier is checked
       ok = wait_bar(sh, bar_dn, 0);
       if (ok && missed && !has_up) ok = wait_bar(sh, bar_miss, 0);
       TR(8);
-      if (ok) ok = run_phase_t<NTD>(sh, dn, x_parity);
+      if (ok) ok = run_phase_t<NTD, true, ONE>(sh, dn, x_parity);
     }
+  }
+  if (ONE) {
+    __syncthreads();
+    if (tid == 0) exch_leave(a.exch);
   }
   TR(9);
   if (ctl->abort_flag) {  // copies that are still in flight get time to land before shared memory is released
@@ -496,18 +547,17 @@ int pick_strip(int q, const int *w, int total, int num_sms) {
   return 0;
 }
 // the instantiated strip widths: up to 32 hidden columns and 16 output columns per CTA
-void (*pick_kernel(int ntu, int ntd))(const FfnDecodeArgs) {
-  if (ntd == 1) {
-    if (ntu == 1) return ffn_decode_kernel<1, 1>;
-    if (ntu == 2) return ffn_decode_kernel<2, 1>;
-    if (ntu == 3) return ffn_decode_kernel<3, 1>;
-    if (ntu == 4) return ffn_decode_kernel<4, 1>;
-  } else if (ntd == 2) {
-    if (ntu == 1) return ffn_decode_kernel<1, 2>;
-    if (ntu == 2) return ffn_decode_kernel<2, 2>;
-    if (ntu == 3) return ffn_decode_kernel<3, 2>;
-    if (ntu == 4) return ffn_decode_kernel<4, 2>;
-  }
+template <int NTD, bool ONE>
+void (*pick_up(int ntu))(const FfnDecodeArgs) {
+  return ntu == 1   ? ffn_decode_kernel<1, NTD, ONE>
+         : ntu == 2 ? ffn_decode_kernel<2, NTD, ONE>
+         : ntu == 3 ? ffn_decode_kernel<3, NTD, ONE>
+         : ntu == 4 ? ffn_decode_kernel<4, NTD, ONE>
+                    : nullptr;
+}
+void (*pick_kernel(int ntu, int ntd, bool one))(const FfnDecodeArgs) {
+  if (ntd == 1) return one ? pick_up<1, true>(ntu) : pick_up<1, false>(ntu);
+  if (ntd == 2) return one ? pick_up<2, true>(ntu) : pick_up<2, false>(ntu);
   return nullptr;
 }
 
@@ -519,7 +569,7 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
   FfnDecodePlan p = {};
   p.su = pick_strip(q, fw, F, num_sms);
   p.sd = pick_strip(q, dw, D, num_sms);
-  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3)) return false;
+  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3, false)) return false;
   p.n_up = F / p.su, p.n_dn = D / p.sd;
   p.wd_bytes = F * p.sd * 2;
   p.wu_bytes = D * p.su * 2;
@@ -533,7 +583,7 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
 }
 
 cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p, cudaStream_t st) {
-  void (*kernel)(const FfnDecodeArgs) = pick_kernel(p.su >> 3, p.sd >> 3);
+  void (*kernel)(const FfnDecodeArgs) = pick_kernel(p.su >> 3, p.sd >> 3, args.M == 1);
   if (!kernel) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   if (e != cudaSuccess) return e;

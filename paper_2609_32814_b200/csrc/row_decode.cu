@@ -10,8 +10,9 @@
 // share of the weight rows); its lanes split the rows, every lane keeps up to 32 loads of 16 bytes in flight and
 // reads the activations it needs straight from global memory -- no staging, one CTA barrier per phase at most.
 // The first weight loads are issued before the launch's dependency resolves (weights do not depend on the previous
-// kernel), those of W_down before the wait between the phases of an FFN.  Phase 1 of an FFN writes the hidden row h
-// (bf16) to global memory; all CTAs meet at a counter (bounded wait); phase 2 is the same routine on h and W_down.
+// kernel), those of W_down before the second phase of an FFN.  Phase 1 of an FFN writes the hidden row h (bf16) to the
+// handle's exchange buffer; phase 2 is the same routine on h and W_down, and a lane waits (bounded) for the values of h
+// it needs -- the two groups its columns take -- not for the whole grid (exchange.cuh).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -19,6 +20,7 @@
 #include <cstdint>
 
 #include "common.cuh"
+#include "exchange.cuh"
 #include "trace.cuh"
 
 namespace algproj {
@@ -107,11 +109,18 @@ __device__ __forceinline__ void load_chunk(uint4 (&w)[kLoads], const Phase &p, c
   }
 }
 
+// Bound of the waits for hidden values.
+struct Wait {
+  long long t0, limit;
+  volatile int *abort_flag;   // shared memory: one wait that ran out ends the others
+  int *status;
+};
+
 // acc[0..8) (gate or plain) and acc[8..16) (up) += x[kk] * w[kk][...] for one chunk.  x is read from global memory
-// (FROM_L2: written by other CTAs of this launch).
-template <bool GATED, bool FROM_L2>
+// (HIDDEN: from the exchange buffer, where it may yet have to arrive).
+template <bool GATED, bool HIDDEN>
 __device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads], const Phase &p, const Lane &l, int type, int c0,
-                                          const __nv_bfloat16 *x, float (&acc)[16]) {
+                                          const __nv_bfloat16 *x, float (&acc)[16], const Wait &wait) {
   constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
   const int step = p.ks * l.rl, first = l.part * l.rl + l.lr;
   const int nr = ((p.s + step - 1) >> (__ffs(step) - 1)) - c0;   // rows of this chunk some lane has (the same in every lane)
@@ -127,9 +136,35 @@ __device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads], const Phase 
       unsigned short raw = 0;
       if (seg_on && kk < p.s) {
         const unsigned short *src = (const unsigned short *)(x + (int64_t)g * p.s + kk);
-        raw = FROM_L2 ? __ldcg(src) : __ldg(src);
+        raw = HIDDEN ? exch_load(src) : __ldg(src);
       }
       xv[sg * RC + u] = __uint_as_float((uint32_t)raw << 16);
+    }
+  }
+  if (HIDDEN) {   // what had not arrived is loaded again
+    uint32_t spins = 0;
+    bool missing = true;
+    while (missing) {
+      missing = false;
+#pragma unroll
+      for (int sg = 0; sg < 2; ++sg) {
+        const int g = sg == 0 ? l.j : type;
+#pragma unroll
+        for (int u = 0; u < RC; ++u) {
+          if (u >= nr) break;
+          if (__float_as_uint(xv[sg * RC + u]) == 0xFFFF0000u) {
+            missing = true;
+            xv[sg * RC + u] = __uint_as_float((uint32_t)exch_load((const unsigned short *)(x + (int64_t)g * p.s + first + (c0 + u) * step)) << 16);
+          }
+        }
+      }
+      if (missing && (++spins & 63u) == 0) {
+        if (*wait.abort_flag) break;
+        if (clock64() - wait.t0 > wait.limit) {
+          *wait.abort_flag = 1;
+          atomicExch(wait.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+        }
+      }
     }
   }
 #pragma unroll
@@ -149,9 +184,9 @@ __device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads], const Phase 
 
 // One phase for the units of this warp.  `w` holds the first chunk of the first unit when have_first.  Results of a
 // piece: lanes with lr == 0 of the warp with part == 0 call `emit(col, acc)`.
-template <bool GATED, bool FROM_L2, typename Emit>
+template <bool GATED, bool HIDDEN, typename Emit>
 __device__ __forceinline__ void run_phase(const Phase &p, int type, const __nv_bfloat16 *x, uint4 (&w)[kLoads], bool have_first,
-                                          int n_units, float *partial, Emit emit) {
+                                          int n_units, float *partial, const Wait &wait, Emit emit) {
   constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total_warps = gridDim.x * kWarps, po = p.pc >> 3;
@@ -166,7 +201,7 @@ __device__ __forceinline__ void run_phase(const Phase &p, int type, const __nv_b
     const int rows_per_lane = (p.s + p.ks * l.rl - 1) >> (__ffs(p.ks * l.rl) - 1);
     for (int c0 = 0; c0 < rows_per_lane; c0 += RC) {
       if (!(have_first && rd == 0 && c0 == 0)) load_chunk<GATED>(w, p, l, type, c0);
-      fma_chunk<GATED, FROM_L2>(w, p, l, type, c0, x, acc);
+      fma_chunk<GATED, HIDDEN>(w, p, l, type, c0, x, acc, wait);
     }
     // sum over the lanes that share the columns
 #pragma unroll
@@ -205,7 +240,7 @@ __device__ __forceinline__ float activate(float z, int act) {
 }
 
 // eight results of a piece: + bias, activation, stored as bf16 or fp32
-__device__ __forceinline__ void store8(const float (&acc)[16], int col, const void *bias, int act, void *out, bool out_bf16) {
+__device__ __forceinline__ void store8(const float (&acc)[16], int col, const void *bias, int act, void *out, bool out_bf16, bool exchange = false) {
   float v[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) v[e] = acc[e];
@@ -226,7 +261,8 @@ __device__ __forceinline__ void store8(const float (&acc)[16], int col, const vo
       __nv_bfloat162 pk = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
       o[e] = *(uint32_t *)&pk;
     }
-    *(uint4 *)((__nv_bfloat16 *)out + col) = make_uint4(o[0], o[1], o[2], o[3]);
+    if (exchange) exch_store4((__nv_bfloat16 *)out + col, o[0], o[1], o[2], o[3]);
+    else *(uint4 *)((__nv_bfloat16 *)out + col) = make_uint4(o[0], o[1], o[2], o[3]);
   } else {
     float4 *dst = (float4 *)((float *)out + col);
     dst[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -249,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
   p2.W = (const __nv_bfloat16 *)a.W2, p2.ldw = a.ldw2, p2.s = a.gr, p2.group_w = a.gs, p2.inv_group_w = a.inv_gs, p2.n_cols = a.D;
   p2.pc = a.pc2, p2.ks = a.ks2;
   const __nv_bfloat16 *X = (const __nv_bfloat16 *)a.X;
-  __nv_bfloat16 *H = (__nv_bfloat16 *)a.H;
+  __nv_bfloat16 *H = nullptr;   // hidden rows in the exchange buffer
   const int warp = threadIdx.x >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) s_abort = 0;
@@ -265,9 +301,17 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
     load_chunk<GATED>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
+  __syncthreads();   // s_abort is set
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 3);
   const int type = read_type(a);   // (in flight while phase 1 runs on the early value)
+  const Wait wait = {clock64(), a.wait_limit, &s_abort, a.status};
+  ExchTurn turn = {0u, 0};
+  if (FFN) {
+    turn = exch_turn(a.exch);
+    H = (__nv_bfloat16 *)(a.exch + kExchHeader + turn.parity * (unsigned)a.exch_bytes);
+  }
+  const bool keep = FFN && a.test_withhold && blockIdx.x == 0;
 
   // ---- phase 1 on the type read early, again if the type has changed since.  Gated: h = silu(x * W_gate) .*
   // (x * W_up); FFN: h = act(x * W_up + b_up); projection: y = act(x * W + b) ----
@@ -275,7 +319,8 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
     const int t = pass == 0 ? t_early : type;
     if (pass == 1 && type == t_early) break;
     if (t < 0) continue;
-    run_phase<GATED, false>(p1, t, X, w, pass == 0, a.units1, partial, [&](int col, const float (&acc)[16]) {
+    run_phase<GATED, false>(p1, t, X, w, pass == 0, a.units1, partial, wait, [&](int col, const float (&acc)[16]) {
+      if (t != type || keep) return;   // (hidden values are taken as soon as they are there: only the right ones are stored)
       if (GATED) {
         uint32_t o[4];
 #pragma unroll
@@ -284,9 +329,9 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
           __nv_bfloat162 pk = __floats2bfloat162_rn(g0 / (1.f + __expf(-g0)) * acc[8 + 2 * e], g1 / (1.f + __expf(-g1)) * acc[8 + 2 * e + 1]);
           o[e] = *(uint32_t *)&pk;
         }
-        *(uint4 *)(H + col) = make_uint4(o[0], o[1], o[2], o[3]);
+        exch_store4(H + col, o[0], o[1], o[2], o[3]);
       } else if (FFN) {
-        store8(acc, col, a.b1, a.act, H, true);
+        store8(acc, col, a.b1, a.act, H, true, true);
       } else {
         store8(acc, col, a.b1, a.act, a.Y, a.y_bf16 != 0);
       }
@@ -304,7 +349,7 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
     return;
   }
 
-  // ---- the first W_down loads go out before the wait between the phases ----
+  // ---- the first W_down loads go out before the hidden values are waited for ----
   {
     const int unit = unit_of(0, p2.ks);
     Lane l = lane_of(p2, unit);
@@ -312,50 +357,23 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
     load_chunk<false>(w, p2, l, max(type, 0), 0);
   }
 
-  // ---- all of h is written before any of it is read: arrive, then wait (bounded) for the other CTAs ----
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ALG_TRACE(0, 8);
-    __threadfence();
-    atomicAdd(a.counters, 1u);
-    const long long t0 = clock64();
-    bool ok = false;
-    while (!ok) {
-      unsigned int seen;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters) : "memory");
-      ok = seen >= gridDim.x + (unsigned int)a.extra_arrivals;
-      if (!ok && clock64() - t0 > a.wait_limit) break;
-    }
-    if (!ok) {
-      s_abort = 1;
-      atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
-    }
-    __threadfence();
-    ALG_TRACE(0, 9);
-  }
-  __syncthreads();
+  exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, 1);
+  if (threadIdx.x == 0) ALG_TRACE(0, 9);
 
   // ---- phase 2: y = h * W_down (+ b_down) ----
-  if (!s_abort) {
-    if (type >= 0) {
-      run_phase<false, true>(p2, type, H, w, true, a.units2, partial,
-                             [&](int col, const float (&acc)[16]) { store8(acc, col, a.b2, ALG_ACT_NONE, a.Y, a.y_bf16 != 0); });
-    } else {   // a row type outside [0, q): the row of Y is zero
-      for (int c = blockIdx.x * kThreads + threadIdx.x; c < a.D; c += gridDim.x * kThreads) {
-        if (a.y_bf16) ((__nv_bfloat16 *)a.Y)[c] = __float2bfloat16_rn(0.f);
-        else ((float *)a.Y)[c] = 0.f;
-      }
+  if (type >= 0) {
+    run_phase<false, true>(p2, type, H, w, true, a.units2, partial, wait,
+                           [&](int col, const float (&acc)[16]) { store8(acc, col, a.b2, ALG_ACT_NONE, a.Y, a.y_bf16 != 0); });
+  } else {   // a row type outside [0, q): the row of Y is zero
+    for (int c = blockIdx.x * kThreads + threadIdx.x; c < a.D; c += gridDim.x * kThreads) {
+      if (a.y_bf16) ((__nv_bfloat16 *)a.Y)[c] = __float2bfloat16_rn(0.f);
+      else ((float *)a.Y)[c] = 0.f;
     }
   }
-  // the last CTA past the wait clears the counters for the next launch
+  __syncthreads();
   if (threadIdx.x == 0) {
     ALG_TRACE(0, 12);
-    const unsigned int left = atomicAdd(a.counters + 1, 1u);
-    if (left == gridDim.x - 1) {
-      a.counters[0] = 0;
-      a.counters[1] = 0;
-      __threadfence();
-    }
+    exch_leave(a.exch);
   }
 }
 
@@ -381,9 +399,9 @@ __device__ __forceinline__ void group_barrier(int id, int threads) {
 
 // A row whose type lies outside [0, q) reads nothing; with LAST (the phase that writes Y) its pieces are stored as zeros
 // and the status word says so.
-template <bool GATED, bool FROM_L2, bool LAST, typename Emit>
+template <bool GATED, bool HIDDEN, bool LAST, typename Emit>
 __device__ __forceinline__ void run_rows_phase(const RowDecodeArgs &a, const Phase &p, const __nv_bfloat16 *x, int64_t ldx,
-                                          uint4 (&w)[kLoads], bool have_first, int t_first, int n_units, float *partial, Emit emit) {
+                                          uint4 (&w)[kLoads], bool have_first, int t_first, int n_units, float *partial, const Wait &wait, Emit emit) {
   constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total_warps = gridDim.x * kWarps, po = p.pc >> 3;
@@ -406,7 +424,7 @@ __device__ __forceinline__ void run_rows_phase(const RowDecodeArgs &a, const Pha
       const int rows_per_lane = (p.s + p.ks * l.rl - 1) >> (__ffs(p.ks * l.rl) - 1);
       for (int c0 = 0; c0 < rows_per_lane; c0 += RC) {
         if (!(have_first && rd == 0 && attempt == 0 && c0 == 0)) load_chunk<GATED>(w, p, l, max(type, 0), c0);
-        fma_chunk<GATED, FROM_L2>(w, p, l, max(type, 0), c0, xm, acc);
+        fma_chunk<GATED, HIDDEN>(w, p, l, max(type, 0), c0, xm, acc, wait);
       }
       // sum over the lanes that share the columns
 #pragma unroll
@@ -462,7 +480,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
   p2.W = (const __nv_bfloat16 *)a.W2, p2.ldw = a.ldw2, p2.s = a.gr, p2.group_w = a.gs, p2.inv_group_w = a.inv_gs, p2.n_cols = a.D;
   p2.pc = a.pc2, p2.ks = a.ks2;
   const __nv_bfloat16 *X = (const __nv_bfloat16 *)a.X;
-  __nv_bfloat16 *H = (__nv_bfloat16 *)a.H;
+  __nv_bfloat16 *H = nullptr;   // hidden rows in the exchange buffer
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (threadIdx.x == 0) s_abort = 0;
 
@@ -478,13 +496,22 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
     load_chunk<GATED>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
+  __syncthreads();   // s_abort is set
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 3);
+  const Wait wait = {clock64(), a.wait_limit, &s_abort, a.status};
+  ExchTurn turn = {0u, 0};
+  if (FFN) {
+    turn = exch_turn(a.exch);
+    H = (__nv_bfloat16 *)(a.exch + kExchHeader + turn.parity * (unsigned)a.exch_bytes);
+  }
+  const bool keep = FFN && a.test_withhold && blockIdx.x == 0;
 
   // ---- phase 1 (its first unit on the type read early).  Gated: h = silu(x * W_gate) .* (x * W_up); FFN:
   // h = act(x * W_up + b_up); projection: y = act(x * W + b) ----
   {
-    run_rows_phase<GATED, false, !FFN>(a, p1, X, a.ldx, w, true, t_early, a.units1, partial, [&](int m, int col, const float (&acc)[16]) {
+    run_rows_phase<GATED, false, !FFN>(a, p1, X, a.ldx, w, true, t_early, a.units1, partial, wait, [&](int m, int col, const float (&acc)[16]) {
+      if (keep) return;
       if (GATED) {
         uint32_t o[4];
 #pragma unroll
@@ -493,9 +520,9 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
           __nv_bfloat162 pk = __floats2bfloat162_rn(g0 / (1.f + __expf(-g0)) * acc[8 + 2 * e], g1 / (1.f + __expf(-g1)) * acc[8 + 2 * e + 1]);
           o[e] = *(uint32_t *)&pk;
         }
-        *(uint4 *)(H + (int64_t)m * a.F + col) = make_uint4(o[0], o[1], o[2], o[3]);
+        exch_store4(H + (int64_t)m * a.F + col, o[0], o[1], o[2], o[3]);
       } else if (FFN) {
-        store8(acc, col, a.b1, a.act, H + (int64_t)m * a.F, true);
+        store8(acc, col, a.b1, a.act, H + (int64_t)m * a.F, true, true);
       } else {
         store8(acc, col, a.b1, a.act, a.y_bf16 ? (void *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy) : (void *)((float *)a.Y + (int64_t)m * a.ldy),
                a.y_bf16 != 0);
@@ -505,7 +532,7 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
   if (threadIdx.x == 0) ALG_TRACE(0, 6);
 
   if (FFN) {
-    // ---- the first W_down loads go out before the wait between the phases ----
+    // ---- the first W_down loads go out before the hidden values are waited for ----
     const int per_row2 = a.M == 1 ? a.units2 : a.units2 / a.M;
     const int unit2 = unit_of(0, p2.ks), m2 = a.M == 1 ? 0 : min(unit2 / per_row2, a.M - 1);
     const int type2 = read_row_type(a, m2);
@@ -515,48 +542,20 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
       load_chunk<false>(w, p2, l, max(type2, 0), 0);
     }
 
-    // ---- all of h is written before any of it is read: arrive, then wait (bounded) for the other CTAs ----
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      ALG_TRACE(0, 8);
-      __threadfence();
-      atomicAdd(a.counters, 1u);
-      const long long t0 = clock64();
-      bool ok = false;
-      while (!ok) {
-        unsigned int seen;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(a.counters) : "memory");
-        ok = seen >= gridDim.x + (unsigned int)a.extra_arrivals;
-        if (!ok && clock64() - t0 > a.wait_limit) break;
-      }
-      if (!ok) {
-        s_abort = 1;
-        atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
-      }
-      __threadfence();
-      ALG_TRACE(0, 9);
-    }
-    __syncthreads();
+    exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, a.M);
+    if (threadIdx.x == 0) ALG_TRACE(0, 9);
 
     // ---- phase 2: y = h * W_down (+ b_down) ----
-    if (!s_abort) {
-      run_rows_phase<false, true, true>(a, p2, H, a.F, w, true, type2, a.units2, partial, [&](int m, int col, const float (&acc)[16]) {
-        store8(acc, col, a.b2, ALG_ACT_NONE,
-               a.y_bf16 ? (void *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy) : (void *)((float *)a.Y + (int64_t)m * a.ldy), a.y_bf16 != 0);
-      });
-    }
-    // the last CTA past the wait clears the counters for the next launch
-    if (threadIdx.x == 0) {
-      ALG_TRACE(0, 12);
-      const unsigned int left = atomicAdd(a.counters + 1, 1u);
-      if (left == gridDim.x - 1) {
-        a.counters[0] = 0;
-        a.counters[1] = 0;
-        __threadfence();
-      }
-    }
+    run_rows_phase<false, true, true>(a, p2, H, a.F, w, true, type2, a.units2, partial, wait, [&](int m, int col, const float (&acc)[16]) {
+      store8(acc, col, a.b2, ALG_ACT_NONE,
+             a.y_bf16 ? (void *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy) : (void *)((float *)a.Y + (int64_t)m * a.ldy), a.y_bf16 != 0);
+    });
+    __syncthreads();
+  if (threadIdx.x == 0) {
+    ALG_TRACE(0, 12);
+    exch_leave(a.exch);
   }
-
+  }
 }
 
 // warps per piece: as many (a power of two, at most the warps of a CTA) as the grid has warps for

@@ -470,3 +470,49 @@ def test_few_rows_one_type_out_of_range_and_types_written_just_before():
     good = [0, 1, 3, 5]
     assert np.all(got[[2, 4]] == 0)
     assert np.array_equal(got[good], oracle.proj(wl.X[good], t[good], wl.W_up, wl.d_widths, wl.f_widths))
+
+
+# ---- the hidden rows' exchange inside a one-launch FFN: buffers alternate from launch to launch, a launch clears what its
+# predecessor wrote, whatever the row counts -------------------------------------------------------------------------
+
+@pytest.mark.parametrize("kind,q,dw,fw,rows", [
+    ("plain", 2, 384, 1536, [1, 5, 1, 1, 16, 1]),     # the staged kernel; more than one row does not use the buffers
+    ("plain", 8, 96, 200, [1, 8, 1, 2, 7, 1, 1, 3]),  # the row kernel
+    ("gated", 32, 64, 24, [8, 1, 1, 4, 8, 2, 1]),
+])
+def test_one_launch_ffn_row_counts_in_turn(kind, q, dw, fw, rows):
+    D, F = q * dw, q * fw
+    wl, Wg = synth.gated_ffn("turns", q, max(rows), D, F, synth.uniform_types(77 + q, max(rows), q), variant=20, integer=False)
+    cls = binding.GatedFFN if kind == "gated" else binding.FFN
+    up = np.concatenate([Wg, wl.W_up], axis=1) if kind == "gated" else wl.W_up
+    X, types, Wu, Wd = H.to_dev(wl.X, "bf16"), H.dev_types(wl.types), H.to_dev(up, "bf16"), H.to_dev(wl.W_down, "bf16")
+
+    def handle():
+        f = cls(wl.d_widths, wl.f_widths, dtype="bf16")
+        if q == 8:
+            f.set_option("small_m_kernel", 3)
+        return f
+    shared = handle()
+    ws = torch.empty(shared.workspace_bytes(max(rows)), dtype=torch.uint8, device="cuda")
+    want = {m: handle().forward(X[-m:], types[-m:], Wu, Wd).clone() for m in set(rows)}
+    outs = [torch.empty((m, D), dtype=torch.bfloat16, device="cuda") for m in rows]
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+
+    def sequence():
+        for m, o in zip(rows, outs):
+            shared.forward(X[-m:], types[-m:], Wu, Wd, out=o, workspace=ws, stream=stream)
+    with torch.cuda.stream(stream):
+        sequence()
+    stream.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        sequence()
+    for _ in range(3):
+        for o in outs:
+            o.fill_(3.0)
+        graph.replay()
+        torch.cuda.synchronize()
+        for m, o in zip(rows, outs):
+            assert torch.equal(o, want[m]), f"{m} rows"
+    assert shared.last_status() == 0
