@@ -215,11 +215,11 @@ __device__ __forceinline__ void stage_hidden(const Shared &sh, const Phase &ph, 
 // memory (deterministic), bias and activation applied, rows < M stored.
 // NT = 8-column tiles of the strip.  HIDDEN: the phase reads the hidden state (down); else it writes it (up).  ONE: one
 // row.  Returns false when a wait ran out.
-template <int NT, bool HIDDEN, bool ONE>
+template <int NT, bool HIDDEN, int MP>
 __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, uint32_t &x_parity) {
   constexpr int SETS = NT <= 2 ? 4 : (NT <= 4 ? 2 : 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const bool HALF = ONE || sh.m_pad == 8;
+  constexpr bool HALF = MP <= 8, ONE = MP == 1;
   const int g = lane >> 2, t4 = lane & 3;
   const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8;
   const int a_row = HALF ? (lane & 7) : frag_row;
@@ -334,8 +334,9 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
 }
 // NTU / NTD: 8-column tiles of the up / down strip (compile-time, so that every kernel gets the
 // registers its own shape needs).  ONE: one row, and the hidden row travels through the exchange buffer.
-template <int NTU, int NTD, bool ONE>
+template <int NTU, int NTD, int MP>
 __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecodeArgs a) {
+  constexpr bool ONE = MP == 1;
   // the next launch of the stream may start now: it only requests its own weights before it waits
   // (triggering later -- after the up phase or after the exchange -- was measured no faster)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -473,7 +474,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
     TR(5);
     up.need = ctl->need_up;
     up.out = hidden;
-    if (ok) ok = run_phase_t<NTU, false, ONE>(sh, up, x_parity);
+    if (ok) ok = run_phase_t<NTU, false, MP>(sh, up, x_parity);
     TR(6);
     if (!ONE) {   // publish: every thread's H stores become visible device-wide, then one arrival per CTA
       __threadfence();
@@ -514,7 +515,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
       ok = wait_bar(sh, bar_dn, 0);
       if (ok && missed && !has_up) ok = wait_bar(sh, bar_miss, 0);
       TR(8);
-      if (ok) ok = run_phase_t<NTD, true, ONE>(sh, dn, x_parity);
+      if (ok) ok = run_phase_t<NTD, true, MP>(sh, dn, x_parity);
     }
   }
   if (ONE) {
@@ -547,17 +548,17 @@ int pick_strip(int q, const int *w, int total, int num_sms) {
   return 0;
 }
 // the instantiated strip widths: up to 32 hidden columns and 16 output columns per CTA
-template <int NTD, bool ONE>
+template <int NTD, int MP>
 void (*pick_up(int ntu))(const FfnDecodeArgs) {
-  return ntu == 1   ? ffn_decode_kernel<1, NTD, ONE>
-         : ntu == 2 ? ffn_decode_kernel<2, NTD, ONE>
-         : ntu == 3 ? ffn_decode_kernel<3, NTD, ONE>
-         : ntu == 4 ? ffn_decode_kernel<4, NTD, ONE>
+  return ntu == 1   ? ffn_decode_kernel<1, NTD, MP>
+         : ntu == 2 ? ffn_decode_kernel<2, NTD, MP>
+         : ntu == 3 ? ffn_decode_kernel<3, NTD, MP>
+         : ntu == 4 ? ffn_decode_kernel<4, NTD, MP>
                     : nullptr;
 }
-void (*pick_kernel(int ntu, int ntd, bool one))(const FfnDecodeArgs) {
-  if (ntd == 1) return one ? pick_up<1, true>(ntu) : pick_up<1, false>(ntu);
-  if (ntd == 2) return one ? pick_up<2, true>(ntu) : pick_up<2, false>(ntu);
+void (*pick_kernel(int ntu, int ntd, int M))(const FfnDecodeArgs) {
+  if (ntd == 1) return M == 1 ? pick_up<1, 1>(ntu) : M <= 8 ? pick_up<1, 8>(ntu) : pick_up<1, 16>(ntu);
+  if (ntd == 2) return M == 1 ? pick_up<2, 1>(ntu) : M <= 8 ? pick_up<2, 8>(ntu) : pick_up<2, 16>(ntu);
   return nullptr;
 }
 
@@ -569,7 +570,7 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
   FfnDecodePlan p = {};
   p.su = pick_strip(q, fw, F, num_sms);
   p.sd = pick_strip(q, dw, D, num_sms);
-  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3, false)) return false;
+  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3, 1)) return false;
   p.n_up = F / p.su, p.n_dn = D / p.sd;
   p.wd_bytes = F * p.sd * 2;
   p.wu_bytes = D * p.su * 2;
@@ -583,7 +584,7 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
 }
 
 cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p, cudaStream_t st) {
-  void (*kernel)(const FfnDecodeArgs) = pick_kernel(p.su >> 3, p.sd >> 3, args.M == 1);
+  void (*kernel)(const FfnDecodeArgs) = pick_kernel(p.su >> 3, p.sd >> 3, args.M);
   if (!kernel) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   if (e != cudaSuccess) return e;
