@@ -1380,7 +1380,7 @@ static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, c
   f->rd_ok = dtype == ALG_BF16 && schedule != ALG_SCHED_INTERVAL && f->up.big.eligible && f->down.big.eligible &&
              row_decode_fits(q, f->D, f->F);
   if (f->fd_ok || f->rd_ok) {   // (the two one-launch decode steps share the exchange)
-    f->exch_bytes = (int)align_up((size_t)(f->rd_ok ? kRowDecodeMaxM : 1) * f->F * 2, 256);
+    f->exch_bytes = (int)align_up((size_t)(f->fd_ok ? kFfnDecodeMaxM : kRowDecodeMaxM) * f->F * 2, 256);
     s = reset_exchange(*f);
     if (s != ALG_OK) {
       if (f->d_exch) cudaFree(f->d_exch);
@@ -1458,11 +1458,9 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
     d.W_up = W_up, d.W_down = W_down;
     d.b_up = b_up, d.b_down = b_down;
     d.act = (int)act;
-    d.H = ws + L.h;
     d.Y = Y;
     d.y_bf16 = y_dtype == ALG_BF16;
     d.D = h->D, d.F = h->F, d.q = u.q;
-    d.counters = (unsigned int *)(h->d_exch + kExchCounters);
     d.exch = h->d_exch, d.exch_bytes = h->exch_bytes;
     d.status = u.d_status;
     d.wait_limit = u.wait_limit;

@@ -291,6 +291,7 @@ constexpr int kFfnDecodeMaxM = 16;
 struct FfnDecodePlan {
   int su, sd;          // columns of the hidden state / of the output one CTA owns (multiples of 8)
   int n_up, n_dn;      // CTAs with an up strip / a down strip
+  int box_up, box_dn;  // weight rows per tiled copy (divide every d / f width, <= 256)
   int wd_bytes, wu_bytes, stage_bytes, p_bytes, ctl_bytes;  // shared-memory regions
 };
 struct FfnDecodeArgs {
@@ -300,16 +301,14 @@ struct FfnDecodeArgs {
   const void *W_up, *W_down;   // canonical banks, packed: [D][F] and [F][D]
   const void *b_up, *b_down;
   int act;
-  void *H;                // [M][F] bf16 scratch in global memory (more than one row)
   void *Y;                // [M][D]
   int y_bf16;
   int D, F, q;
-  int su, sd, n_up, n_dn;
+  int su, sd, n_up, n_dn, box_up, box_dn;
   int off_wu, off_stage, off_p, off_ctl;   // shared-memory offsets (the W_down slice sits at 0)
   int kc_up, kc_dn, m_pad;                 // K-chunk lengths of the staged activations; staged rows (8 or 16)
-  uint8_t *exch;                           // one row: its hidden row between the phases (exchange.cuh), buffers of exch_bytes
+  uint8_t *exch;                           // hidden rows between the phases (exchange.cuh), buffers of exch_bytes
   int exch_bytes;
-  unsigned int *counters;                  // more rows: [0] producers arrived, [1] consumers past the wait; zero between launches
   int *status;
   long long wait_limit;
   int extra_expect_bytes;

@@ -8,8 +8,10 @@
 // only -- no fence, no arrival counter to add to and poll, no wait for the slowest CTA of the grid.
 // Per layer in a graph of layers: 768 -> 3072 -> 768 at q = 2, one row, 9.2 -> 7.5 us; gated 2048 -> 6144 at q = 32, one
 // row, 9.8 -> 8.3 us, four rows 17.8 -> 16.7 us.
-// (Where many CTAs poll many lines the polls get in the way of the values: with several rows that all CTAs read whole,
-// ffn_decode.cu counts arrivals instead.)
+// Where every CTA reads the whole hidden state (ffn_decode.cu) loading it over and over would get in the way of the
+// values themselves (96 CTAs, 8 rows of 3072: 12.1 us a layer): there one thread of a CTA waits for a hint first, a count
+// of the CTAs whose values are on their way.  The hint is not ordered behind the values, so it costs no fence; it says
+// when to look, the values say what is there.
 //
 // Meanwhile every launch fills the OTHER buffer (the rows its predecessor used) with 0xFFFF for its successor.  All of it
 // happens behind griddepcontrol.wait, so the predecessor is done with that buffer, and the successor starts reading only
@@ -18,18 +20,19 @@
 // grid.  A launch that gave up leaves behind the same state as any other.
 #pragma once
 
+#include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace algproj {
 
 constexpr int kExchHeader = 256;         // ExchHead, then the two buffers
-constexpr int kExchCounters = 128;       // in the header: two counters for kernels that count arrivals instead
 constexpr unsigned kExchTurn = 1u << 20;
 
 struct ExchHead {
   unsigned long long turns;   // turn << 20
   int rows[2];                // rows the last launch that used a buffer wrote there
+  unsigned hints[2];          // CTAs of the turn whose values are on their way
 };
 
 struct ExchTurn {
@@ -54,7 +57,16 @@ __device__ __forceinline__ void exch_clear(uint8_t *exch, int exch_bytes, const 
   uint8_t *buf = exch + kExchHeader + (turn.parity ^ 1u) * (unsigned)exch_bytes;
   for (int e = (blockIdx.x + threadIdx.x * gridDim.x) * 16; e < bytes; e += gridDim.x * blockDim.x * 16)
     *(uint4 *)(buf + e) = make_uint4(~0u, ~0u, ~0u, ~0u);
-  if (blockIdx.x == 0 && threadIdx.x == 0) ((ExchHead *)exch)->rows[turn.parity] = rows;
+  if (blockIdx.x == 0 && threadIdx.x == 0) ((ExchHead *)exch)->rows[turn.parity] = rows, ((ExchHead *)exch)->hints[turn.parity ^ 1u] = 0u;
+}
+// "My values are on their way": not ordered behind them, so that it costs no fence, and no proof that they are there.
+__device__ __forceinline__ void exch_hint(uint8_t *exch, const ExchTurn &turn) {
+  asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(&((ExchHead *)exch)->hints[turn.parity]) : "memory");
+}
+__device__ __forceinline__ bool exch_hinted(const uint8_t *exch, const ExchTurn &turn, int ctas) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&((const ExchHead *)exch)->hints[turn.parity]) : "memory");
+  return v >= (unsigned)ctas;
 }
 // Two bf16 values on their way into the buffer.
 __device__ __forceinline__ uint32_t exch_value(uint32_t v) {
@@ -80,6 +92,18 @@ __device__ __forceinline__ unsigned short exch_load(const void *src) {
   asm volatile("ld.relaxed.gpu.global.u16 %0, [%1];" : "=h"(v) : "l"(src) : "memory");
   return v;
 }
+// Single values, and pairs of them.
+__device__ __forceinline__ void exch_store1(void *dst, float z) {
+  unsigned short v = __bfloat16_as_ushort(__float2bfloat16_rn(z));
+  if (v == 0xFFFFu) v = 0x7FFFu;
+  asm volatile("st.relaxed.gpu.global.u16 [%0], %1;" ::"l"(dst), "h"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t exch_load2(const void *src) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(src) : "memory");
+  return v;
+}
+__device__ __forceinline__ bool exch_ready2(uint32_t v) { return (v & 0xFFFFu) != 0xFFFFu && v < 0xFFFF0000u; }
 // (a producer stores whole 32-bit words, so a word is there or not)
 __device__ __forceinline__ bool exch_ready(const uint4 &v) { return v.x != ~0u && v.y != ~0u && v.z != ~0u && v.w != ~0u; }
 

@@ -12,25 +12,20 @@
 // Decomposition.  No reduction across CTAs anywhere: CTA c owns `su` columns of the hidden state
 // (all D input rows of W_up for them) and `sd` columns of the output (all F rows of W_down).
 //   before the wait : row types read speculatively -> input groups some row needs (blocks W_kj that
-//                     no present row type uses are never fetched) -> both slices requested with
-//                     16-byte asynchronous copies (a slice is only 16-48 bytes wide per weight row;
-//                     tiled TMA boxes that narrow were measured no faster), each asking L2 for the
-//                     whole 128-byte line the neighbouring CTAs need too.
+//                     no present row type uses are never fetched) -> both slices requested by one
+//                     thread with tiled copies (request_slice).
 //   after the wait  : X staged in shared memory (all groups, unmasked) while the row types are read
 //                     again; if they differ, the blocks that are missing are requested now.
 //   up phase        : 8 warps split the K steps; mma.sync m16n8k16 (bf16 x bf16 -> fp32); the rule
 //                     "row b uses block k only if k in B(t_b, j)" is applied by clearing the A
 //                     fragment rows that do not use the block; the 8 partial tiles are summed in a
-//                     fixed order through shared memory; bias, activation, bf16 -> H in global memory.
-//   exchange        : one row: H goes through the handle's exchange buffer, whose consumers load again what
-//                     is not there yet (exchange.cuh).  Several rows: producers publish with fence + one
-//                     atomic add on a counter; consumers poll it (bounded), the last consumer clears the
-//                     counters for the next launch (96 CTAs polling 8 rows: 12.1 us a layer against 9.6).
-//                     One row has a kernel of its own: the branch alone cost 0.6 us a layer of both, the
-//                     step is that sensitive to the code it has to fetch.
+//                     fixed order through shared memory; bias, activation, bf16 -> H.
+//   exchange        : H goes through the handle's exchange buffer: no fence, no barrier over the grid
+//                     (exchange.cuh).
 //   down phase      : H staged from L2 over the shared memory the W_up slice no longer needs; same
 //                     MMA / reduction; bias; Y stored.
-// Every wait (mbarriers the copies arrive on, a counter or the values of H) is bounded by the handle's wait limit; on expiry the CTA
+// Up to kRowsMax rows take a kernel on plain FMAs of the same decomposition (ffn_rows.cuh).
+// Every wait (mbarriers the copies arrive on, values of H) is bounded by the handle's wait limit; on expiry the CTA
 // raises ALG_ERR_DEVICE_TIMEOUT, skips its arithmetic, gives copies in flight time to land and
 // returns.
 #include <algorithm>
@@ -49,7 +44,6 @@ namespace {
 constexpr int kThreads = 256, kWarps = 8;
 constexpr int kSmemBudget = 112 * 1024;   // two CTAs (this launch and the next layer's) per SM
 
-constexpr int kLoaders = 64;    // threads per weight slice: warps 0-1 fetch W_up, warps 2-3 fetch W_down
 constexpr int kStagers = 128;   // warps 4-7 stage the activations
 
 struct Ctl {
@@ -60,14 +54,10 @@ struct Ctl {
   uint32_t rows_up[kMaxQ], rows_dn[kMaxQ];  // bit m: row m uses input group k
   uint32_t bad_rows;
   volatile int abort_flag;
-  volatile int go;
 };
 
 __device__ __forceinline__ void cp_async_16_zfill(uint32_t dst, const void *src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_16_l2line(uint32_t dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 // arrives on the barrier once every copy this thread has issued so far has landed
 __device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
@@ -89,11 +79,6 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
 __device__ __forceinline__ float act_f(float z, int act) {
   if (act == ALG_ACT_GELU_ERF) return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f));
   if (act == ALG_ACT_GELU_TANH) {
@@ -105,6 +90,21 @@ __device__ __forceinline__ float act_f(float z, int act) {
 // staged activations: [m_pad][kc] bf16, 16-byte pieces XOR-swizzled by the row (conflict-free ldmatrix)
 __device__ __forceinline__ uint32_t x_off(int m, int chunk, int pitch_bytes) {
   return (uint32_t)(m * pitch_bytes + ((chunk ^ (m & 7)) << 4));
+}
+
+// One thread requests the rows of the input groups in `mask` of a weight slice (tiled copies; `so` = group offsets) and
+// tells the barrier how many bytes will come.  (16-byte asynchronous copies by 128 threads cost the SM's load path
+// about 5 k cycles per layer -- a slice is 16 to 64 bytes wide, a warp's copies touch 32 lines -- beside the CTA of
+// the running layer: one row of 768 -> 3072 -> 768 at q = 2 took 7.0 us a layer with them and 5.7 with tiled copies.)
+__device__ __forceinline__ void request_slice(const CUtensorMap *map, uint32_t bar, uint32_t dst, const int *so, uint32_t mask, int q,
+                                              int col0, int pitch, int box, int extra) {
+  uint32_t bytes = (uint32_t)extra;   // (test aid: bytes that never come)
+  for (int k = 0; k < q; ++k)
+    if ((mask >> k) & 1u) bytes += (uint32_t)((so[k + 1] - so[k]) * pitch);
+  mbar_expect_tx(bar, bytes);
+  for (int k = 0; k < q; ++k)
+    if ((mask >> k) & 1u)
+      for (int r = so[k]; r < so[k + 1]; r += box) tma_load_2d(dst + (uint32_t)(r * pitch), map, bar, col0, r);
 }
 
 // Warp 0: from the types of the M rows (lane m holds the type of row m, -1 = out of range) to the
@@ -181,15 +181,24 @@ __device__ __forceinline__ void stage_chunk(const Shared &sh, const Phase &ph, i
   cp_async_arrive(sh.bar_x);
 }
 
-// One row, all threads: one K chunk of the hidden row, out of the exchange buffer as its values arrive.  (The other
-// staged rows keep whatever is there: the row rule clears their A fragments.)
+// All threads: rows < M of one K chunk of the hidden state out of the exchange buffer, copied like any activation; what
+// a copy found missing (exchange.cuh) is loaded again.  (The other staged rows keep whatever is there: the row rule
+// clears their A fragments.)
+template <int MP>
 __device__ __forceinline__ void stage_hidden(const Shared &sh, const Phase &ph, int kc0, int len) {
-  const int pieces = len >> 3;
+  constexpr int TPR = kThreads / MP;   // threads that walk along a row
+  const int cpr = len >> 3, m = threadIdx.x / TPR, ch0 = threadIdx.x % TPR;
+  if (m >= sh.M) return;
+  const __nv_bfloat16 *row = ph.src + (int64_t)m * ph.ld + kc0;
+  for (int ch = ch0; ch < cpr; ch += TPR) cp_async_16_zfill(ph.stage_base + x_off(m, ch, ph.pitch_bytes), row + ch * 8, true);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   const long long t0 = clock64();
   uint32_t spins = 0;
-  for (int p = threadIdx.x; p < pieces; p += kThreads) {
-    const __nv_bfloat16 *src = ph.src + kc0 + p * 8;
-    uint4 v = exch_load4(src);
+  for (int ch = ch0; ch < cpr; ch += TPR) {
+    const uint32_t dst = ph.stage_base + x_off(m, ch, ph.pitch_bytes);
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(dst) : "memory");
+    if (exch_ready(v)) continue;
     while (!exch_ready(v)) {
       if ((++spins & 63u) == 0) {
         if (sh.ctl->abort_flag) return;
@@ -199,9 +208,9 @@ __device__ __forceinline__ void stage_hidden(const Shared &sh, const Phase &ph, 
           return;
         }
       }
-      v = exch_load4(src);
+      v = exch_load4(row + ch * 8);
     }
-    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(ph.stage_base + (uint32_t)(p << 4)), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
   }
 }
 
@@ -213,13 +222,13 @@ __device__ __forceinline__ void stage_hidden(const Shared &sh, const Phase &ph, 
 // "row b uses block k only if k in B(t_b, j)" is applied by clearing the rows of the A fragment that
 // do not use the block.  The 8 warps' partial tiles are then summed in warp order through shared
 // memory (deterministic), bias and activation applied, rows < M stored.
-// NT = 8-column tiles of the strip.  HIDDEN: the phase reads the hidden state (down); else it writes it (up).  ONE: one
-// row.  Returns false when a wait ran out.
+// NT = 8-column tiles of the strip, MP = staged rows (8 or 16).  HIDDEN: the phase reads the hidden state (down); else
+// it writes it (up).  Returns false when a wait ran out.
 template <int NT, bool HIDDEN, int MP>
 __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, uint32_t &x_parity) {
   constexpr int SETS = NT <= 2 ? 4 : (NT <= 4 ? 2 : 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr bool HALF = MP <= 8, ONE = MP == 1;
+  constexpr bool HALF = MP == 8;
   const int g = lane >> 2, t4 = lane & 3;
   const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8;
   const int a_row = HALF ? (lane & 7) : frag_row;
@@ -236,9 +245,9 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
   bool ok = true;
   for (int kc0 = 0; kc0 < ph.K && ok; kc0 += ph.kc) {
     const int len = min(ph.kc, ph.K - kc0);
-    if (HIDDEN && ONE) {
+    if (HIDDEN) {
       if (kc0) __syncthreads();   // the previous chunk has been consumed
-      stage_hidden(sh, ph, kc0, len);
+      stage_hidden<MP>(sh, ph, kc0, len);
       __syncthreads();
       ok = !sh.ctl->abort_flag;
     } else {
@@ -320,7 +329,7 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
     }
     z0 = act_f(z0, ph.act), z1 = act_f(z1, ph.act);
     if ((sh.ctl->bad_rows >> m) & 1u) z0 = z1 = 0.f;   // out-of-range type: the row's output is defined to be zero
-    if (!HIDDEN && ONE) {
+    if (!HIDDEN) {
       __nv_bfloat162 v = __floats2bfloat162_rn(z0, z1);
       exch_store((__nv_bfloat16 *)ph.out + (int64_t)m * ph.out_ld + col, *(uint32_t *)&v);
     } else if (ph.out_bf16) {
@@ -335,8 +344,7 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
 // NTU / NTD: 8-column tiles of the up / down strip (compile-time, so that every kernel gets the
 // registers its own shape needs).  ONE: one row, and the hidden row travels through the exchange buffer.
 template <int NTU, int NTD, int MP>
-__global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecodeArgs a) {
-  constexpr bool ONE = MP == 1;
+__global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const __grid_constant__ CUtensorMap tm_up, const __grid_constant__ CUtensorMap tm_dn, const FfnDecodeArgs a) {
   // the next launch of the stream may start now: it only requests its own weights before it waits
   // (triggering later -- after the up phase or after the exchange -- was measured no faster)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -347,7 +355,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   uint8_t *st_sm = smem + a.off_stage;          // X stage; the H stage starts at wu_sm and runs through here
   Ctl *ctl = (Ctl *)(smem + a.off_ctl);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int c = blockIdx.x, q = a.q, M = ONE ? 1 : a.M;
+  const int c = blockIdx.x, q = a.q, M = a.M;
   const bool has_up = c < a.n_up, has_dn = c < a.n_dn;
   const int col_u = c * a.su, col_d = c * a.sd;
   const int D = a.D, F = a.F;
@@ -364,12 +372,11 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   const uint32_t bar_up = smem_u32(&ctl->bar_up), bar_dn = smem_u32(&ctl->bar_dn);
   const uint32_t bar_miss = smem_u32(&ctl->bar_miss), bar_x = smem_u32(&ctl->bar_x);
   if (tid == 0) {
-    mbar_init(bar_up, kLoaders);        // every loader thread arrives once its copies have landed
-    mbar_init(bar_dn, kLoaders);
-    mbar_init(bar_miss, 2 * kLoaders);
+    mbar_init(bar_up, 1);
+    mbar_init(bar_dn, 1);
+    mbar_init(bar_miss, 2);   // both slices
     mbar_init(bar_x, kStagers);
     ctl->abort_flag = 0;
-    ctl->go = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   int spec_type = -1;
@@ -392,42 +399,17 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   __syncthreads();
   const uint32_t spec_up = ctl->need_up, spec_dn = ctl->need_dn;
 
-  // Requests the rows of the input groups in `mask` of one weight slice: `cols` columns starting at
-  // col0, 16 bytes per copy, neighbouring lanes on neighbouring pieces of a row.  t = index of the
-  // thread among the `kLoaders` threads of this slice.
-  auto request_slice = [&](const __nv_bfloat16 *W, int ld, uint32_t dst, const int *so, uint32_t mask, int col0, int cols,
-                           int t) {
-    const int ppr = cols >> 3;   // 16-byte pieces per row
-    // piece e of a group = (row e / ppr, piece e % ppr); a thread steps by kLoaders pieces at a time,
-    // i.e. by (kLoaders / ppr) rows and (kLoaders % ppr) pieces: no division inside the loops
-    const int dr = kLoaders / ppr, dp = kLoaders % ppr;
-    const int tr0 = t / ppr, tp0 = t % ppr;
-    for (int k = 0; k < q; ++k) {
-      if (!((mask >> k) & 1u)) continue;
-      const int r0 = so[k], rows = so[k + 1] - r0;
-      int r = tr0, pc = tp0;
-      while (r < rows) {
-        cp_async_16_l2line(dst + (uint32_t)(((r0 + r) * ppr + pc) << 4), W + (int64_t)(r0 + r) * ld + col0 + pc * 8);
-        r += dr, pc += dp;
-        if (pc >= ppr) pc -= ppr, ++r;
-      }
-    }
-  };
   // ---- both weight slices, requested before anything else is waited for ----
-  if (tid < kLoaders) {
-    if (has_up) request_slice((const __nv_bfloat16 *)a.W_up, F, smem_u32(wu_sm), ctl->so_d, spec_up, col_u, a.su, tid);
-    if (!(a.extra_expect_bytes && tid == 0)) cp_async_arrive(bar_up);   // test aid: one arrival short, the barrier never completes
-  } else if (tid < 2 * kLoaders) {
-    if (has_dn) request_slice((const __nv_bfloat16 *)a.W_down, D, smem_u32(wd_sm), ctl->so_f, spec_dn, col_d, a.sd, tid - kLoaders);
-    cp_async_arrive(bar_dn);
+  if (tid == 0) {
+    request_slice(&tm_up, bar_up, smem_u32(wu_sm), ctl->so_d, has_up ? spec_up : 0u, q, col_u, a.su * 2, a.box_up, a.extra_expect_bytes);
+    request_slice(&tm_dn, bar_dn, smem_u32(wd_sm), ctl->so_f, has_dn ? spec_dn : 0u, q, col_d, a.sd * 2, a.box_dn, a.extra_expect_bytes);
   }
   TR(2);
   // ---- everything below may depend on the previous kernel of the stream ----
   asm volatile("griddepcontrol.wait;" ::: "memory");
   TR(3);
 
-  ExchTurn turn = {0u, 0};
-  if (ONE) turn = exch_turn(a.exch);   // (on its way while the activations are staged)
+  const ExchTurn turn = exch_turn(a.exch);   // (on its way while the activations are staged)
   Shared sh;
   sh.ctl = ctl, sh.p_sm = (float *)(smem + a.off_p), sh.bar_x = bar_x;
   sh.M = M, sh.m_pad = a.m_pad, sh.q = q, sh.wait_limit = a.wait_limit, sh.status = a.status;
@@ -454,18 +436,13 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   }
   __syncthreads();   // final masks visible
   const bool missed = (ctl->miss_up | ctl->miss_dn) != 0u;
-  if (missed) {   // rare: blocks the final types need and the early request did not cover
-    if (tid < kLoaders) {
-      if (has_up) request_slice((const __nv_bfloat16 *)a.W_up, F, smem_u32(wu_sm), ctl->so_d, ctl->miss_up, col_u, a.su, tid);
-      cp_async_arrive(bar_miss);
-    } else if (tid < 2 * kLoaders) {
-      if (has_dn) request_slice((const __nv_bfloat16 *)a.W_down, D, smem_u32(wd_sm), ctl->so_f, ctl->miss_dn, col_d, a.sd, tid - kLoaders);
-      cp_async_arrive(bar_miss);
-    }
+  if (missed && tid == 0) {   // rare: blocks the final types need and the early request did not cover
+    request_slice(&tm_up, bar_miss, smem_u32(wu_sm), ctl->so_d, has_up ? ctl->miss_up : 0u, q, col_u, a.su * 2, a.box_up, 0);
+    request_slice(&tm_dn, bar_miss, smem_u32(wd_sm), ctl->so_f, has_dn ? ctl->miss_dn : 0u, q, col_d, a.sd * 2, a.box_dn, 0);
   }
   TR(4);
   bool ok = true;
-  void *const hidden = ONE ? (void *)(a.exch + kExchHeader + turn.parity * (unsigned)a.exch_bytes) : a.H;
+  void *const hidden = a.exch + kExchHeader + turn.parity * (unsigned)a.exch_bytes;
 
   // ---------------- up phase: H[:, strip] = act(X *_q W_up + b_up) ----------------
   if (has_up) {
@@ -476,33 +453,24 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
     up.out = hidden;
     if (ok) ok = run_phase_t<NTU, false, MP>(sh, up, x_parity);
     TR(6);
-    if (!ONE) {   // publish: every thread's H stores become visible device-wide, then one arrival per CTA
-      __threadfence();
-      __syncthreads();
-      if (tid == 0 && ok) atomicAdd(a.counters, 1u);
-    }
+    if (tid == 0 && ok) exch_hint(a.exch, turn);
+  } else {
+    __syncthreads();   // every thread has asked for the turn
   }
-  if (ONE) exch_clear(a.exch, a.exch_bytes, turn, F * 2, 1);
+  if (tid == 96) exch_leave(a.exch);   // (not the thread that waits for the hints)
+  exch_clear(a.exch, a.exch_bytes, turn, F * 2, M);
   if (has_dn) {
-    if (!ONE) {
-      // ---------------- exchange: all of H must be there ----------------
-      if (tid == 0) {
-        const long long t0 = clock64();
-        int go = ctl->abort_flag ? 0 : 1;
-        while (go && ld_acquire_u32(a.counters) < (unsigned)a.n_up) {
-          if (clock64() - t0 > a.wait_limit) {
-            atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
-            ctl->abort_flag = 1;
-            go = 0;
-          }
+    // ---------------- exchange: most of H is on its way ----------------
+    if (tid == 0) {
+      const long long t0 = clock64();
+      while (!ctl->abort_flag && !exch_hinted(a.exch, turn, a.n_up - (a.n_up >> 2)))
+        if (clock64() - t0 > a.wait_limit) {
+          atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+          ctl->abort_flag = 1;
         }
-        ctl->go = go;
-      }
-      __syncthreads();   // also: every warp is done with the W_up slice and the partial-sum buffer
-      ok = ctl->go != 0;
-      // the last consumer past the wait clears the counters: the next launch starts from zero
-      if (tid == 0 && ok && atomicAdd(a.counters + 1, 1u) == (unsigned)(a.n_dn - 1)) a.counters[0] = 0u, a.counters[1] = 0u;
     }
+    __syncthreads();   // also: every warp is done with the W_up slice and the partial-sum buffer
+    ok = !ctl->abort_flag;
     TR(7);
     // ---------------- down phase: Y[:, strip] = H *_q W_down + b_down ----------------
     if (ok) {
@@ -511,16 +479,11 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
       dn.stage_base = smem_u32(wu_sm), dn.w_base = smem_u32(wd_sm), dn.cols = a.sd, dn.col0 = col_d;
       dn.so = ctl->so_f, dn.rows_k = ctl->rows_dn, dn.need = ctl->need_dn, dn.bias = a.b_down, dn.act = ALG_ACT_NONE;
       dn.out = a.Y, dn.out_ld = D, dn.out_bf16 = a.y_bf16;
-      if (!ONE) stage_chunk(sh, dn, 0, min(a.kc_dn, F));   // H travels while the weight barrier is checked
       ok = wait_bar(sh, bar_dn, 0);
       if (ok && missed && !has_up) ok = wait_bar(sh, bar_miss, 0);
       TR(8);
       if (ok) ok = run_phase_t<NTD, true, MP>(sh, dn, x_parity);
     }
-  }
-  if (ONE) {
-    __syncthreads();
-    if (tid == 0) exch_leave(a.exch);
   }
   TR(9);
   if (ctl->abort_flag) {  // copies that are still in flight get time to land before shared memory is released
@@ -530,6 +493,8 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const FfnDecode
   }
 #undef TR
 }
+
+#include "ffn_rows.cuh"
 
 int gcd_i(int x, int y) {
   while (y) {
@@ -548,18 +513,22 @@ int pick_strip(int q, const int *w, int total, int num_sms) {
   return 0;
 }
 // the instantiated strip widths: up to 32 hidden columns and 16 output columns per CTA
-template <int NTD, int MP>
-void (*pick_up(int ntu))(const FfnDecodeArgs) {
-  return ntu == 1   ? ffn_decode_kernel<1, NTD, MP>
-         : ntu == 2 ? ffn_decode_kernel<2, NTD, MP>
-         : ntu == 3 ? ffn_decode_kernel<3, NTD, MP>
-         : ntu == 4 ? ffn_decode_kernel<4, NTD, MP>
+using Kernel = void (*)(const CUtensorMap, const CUtensorMap, const FfnDecodeArgs);
+template <int NTU, int NTD>
+Kernel pick_rows(bool fma, int M) {
+  if (fma) return M == 1 ? ffn_rows_kernel<NTU, NTD, 1> : ffn_rows_kernel<NTU, NTD, 2>;
+  return M <= 8 ? ffn_decode_kernel<NTU, NTD, 8> : ffn_decode_kernel<NTU, NTD, 16>;
+}
+template <int NTD>
+Kernel pick_up(int ntu, bool fma, int M) {
+  return ntu == 1   ? pick_rows<1, NTD>(fma, M)
+         : ntu == 2 ? pick_rows<2, NTD>(fma, M)
+         : ntu == 3 ? pick_rows<3, NTD>(fma, M)
+         : ntu == 4 ? pick_rows<4, NTD>(fma, M)
                     : nullptr;
 }
-void (*pick_kernel(int ntu, int ntd, int M))(const FfnDecodeArgs) {
-  if (ntd == 1) return M == 1 ? pick_up<1, 1>(ntu) : M <= 8 ? pick_up<1, 8>(ntu) : pick_up<1, 16>(ntu);
-  if (ntd == 2) return M == 1 ? pick_up<2, 1>(ntu) : M <= 8 ? pick_up<2, 8>(ntu) : pick_up<2, 16>(ntu);
-  return nullptr;
+Kernel pick_kernel(int ntu, int ntd, bool fma, int M) {
+  return ntd == 1 ? pick_up<1>(ntu, fma, M) : ntd == 2 ? pick_up<2>(ntu, fma, M) : nullptr;
 }
 
 }  // namespace
@@ -570,8 +539,17 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
   FfnDecodePlan p = {};
   p.su = pick_strip(q, fw, F, num_sms);
   p.sd = pick_strip(q, dw, D, num_sms);
-  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3, 1)) return false;
+  if (!p.su || !p.sd || !pick_kernel(p.su >> 3, p.sd >> 3, false, 1)) return false;
   p.n_up = F / p.su, p.n_dn = D / p.sd;
+  auto box = [&](const int *w) {   // widths are multiples of 16
+    int g = 0;
+    for (int k = 0; k < q; ++k) g = gcd_i(g, w[k]);
+    int b = 16;
+    for (int v = 16; v <= 256; v += 16)
+      if (g % v == 0) b = v;
+    return b;
+  };
+  p.box_up = box(dw), p.box_dn = box(fw);
   p.wd_bytes = F * p.sd * 2;
   p.wu_bytes = D * p.su * 2;
   p.p_bytes = kWarps * 16 * (p.su > p.sd ? p.su : p.sd) * 4;   // for 16 staged rows; half of it for 8
@@ -584,35 +562,49 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
 }
 
 cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p, cudaStream_t st) {
-  void (*kernel)(const FfnDecodeArgs) = pick_kernel(p.su >> 3, p.sd >> 3, args.M);
+  FfnDecodeArgs a = args;
+  a.su = p.su, a.sd = p.sd, a.n_up = p.n_up, a.n_dn = p.n_dn, a.box_up = p.box_up, a.box_dn = p.box_dn;
+  // up to kRowsMax rows on plain FMAs (tables in the kernel parameters only)
+  const bool rows = a.M <= kRowsMax && a.small_q && a.D <= 512 * kRowsUp && a.F <= 512 * kRowsDn;
+  const Kernel kernel = pick_kernel(p.su >> 3, p.sd >> 3, rows, a.M);
   if (!kernel) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   if (e != cudaSuccess) return e;
-  FfnDecodeArgs a = args;
-  a.su = p.su, a.sd = p.sd, a.n_up = p.n_up, a.n_dn = p.n_dn;
-  a.m_pad = a.M <= 8 ? 8 : 16;
-  // the partial-sum buffer shrinks with the staged rows; what it gives up goes to the activation stage
-  const int p_bytes = p.p_bytes * a.m_pad / 16;
-  const int stage_bytes = p.stage_bytes + (p.p_bytes - p_bytes);
+  int ctl_bytes = p.ctl_bytes;
   a.off_wu = p.wd_bytes;
-  a.off_stage = a.off_wu + p.wu_bytes;
-  a.off_p = a.off_stage + stage_bytes;
-  a.off_ctl = a.off_p + p_bytes;
-  auto round64 = [](int v) { return (v + 63) & ~63; };
-  a.kc_up = std::min(round64(a.D), (stage_bytes / (a.m_pad * 2)) & ~63);
-  a.kc_dn = std::min(round64(a.F), ((p.wu_bytes + stage_bytes) / (a.m_pad * 2)) & ~63);
-  if (a.kc_up < 64 || a.kc_dn < 64) return cudaErrorInvalidConfiguration;
+  if (rows) {
+        a.off_p = a.off_wu + p.wu_bytes;
+    a.off_ctl = (a.off_p + kWarps * (p.su + p.sd) * a.M * 4 + 127) & ~127;
+    ctl_bytes = (int)sizeof(RowsCtl);
+  } else {
+    a.m_pad = a.M <= 8 ? 8 : 16;
+    // the partial-sum buffer shrinks with the staged rows; what it gives up goes to the activation stage
+    const int p_bytes = p.p_bytes * a.m_pad / 16;
+    const int stage_bytes = p.stage_bytes + (p.p_bytes - p_bytes);
+    a.off_stage = a.off_wu + p.wu_bytes;
+    a.off_p = a.off_stage + stage_bytes;
+    a.off_ctl = a.off_p + p_bytes;
+    auto round64 = [](int v) { return (v + 63) & ~63; };
+    a.kc_up = std::min(round64(a.D), (stage_bytes / (a.m_pad * 2)) & ~63);
+    a.kc_dn = std::min(round64(a.F), ((p.wu_bytes + stage_bytes) / (a.m_pad * 2)) & ~63);
+    if (a.kc_up < 64 || a.kc_dn < 64) return cudaErrorInvalidConfiguration;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(std::max(a.n_up, a.n_dn), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = a.off_ctl + p.ctl_bytes + 128;
+  cfg.dynamicSmemBytes = a.off_ctl + ctl_bytes + (rows ? 512 : 128);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kernel, a);
+  CUtensorMap up, dn;
+  auto swizzle = [&](int strip) { return rows && (strip == 16 || strip == 32) ? strip * 2 : 0; };
+  e = make_map_2d_sw(&up, a.W_up, (uint64_t)a.F, (uint64_t)a.D, (uint64_t)a.F * 2, (uint32_t)a.su, (uint32_t)a.box_up, swizzle(a.su));
+  if (e == cudaSuccess)
+    e = make_map_2d_sw(&dn, a.W_down, (uint64_t)a.D, (uint64_t)a.F, (uint64_t)a.D * 2, (uint32_t)a.sd, (uint32_t)a.box_dn, swizzle(a.sd));
+  if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kernel, up, dn, a);
   count_launch(1);
   return e;
 }
