@@ -42,7 +42,10 @@ ALG_TRACE_DEFINE(ffn_decode)
 namespace {
 
 constexpr int kThreads = 256, kWarps = 8;
-constexpr int kSmemBudget = 112 * 1024;   // two CTAs (this launch and the next layer's) per SM
+// Two CTAs (this launch and the next layer's) per SM where the weight slices leave room for that, else one: the next
+// layer's weights then come after this layer's, still in one launch (1024 -> 4096 -> 1024, q = 2, per layer of a graph:
+// M = 1 19.7 -> 7.8 us, M = 8 16.5 -> 11.5 us against two launches).
+constexpr int kSmemBudget = 112 * 1024, kSmemBudgetOne = 220 * 1024;
 
 constexpr int kStagers = 128;   // warps 4-7 stage the activations
 
@@ -554,8 +557,10 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
   p.wu_bytes = D * p.su * 2;
   p.p_bytes = kWarps * 16 * (p.su > p.sd ? p.su : p.sd) * 4;   // for 16 staged rows; half of it for 8
   p.ctl_bytes = ((int)sizeof(Ctl) + 127) & ~127;
-  p.stage_bytes = kSmemBudget - 128 - p.wd_bytes - p.wu_bytes - p.p_bytes - p.ctl_bytes;
-  p.stage_bytes &= ~127;
+  for (int budget : {kSmemBudget, kSmemBudgetOne}) {
+    p.stage_bytes = (budget - 128 - p.wd_bytes - p.wu_bytes - p.p_bytes - p.ctl_bytes) & ~127;
+    if (p.stage_bytes >= 16 * 64 * 2) break;
+  }
   if (p.stage_bytes < 16 * 64 * 2) return false;   // at least one 64-deep chunk of 16 rows
   *plan = p;
   return true;
@@ -568,7 +573,7 @@ cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p,
   const bool rows = a.M <= kRowsMax && a.small_q && a.D <= 512 * kRowsUp && a.F <= 512 * kRowsDn;
   const Kernel kernel = pick_kernel(p.su >> 3, p.sd >> 3, rows, a.M);
   if (!kernel) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudgetOne);
   if (e != cudaSuccess) return e;
   int ctl_bytes = p.ctl_bytes;
   a.off_wu = p.wd_bytes;

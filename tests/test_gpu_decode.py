@@ -516,3 +516,41 @@ def test_one_launch_ffn_row_counts_in_turn(kind, q, dw, fw, rows):
         for m, o in zip(rows, outs):
             assert torch.equal(o, want[m]), f"{m} rows"
     assert shared.last_status() == 0
+
+
+# ---- one-launch FFN: the strip widths (8 .. 32 hidden columns, 8 or 16 output columns per CTA, each with its own
+# shared-memory layout), one or two rows on plain FMAs and more on the matrix path, slices too large for two CTAs per SM,
+# group widths off the powers of two, row types written by the kernel just before --------------------------------------
+
+@pytest.mark.parametrize("dw,fw", [
+    ([256, 256], [512, 512]),          # 8 hidden columns
+    ([256, 256], [1024, 1024]),        # 16
+    ([384, 384], [1536, 1536]),        # 24
+    ([512, 512], [2048, 2048]),        # 32; one CTA per SM
+    ([1024, 1024], [512, 512]),        # 16 output columns, four row pairs per thread
+    ([208, 48, 128], [304, 80, 128]),  # unequal, short copies
+])
+@pytest.mark.parametrize("M", [1, 2, 3, 8, 9, 16])
+def test_one_launch_ffn_strip_widths_and_rows(dw, fw, M):
+    q = len(dw)
+    wl = synth.make_workload("strips", config=7, variant=90 + M, dtype="bf16", q=q, M=M, D=sum(dw), F=sum(fw),
+                             types=synth.uniform_types(5 + M, M, q), integer=True, d_widths=dw, f_widths=fw)
+    wl.X[:] = np.sign(wl.X)                       # |h| <= 3 * sum(dw): small enough for exact bf16 hidden values
+    wl.W_up[:] = np.where(np.arange(wl.W_up.size).reshape(wl.W_up.shape) % 7 == 0, np.sign(wl.W_up), 0)
+    ffn = binding.FFN(dw, fw, dtype="bf16")
+    X, Wu, Wd = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.to_dev(wl.W_down, "bf16")
+    real = H.dev_types(wl.types)
+    h = oracle.proj(wl.X, wl.types, wl.W_up, dw, fw)
+    assert np.abs(h).max() <= 256                 # exact in bf16
+    ref = oracle.proj(h.astype(np.float32), wl.types, wl.W_down, fw, dw)
+    ffn.forward(X, real, Wu, Wd, act=None)
+    types = torch.full_like(real, int((wl.types[0] + 1) % q))
+    for _ in range(2):
+        torch.cuda.synchronize()
+        types.copy_(real)                          # still running when the call reads the types for the first time
+        before = binding.launch_count()
+        got = ffn.forward(X, types, Wu, Wd, act=None, out_dtype=torch.float32)
+        assert binding.launch_count() - before == 1
+        assert np.array_equal(H.to_np(got), ref)
+        types.fill_(int((wl.types[0] + 1) % q))
+    assert ffn.last_status() == 0
