@@ -7,7 +7,7 @@
 // (Eqs. typed-diag / typed-off): 2 s of the q s weight rows above every output column.  The step is a pair of
 // matrix-vector products bound by memory LATENCY, so it runs on plain FMAs and is organised around the dependent
 // round trips.  A warp owns a piece of 8 or 16 output columns (and, while there are more warps than pieces, a
-// share of the weight rows); its lanes split the rows, every lane keeps up to 32 loads of 16 bytes in flight and
+// share of the weight rows); its lanes split the rows, every lane keeps all its loads of 16 bytes in flight and
 // reads the activations it needs straight from global memory -- no staging, one CTA barrier per phase at most.
 // The first weight loads are issued before the launch's dependency resolves (weights do not depend on the previous
 // kernel), those of W_down before the second phase of an FFN.  Phase 1 of an FFN writes the hidden row h (bf16) to the
@@ -21,6 +21,7 @@
 
 #include "common.cuh"
 #include "exchange.cuh"
+#include "tc_common.cuh"
 #include "trace.cuh"
 
 namespace algproj {
@@ -29,9 +30,16 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
-constexpr int kLoads = 32;   // 16-byte weight loads a lane keeps in flight
-constexpr int kMaxPo = 8;     // a piece has at most 8 x 8 columns
 constexpr int kPieceCols = 16;   // columns of a piece where the group width allows (32 and 64 measured the same or slower)
+
+// 16-byte weight loads a lane keeps in flight: RC rows of two segments, for the gate and the up columns.  RC (2, 4, 8 or,
+// projections only, 16) is what the shape needs: code for more rows is code the one pass has to fetch around, and up to
+// four rows leave registers for two CTAs per SM, so that the next launch's loads go out while this one computes.  Gated
+// 2048 -> 6144 -> 2048 at q = 32, one row, per layer of a graph of layers: 8.3 us with 8 rows for every shape, 6.6 with
+// RC = 2, 6.0 with the sums halved across the lanes and one lane per column at the end.  Shapes that need 8 rows are
+// better off with all of them in flight than with two passes of 4 (4096 -> 12288: 13.2 against 13.8 us).
+template <bool GATED, int RC>
+constexpr int kLoads = RC * (GATED ? 4 : 2);
 
 // One matrix-vector phase as the kernel sees it.
 struct Phase {
@@ -41,18 +49,9 @@ struct Phase {
   int group_w;              // columns of one output group
   float inv_group_w;
   int n_cols;               // output columns (GATED: the up columns sit n_cols further in the bank)
-  int pc;                   // columns of a piece: 8, 16, 32 or 64
+  int pc;                   // columns of a piece: 8 or 16
   int ks;                   // warps that share the rows of a piece: 1, 2, 4 or 8
 };
-
-__device__ __forceinline__ void unpack8(const uint4 &v, float *f) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int e = 0; e < 4; ++e) {
-    f[2 * e] = __uint_as_float(w[e] << 16);
-    f[2 * e + 1] = __uint_as_float(w[e] & 0xFFFF0000u);
-  }
-}
 
 // Where a lane stands in a piece: `sub` = which 8 columns, `lr` = which share of the rows.
 struct Lane {
@@ -87,9 +86,8 @@ __device__ __forceinline__ int unit_of(int rd, int ks) {
 
 // Loads of one chunk: rows r0 .. of both segments (the diagonal block of group j, then -- unless the row's own type is
 // j -- its panel block), for the gate and, GATED, the up columns.  RC rows per segment and chunk.
-template <bool GATED>
-__device__ __forceinline__ void load_chunk(uint4 (&w)[kLoads], const Phase &p, const Lane &l, int type, int c0) {
-  constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
+template <bool GATED, int RC>
+__device__ __forceinline__ void load_chunk(uint4 (&w)[kLoads<GATED, RC>], const Phase &p, const Lane &l, int type, int c0) {
   const int step = p.ks * l.rl, first = l.part * l.rl + l.lr;
   const int nr = ((p.s + step - 1) >> (__ffs(step) - 1)) - c0;   // rows of this chunk some lane has (the same in every lane)
 #pragma unroll
@@ -118,10 +116,9 @@ struct Wait {
 
 // acc[0..8) (gate or plain) and acc[8..16) (up) += x[kk] * w[kk][...] for one chunk.  x is read from global memory
 // (HIDDEN: from the exchange buffer, where it may yet have to arrive).
-template <bool GATED, bool HIDDEN>
-__device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads], const Phase &p, const Lane &l, int type, int c0,
-                                          const __nv_bfloat16 *x, float (&acc)[16], const Wait &wait) {
-  constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
+template <bool GATED, bool HIDDEN, int RC>
+__device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads<GATED, RC>], const Phase &p, const Lane &l, int type, int c0,
+                                          const __nv_bfloat16 *x, uint64_t (&acc)[GATED ? 8 : 4], const Wait &wait) {
   const int step = p.ks * l.rl, first = l.part * l.rl + l.lr;
   const int nr = ((p.s + step - 1) >> (__ffs(step) - 1)) - c0;   // rows of this chunk some lane has (the same in every lane)
   float xv[2 * RC];
@@ -170,61 +167,81 @@ __device__ __forceinline__ void fma_chunk(const uint4 (&w)[kLoads], const Phase 
 #pragma unroll
   for (int e = 0; e < 2 * RC; ++e) {
     if ((e % RC) >= nr) continue;
-    float f[8];
-    unpack8(w[e * (GATED ? 2 : 1)], f);
+    const uint64_t xx = tc::pack2(xv[e], xv[e]);
 #pragma unroll
-    for (int cc = 0; cc < 8; ++cc) acc[cc] = fmaf(xv[e], f[cc], acc[cc]);
-    if (GATED) {
-      unpack8(w[e * 2 + 1], f);
+    for (int h = 0; h < (GATED ? 2 : 1); ++h) {
+      const uint4 &v = w[e * (GATED ? 2 : 1) + h];
+      const uint32_t p[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-      for (int cc = 0; cc < 8; ++cc) acc[8 + cc] = fmaf(xv[e], f[cc], acc[8 + cc]);
+      for (int c = 0; c < 4; ++c)
+        acc[h * 4 + c] = tc::fma2(xx, tc::pack2(__uint_as_float(p[c] << 16), __uint_as_float(p[c] & 0xFFFF0000u)), acc[h * 4 + c]);
     }
   }
 }
 
-// One phase for the units of this warp.  `w` holds the first chunk of the first unit when have_first.  Results of a
-// piece: lanes with lr == 0 of the warp with part == 0 call `emit(col, acc)`.
-template <bool GATED, bool HIDDEN, typename Emit>
-__device__ __forceinline__ void run_phase(const Phase &p, int type, const __nv_bfloat16 *x, uint4 (&w)[kLoads], bool have_first,
+// The sums of a piece: NV values of every lane over the lanes that share its columns, halved step by step (a lane ends
+// with one value), then over the warps that share the piece, through shared memory.  One lane per column calls emit(column
+// of the piece, gate or plain value, up value).  `meet` is the barrier of those warps.
+template <bool GATED, typename Meet, typename Emit>
+__device__ __forceinline__ void finish_piece(const uint64_t (&acc)[GATED ? 8 : 4], const Phase &p, const Lane &l, float *partial, Meet meet,
+                                             Emit emit) {
+  constexpr int NV = GATED ? 16 : 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, po = p.pc >> 3;
+  float v[NV];
+#pragma unroll
+  for (int i = 0; i < NV / 2; ++i) v[2 * i] = __uint_as_float((uint32_t)acc[i]), v[2 * i + 1] = __uint_as_float((uint32_t)(acc[i] >> 32));
+  int n = NV;
+#pragma unroll
+  for (int d = 16; d >= 1; d >>= 1) {
+    if (n > 1) {   // (16 or 8 lanes away at least: never a lane with other columns)
+      n >>= 1;
+      const bool hi = lane & d;
+#pragma unroll
+      for (int i = 0; i < NV / 2; ++i)
+        if (i < n) {
+          const float send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+          v[i] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+        }
+    } else if (d >= po) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], d);
+    }
+  }
+  // lane: value lane / (32 / NV) of the columns l.sub
+  partial[(warp * 2 + l.sub) * 16 + lane / (32 / NV)] = v[0];
+  if (p.ks > 1) meet(); else __syncwarp();
+  if (l.part == 0 && lane < p.pc) {
+    const float *src = partial + (warp * 2 + (lane >> 3)) * 16 + (lane & 7);
+    float g = 0.f, u = 0.f;
+    for (int o = 0; o < p.ks; ++o) {
+      g += src[o * 32];
+      if (GATED) u += src[o * 32 + 8];
+    }
+    emit(lane, g, u);
+  }
+  if (p.ks > 1) meet(); else __syncwarp();
+}
+
+// One phase for the units of this warp.  `w` holds the first chunk of the first unit when have_first.  Results:
+// emit(column, gate or plain value, up value), one lane per column.
+template <bool GATED, bool HIDDEN, int RC, typename Emit>
+__device__ __forceinline__ void run_phase(const Phase &p, int type, const __nv_bfloat16 *x, uint4 (&w)[kLoads<GATED, RC>], bool have_first,
                                           int n_units, float *partial, const Wait &wait, Emit emit) {
-  constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total_warps = gridDim.x * kWarps, po = p.pc >> 3;
+  const int total_warps = gridDim.x * kWarps;
   const int rounds = (n_units + total_warps - 1) / total_warps;
   for (int rd = 0; rd < rounds; ++rd) {
     const int unit = unit_of(rd, p.ks);
     Lane l = lane_of(p, unit);
     if (unit >= n_units) l.on = false;
-    float acc[16];
-#pragma unroll
-    for (int cc = 0; cc < 16; ++cc) acc[cc] = 0.f;
+    uint64_t acc[GATED ? 8 : 4] = {};
     const int rows_per_lane = (p.s + p.ks * l.rl - 1) >> (__ffs(p.ks * l.rl) - 1);
     for (int c0 = 0; c0 < rows_per_lane; c0 += RC) {
-      if (!(have_first && rd == 0 && c0 == 0)) load_chunk<GATED>(w, p, l, type, c0);
-      fma_chunk<GATED, HIDDEN>(w, p, l, type, c0, x, acc, wait);
+      if (!(have_first && rd == 0 && c0 == 0)) load_chunk<GATED, RC>(w, p, l, type, c0);
+      fma_chunk<GATED, HIDDEN, RC>(w, p, l, type, c0, x, acc, wait);
     }
-    // sum over the lanes that share the columns
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-      if (d >= po) {
-#pragma unroll
-        for (int cc = 0; cc < (GATED ? 16 : 8); ++cc) acc[cc] += __shfl_xor_sync(0xffffffffu, acc[cc], d);
-      }
-    }
-    if (p.ks > 1) {   // the warps of a piece sit in one CTA
-      if (lane < po) {
-#pragma unroll
-        for (int cc = 0; cc < 16; ++cc) partial[(warp * kMaxPo + lane) * 16 + cc] = acc[cc];
-      }
-      __syncthreads();
-      if (l.part == 0 && lane < po) {
-        for (int o = 1; o < p.ks; ++o)
-#pragma unroll
-          for (int cc = 0; cc < 16; ++cc) acc[cc] += partial[((warp + o) * kMaxPo + lane) * 16 + cc];
-      }
-      __syncthreads();
-    }
-    if (l.on && l.part == 0 && lane < po) emit(l.col, acc);
+    const int col0 = l.piece * p.pc;
+    finish_piece<GATED>(acc, p, l, partial, [] { __syncthreads(); }, [&](int c, float g, float u) {
+      if (unit < n_units && col0 + c < p.n_cols) emit(col0 + c, g, u);
+    });
   }
 }
 
@@ -239,42 +256,22 @@ __device__ __forceinline__ float activate(float z, int act) {
   return z;
 }
 
-// eight results of a piece: + bias, activation, stored as bf16 or fp32
-__device__ __forceinline__ void store8(const float (&acc)[16], int col, const void *bias, int act, void *out, bool out_bf16, bool exchange = false) {
-  float v[8];
-#pragma unroll
-  for (int e = 0; e < 8; ++e) v[e] = acc[e];
-  if (bias) {
-    float b[8];
-    unpack8(__ldg((const uint4 *)((const __nv_bfloat16 *)bias + col)), b);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] += b[e];
-  }
-  if (act != ALG_ACT_NONE) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = activate(v[e], act);
-  }
-  if (out_bf16) {
-    uint32_t o[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      __nv_bfloat162 pk = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-      o[e] = *(uint32_t *)&pk;
-    }
-    if (exchange) exch_store4((__nv_bfloat16 *)out + col, o[0], o[1], o[2], o[3]);
-    else *(uint4 *)((__nv_bfloat16 *)out + col) = make_uint4(o[0], o[1], o[2], o[3]);
-  } else {
-    float4 *dst = (float4 *)((float *)out + col);
-    dst[0] = make_float4(v[0], v[1], v[2], v[3]);
-    dst[1] = make_float4(v[4], v[5], v[6], v[7]);
-  }
+// one result: + bias, activation
+__device__ __forceinline__ float finish1(float z, int col, const void *bias, int act) {
+  if (bias) z += __bfloat162float(__ldg((const __nv_bfloat16 *)bias + col));
+  return act == ALG_ACT_NONE ? z : activate(z, act);
 }
+__device__ __forceinline__ void store1(void *out, int64_t at, bool out_bf16, float z) {
+  if (out_bf16) ((__nv_bfloat16 *)out)[at] = __float2bfloat16_rn(z);
+  else ((float *)out)[at] = z;
+}
+__device__ __forceinline__ float gated1(float g, float u) { return g / (1.f + __expf(-g)) * u; }   // silu(g) * u
 
 // MODE 0: gated FFN, 1: FFN, 2: projection (W1 only)
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecodeArgs a) {
+template <int MODE, int RC>
+__global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(const RowDecodeArgs a) {
   constexpr bool GATED = MODE == 0, FFN = MODE != 2;
-  __shared__ float partial[kWarps * kMaxPo * 16];
+  __shared__ float partial[kWarps * 2 * 16];   // a piece has at most 2 x 8 columns
   __shared__ int s_abort;
   ALG_TRACE_VARS;
   if (threadIdx.x == 0) ALG_TRACE(0, 1);
@@ -293,12 +290,12 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
   // ---- before the dependency resolves: the row type as it stands now and the first W1 loads it asks for (the type
   // is read again after the wait) ----
   const int t_early = read_type(a);
-  uint4 w[kLoads];
+  uint4 w[kLoads<GATED, RC>];
   {
     const int unit = unit_of(0, p1.ks);
     Lane l = lane_of(p1, unit);
     if (unit >= a.units1 || t_early < 0) l.on = false;
-    load_chunk<GATED>(w, p1, l, max(t_early, 0), 0);
+    load_chunk<GATED, RC>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
   __syncthreads();   // s_abort is set
@@ -319,22 +316,11 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
     const int t = pass == 0 ? t_early : type;
     if (pass == 1 && type == t_early) break;
     if (t < 0) continue;
-    run_phase<GATED, false>(p1, t, X, w, pass == 0, a.units1, partial, wait, [&](int col, const float (&acc)[16]) {
+    run_phase<GATED, false, RC>(p1, t, X, w, pass == 0, a.units1, partial, wait, [&](int col, float g, float u) {
       if (t != type || keep) return;   // (hidden values are taken as soon as they are there: only the right ones are stored)
-      if (GATED) {
-        uint32_t o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float g0 = acc[2 * e], g1 = acc[2 * e + 1];
-          __nv_bfloat162 pk = __floats2bfloat162_rn(g0 / (1.f + __expf(-g0)) * acc[8 + 2 * e], g1 / (1.f + __expf(-g1)) * acc[8 + 2 * e + 1]);
-          o[e] = *(uint32_t *)&pk;
-        }
-        exch_store4(H + col, o[0], o[1], o[2], o[3]);
-      } else if (FFN) {
-        store8(acc, col, a.b1, a.act, H, true, true);
-      } else {
-        store8(acc, col, a.b1, a.act, a.Y, a.y_bf16 != 0);
-      }
+      if (GATED) exch_store1(H + col, gated1(g, u));
+      else if (FFN) exch_store1(H + col, finish1(g, col, a.b1, a.act));
+      else store1(a.Y, col, a.y_bf16 != 0, finish1(g, col, a.b1, a.act));
     });
   }
   if (type < 0 && threadIdx.x == 0 && blockIdx.x == 0) atomicExch(a.status, (int)ALG_ERR_BAD_TYPE);   // y = 0
@@ -350,11 +336,12 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
   }
 
   // ---- the first W_down loads go out before the hidden values are waited for ----
+  uint4 w2[kLoads<false, RC>];
   {
     const int unit = unit_of(0, p2.ks);
     Lane l = lane_of(p2, unit);
     if (unit >= a.units2 || type < 0) l.on = false;
-    load_chunk<false>(w, p2, l, max(type, 0), 0);
+    load_chunk<false, RC>(w2, p2, l, max(type, 0), 0);
   }
 
   exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, 1);
@@ -362,8 +349,8 @@ __global__ void __launch_bounds__(kThreads, 1) row_decode_kernel(const RowDecode
 
   // ---- phase 2: y = h * W_down (+ b_down) ----
   if (type >= 0) {
-    run_phase<false, true>(p2, type, H, w, true, a.units2, partial, wait,
-                           [&](int col, const float (&acc)[16]) { store8(acc, col, a.b2, ALG_ACT_NONE, a.Y, a.y_bf16 != 0); });
+    run_phase<false, true, RC>(p2, type, H, w2, true, a.units2, partial, wait,
+                                [&](int col, float z, float) { store1(a.Y, col, a.y_bf16 != 0, finish1(z, col, a.b2, ALG_ACT_NONE)); });
   } else {   // a row type outside [0, q): the row of Y is zero
     for (int c = blockIdx.x * kThreads + threadIdx.x; c < a.D; c += gridDim.x * kThreads) {
       if (a.y_bf16) ((__nv_bfloat16 *)a.Y)[c] = __float2bfloat16_rn(0.f);
@@ -384,7 +371,7 @@ __device__ __forceinline__ int read_row_type(const RowDecodeArgs &a, int m) {
 
 // The same phase for several rows: unit = (row, piece, share of the piece's weight rows), rows outermost.  `w` holds
 // the first chunk of the first unit when have_first, fetched for row type t_first; the other units read their row's
-// type themselves.  Results of a piece: lanes with lr == 0 of the warp with part == 0 call `emit(row, col, acc)`.
+// type themselves.  Results: emit(row, column, gate or plain value, up value), one lane per column.
 // Barrier of the warps that share a piece (2, 4 or 8 of them: at most four groups per CTA).  The ids are literals so
 // that the kernel reserves five hardware barriers, not all sixteen -- with sixteen a second CTA (the next launch's,
 // which starts early to request its weights) could not become resident beside this one.
@@ -399,12 +386,11 @@ __device__ __forceinline__ void group_barrier(int id, int threads) {
 
 // A row whose type lies outside [0, q) reads nothing; with LAST (the phase that writes Y) its pieces are stored as zeros
 // and the status word says so.
-template <bool GATED, bool HIDDEN, bool LAST, typename Emit>
+template <bool GATED, bool HIDDEN, bool LAST, int RC, typename Emit>
 __device__ __forceinline__ void run_rows_phase(const RowDecodeArgs &a, const Phase &p, const __nv_bfloat16 *x, int64_t ldx,
-                                          uint4 (&w)[kLoads], bool have_first, int t_first, int n_units, float *partial, const Wait &wait, Emit emit) {
-  constexpr int RC = GATED ? kLoads / 4 : kLoads / 2;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total_warps = gridDim.x * kWarps, po = p.pc >> 3;
+                                          uint4 (&w)[kLoads<GATED, RC>], bool have_first, int t_first, int n_units, float *partial, const Wait &wait, Emit emit) {
+  const int warp = threadIdx.x >> 5;
+  const int total_warps = gridDim.x * kWarps;
   const int rounds = (n_units + total_warps - 1) / total_warps;
   const int per_row = a.M == 1 ? n_units : n_units / a.M;   // (one row: no division on the way to the first load)
   for (int rd = 0; rd < rounds; ++rd) {
@@ -418,47 +404,25 @@ __device__ __forceinline__ void run_rows_phase(const RowDecodeArgs &a, const Pha
     for (int attempt = 0; attempt < 2; ++attempt) {
       Lane l = lane_of(p, unit - m * per_row);
       if (unit >= n_units || type < 0) l.on = false;
-      float acc[16];
-#pragma unroll
-      for (int cc = 0; cc < 16; ++cc) acc[cc] = 0.f;
+      uint64_t acc[GATED ? 8 : 4] = {};
       const int rows_per_lane = (p.s + p.ks * l.rl - 1) >> (__ffs(p.ks * l.rl) - 1);
       for (int c0 = 0; c0 < rows_per_lane; c0 += RC) {
-        if (!(have_first && rd == 0 && attempt == 0 && c0 == 0)) load_chunk<GATED>(w, p, l, max(type, 0), c0);
-        fma_chunk<GATED, HIDDEN>(w, p, l, max(type, 0), c0, xm, acc, wait);
+        if (!(have_first && rd == 0 && attempt == 0 && c0 == 0)) load_chunk<GATED, RC>(w, p, l, max(type, 0), c0);
+        fma_chunk<GATED, HIDDEN, RC>(w, p, l, max(type, 0), c0, xm, acc, wait);
       }
-      // sum over the lanes that share the columns
-#pragma unroll
-      for (int d = 16; d >= 1; d >>= 1) {
-        if (d >= po) {
-#pragma unroll
-          for (int cc = 0; cc < (GATED ? 16 : 8); ++cc) acc[cc] += __shfl_xor_sync(0xffffffffu, acc[cc], d);
+      const int col0 = l.piece * p.pc;
+      const bool again = attempt == 0 && type != real;
+      finish_piece<GATED>(acc, p, l, partial, [&] { group_barrier(1 + warp / p.ks, 32 * p.ks); }, [&](int c, float g, float u) {
+        if (again || unit >= n_units || col0 + c >= p.n_cols) return;
+        if (type >= 0) {
+          emit(m, col0 + c, g, u);
+        } else if (LAST) {
+          store1(a.Y, (int64_t)m * a.ldy + col0 + c, a.y_bf16 != 0, 0.f);
+          if (c == 0) atomicExch(a.status, (int)ALG_ERR_BAD_TYPE);
         }
-      }
-      if (p.ks > 1) {   // the warps of a piece sit side by side in one CTA
-        const int bar_id = 1 + warp / p.ks, bar_threads = 32 * p.ks;
-        if (lane < po) {
-#pragma unroll
-          for (int cc = 0; cc < 16; ++cc) partial[(warp * kMaxPo + lane) * 16 + cc] = acc[cc];
-        }
-        group_barrier(bar_id, bar_threads);
-        if (l.part == 0 && lane < po) {
-          for (int o = 1; o < p.ks; ++o)
-#pragma unroll
-            for (int cc = 0; cc < 16; ++cc) acc[cc] += partial[((warp + o) * kMaxPo + lane) * 16 + cc];
-        }
-        group_barrier(bar_id, bar_threads);
-      }
-      if (attempt == 0 && type != real) {
-        type = real;
-        continue;
-      }
-      if (l.on && l.part == 0 && lane < po) emit(m, l.col, acc);
-      if (LAST && type < 0 && unit < n_units && l.part == 0 && lane < po && l.col < p.n_cols) {
-        if (a.y_bf16) *(uint4 *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy + l.col) = make_uint4(0, 0, 0, 0);
-        else ((float4 *)((float *)a.Y + (int64_t)m * a.ldy + l.col))[0] = ((float4 *)((float *)a.Y + (int64_t)m * a.ldy + l.col))[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (lane == 0) atomicExch(a.status, (int)ALG_ERR_BAD_TYPE);
-      }
-      break;
+      });
+      if (!again) break;
+      type = real;
     }
   }
 }
@@ -466,10 +430,10 @@ __device__ __forceinline__ void run_rows_phase(const RowDecodeArgs &a, const Pha
 // Several rows (2 .. kRowDecodeMaxM): the row is the outermost dimension of the units; every warp reads the type of the
 // rows it works on.  (A kernel of its own: the index arithmetic of the general form costs the one-row step 0.4-1 us.)
 // MODE 0: gated FFN, 1: FFN, 2: projection (W1 only)
-template <int MODE>
-__global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecodeArgs a) {
+template <int MODE, int RC>
+__global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(const RowDecodeArgs a) {
   constexpr bool GATED = MODE == 0, FFN = MODE != 2;
-  __shared__ float partial[kWarps * kMaxPo * 16];
+  __shared__ float partial[kWarps * 2 * 16];   // a piece has at most 2 x 8 columns
   __shared__ int s_abort;
   ALG_TRACE_VARS;
   if (threadIdx.x == 0) ALG_TRACE(0, 1);
@@ -489,11 +453,11 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
   const int per_row1 = a.M == 1 ? a.units1 : a.units1 / a.M;
   const int unit1 = unit_of(0, p1.ks), m1 = a.M == 1 ? 0 : min(unit1 / per_row1, a.M - 1);
   const int t_early = read_row_type(a, m1);
-  uint4 w[kLoads];
+  uint4 w[kLoads<GATED, RC>];
   {
     Lane l = lane_of(p1, unit1 - m1 * per_row1);
     if (unit1 >= a.units1 || t_early < 0) l.on = false;
-    load_chunk<GATED>(w, p1, l, max(t_early, 0), 0);
+    load_chunk<GATED, RC>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
   __syncthreads();   // s_abort is set
@@ -510,45 +474,33 @@ __global__ void __launch_bounds__(kThreads, 1) rows_decode_kernel(const RowDecod
   // ---- phase 1 (its first unit on the type read early).  Gated: h = silu(x * W_gate) .* (x * W_up); FFN:
   // h = act(x * W_up + b_up); projection: y = act(x * W + b) ----
   {
-    run_rows_phase<GATED, false, !FFN>(a, p1, X, a.ldx, w, true, t_early, a.units1, partial, wait, [&](int m, int col, const float (&acc)[16]) {
+    run_rows_phase<GATED, false, !FFN, RC>(a, p1, X, a.ldx, w, true, t_early, a.units1, partial, wait, [&](int m, int col, float g, float u) {
       if (keep) return;
-      if (GATED) {
-        uint32_t o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float g0 = acc[2 * e], g1 = acc[2 * e + 1];
-          __nv_bfloat162 pk = __floats2bfloat162_rn(g0 / (1.f + __expf(-g0)) * acc[8 + 2 * e], g1 / (1.f + __expf(-g1)) * acc[8 + 2 * e + 1]);
-          o[e] = *(uint32_t *)&pk;
-        }
-        exch_store4(H + (int64_t)m * a.F + col, o[0], o[1], o[2], o[3]);
-      } else if (FFN) {
-        store8(acc, col, a.b1, a.act, H + (int64_t)m * a.F, true, true);
-      } else {
-        store8(acc, col, a.b1, a.act, a.y_bf16 ? (void *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy) : (void *)((float *)a.Y + (int64_t)m * a.ldy),
-               a.y_bf16 != 0);
-      }
+      if (GATED) exch_store1(H + (int64_t)m * a.F + col, gated1(g, u));
+      else if (FFN) exch_store1(H + (int64_t)m * a.F + col, finish1(g, col, a.b1, a.act));
+      else store1(a.Y, (int64_t)m * a.ldy + col, a.y_bf16 != 0, finish1(g, col, a.b1, a.act));
     });
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 6);
 
   if (FFN) {
     // ---- the first W_down loads go out before the hidden values are waited for ----
+    uint4 w2[kLoads<false, RC>];
     const int per_row2 = a.M == 1 ? a.units2 : a.units2 / a.M;
     const int unit2 = unit_of(0, p2.ks), m2 = a.M == 1 ? 0 : min(unit2 / per_row2, a.M - 1);
     const int type2 = read_row_type(a, m2);
     {
       Lane l = lane_of(p2, unit2 - m2 * per_row2);
       if (unit2 >= a.units2 || type2 < 0) l.on = false;
-      load_chunk<false>(w, p2, l, max(type2, 0), 0);
+      load_chunk<false, RC>(w2, p2, l, max(type2, 0), 0);
     }
 
     exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, a.M);
     if (threadIdx.x == 0) ALG_TRACE(0, 9);
 
     // ---- phase 2: y = h * W_down (+ b_down) ----
-    run_rows_phase<false, true, true>(a, p2, H, a.F, w, true, type2, a.units2, partial, wait, [&](int m, int col, const float (&acc)[16]) {
-      store8(acc, col, a.b2, ALG_ACT_NONE,
-             a.y_bf16 ? (void *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy) : (void *)((float *)a.Y + (int64_t)m * a.ldy), a.y_bf16 != 0);
+    run_rows_phase<false, true, true, RC>(a, p2, H, a.F, w2, true, type2, a.units2, partial, wait, [&](int m, int col, float z, float) {
+      store1(a.Y, (int64_t)m * a.ldy + col, a.y_bf16 != 0, finish1(z, col, a.b2, ALG_ACT_NONE));
     });
     __syncthreads();
   if (threadIdx.x == 0) {
@@ -565,8 +517,8 @@ int pick_ks(int pieces, int grid) {
   return ks;
 }
 
-template <int MODE>
-cudaError_t launch_mode(const RowDecodeArgs &a, int grid, cudaStream_t st) {
+template <int MODE, int RC>
+cudaError_t launch_rc(const RowDecodeArgs &a, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -577,9 +529,22 @@ cudaError_t launch_mode(const RowDecodeArgs &a, int grid, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaError_t e = a.M == 1 ? cudaLaunchKernelEx(&cfg, row_decode_kernel<MODE>, a) : cudaLaunchKernelEx(&cfg, rows_decode_kernel<MODE>, a);
+  cudaError_t e = a.M == 1 ? cudaLaunchKernelEx(&cfg, row_decode_kernel<MODE, RC>, a) : cudaLaunchKernelEx(&cfg, rows_decode_kernel<MODE, RC>, a);
   count_launch(1);
   return e;
+}
+
+template <int MODE>
+cudaError_t launch_mode(const RowDecodeArgs &a, int grid, cudaStream_t st) {
+  // rows of a segment per lane in the wider of the two phases
+  auto rows = [](int s, int pc, int ks) { return ceil_div(s, ks * (32 / (pc / 8))); };
+  const int need = std::max(rows(a.gs, a.pc1, a.ks1), a.units2 ? rows(a.gr, a.pc2, a.ks2) : 0);
+  if (need <= 2) return launch_rc<MODE, 2>(a, grid, st);
+  if (need <= 4) return launch_rc<MODE, 4>(a, grid, st);
+  if constexpr (MODE == 2) {
+    if (need > 8) return launch_rc<MODE, 16>(a, grid, st);
+  }
+  return launch_rc<MODE, 8>(a, grid, st);
 }
 
 }  // namespace
