@@ -250,6 +250,7 @@ struct DecodePlan {
   int sn;            // strip width in columns (64 or 32)
   int splits;        // K splits = cluster size (1..8)
   int box_rows;      // rows per TMA box of the weight slice (divides every s[k] / splits, <= 256)
+  int x_box;         // columns per TMA box of X: 64, 32 or 16 (divides every s[k] / splits)
   int w_smem_bytes;  // worst-case weight slice of one CTA
   int x_smem_bytes;  // worst-case staged X slice
   int p_smem_bytes;  // partial sums
@@ -271,7 +272,7 @@ struct DecodeArgs {
   int N;
   int splits;
   uint32_t inv_splits;    // ceil(2^32 / splits): x / splits = umulhi(x, inv_splits) for x < 2^29, splits > 1 (set by the launcher)
-  int box_rows;
+  int box_rows, x_box;
   int w_smem_bytes;
   int x_smem_bytes;
   int *status;

@@ -12,12 +12,17 @@
 // waits for the previous kernel in the stream (programmatic dependent launch), because weights do
 // not depend on it.  Which groups are needed follows from the row types, which MAY come from that
 // previous kernel: they are read once before the wait to choose the boxes and once more after it;
-// if the second reading differs, the slice is fetched again for the types that count.  It then stages the matching columns of X with 16-byte asynchronous copies (rows
-// that do not use a block are staged as zeros, which is how the row-type rule is applied),
-// multiplies with warp-level mma.sync (bf16 x bf16 -> fp32), and pushes its partial sums into the
-// shared memory of the CTA that owns the output row (row m belongs to CTA m mod splits).  After
-// one cluster barrier every CTA adds the partial sums of its rows in split order (deterministic,
-// nothing goes through global memory), applies bias / activation and stores Y.
+// if the second reading differs, the slice is fetched again for the types that count.  The
+// matching columns of X come by tiled copies too, requested the moment the wait is over (they do not
+// depend on the types); the row-type rule is applied by clearing the rows of an A fragment that do
+// not use the segment's block.  Warp-level mma.sync (bf16 x bf16 -> fp32); the partial sums are sent
+// into the shared memory of the CTA that owns the output row (row m belongs to CTA m mod splits) by
+// asynchronous stores that count their bytes on the owner's mbarrier, so nobody waits for a
+// barrier over the cluster.  The owner adds them in split order (deterministic, nothing goes through
+// global memory), applies bias / activation and stores Y.
+// What bounds it: latency (a launch reads 3-5 MB).  Two launches, 768 -> 3072 -> 768 at q = 2, per layer of a graph of layers: M = 17 12.9 -> 10.5 us, M = 40
+// 14.8 -> 12.6 us, M = 64 17.0 -> 14.7 us against X staged after the types with asynchronous copies, remote
+// stores and a cluster barrier, and 192 CTAs on 148 SMs.
 #include <cuda_runtime.h>
 
 #include "tc_common.cuh"
@@ -40,12 +45,6 @@ struct Seg {
   uint32_t rows_lo, rows_hi;  // bit b set: row b of X uses this block
 };
 
-__device__ __forceinline__ void cp_async_16_zfill(uint32_t dst, const void *src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t (&r)[4]) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -64,42 +63,31 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void st_remote_f32x2(uint32_t local_addr, uint32_t rank, float x, float y) {
-  uint32_t remote;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local_addr), "r"(rank));
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(remote), "f"(x), "f"(y) : "memory");
-}
-__device__ __forceinline__ float act_f(float z, int act) {
-  if (act == ALG_ACT_GELU_ERF) return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f));
-  if (act == ALG_ACT_GELU_TANH) {
-    float u = 0.7978845608028654f * (z + 0.044715f * z * z * z);
-    return 0.5f * z * (1.0f + tanhf(u));
-  }
-  return z;
+// eight bytes into the shared memory of CTA `rank` of the cluster, counted on the barrier at the same place there
+__device__ __forceinline__ void send_f32x2(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float x, float y) {
+  uint32_t addr, bar;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local_addr), "r"(rank));
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(local_bar), "r"(rank));
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
 }
 
 // Shared-memory images.  W slice: [rows][SN] bf16 as the TMA writes it with its 128-byte (SN = 64)
 // or 64-byte (SN = 32) swizzle: 16-byte chunk c of row r sits at chunk c ^ (r & 7), resp.
-// c ^ ((r >> 1) & 3), so the 8 rows an ldmatrix touches fall into different banks.  X slice:
-// [m_pad][x_pitch] bf16, written by this kernel with the same kind of XOR.
+// c ^ ((r >> 1) & 3), so the 8 rows an ldmatrix touches fall into different banks.  X slice: boxes of
+// [16 MT rows][x_box columns] with the swizzle of their row length, side by side along k.
 template <int SN>
 __device__ __forceinline__ uint32_t w_off(int row, int chunk) {
   constexpr int kChunks = SN / 8;
   const int sw = (kChunks == 8) ? (row & 7) : ((row >> 1) & 3);
   return (uint32_t)(row * SN * 2 + ((chunk ^ sw) << 4));
 }
-__device__ __forceinline__ uint32_t x_off(int m, int chunk, int x_pitch_bytes) {
-  return (uint32_t)(m * x_pitch_bytes + ((chunk ^ (m & 7)) << 4));
-}
 
 #define DTR() ALG_TRACE(0, 0)
 
-template <int SN>
-__global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant__ CUtensorMap tmW, const DecodeArgs a) {
+// MT = 16-row tiles of the batch
+template <int SN, int MT>
+__global__ void __launch_bounds__(kThreads, 2)
+decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const DecodeArgs a) {
   constexpr int NT = SN / 32;          // 8-column n-tiles per warp (4 warps share the strip)
   extern __shared__ uint8_t smem_raw[];
   __shared__ Seg s_seg[kMaxQ];
@@ -107,7 +95,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
   __shared__ int s_so[kMaxQ + 1], s_ro[kMaxQ + 1];
   __shared__ uint32_t s_keep[kMaxPairs];
   __shared__ uint32_t s_rows32[kMaxQ][2], s_bad32[2];
-  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ __align__(8) uint64_t s_bar, s_bar_x, s_bar_p;   // weights, X, partial sums of this CTA's rows
 
   const DevTable *__restrict__ tab = a.tab;
   const int q = a.q;
@@ -118,7 +106,7 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
   auto div_splits = [&](int x) { return splits == 1 ? x : (int)__umulhi((uint32_t)x, inv_splits); };
   const int n0 = strip * SN;
   const int M = a.M;
-  const int m_tiles = (M + 15) >> 4, m_pad = m_tiles << 4;
+  constexpr int kMPad = 16 * MT;
   ALG_TRACE_VARS;
   DTR();
 
@@ -132,11 +120,20 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
   }
   if (tid == 0) {
     mbar_init(smem_u32(&s_bar), 1);
+    mbar_init(smem_u32(&s_bar_x), 1);
+    mbar_init(smem_u32(&s_bar_p), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmW) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&tmX) : "memory");
+    const int my_rows = div_splits(M - split + splits - 1);   // rows m = split + splits * slot < M
+    mbar_expect_tx(smem_u32(&s_bar_p), (uint32_t)(my_rows * splits * SN * 4));
+  }
+  if (splits > 1) {   // the cluster's barriers are ready before anybody sends (waited for below)
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
   }
   int j = 0;
-  const uint32_t bar = smem_u32(&s_bar);
+  const uint32_t bar = smem_u32(&s_bar), bar_x = smem_u32(&s_bar_x), bar_p = smem_u32(&s_bar_p);
   uint8_t *w_sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *x_sm = w_sm + (size_t)a.w_smem_bytes;
   float *r_sm = (float *)(x_sm + (size_t)a.x_smem_bytes);   // [splits][rows owned][SN] partial sums of my rows
@@ -197,10 +194,20 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
       }
     }
   };
-  // Bounded wait for the weight slice (parity = phase of the barrier).
-  auto wait_weights = [&](uint32_t parity) {
+  // the columns of X that go with the slice; rows past M read as zero
+  auto fetch_x = [&]() {
+    if (tid == 0) {
+      const int box_bytes = kMPad * a.x_box * 2;
+      mbar_expect_tx(bar_x, (uint32_t)(s_rows * kMPad * 2));
+      uint32_t dst = smem_u32(x_sm);
+      for (int s = 0; s < s_nseg; ++s)
+        for (int c = 0; c < s_seg[s].len; c += a.x_box, dst += box_bytes) tma_load_2d(dst, &tmX, bar_x, s_seg[s].grow0 + c, 0);
+    }
+  };
+  // Bounded wait (parity = phase of the barrier).
+  auto wait_bar = [&](uint32_t b, uint32_t parity) {
     const long long t0 = clock64();
-    while (!mbar_try_wait(bar, parity)) {
+    while (!mbar_try_wait(b, parity)) {
       if (clock64() - t0 > a.wait_limit) {
         atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
         while (clock64() - t0 < a.wait_limit + 2000000LL) {  // copies still in flight get time to land
@@ -217,8 +224,9 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   DTR();
-  uint32_t w_parity = 0;
-  bool weights_ok = true;
+  fetch_x();
+  uint32_t parity = 0;
+  bool landed = true;
   {  // the row types as the previous kernel left them: the ones that count
     int t_now = -1;
     if (tid < M) {
@@ -230,97 +238,98 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
     }
     if (__syncthreads_or(t_now != my_type)) {
       // fetched for other types than the final ones: let those copies land, then fetch again
-      weights_ok = wait_weights(0);
-      __syncthreads();
-      if (weights_ok) {
+      landed = wait_bar(bar, 0) && wait_bar(bar_x, 0);
+      if (__syncthreads_and(landed)) {
         plan_and_fetch();
-        w_parity = 1;
-      }
-    }
-  }
-  const int nseg = s_nseg, rows_cta = s_rows;
-  const int x_pitch_bytes = ((rows_cta + 63) & ~63) * 2;  // whole groups of eight 16-byte chunks
-  // ---- the matching columns of X; rows that do not use a block are staged as zeros ----
-  {
-    const __nv_bfloat16 *X = (const __nv_bfloat16 *)a.X;
-    const uint32_t x_base = smem_u32(x_sm);
-    // thread -> (row m = tid / 8 + 16 i, chunk ch = tid % 8 + 8 jj): no divisions in the loop
-    const int m_lo = tid >> 3, ch_lo = tid & 7;
-    for (int s = 0; s < nseg; ++s) {
-      const Seg sg = s_seg[s];
-      const int seg_chunks = sg.len >> 3;
-      for (int m = m_lo; m < m_pad; m += kThreads / 8) {
-        const bool use = m < M && (((m < 32 ? sg.rows_lo : sg.rows_hi) >> (m & 31)) & 1u);
-        const __nv_bfloat16 *src = X + (int64_t)(use ? m : 0) * a.ldx + sg.grow0;
-        for (int ch = ch_lo; ch < seg_chunks; ch += 8)
-          cp_async_16_zfill(x_base + x_off(m, (sg.loc0 >> 3) + ch, x_pitch_bytes), src + ch * 8, use);
+        fetch_x();
+        parity = 1;
       }
     }
   }
   DTR();
-  cp_async_wait_all();
-  if (weights_ok) wait_weights(w_parity);   // on expiry: status raised, the result is invalid, the kernel still ends
-  __syncthreads();
+  // on expiry: status raised, the result is invalid, the kernel still ends
+  if (landed && wait_bar(bar_x, parity)) wait_bar(bar, parity);
   DTR();
 
   // ---- warp-level MMA: warp w owns columns [w * SN/4, +SN/4) of the strip, all rows ----
-  float acc[4][NT][4];
+  float acc[MT][NT][4];
 #pragma unroll
-  for (int mt = 0; mt < 4; ++mt)
+  for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
-  const uint32_t w_base = smem_u32(w_sm), x_base = smem_u32(x_sm);
-  const int wcol_chunk = warp * (SN / 32);  // first 16-byte chunk of this warp's columns
-  const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8;
-#pragma unroll 2
-  for (int k0 = 0; k0 < rows_cta; k0 += 16) {
-    uint32_t b[4];
-    if (NT == 2) {
-      ldmatrix_x4_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk + (lane >> 4)), b);
-    } else {
-      uint32_t r2[2];
-      ldmatrix_x2_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk), r2);
-      b[0] = r2[0], b[1] = r2[1], b[2] = 0, b[3] = 0;
-    }
-    uint32_t af[4][4];
+  {
+    const uint32_t w_base = smem_u32(w_sm);
+    const int wcol_chunk = warp * (SN / 32);  // first 16-byte chunk of this warp's columns
+    const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8, g = lane >> 2;
+    const int xb = a.x_box, x_sw = xb == 64 ? frag_row & 7 : xb == 32 ? (frag_row >> 1) & 3 : (frag_row >> 2) & 1;
+    const uint32_t x_row = smem_u32(x_sm) + (uint32_t)(frag_row * xb * 2);
+    const int box_bytes = kMPad * xb * 2, x_tile = 16 * xb * 2;
+    const int nseg = s_nseg;
+    for (int s = 0; s < nseg; ++s) {
+      const Seg sg = s_seg[s];
+      uint32_t keep[MT][2];   // rows g and g + 8 of every tile: all ones if the row uses the segment
 #pragma unroll
-    for (int mt = 0; mt < 4; ++mt)
-      if (mt < m_tiles) ldmatrix_x4(x_base + x_off(mt * 16 + frag_row, (k0 >> 3) + (lane >> 4), x_pitch_bytes), af[mt]);
-#pragma unroll
-    for (int mt = 0; mt < 4; ++mt)
-      if (mt < m_tiles) {
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af[mt], b[nt * 2], b[nt * 2 + 1]);
+      for (int mt = 0; mt < MT; ++mt) {
+        const uint32_t rows = (mt < 2 ? sg.rows_lo : sg.rows_hi) >> (16 * (mt & 1) + g);
+        keep[mt][0] = 0u - (rows & 1u), keep[mt][1] = 0u - ((rows >> 8) & 1u);
       }
+      uint32_t x_box = x_row + (uint32_t)(sg.loc0 / xb * box_bytes);
+      int c = 0;   // 16-byte chunk of the current k inside its box
+#pragma unroll 2
+      for (int k0 = sg.loc0; k0 < sg.loc0 + sg.len; k0 += 16) {
+        uint32_t b[4];
+        if (NT == 2) {
+          ldmatrix_x4_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk + (lane >> 4)), b);
+        } else {
+          uint32_t r2[2];
+          ldmatrix_x2_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk), r2);
+          b[0] = r2[0], b[1] = r2[1], b[2] = 0, b[3] = 0;
+        }
+        uint32_t af[MT][4];
+        const uint32_t x_at = x_box + (uint32_t)(((c + (lane >> 4)) ^ x_sw) << 4);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) ldmatrix_x4(x_at + (uint32_t)(mt * x_tile), af[mt]);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          af[mt][0] &= keep[mt][0], af[mt][2] &= keep[mt][0], af[mt][1] &= keep[mt][1], af[mt][3] &= keep[mt][1];
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af[mt], b[nt * 2], b[nt * 2 + 1]);
+        }
+        c += 2;
+        if (c == xb >> 3) c = 0, x_box += (uint32_t)box_bytes;
+      }
+    }
   }
   DTR();
+  if (splits > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // long since complete
   // ---- push the partial sums to the owners of the rows: row m -> CTA m % splits, slot m / splits ----
-  const int rows_owned_max = div_splits(m_pad + splits - 1);
+  const int rows_owned_max = div_splits(kMPad + splits - 1);
   {
     const uint32_t r_base = smem_u32(r_sm);
     const int g = lane >> 2, t4 = lane & 3;
 #pragma unroll
-    for (int mt = 0; mt < 4; ++mt) {
-      if (mt < m_tiles) {
+    for (int mt = 0; mt < MT; ++mt) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int m = mt * 16 + g + h * 8;
-          const int slot = div_splits(m);
-          const uint32_t owner = (uint32_t)(m - slot * splits);
+      for (int h = 0; h < 2; ++h) {
+        const int m = mt * 16 + g + h * 8;
+        const int slot = div_splits(m);
+        const uint32_t owner = (uint32_t)(m - slot * splits);
+        if (m < M) {
 #pragma unroll
           for (int nt = 0; nt < NT; ++nt) {
             const int col = warp * (SN / 4) + nt * 8 + t4 * 2;
-            const uint32_t off = r_base + (uint32_t)(((split * rows_owned_max + slot) * SN + col) * 4);
-            if (splits > 1) st_remote_f32x2(off, owner, acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
-            else *(float2 *)(r_sm + (slot * SN + col)) = make_float2(acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
+            if (splits > 1)
+              send_f32x2(r_base + (uint32_t)(((split * rows_owned_max + slot) * SN + col) * 4), bar_p, owner, acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
+            else
+              *(float2 *)(r_sm + (slot * SN + col)) = make_float2(acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
           }
         }
       }
     }
   }
-  if (splits > 1) cluster_sync_all();  // all partial sums of my rows have arrived; no remote access after this
+  if (splits > 1) wait_bar(bar_p, 0);   // every partial sum of my rows has arrived
   else __syncthreads();
   DTR();
 
@@ -339,12 +348,18 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
       const int col = n0 + n;
       const bool bad = ((m < 32 ? s_bad32[0] : s_bad32[1]) >> (m & 31)) & 1u;
       float v[4] = {z.x, z.y, z.z, z.w};
+      if (a.bias) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        if (a.bias) v[c] += __bfloat162float(((const __nv_bfloat16 *)a.bias)[col + c]);
-        v[c] = act_f(v[c], a.act);
-        if (bad) v[c] = 0.f;  // out-of-range type: the row's output is defined to be zero
+        for (int c = 0; c < 4; ++c) v[c] += __bfloat162float(((const __nv_bfloat16 *)a.bias)[col + c]);
       }
+      if (a.act == ALG_ACT_GELU_ERF) {
+        gelu_erf2(v[0], v[1]);
+        gelu_erf2(v[2], v[3]);
+      } else if (a.act == ALG_ACT_GELU_TANH) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) v[c] = gelu_tanh(v[c]);
+      }
+      if (bad) v[0] = v[1] = v[2] = v[3] = 0.f;  // out-of-range type: the row's output is defined to be zero
       if (a.y_bf16) {
         __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
         *(uint2 *)((__nv_bfloat16 *)a.Y + (int64_t)m * a.ldy + col) = make_uint2(*(uint32_t *)&lo, *(uint32_t *)&hi);
@@ -356,17 +371,19 @@ __global__ void __launch_bounds__(kThreads) decode_kernel(const __grid_constant_
   DTR();
 }
 
-template <int SN>
+template <int SN, int MT>
 cudaError_t launch_t(const DecodeArgs &a, size_t smem_bytes, cudaStream_t st) {
   static bool attr = false;
   if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(decode_kernel<SN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    cudaError_t e = cudaFuncSetAttribute(decode_kernel<SN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  CUtensorMap tmW;
+  CUtensorMap tmW, tmX;
   cudaError_t e = make_map_2d_sw(&tmW, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.ldw * 2, SN, (uint32_t)a.box_rows,
                                  SN * 2);
+  if (e != cudaSuccess) return e;
+  e = make_map_2d_sw(&tmX, a.X, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.ldx * 2, (uint32_t)a.x_box, 16 * MT, a.x_box * 2);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.N / SN, a.splits, 1);
@@ -384,7 +401,15 @@ cudaError_t launch_t(const DecodeArgs &a, size_t smem_bytes, cudaStream_t st) {
   at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, decode_kernel<SN>, tmW, a);
+  return cudaLaunchKernelEx(&cfg, decode_kernel<SN, MT>, tmW, tmX, a);
+}
+
+template <int SN>
+cudaError_t launch_mt(const DecodeArgs &a, size_t smem_bytes, cudaStream_t st) {
+  if (a.M <= 16) return launch_t<SN, 1>(a, smem_bytes, st);
+  if (a.M <= 32) return launch_t<SN, 2>(a, smem_bytes, st);
+  if (a.M <= 48) return launch_t<SN, 3>(a, smem_bytes, st);
+  return launch_t<SN, 4>(a, smem_bytes, st);
 }
 
 }  // namespace
@@ -417,16 +442,20 @@ bool decode_plan(int q, const int *s, int K, int N, int num_sms, DecodePlan *pla
       if (box % 8) continue;
       const int rows_max = K / sp;  // worst case: every input group needed by the strip
       const size_t w_bytes = (size_t)rows_max * sn * 2;
-      const size_t x_bytes = (size_t)kDecodeMaxM * (((rows_max + 63) & ~63) * 2);
+      const size_t x_bytes = (size_t)kDecodeMaxM * rows_max * 2;
+      int xb = 64;
+      for (int k = 0; k < q; ++k)
+        while (s[k] / sp % xb) xb /= 2;
       const size_t p_bytes = (size_t)(kDecodeMaxM + 8) * sn * 4;
       if (w_bytes + x_bytes + p_bytes + 1024 > 190 * 1024) continue;
       const int ctas = (N / sn) * sp;
-      // prefer filling the machine, then not overshooting it, then the wider strip
-      long long score = ctas >= num_sms ? (1000000 - (ctas - num_sms)) * 4 : (long long)ctas * 4;
+      // one CTA per SM as far as that goes (two of them on some SMs take as long as two everywhere), then not
+      // overshooting, then the wider strip
+      long long score = ctas <= num_sms ? 4000000 + (long long)ctas * 4 : (1000000 - (long long)ctas) * 4;
       score += (sn == 64) ? 1 : 0;
       if (score > best_score) {
         best_score = score;
-        best.sn = sn, best.splits = sp, best.box_rows = box;
+        best.sn = sn, best.splits = sp, best.box_rows = box, best.x_box = xb;
         best.w_smem_bytes = (int)w_bytes, best.x_smem_bytes = (int)x_bytes, best.p_smem_bytes = (int)p_bytes;
       }
     }
@@ -440,11 +469,11 @@ cudaError_t launch_decode(const DecodeArgs &a, const DecodePlan &plan, cudaStrea
   DecodeArgs b = a;
   b.splits = plan.splits;
   b.inv_splits = (uint32_t)((0x100000000ull + (uint64_t)plan.splits - 1) / (uint64_t)plan.splits);
-  b.box_rows = plan.box_rows;
+  b.box_rows = plan.box_rows, b.x_box = plan.x_box;
   b.w_smem_bytes = plan.w_smem_bytes;
   b.x_smem_bytes = plan.x_smem_bytes;
   const size_t smem = (size_t)plan.w_smem_bytes + plan.x_smem_bytes + plan.p_smem_bytes + 1024;
-  cudaError_t e = plan.sn == 64 ? launch_t<64>(b, smem, st) : launch_t<32>(b, smem, st);
+  cudaError_t e = plan.sn == 64 ? launch_mt<64>(b, smem, st) : launch_mt<32>(b, smem, st);
   count_launch(1);
   return e;
 }
