@@ -807,7 +807,6 @@ alg_status_t run_decode(const alg_proj_s &p, const void *X, int64_t ldx, const i
   d.splits = p.decode.splits;
   d.box_rows = p.decode.box_rows;
   d.w_smem_bytes = p.decode.w_smem_bytes;
-  d.x_smem_bytes = p.decode.x_smem_bytes;
   d.status = p.d_status;
   d.wait_limit = p.wait_limit;
   d.extra_expect_bytes = p.test_extra_expect;
@@ -1380,7 +1379,8 @@ static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, c
   f->rd_ok = dtype == ALG_BF16 && schedule != ALG_SCHED_INTERVAL && f->up.big.eligible && f->down.big.eligible &&
              row_decode_fits(q, f->D, f->F);
   if (f->fd_ok || f->rd_ok) {   // (the two one-launch decode steps share the exchange)
-    f->exch_bytes = (int)align_up((size_t)(f->fd_ok ? kFfnDecodeMaxM : kRowDecodeMaxM) * f->F * 2, 256);
+    const int rows = std::max(f->fd_ok ? kFfnDecodeMaxM : 0, f->rd_ok ? kRowDecodeMaxM : 0);   // either may serve a call
+    f->exch_bytes = (int)align_up((size_t)rows * f->F * 2, 256);
     s = reset_exchange(*f);
     if (s != ALG_OK) {
       if (f->d_exch) cudaFree(f->d_exch);

@@ -252,7 +252,7 @@ struct DecodePlan {
   int box_rows;      // rows per TMA box of the weight slice (divides every s[k] / splits, <= 256)
   int x_box;         // columns per TMA box of X: 64, 32 or 16 (divides every s[k] / splits)
   int w_smem_bytes;  // worst-case weight slice of one CTA
-  int x_smem_bytes;  // worst-case staged X slice
+  int operand_bytes; // worst-case slices of W and X, at least the partial tiles that replace them
   int p_smem_bytes;  // partial sums
 };
 struct DecodeArgs {
@@ -274,7 +274,7 @@ struct DecodeArgs {
   uint32_t inv_splits;    // ceil(2^32 / splits): x / splits = umulhi(x, inv_splits) for x < 2^29, splits > 1 (set by the launcher)
   int box_rows, x_box;
   int w_smem_bytes;
-  int x_smem_bytes;
+  int operand_bytes;
   int *status;
   long long wait_limit;   // bound of every device-side wait, in SM clock cycles
   int extra_expect_bytes; // test aid: bytes added to the weight barrier's expectation that never arrive

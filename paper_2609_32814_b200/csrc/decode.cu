@@ -20,9 +20,10 @@
 // asynchronous stores that count their bytes on the owner's mbarrier, so nobody waits for a
 // barrier over the cluster.  The owner adds them in split order (deterministic, nothing goes through
 // global memory), applies bias / activation and stores Y.
-// What bounds it: latency (a launch reads 3-5 MB).  Two launches, 768 -> 3072 -> 768 at q = 2, per layer of a graph of layers: M = 17 12.9 -> 10.5 us, M = 40
-// 14.8 -> 12.6 us, M = 64 17.0 -> 14.7 us against X staged after the types with asynchronous copies, remote
-// stores and a cluster barrier, and 192 CTAs on 148 SMs.
+// What bounds it: latency (a launch reads 3-5 MB).  Two launches, 768 -> 3072 -> 768 at q = 2, per layer of a graph of
+// layers: M = 17 12.8 -> 9.6 us, M = 40 14.7 -> 10.9 us, M = 64 16.9 -> 12.5 us against X staged after the
+// types with asynchronous copies, remote stores and a cluster barrier, warps that split the columns, and
+// 192 CTAs on 148 SMs.
 #include <cuda_runtime.h>
 
 #include "tc_common.cuh"
@@ -55,20 +56,19 @@ __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t (&r)[4
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
 }
-__device__ __forceinline__ void ldmatrix_x2_trans(uint32_t addr, uint32_t (&r)[2]) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// eight bytes into the shared memory of CTA `rank` of the cluster, counted on the barrier at the same place there
-__device__ __forceinline__ void send_f32x2(uint32_t local_addr, uint32_t local_bar, uint32_t rank, float x, float y) {
+// sixteen bytes into the shared memory of CTA `rank` of the cluster, counted on the barrier at the same place there
+__device__ __forceinline__ void send_f32x4(uint32_t local_addr, uint32_t local_bar, uint32_t rank, const float4 &v) {
   uint32_t addr, bar;
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(local_addr), "r"(rank));
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(local_bar), "r"(rank));
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(addr), "f"(x), "f"(y), "r"(bar) : "memory");
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "f"(v.x), "f"(v.y),
+               "f"(v.z), "f"(v.w), "r"(bar)
+               : "memory");
 }
 
 // Shared-memory images.  W slice: [rows][SN] bf16 as the TMA writes it with its 128-byte (SN = 64)
@@ -88,7 +88,8 @@ __device__ __forceinline__ uint32_t w_off(int row, int chunk) {
 template <int SN, int MT>
 __global__ void __launch_bounds__(kThreads, 2)
 decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const DecodeArgs a) {
-  constexpr int NT = SN / 32;          // 8-column n-tiles per warp (4 warps share the strip)
+  constexpr int NT = SN / 8;           // 8-column n-tiles; the warps split k
+  constexpr int kPartPitch = SN + 8;   // floats per row of a warp's partial tile
   extern __shared__ uint8_t smem_raw[];
   __shared__ Seg s_seg[kMaxQ];
   __shared__ int s_nseg, s_rows;
@@ -136,7 +137,8 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
   const uint32_t bar = smem_u32(&s_bar), bar_x = smem_u32(&s_bar_x), bar_p = smem_u32(&s_bar_p);
   uint8_t *w_sm = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *x_sm = w_sm + (size_t)a.w_smem_bytes;
-  float *r_sm = (float *)(x_sm + (size_t)a.x_smem_bytes);   // [splits][rows owned][SN] partial sums of my rows
+  float *part = (float *)w_sm;   // [warp][row][kPartPitch] partial tiles of the warps, over the operands once they are used up
+  float *r_sm = (float *)(w_sm + (size_t)a.operand_bytes);   // [splits][rows owned][SN] partial sums of my rows
   int my_type = -1;
   // Reads the row types (L2, never a stale L1 line), derives the support of this strip and the
   // segment list, and requests the weight slice: one TMA box per segment (more when a segment
@@ -196,7 +198,7 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
   };
   // the columns of X that go with the slice; rows past M read as zero
   auto fetch_x = [&]() {
-    if (tid == 0) {
+    if (tid == 96) {   // (a thread that has no row type to read)
       const int box_bytes = kMPad * a.x_box * 2;
       mbar_expect_tx(bar_x, (uint32_t)(s_rows * kMPad * 2));
       uint32_t dst = smem_u32(x_sm);
@@ -251,7 +253,9 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
   if (landed && wait_bar(bar_x, parity)) wait_bar(bar, parity);
   DTR();
 
-  // ---- warp-level MMA: warp w owns columns [w * SN/4, +SN/4) of the strip, all rows ----
+  // ---- warp-level MMA: warp w takes the k steps w, w + 4, ... of the slice, all rows and columns ----
+  // (Splitting the columns instead, every warp read all of X: 8 KB of shared memory per k step of 48 rows x 64 columns
+  // against 3.5 KB, with 6 independent products per step against 24.)
   float acc[MT][NT][4];
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
@@ -259,11 +263,11 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[mt][nt][e] = 0.f;
+  const int g = lane >> 2, t4 = lane & 3;
   {
     const uint32_t w_base = smem_u32(w_sm);
-    const int wcol_chunk = warp * (SN / 32);  // first 16-byte chunk of this warp's columns
-    const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8, g = lane >> 2;
-    const int xb = a.x_box, x_sw = xb == 64 ? frag_row & 7 : xb == 32 ? (frag_row >> 1) & 3 : (frag_row >> 2) & 1;
+    const int frag_row = (lane & 7) + ((lane >> 3) & 1) * 8;
+    const int xb = a.x_box, xb_sh = 31 - __clz(xb), x_sw = xb == 64 ? frag_row & 7 : xb == 32 ? (frag_row >> 1) & 3 : (frag_row >> 2) & 1;
     const uint32_t x_row = smem_u32(x_sm) + (uint32_t)(frag_row * xb * 2);
     const int box_bytes = kMPad * xb * 2, x_tile = 16 * xb * 2;
     const int nseg = s_nseg;
@@ -275,59 +279,48 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
         const uint32_t rows = (mt < 2 ? sg.rows_lo : sg.rows_hi) >> (16 * (mt & 1) + g);
         keep[mt][0] = 0u - (rows & 1u), keep[mt][1] = 0u - ((rows >> 8) & 1u);
       }
-      uint32_t x_box = x_row + (uint32_t)(sg.loc0 / xb * box_bytes);
-      int c = 0;   // 16-byte chunk of the current k inside its box
-#pragma unroll 2
-      for (int k0 = sg.loc0; k0 < sg.loc0 + sg.len; k0 += 16) {
-        uint32_t b[4];
-        if (NT == 2) {
-          ldmatrix_x4_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk + (lane >> 4)), b);
-        } else {
-          uint32_t r2[2];
-          ldmatrix_x2_trans(w_base + w_off<SN>(k0 + frag_row, wcol_chunk), r2);
-          b[0] = r2[0], b[1] = r2[1], b[2] = 0, b[3] = 0;
-        }
-        uint32_t af[MT][4];
-        const uint32_t x_at = x_box + (uint32_t)(((c + (lane >> 4)) ^ x_sw) << 4);
+#pragma unroll 1
+      for (int k0 = sg.loc0 + 16 * ((warp - (sg.loc0 >> 4)) & 3); k0 < sg.loc0 + sg.len; k0 += 64) {
+        uint32_t b[NT / 2][4], af[MT][4];
+        const uint32_t x_at = x_row + (uint32_t)((k0 >> xb_sh) * box_bytes) + (uint32_t)(((((k0 & (xb - 1)) >> 3) + (lane >> 4)) ^ x_sw) << 4);
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) ldmatrix_x4(x_at + (uint32_t)(mt * x_tile), af[mt]);
+#pragma unroll
+        for (int n = 0; n < NT / 2; ++n) ldmatrix_x4_trans(w_base + w_off<SN>(k0 + frag_row, 2 * n + (lane >> 4)), b[n]);
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
           af[mt][0] &= keep[mt][0], af[mt][2] &= keep[mt][0], af[mt][1] &= keep[mt][1], af[mt][3] &= keep[mt][1];
 #pragma unroll
-          for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af[mt], b[nt * 2], b[nt * 2 + 1]);
+          for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af[mt], b[nt >> 1][(nt & 1) * 2], b[nt >> 1][(nt & 1) * 2 + 1]);
         }
-        c += 2;
-        if (c == xb >> 3) c = 0, x_box += (uint32_t)box_bytes;
       }
     }
   }
+  __syncthreads();   // the operands are used up
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt)
+        *(float2 *)(part + ((warp * kMPad + mt * 16 + h * 8 + g) * kPartPitch + nt * 8 + t4 * 2)) = make_float2(acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
+  __syncthreads();
   DTR();
   if (splits > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // long since complete
   // ---- push the partial sums to the owners of the rows: row m -> CTA m % splits, slot m / splits ----
   const int rows_owned_max = div_splits(kMPad + splits - 1);
-  {
-    const uint32_t r_base = smem_u32(r_sm);
-    const int g = lane >> 2, t4 = lane & 3;
+  for (int e = tid; e < M * (SN / 4); e += kThreads) {   // the warps' sum, four columns at a time, to the owner of the row
+    const int m = e / (SN / 4), n = (e % (SN / 4)) * 4;
+    float4 z = *(const float4 *)(part + m * kPartPitch + n);
 #pragma unroll
-    for (int mt = 0; mt < MT; ++mt) {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int m = mt * 16 + g + h * 8;
-        const int slot = div_splits(m);
-        const uint32_t owner = (uint32_t)(m - slot * splits);
-        if (m < M) {
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int col = warp * (SN / 4) + nt * 8 + t4 * 2;
-            if (splits > 1)
-              send_f32x2(r_base + (uint32_t)(((split * rows_owned_max + slot) * SN + col) * 4), bar_p, owner, acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
-            else
-              *(float2 *)(r_sm + (slot * SN + col)) = make_float2(acc[mt][nt][h * 2], acc[mt][nt][h * 2 + 1]);
-          }
-        }
-      }
+    for (int w = 1; w < 4; ++w) {
+      const float4 v = *(const float4 *)(part + (w * kMPad + m) * kPartPitch + n);
+      z.x += v.x, z.y += v.y, z.z += v.z, z.w += v.w;
     }
+    const int slot = div_splits(m);
+    float *at = r_sm + ((split * rows_owned_max + slot) * SN + n);
+    if (splits > 1) send_f32x4(smem_u32(at), bar_p, (uint32_t)(m - slot * splits), z);
+    else *(float4 *)at = z;
   }
   if (splits > 1) wait_bar(bar_p, 0);   // every partial sum of my rows has arrived
   else __syncthreads();
@@ -447,7 +440,9 @@ bool decode_plan(int q, const int *s, int K, int N, int num_sms, DecodePlan *pla
       for (int k = 0; k < q; ++k)
         while (s[k] / sp % xb) xb /= 2;
       const size_t p_bytes = (size_t)(kDecodeMaxM + 8) * sn * 4;
-      if (w_bytes + x_bytes + p_bytes + 1024 > 190 * 1024) continue;
+      const size_t part_bytes = (size_t)4 * kDecodeMaxM * (sn + 8) * 4;   // the warps' partial tiles lie over the operands
+      const size_t operand_bytes = w_bytes + x_bytes > part_bytes ? w_bytes + x_bytes : part_bytes;
+      if (operand_bytes + p_bytes + 1024 > 190 * 1024) continue;
       const int ctas = (N / sn) * sp;
       // one CTA per SM as far as that goes (two of them on some SMs take as long as two everywhere), then not
       // overshooting, then the wider strip
@@ -456,7 +451,7 @@ bool decode_plan(int q, const int *s, int K, int N, int num_sms, DecodePlan *pla
       if (score > best_score) {
         best_score = score;
         best.sn = sn, best.splits = sp, best.box_rows = box, best.x_box = xb;
-        best.w_smem_bytes = (int)w_bytes, best.x_smem_bytes = (int)x_bytes, best.p_smem_bytes = (int)p_bytes;
+        best.w_smem_bytes = (int)w_bytes, best.operand_bytes = (int)operand_bytes, best.p_smem_bytes = (int)p_bytes;
       }
     }
   }
@@ -471,8 +466,8 @@ cudaError_t launch_decode(const DecodeArgs &a, const DecodePlan &plan, cudaStrea
   b.inv_splits = (uint32_t)((0x100000000ull + (uint64_t)plan.splits - 1) / (uint64_t)plan.splits);
   b.box_rows = plan.box_rows, b.x_box = plan.x_box;
   b.w_smem_bytes = plan.w_smem_bytes;
-  b.x_smem_bytes = plan.x_smem_bytes;
-  const size_t smem = (size_t)plan.w_smem_bytes + plan.x_smem_bytes + plan.p_smem_bytes + 1024;
+  b.operand_bytes = plan.operand_bytes;
+  const size_t smem = (size_t)plan.operand_bytes + plan.p_smem_bytes + 1024;
   cudaError_t e = plan.sn == 64 ? launch_mt<64>(b, smem, st) : launch_mt<32>(b, smem, st);
   count_launch(1);
   return e;
