@@ -61,6 +61,10 @@ struct alg_proj_s {
   bool tall_ok = false;
   DevTable tab_tall;
   DevTable *d_tab_tall = nullptr;
+  // CTA pairs (256-row x 256-column tiles) by the library's choice, for batches that fill them; their tile classes
+  int pair_min_klen = 0;    // shortest reduction of a tile where the shape allows them, else 0
+  DevTable tab_pair;
+  DevTable *d_tab_pair = nullptr;
   int device = 0;
   int num_sms = 148;
   int n_workers = 1;        // persistent CTAs (or CTA pairs) of the tensor-core kernel
@@ -162,8 +166,6 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     p.tile_n = p.opt_tile_n;
   else if (p.opt_tile_n != 0)
     return ALG_ERR_UNSUPPORTED_SHAPE;
-  // CTA-pair kernel whenever every output group splits into 256-wide tiles plus a 128-wide rest
-  // (measured: it wins only when every tile has a long K loop; short loops favour the one-CTA kernel)
   int min_klen = 1 << 30;
   for (int pr = 0; pr < q * q; ++pr) {
     int len = 0;
@@ -171,7 +173,7 @@ alg_status_t configure_kernels(alg_proj_s &p) {
       if ((p.tab.keep[pr] >> k) & 1u) len += p.s[k];
     min_klen = std::min(min_klen, len);
   }
-  p.pair_kernel = p.tc_ok && all128 && min_klen >= 4096;
+  p.pair_kernel = false;
   if (p.gated && !(p.tc_ok && all128)) {
     // hidden groups off the 128-column grid: only the large-algebra kernel has a gated form for them (the caller
     // checks that the handle fits it)
@@ -182,13 +184,17 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     p.tile_n = 128;
     p.pair_kernel = false;
   }
-  if (p.w_kmajor || p.dyn_segments) p.pair_kernel = false;   // the gradient passes run on the one-CTA kernel
-  if (p.sched == ALG_SCHED_INTERVAL) p.pair_kernel = false;  // runs of a type are read in place by the one-CTA kernel only
-  if (p.opt_kernel == 1) p.pair_kernel = false;
   if (p.opt_kernel == 2) {
     if (!(p.tc_ok && all128)) return ALG_ERR_UNSUPPORTED_SHAPE;
     p.pair_kernel = true;
   }
+  // CTA pairs by the library's choice (use_pairs decides per call): output groups that split into 256-wide tiles, or
+  // reductions so long that a 128-wide rest does not matter.  The gradient passes and the interval schedule (runs of a
+  // type read in place) exist on the one-CTA kernel only.
+  p.pair_min_klen = 0;
+  if (p.tc_ok && !p.gated && !p.w_kmajor && !p.dyn_segments && p.sched != ALG_SCHED_INTERVAL && p.opt_kernel == 0 && p.opt_tile_n == 0 &&
+      ((all256 && min_klen >= 512) || (all128 && min_klen >= 4096)))
+    p.pair_min_klen = min_klen;
 
   alg_status_t bs = build_classes(p, tile_n_of(p), p.tab);
   if (bs != ALG_OK) return bs;
@@ -206,6 +212,11 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     if (bs != ALG_OK) return bs;
   }
 
+  if (p.pair_min_klen) {
+    p.tab_pair = p.tab;
+    bs = build_classes(p, kTc2TileN, p.tab_pair);
+    if (bs != ALG_OK) return bs;
+  }
   return ALG_OK;
 }
 
@@ -333,6 +344,8 @@ alg_status_t init_proj(alg_proj_s &p, int q, const int32_t *in_w, const int32_t 
   if (cudaMemcpy(p.d_tab, &p.tab, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMalloc(&p.d_tab_tall, sizeof(DevTable)) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemcpy(p.d_tab_tall, &p.tab_tall, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
+  if (cudaMalloc(&p.d_tab_pair, sizeof(DevTable)) != cudaSuccess) return ALG_ERR_CUDA;
+  if (cudaMemcpy(p.d_tab_pair, &p.tab_pair, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
   if (shared_status) {
     p.d_status = shared_status;
     p.shared_status = true;
@@ -375,6 +388,8 @@ void free_proj(alg_proj_s &p) {
   if (p.d_tab) cudaFree(p.d_tab);
   if (p.d_tab_tall) cudaFree(p.d_tab_tall);
   p.d_tab_tall = nullptr;
+  if (p.d_tab_pair) cudaFree(p.d_tab_pair);
+  p.d_tab_pair = nullptr;
   if (p.d_status && !p.shared_status) cudaFree(p.d_status);
   p.d_tab = nullptr;
   p.d_status = nullptr;
@@ -423,12 +438,29 @@ struct TcChoice {
   int tile_m, tile_n;
   const DevTable *tab;   // host copy with the tile classes of this tiling
   const DevTable *d_tab;
+  bool pair;             // CTA pairs
 };
+// CTA pairs need two thirds of the operand bytes of one-CTA 128 x 256 tiles, but a stage's round trip through two SMs is
+// longer, so they want reductions of at least 512, enough 256 x 256 tiles for the 74 pairs and row types that fill
+// them.  Measured one CTA / pairs, one projection, us: 4096 -> 16384 at q = 4 (reductions of 1024 and 2048), M = 32768
+// 1459 / 1255; 8192 -> 2048 at q = 4 (2048, 4096), M = 8192 100.6 / 89.3, M = 2048 (64 tiles) 31.6 / 31.6; 4096 -> 1024
+// at q = 4 (1024, 2048), M = 16384 56.7 / 51.9, M = 4096 (64 tiles) 18.6 / 19.6; 1024 -> 4096 at q = 2 (512, 1024),
+// M = 8192 48.7 / 47.4, M = 2048 (128 tiles) 17.4 / 19.9; reductions of 256: 2048 -> 8192 at q = 8, M = 32768
+// 280.7 / 290.6.  With explicit types every type ends in a ragged tile, half of 256 rows on average, which eats the gain
+// at 1024 rows a type (FFN 4096 -> 16384 at q = 16, M = 16384: 605 / 616).
+bool use_pairs(const alg_proj_s &p, int64_t M) {
+  if (!p.pair_min_klen) return false;
+  const int64_t tiles = ceil_div((int)M, kTc2TileM) * (int64_t)ceil_div(p.N, kTc2TileN);
+  const bool ragged = p.sched == ALG_SCHED_EXPLICIT;
+  if (p.pair_min_klen >= 1024) return tiles >= 96 && M / p.q >= (ragged ? 2048 : 256);
+  return tiles >= 192 && M / p.q >= (ragged ? 2048 : 512);
+}
 // 256-row tiles pay when every row type fills several of them (a ragged last tile then wastes
 // little); with explicit types the rows per type are not known on the host: assume an even mix.
 TcChoice choose_tiling(const alg_proj_s &p, int64_t M) {
-  if (p.tall_ok && (p.opt_kernel == 3 || M / p.q >= 1024)) return {256, 128, &p.tab_tall, p.d_tab_tall};
-  return {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab};
+  if (p.tall_ok && (p.opt_kernel == 3 || M / p.q >= 1024)) return {256, 128, &p.tab_tall, p.d_tab_tall, false};
+  if (use_pairs(p, M)) return {kTc2TileM, kTc2TileN, &p.tab_pair, p.d_tab_pair, true};
+  return {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, p.pair_kernel};
 }
 
 // Host twin of the in-kernel tile enumeration for the cyclic schedule (equal buckets of M/q rows):
@@ -441,7 +473,7 @@ TcChoice choose_tiling(const alg_proj_s &p, int64_t M) {
 // not depend on handle state that later calls rewrite), when every slot's last upload is still in
 // flight, or when the sequences do not fit.
 const PlanSlot *prepare_cyclic_plan(alg_proj_s &p, const TcChoice &tc, int64_t M, cudaStream_t st) {
-  if (!p.opt_host_plan || p.pair_kernel || !p.plan[0].d) return nullptr;
+  if (!p.opt_host_plan || tc.pair || !p.plan[0].d) return nullptr;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return nullptr;
   ++p.plan_clock;
@@ -629,7 +661,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
   a.w_kmajor = p.w_kmajor ? 1 : 0;
   a.dyn_so = nullptr;
   a.seg_rows = 0;
-  a.block_k = block_k_of(p);
+  a.block_k = tc.pair ? kTcBlockK : block_k_of(p);
   a.y_staged = 0;
   a.plan = nullptr;
   a.plan_stride = a.plan_rounds = a.plan_tag = 0;
@@ -647,7 +679,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
     if (x_bucketed || cyclic) {
       a.X = X;
       a.ldx = ldx;
-    } else if (p.opt_row_gather == 2 && !p.pair_kernel && !p.w_kmajor && !p.dyn_segments && block_k_of(p) == 64) {
+    } else if (p.opt_row_gather == 2 && !tc.pair && !p.w_kmajor && !p.dyn_segments && block_k_of(p) == 64) {
       // explicit types: the producer warps of the one-CTA kernel fetch the rows of a tile through the permutation,
       // four per copy instruction; X is read in place and no bucketed copy is written.  An option, not the
       // default: the copy engine needs longer for gathered rows than for a box (reductions of 1024..2048 columns:
@@ -668,7 +700,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
     }
     if (after_gather) cudaEventRecord(after_gather, st);
     if (p.gated) return cuda_status(launch_proj_tc_gated(a, p.n_workers, st));
-    if (p.pair_kernel) return cuda_status(launch_proj_tc2(a, p.num_sms, st));
+    if (tc.pair) return cuda_status(launch_proj_tc2(a, p.num_sms, st));
     return cuda_status(launch_proj_tc(a, tc.tile_n, p.n_workers, st));
   }
   if (p.gated) return ALG_ERR_UNSUPPORTED_SHAPE;
@@ -877,6 +909,7 @@ static alg_status_t set_option(alg_proj_s &p, alg_option_t option, int64_t value
       // the device copy of the table may still be read by kernels in flight
       if (cudaDeviceSynchronize() != cudaSuccess) return ALG_ERR_CUDA;
       if (cudaMemcpy(p.d_tab, &p.tab, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
+      if (cudaMemcpy(p.d_tab_pair, &p.tab_pair, sizeof(DevTable), cudaMemcpyHostToDevice) != cudaSuccess) return ALG_ERR_CUDA;
       return cuda_status(cudaMemcpy(p.d_tab_tall, &p.tab_tall, sizeof(DevTable), cudaMemcpyHostToDevice));
     }
     case ALG_OPT_STAGE_K:
@@ -1289,7 +1322,7 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   }
   // 3. the grouped GEMM: rows = input features (type = their group), reduction over the padded buckets
   ProjArgs a;
-  const TcChoice tc = {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab};
+  const TcChoice tc = {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, false};
   const DevTable &tab = p.tab;
   a.tab = tc.d_tab;
   a.offsets = h->d_feat_offsets;

@@ -470,3 +470,22 @@ def test_f32_buckets_tiles_and_copies(q, M, s, r, schedule):
     if bad is not None:
         ref[bad] = 0
     assert np.array_equal(H.to_np(Y), ref)
+
+
+# ---- CTA pairs by the library's choice: batches on both sides of the rule ---------------------------------------------
+
+@pytest.mark.parametrize("schedule,M", [("cyclic", 6144), ("cyclic", 5888), ("explicit", 6145), ("explicit", 4000)])
+def test_pair_choice_is_exact_on_both_sides_of_the_rule(schedule, M):
+    q, s, r = 2, 512, 1024                        # reductions of 512 and 1024, eight 256-wide tiles per 256 rows
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    wl = _tc_workload(q, M, s, r, types=types, seed=61)
+    X, W = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16")
+    tt = None if schedule == "cyclic" else H.dev_types(types)
+    proj = binding.Proj([s] * q, [r] * q, schedule=schedule)
+    got = proj.forward(X, tt, W, out_dtype=torch.float32)
+    assert proj.last_status() == 0
+    rows = np.unique(np.r_[0:40, M // 2:M // 2 + 40, M - 40:M])
+    ref = oracle.proj(wl.X[rows], types[rows], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(got[torch.from_numpy(rows).cuda()]), ref)
+    proj.set_option("gemm_kernel", 1)             # the one-CTA kernel: same integers everywhere
+    assert torch.equal(got, proj.forward(X, tt, W, out_dtype=torch.float32))
