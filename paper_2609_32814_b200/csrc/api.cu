@@ -59,9 +59,11 @@ struct alg_proj_s {
   bool w_kmajor = false;    // input-gradient pass: W (N x K here) is used transposed
   bool dyn_segments = false;  // weight-gradient pass: the reduction segments are the padded row buckets of the call
   bool tall_ok = false;
+  bool all128 = false, all256 = false;   // every output group is a multiple: tab_tall / tab_pair hold classes of one width
   DevTable tab_tall;
   DevTable *d_tab_tall = nullptr;
   // CTA pairs (256-row x 256-column tiles) by the library's choice, for batches that fill them; their tile classes
+  int max_klen = 0, max_groups = 0;   // longest reduction of a tile: columns, input groups
   int pair_min_klen = 0;    // shortest reduction of a tile where the shape allows them, else 0
   DevTable tab_pair;
   DevTable *d_tab_pair = nullptr;
@@ -172,6 +174,7 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     for (int k = 0; k < q; ++k)
       if ((p.tab.keep[pr] >> k) & 1u) len += p.s[k];
     min_klen = std::min(min_klen, len);
+    p.max_klen = std::max(p.max_klen, len), p.max_groups = std::max(p.max_groups, __builtin_popcount(p.tab.keep[pr]));
   }
   p.pair_kernel = false;
   if (p.gated && !(p.tc_ok && all128)) {
@@ -206,13 +209,13 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     p.pair_kernel = false;
     p.tall_ok = true;
   }
-  if (p.tall_ok) {
+  p.all128 = p.tc_ok && all128, p.all256 = p.tc_ok && all256;
+  if (p.all128) {
     p.tab_tall = p.tab;
     bs = build_classes(p, 128, p.tab_tall);
     if (bs != ALG_OK) return bs;
   }
-
-  if (p.pair_min_klen) {
+  if (p.pair_min_klen || p.all256) {
     p.tab_pair = p.tab;
     bs = build_classes(p, kTc2TileN, p.tab_pair);
     if (bs != ALG_OK) return bs;
@@ -455,6 +458,44 @@ bool use_pairs(const alg_proj_s &p, int64_t M) {
   if (p.pair_min_klen >= 1024) return tiles >= 96 && M / p.q >= (ragged ? 2048 : 256);
   return tiles >= 192 && M / p.q >= (ragged ? 2048 : 512);
 }
+// Few output tiles: clusters of CTAs share a tile and split its reduction (proj_split.cu).
+struct SplitChoice {
+  int splits = 1, tile_n = 0;
+  const DevTable *tab = nullptr, *d_tab = nullptr;
+};
+// m_tiles = expected 128-row tiles of the launch over all row types, stages = 64-deep stages of its longest reduction.
+// Compares the cycles of the longest chain, (stages of a CTA) x (cycles of a stage) + epilogue + the exchange, over tile
+// widths and 1, 2, 4 or 8 CTAs per tile; a choice needs its clusters resident at once (one CTA per SM, clusters of 4 and 8
+// leave some SMs of a GPC over).  Stage cycles are what the copy engine takes for the rows of a stage (about 1.75 a row).
+// Measured, whole FFN, one CTA per tile / split, us: 768 -> 3072 at q = 2, M = 700 35.4 / 29.0, M = 1777 40.8 / 36.5;
+// 1024 -> 4096 at q = 2, M = 1000 48.5 / 42.2, M = 2000 53.1 / 48.2; forward and both gradients 768 -> 3072 at q = 2,
+// M = 8003 174.0 / 168.5.
+SplitChoice choose_split(const alg_proj_s &p, int64_t m_tiles, int64_t stages, bool act) {
+  SplitChoice best;
+  if (!use_tc(p) || p.gated || p.pair_kernel || p.opt_kernel != 0 || p.sched == ALG_SCHED_INTERVAL || p.opt_stage_k == 32 ||
+      (p.opt_tile_n != 0 && !p.dyn_segments) || p.opt_row_gather == 2)
+    return best;
+  struct { int tile_n; const DevTable *tab, *d_tab; bool on; } width[3] = {
+      {256, &p.tab_pair, p.d_tab_pair, p.all256}, {192, &p.tab, p.d_tab, p.tile_n == 192}, {128, &p.tab_tall, p.d_tab_tall, p.all128}};
+  double best_cost = 1e30;
+  for (const auto &w : width) {
+    if (!w.on) continue;
+    const int64_t tiles = m_tiles * (p.N / w.tile_n);
+    for (int s = 1; s <= 8; s *= 2) {
+      const int resident = s == 1 ? 148 : s == 2 ? 74 : s == 4 ? 33 : 15;
+      if (s == 8 && w.tile_n == 192) continue;
+      if (s > 1 && (tiles > resident || stages < 2 * s)) continue;
+      const int64_t rounds = (tiles + resident - 1) / resident;
+      const double stage = w.tile_n == 256 ? 672 : w.tile_n == 192 ? 560 : 450;
+      const double cost = rounds * ((double)((stages + s - 1) / s) * stage) + w.tile_n * (act ? 16.0 : 8.0) / s + (s > 1 ? 2000 : 0);
+      if (cost < best_cost * 0.97) {
+        best_cost = cost;
+        best.splits = s, best.tile_n = w.tile_n, best.tab = w.tab, best.d_tab = w.d_tab;
+      }
+    }
+  }
+  return best;
+}
 // 256-row tiles pay when every row type fills several of them (a ragged last tile then wastes
 // little); with explicit types the rows per type are not known on the host: assume an even mix.
 TcChoice choose_tiling(const alg_proj_s &p, int64_t M) {
@@ -548,9 +589,12 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // (at most two 128-row tiles per type on average) -- there the table-driven kernel spends its time on tile
 // records and half-empty tiles (4096 -> 12288 at q = 32, M = 2048: 95.7 -> 70.1 us; FFN 187.6 -> 139.0 us),
 // while with large buckets its tuned main loop and epilogue win (q = 8, M = 16384 FFN: 125.9 against 138.3 us).
+// With up to 8 groups the table-driven kernels are the better ones for small batches too, now that clusters split the
+// few tiles' reductions: FFN 768 -> 3072 at q = 2, M = 100 / 300 / 500: 38.3 / 39.4 / 39.1 us here, 22.3 / 27.2 / 27.8 there;
+// 1024 -> 4096 at q = 8, M = 300 / 1900: 30.7 / 40.5 here, 27.5 / 36.7 there.
 bool use_big_counted(const alg_proj_s &p, int64_t M) {
   if (p.big.repack) return false;
-  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && M <= 256 * (int64_t)p.q);
+  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok) && M <= 256 * (int64_t)p.q);
 }
 // Equal buckets (cyclic schedule, q | M): by the library's choice when a type has at most 128 rows -- the
 // large-algebra kernel then packs several types into a tile (FFN 4096 -> 12288 -> 4096 at q = 32, M = 2048:
@@ -558,7 +602,7 @@ bool use_big_counted(const alg_proj_s &p, int64_t M) {
 // FFN at M = 8192).
 bool use_big_equal(const alg_proj_s &p, int64_t M) {
   if (p.big.repack) return false;
-  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && M <= 128 * (int64_t)p.q);
+  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok) && M <= 128 * (int64_t)p.q);
 }
 
 
@@ -625,7 +669,12 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
     return cuda_status(launch_proj_big(g, p.num_sms, st));
   }
   ProjArgs a;
-  const TcChoice tc = choose_tiling(p, M);
+  TcChoice tc = choose_tiling(p, M);
+  SplitChoice sp;
+  if (!tc.pair && !run_rows) {
+    sp = choose_split(p, (int64_t)p.q * ((M + (int64_t)p.q * 128 - 1) / ((int64_t)p.q * 128)), p.max_klen / 64, act != ALG_ACT_NONE);
+    if (sp.splits > 1) tc = {128, sp.tile_n, sp.tab, sp.d_tab, false};
+  }
   const DevTable &tab = *tc.tab;
   a.tab = tc.d_tab;
   a.offsets = cyclic ? nullptr : ((const WsHeader *)(ws + L.hdr))->offsets;
@@ -666,7 +715,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
   a.plan = nullptr;
   a.plan_stride = a.plan_rounds = a.plan_tag = 0;
   a.wait_limit = p.wait_limit;
-  if (cyclic) {
+  if (cyclic && sp.splits == 1) {
     if (const PlanSlot *sl = prepare_cyclic_plan(p, tc, M, st)) {
       a.plan = sl->d;
       a.plan_stride = p.plan_stride;
@@ -701,6 +750,10 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
     if (after_gather) cudaEventRecord(after_gather, st);
     if (p.gated) return cuda_status(launch_proj_tc_gated(a, p.n_workers, st));
     if (tc.pair) return cuda_status(launch_proj_tc2(a, p.num_sms, st));
+    if (sp.splits > 1) {
+      const int64_t m_tiles = cyclic ? p.q * ((M / p.q + 127) / 128) : (M + 127 * (int64_t)p.q) / 128;   // at most
+      return cuda_status(launch_proj_split(a, sp.tile_n, sp.splits, (int)(m_tiles * (p.N / sp.tile_n)), st));
+    }
     return cuda_status(launch_proj_tc(a, tc.tile_n, p.n_workers, st));
   }
   if (p.gated) return ALG_ERR_UNSUPPORTED_SHAPE;
@@ -1322,8 +1375,12 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   }
   // 3. the grouped GEMM: rows = input features (type = their group), reduction over the padded buckets
   ProjArgs a;
-  const TcChoice tc = {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, false};
-  const DevTable &tab = p.tab;
+  TcChoice tc = {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, false};
+  int64_t m_tiles = 0;   // 128-row tiles of the feature groups
+  for (int e = 0; e < p.q; ++e) m_tiles += (h->dx.r[e] + 127) / 128;
+  const SplitChoice sp = choose_split(p, m_tiles, p.max_groups * ((M / p.q + 63) / 64), false);
+  if (sp.splits > 1) tc = {128, sp.tile_n, sp.tab, sp.d_tab, false};
+  const DevTable &tab = *tc.tab;
   a.tab = tc.d_tab;
   a.offsets = h->d_feat_offsets;
   a.cyclic_rows = 0;
@@ -1366,6 +1423,7 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   a.plan = nullptr;
   a.plan_stride = a.plan_rounds = a.plan_tag = 0;
   a.wait_limit = p.wait_limit;
+  if (sp.splits > 1) return cuda_status(launch_proj_split(a, sp.tile_n, sp.splits, (int)(m_tiles * (p.N / sp.tile_n)), st));
   return cuda_status(launch_proj_tc(a, tc.tile_n, p.n_workers, st));
 }
 

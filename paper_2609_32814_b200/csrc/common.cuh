@@ -239,6 +239,9 @@ constexpr int kTc2TileN = 256;
 cudaError_t launch_proj_tc(const ProjArgs &a, int tile_n, int num_sms, cudaStream_t st);
 cudaError_t launch_proj_tc_gated(const ProjArgs &a, int num_sms, cudaStream_t st);  // 128 output columns per tile
 cudaError_t launch_proj_tc2(const ProjArgs &a, int num_sms, cudaStream_t st);
+// few tiles: clusters of `splits` CTAs (2, 4, 8) share a 128 x tile_n tile (128, 192, 256) and split its reduction;
+// `tiles` = upper bound of the tile count
+cudaError_t launch_proj_split(const ProjArgs &a, int tile_n, int splits, int tiles, cudaStream_t st);
 int tc2_max_pairs(int num_sms);  // CTA pairs that can be co-resident (0 on failure)
 constexpr int kMaxWorkers = 256;
 cudaError_t tc_init();  // resolves the driver entry point for tensor-map encoding

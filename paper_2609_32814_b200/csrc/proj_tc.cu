@@ -565,37 +565,9 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   int smem_bytes = C::kFixedSmemBytes + (int)tile_map_bytes(a.n_classes);
   if (smem_bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
   CUtensorMap tmA, tmB;
-  cudaError_t e;
   ProjArgs b = a;
-  if (a.seg_rows) {
-    // X and G as {columns, type, position in the type}: rows t, t + q, ... are the reduction segment of type t
-    if (GATED || a.w_kmajor || TILE_M != 128 || BK != 64) return cudaErrorInvalidValue;
-    const uint64_t da[3] = {(uint64_t)a.M, (uint64_t)a.q, (uint64_t)a.seg_rows};
-    const uint64_t sa[2] = {(uint64_t)a.ldx * 2, (uint64_t)a.ldx * 2 * (uint64_t)a.q};
-    const uint64_t db[3] = {(uint64_t)a.N, (uint64_t)a.q, (uint64_t)a.seg_rows};
-    const uint64_t sb[2] = {(uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.q};
-    const uint32_t box[3] = {64, 1, 64};
-    e = make_map_nd(&tmA, a.X, 3, da, sa, box, 128);
-    if (e == cudaSuccess) e = make_map_nd(&tmB, a.W, 3, db, sb, box, 128);
-    if (e != cudaSuccess) return e;
-    b.b_3d = 0;
-  } else {
-  e = make_map_a(&tmA, a);
+  cudaError_t e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
   if (e != cudaSuccess) return e;
-  if (a.w_kmajor) {   // W is N x K here (rows = output columns, contiguous along the reduction): boxes of 64 x TILE_N
-    if (GATED) return cudaErrorInvalidValue;
-    b.b_3d = 0;
-    e = make_map_2d_sw(&tmB, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.ldw * 2, BK, TILE_N, BK * 2);
-    if (e != cudaSuccess) return e;
-  } else {
-    b.b_3d = make_map_b3d(&tmB, a, GATED ? 2 : TILE_N / 64) == cudaSuccess;
-  }
-  if (GATED && !b.b_3d) return cudaErrorInvalidValue;
-  if (!b.b_3d && !a.w_kmajor) {
-    e = make_map_2d(&tmB, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.ldw * 2, 64, BK);
-    if (e != cudaSuccess) return e;
-  }
-  }
   // staging buffers for the transposing epilogue, when they fit and the output rows are 16-byte aligned
   b.y_staged = !GATED && a.y_bf16 && smem_bytes + kEpiWarps * C::kStoreBufBytes <= 227 * 1024 && ((uintptr_t)a.Y & 15u) == 0 &&
                (a.ldy * 2) % 16 == 0;
@@ -629,6 +601,32 @@ cudaError_t launch_t(const ProjArgs &a, int num_sms, cudaStream_t st) {
 }  // namespace
 
 namespace tc {
+// Tensor maps of both operands of the one-CTA kernels; sets a->b_3d.
+cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int tile_n, int tile_m, bool gated, int bk) {
+  a->b_3d = 0;
+  if (a->seg_rows) {
+    // X and G as {columns, type, position in the type}: rows t, t + q, ... are the reduction segment of type t
+    if (gated || a->w_kmajor || tile_m != 128 || bk != 64) return cudaErrorInvalidValue;
+    const uint64_t da[3] = {(uint64_t)a->M, (uint64_t)a->q, (uint64_t)a->seg_rows};
+    const uint64_t sa[2] = {(uint64_t)a->ldx * 2, (uint64_t)a->ldx * 2 * (uint64_t)a->q};
+    const uint64_t db[3] = {(uint64_t)a->N, (uint64_t)a->q, (uint64_t)a->seg_rows};
+    const uint64_t sb[2] = {(uint64_t)a->ldw * 2, (uint64_t)a->ldw * 2 * (uint64_t)a->q};
+    const uint32_t box[3] = {64, 1, 64};
+    const cudaError_t e = make_map_nd(tmA, a->X, 3, da, sa, box, 128);
+    return e == cudaSuccess ? make_map_nd(tmB, a->W, 3, db, sb, box, 128) : e;
+  }
+  const cudaError_t e = make_map_a(tmA, *a);
+  if (e != cudaSuccess) return e;
+  if (a->w_kmajor) {   // W is N x K here (rows = output columns, contiguous along the reduction): boxes of 64 x tile_n
+    if (gated) return cudaErrorInvalidValue;
+    return make_map_2d_sw(tmB, a->W, (uint64_t)a->K, (uint64_t)a->N, (uint64_t)a->ldw * 2, (uint32_t)bk, (uint32_t)tile_n, bk * 2);
+  }
+  a->b_3d = make_map_b3d(tmB, *a, gated ? 2 : tile_n / 64) == cudaSuccess;
+  if (a->b_3d) return cudaSuccess;
+  if (gated) return cudaErrorInvalidValue;
+  return make_map_2d(tmB, a->W, (uint64_t)a->N, (uint64_t)a->K, (uint64_t)a->ldw * 2, 64, (uint32_t)bk);
+}
+
 cudaError_t make_map_2d_sw(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_bytes,
                            uint32_t box_inner, uint32_t box_outer, int swizzle_bytes) {
   cudaError_t e0 = tc_init();

@@ -236,6 +236,7 @@ cudaError_t make_map_nd(CUtensorMap *map, const void *base, int rank, const uint
 // {K, q, M/q} of X with strides {ld, q*ld} and a box of 64 x 1 x 128 (same shared-memory image).
 cudaError_t make_map_a(CUtensorMap *map, const ProjArgs &a);
 cudaError_t make_map_b3d(CUtensorMap *map, const ProjArgs &a, int chunks);
+cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int tile_n, int tile_m, bool gated, int bk);
 
 }  // namespace tc
 }  // namespace algproj

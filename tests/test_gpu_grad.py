@@ -102,3 +102,23 @@ def test_grad_refusals():
     with pytest.raises(binding.AlgError) as e:
         binding.ProjGrad([64, 64], [72, 72])      # output groups the tensor-core tiles do not divide
     assert e.value.code == 2
+
+
+@pytest.mark.parametrize("q,M,s_w,r_w,schedule", [
+    (2, 1024, 384, 1536, "cyclic"),      # dW in place, 72 tiles of 256 columns
+    (2, 1000, 384, 1536, "explicit"),    # dW through the padded copies, dX too
+    (2, 300, 256, 256, "explicit"),      # four and eight CTAs per tile
+    (4, 512, 128, 256, "cyclic"),
+])
+def test_grad_maps_on_split_reductions(q, M, s_w, r_w, schedule):
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    X, G = synth.small_ints(1, (M, q * s_w), -1, 1), synth.small_ints(2, (M, q * r_w), -1, 1)
+    W = synth.small_ints(3, (q * s_w, q * r_w), -1, 1)
+    grad = binding.ProjGrad([s_w] * q, [r_w] * q, schedule=schedule)
+    tt = None if schedule == "cyclic" else H.dev_types(types)
+    dX = grad.grad_input(H.to_dev(G, "bf16"), tt, H.to_dev(W, "bf16"), out_dtype=torch.float32)
+    dW = grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), tt)
+    assert grad.last_status() == 0
+    widths = [s_w] * q, [r_w] * q
+    assert np.array_equal(H.to_np(dX), oracle.proj_vjp_x(G, types, W, *widths))
+    assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X, G, types, *widths))

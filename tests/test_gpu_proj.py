@@ -489,3 +489,52 @@ def test_pair_choice_is_exact_on_both_sides_of_the_rule(schedule, M):
     assert np.array_equal(H.to_np(got[torch.from_numpy(rows).cuda()]), ref)
     proj.set_option("gemm_kernel", 1)             # the one-CTA kernel: same integers everywhere
     assert torch.equal(got, proj.forward(X, tt, W, out_dtype=torch.float32))
+
+
+# ---- clusters that split a tile's reduction (few output tiles): 2, 4 and 8 CTAs per tile, 256-, 192- and 128-wide tiles,
+# ragged, absent and out-of-range types, short reductions, every kind of result ----------------------------------------
+
+@pytest.mark.parametrize("q,M,s_w,r_w", [
+    (2, 1500, 1536, 384),    # two CTAs, 192 wide, 24 and 48 stages
+    (2, 600, 1536, 384),     # four
+    (2, 130, 1536, 512),     # eight, one full and one nearly empty tile per type
+    (1, 140, 1024, 256),     # eight, 256 wide: one type, 16 stages
+    (2, 700, 256, 1024),     # short reductions: 4 and 8 stages
+    (3, 390, 192, 128),      # 3 and 6 stages, 128 wide
+    (4, 900, 512, 256),
+])
+@pytest.mark.parametrize("schedule", ["explicit", "cyclic"])
+def test_split_reduction_is_exact(q, M, s_w, r_w, schedule):
+    if schedule == "cyclic":
+        M = M // q * q
+        types = synth.cyclic_types(M, q)
+    else:
+        types = synth.uniform_types(17 * q + M, M, q)
+        if q == 4:
+            types[types == 2] = 0                 # a type without rows
+    wl = _tc_workload(q, M, s_w, r_w, types=types, seed=71)
+    wl.W_up[:] = np.sign(wl.W_up)                 # results stay below 2^24 and, for the activation, small
+    bias = synth.small_ints(72, (q * r_w,))
+    X, W, b = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.to_dev(bias, "bf16")
+    tt = None
+    bad = None
+    if schedule == "explicit":
+        bad = M // 3
+        t2 = types.copy()
+        t2[bad] = -1
+        tt = H.dev_types(t2)
+    proj = binding.Proj([s_w] * q, [r_w] * q, schedule=schedule)
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths, bias=bias)
+    if bad is not None:
+        ref[bad] = 0
+    for out_dtype in (torch.float32, torch.bfloat16):
+        got = H.to_np(proj.forward(X, tt, W, bias=b, out_dtype=out_dtype))
+        assert np.array_equal(got, ref if out_dtype == torch.float32 else H.bf16_rne(ref))
+    assert proj.last_status() == (0 if bad is None else 5)
+    again = proj.forward(X, tt, W, bias=b, act="gelu", out_dtype=torch.float32)
+    assert torch.equal(again, proj.forward(X, tt, W, bias=b, act="gelu", out_dtype=torch.float32))   # bitwise repeatable
+    g = H.to_np(again)
+    want = oracle.gelu_array(ref)
+    if bad is not None:
+        want[bad] = 0
+    assert np.abs(g - want).max() <= 1e-6 * (1 + np.abs(want).max())   # the GELU's own error is below 1e-7 |z|
