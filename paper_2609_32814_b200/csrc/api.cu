@@ -643,7 +643,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
     BigArgs g;
     g.X = X, g.ldx = ldx;
     if (!x_bucketed) {
-      if (launch_gather_rows(X, ldx, (const int *)(ws + L.perm), (int)M, p.K, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
+      if (launch_gather_rows(X, ldx, (const int *)(ws + L.perm), (int)M, p.K, 2, ws + L.xb, p.d_status, p.wait_limit, st) != cudaSuccess) return ALG_ERR_CUDA;
       g.X = ws + L.xb, g.ldx = p.K;
     }
     if (after_gather) cudaEventRecord(after_gather, st);
@@ -709,7 +709,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
   a.gated_f = p.gated ? p.N : 0;
   a.w_kmajor = p.w_kmajor ? 1 : 0;
   a.dyn_so = nullptr;
-  a.seg_rows = 0;
+  a.a_mn = 0, a.seg_rows = 0;
   a.block_k = tc.pair ? kTcBlockK : block_k_of(p);
   a.y_staged = 0;
   a.plan = nullptr;
@@ -742,7 +742,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
       // the GEMM's producer warps fetch the rows through the permutation themselves, with 16-byte
       // asynchronous copies into the swizzled image, was measured slower: the up projection of the
       // q = 4, M = 16384 configuration took 49 us against 36 us + 9 us for the copy.)
-      cudaError_t e = launch_gather_rows(X, ldx, (const int *)(ws + L.perm), (int)M, p.K, 2, ws + L.xb, st);
+      cudaError_t e = launch_gather_rows(X, ldx, (const int *)(ws + L.perm), (int)M, p.K, 2, ws + L.xb, p.d_status, p.wait_limit, st);
       if (e != cudaSuccess) return ALG_ERR_CUDA;
       a.X = ws + L.xb;
       a.ldx = p.K;
@@ -848,7 +848,7 @@ alg_status_t run_big(alg_proj_s &p, const WsLayout &L, char *ws, const void *X, 
     if (launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
     a.sched = 0;
     if (!p.big.repack) {   // (the repacking pass below gathers the rows itself)
-      if (launch_gather_rows(X, ldx, b.perm, (int)M, p.K, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
+      if (launch_gather_rows(X, ldx, b.perm, (int)M, p.K, 2, ws + L.xb, p.d_status, p.wait_limit, st) != cudaSuccess) return ALG_ERR_CUDA;
       a.X = ws + L.xb, a.ldx = p.K;
     }
     a.offsets = (const int *)(ws + L.hdr);   // WsHeader starts with its offsets
@@ -1292,7 +1292,7 @@ alg_status_t alg_proj_grad_destroy(alg_proj_grad_t h) {
 namespace {
 int padded_rows(const alg_proj_grad_s &g, int64_t M) { return (int)((M + 63) / 64 * 64) + 64 * g.q; }
 struct GradLayout {
-  size_t hdr, chunks, perm, xt, gp, total;
+  size_t hdr, chunks, perm, xp, gp, total;
 };
 GradLayout grad_layout(const alg_proj_grad_s &g, int64_t M) {
   GradLayout L;
@@ -1304,7 +1304,7 @@ GradLayout grad_layout(const alg_proj_grad_s &g, int64_t M) {
   L.perm = off;
   off = align_up(off + (size_t)M * sizeof(int));
   const size_t mp = (size_t)padded_rows(g, M);
-  L.xt = off;
+  L.xp = off;
   off = align_up(off + mp * g.K * 2, 1024);
   L.gp = off;
   off = align_up(off + mp * g.N * 2, 1024);
@@ -1348,7 +1348,10 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   // Cyclic schedule with whole 64-row blocks per type: the buckets are rows t, t + q, ... of X and of G as they
   // lie in memory, nothing is counted, permuted, transposed or copied (the kernel reads both through
   // type-strided views and takes the X block as an MN-major A operand).
-  const bool in_place = h->sched == ALG_SCHED_CYCLIC && M > 0 && M % (64 * (int64_t)h->q) == 0 && block_k_of(p) == 64;
+  // (tiled copies of feature columns start on 16 bytes: groups of a multiple of 8 features)
+  bool mn = true;
+  for (int e = 0; e < h->q; ++e) mn = mn && h->dx.r[e] % 8 == 0;
+  const bool in_place = mn && h->sched == ALG_SCHED_CYCLIC && M > 0 && M % (64 * (int64_t)h->q) == 0 && block_k_of(p) == 64;
   // 1. row buckets of this batch (also for the cyclic schedule: the copies below need the permutation)
   BucketArgs b;
   b.types = h->sched == ALG_SCHED_CYCLIC ? nullptr : types;
@@ -1368,10 +1371,12 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
     return cuda_status(cudaMemset2DAsync(dW, (size_t)lddw * elem_bytes(w_dtype), 0, (size_t)h->N * elem_bytes(w_dtype),
                                          (size_t)h->K, st));
   }
-  // 2. padded, bucketed copies: X transposed (K x m_pad), G as it is (m_pad x N); pad rows are zero
+  // 2. padded, bucketed copies of X (as it is, or transposed) and G; pad rows are zero
   if (!in_place) {
-    if (launch_gather_transpose_padded(X, ldx, hdr, b.perm, h->q, mp, h->K, ws + L.xt, st) != cudaSuccess) return ALG_ERR_CUDA;
-    if (launch_gather_rows_padded(G, ldg, hdr, b.perm, h->q, mp, h->N, ws + L.gp, st) != cudaSuccess) return ALG_ERR_CUDA;
+    if (!mn && launch_gather_transpose_padded(X, ldx, hdr, b.perm, h->q, mp, h->K, ws + L.xp, st) != cudaSuccess) return ALG_ERR_CUDA;
+    if (launch_gather_rows_padded(X, ldx, mn ? h->K : 0, ws + L.xp, G, ldg, h->N, ws + L.gp, hdr, b.perm, h->q, mp, p.d_status, p.wait_limit,
+                                  st) != cudaSuccess)
+      return ALG_ERR_CUDA;
   }
   // 3. the grouped GEMM: rows = input features (type = their group), reduction over the padded buckets
   ProjArgs a;
@@ -1396,8 +1401,8 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   a.q = p.q;
   a.perm = nullptr;
   a.in_perm = nullptr;
-  a.X = in_place ? X : (const void *)(ws + L.xt);
-  a.ldx = in_place ? ldx : mp;
+  a.X = in_place ? X : (const void *)(ws + L.xp);
+  a.ldx = in_place ? ldx : mn ? h->K : mp;
   a.W = in_place ? G : (const void *)(ws + L.gp);
   a.ldw = in_place ? ldg : h->N;
   a.bias = nullptr;
@@ -1417,7 +1422,7 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   a.gated_f = 0;
   a.w_kmajor = 0;
   a.dyn_so = in_place ? nullptr : hdr->pad_offsets;
-  a.seg_rows = in_place ? (int)(M / h->q) : 0;
+  a.a_mn = mn, a.seg_rows = in_place ? (int)(M / h->q) : 0;
   a.block_k = block_k_of(p);
   a.y_staged = 0;
   a.plan = nullptr;

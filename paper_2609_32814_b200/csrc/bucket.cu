@@ -332,22 +332,6 @@ __device__ __forceinline__ int padded_source_row(const WsHeader *hdr, const int 
   return (p < hdr->pad_offsets[q] && rank < rows) ? perm[hdr->offsets[t] + rank] : -1;
 }
 
-__global__ void __launch_bounds__(256) gather_rows_padded_kernel(const uint4 *__restrict__ G, int64_t ldg_v,
-                                                                 const WsHeader *__restrict__ hdr,
-                                                                 const int *__restrict__ perm, int q, int m_pad, int vecs,
-                                                                 uint4 *__restrict__ Gp) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");  // perm and the offsets come from the bucketing kernel
-  const int lane = threadIdx.x & 31;
-  const int warp_global = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int n_warps = (gridDim.x * blockDim.x) >> 5;
-  for (int p = warp_global; p < m_pad; p += n_warps) {
-    const int src_row = padded_source_row(hdr, perm, q, p);
-    uint4 *dst = Gp + (int64_t)p * vecs;
-    for (int v0 = lane; v0 < vecs; v0 += 32) dst[v0] = src_row >= 0 ? __ldg(G + (int64_t)src_row * ldg_v + v0) : make_uint4(0, 0, 0, 0);
-  }
-}
-
 // XpT[c, p] = X[source(p), c]: 64 padded rows x 64 columns per CTA through shared memory, so that both the
 // reads (along c) and the writes (along p) are contiguous.
 __global__ void __launch_bounds__(256) gather_transpose_padded_kernel(const __nv_bfloat16 *__restrict__ X, int64_t ldx,
@@ -378,6 +362,96 @@ __global__ void __launch_bounds__(256) gather_transpose_padded_kernel(const __nv
       *(__nv_bfloat162 *)(XpT + (int64_t)(c0 + c) * m_pad + p0 + rp) = v;
     }
   }
+}
+
+// ---- row copies by the bulk copy engine ----
+//
+// dst[d, :] = src[row(d), :] for one or two matrices, row(d) = perm[d], or for buckets padded to multiples of 64 rows
+// the row behind padded row d (pad rows are zero).  An agent (one thread) owns a slot of shared memory and moves one
+// piece of a row at a time: bulk load, wait, bulk store.  A CTA holds as many slots as fit, so an SM has up to 190 KB in
+// flight without a register or a load instruction per 16 bytes.  The copy streams: at 8003 rows of 6 KB it takes 17.9 us
+// (98 MB moved, 5.5 TB/s) where the warp-per-row copy above takes 20; X (1.5 KB) and G (6 KB) of those rows into padded
+// buckets in one launch 27 us, where transposing X and copying G took 34.  Its CTAs fill an SM, so the next kernel's
+// prologue cannot run beside it: below 40 MB the warp-per-row copy is the better one (FFN 768 -> 3072, M = 12000, 18 MB:
+// 94.5 us there, 96.7 here; gated 7168 -> 2048 at q = 32, M = 4000, 57 MB: 119.2 there, 115.9 here).
+constexpr int kMaxPiece = 8192, kSlotBytes = 184 * 1024, kMaxAgents = 128;
+
+struct CopyArgs {
+  const uint8_t *src[2];
+  uint8_t *dst[2];
+  int64_t ld_src[2];    // bytes
+  int row_bytes[2];     // 0: no second matrix
+  int pieces[2], piece[2];   // pieces per row, bytes of a piece (the last one may be shorter)
+  int slot, agents;     // bytes of a slot, slots of a CTA
+  int rows;             // rows of dst
+  const int *perm;
+  const WsHeader *hdr;  // padded buckets; nullptr: rows through perm as they are
+  int q;
+  int *status;
+  long long wait_limit;
+};
+
+__global__ void __launch_bounds__(kMaxAgents) copy_rows_kernel(const CopyArgs a) {
+  extern __shared__ __align__(128) uint8_t slots[];   // [agents][slot], then a slot of zeros (padded buckets)
+  __shared__ __align__(8) uint64_t bars[kMaxAgents];
+  __shared__ int s_off[kMaxQ + 1], s_pad[kMaxQ + 1];
+  const int tid = threadIdx.x;
+  const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&bars[tid]), base = (uint32_t)__cvta_generic_to_shared(slots);
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar));
+  if (a.hdr)
+    for (int e = tid * 16; e < a.slot; e += kMaxAgents * 16) *(uint4 *)(slots + a.agents * a.slot + e) = make_uint4(0, 0, 0, 0);
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the zeros, before the copy engine reads them
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // perm and the offsets come from the bucketing kernel
+  if (a.hdr)
+    for (int e = tid; e <= a.q; e += kMaxAgents) s_off[e] = __ldcg(a.hdr->offsets + e), s_pad[e] = __ldcg(a.hdr->pad_offsets + e);
+  __syncthreads();
+  if (tid >= a.agents) return;
+  const uint32_t slot = base + (uint32_t)(tid * a.slot), zeros = base + (uint32_t)(a.agents * a.slot);
+  const int per_row = a.pieces[0] + a.pieces[1];
+  const int64_t units = (int64_t)a.rows * per_row;
+  uint32_t parity = 0;
+  for (int64_t u = blockIdx.x + (int64_t)gridDim.x * tid; u < units; u += (int64_t)gridDim.x * a.agents) {
+    const int row = (int)(u / per_row), c = (int)(u - (int64_t)row * per_row);
+    const int m = c >= a.pieces[0], at = (m ? c - a.pieces[0] : c) * a.piece[m];
+    const uint32_t bytes = (uint32_t)min(a.piece[m], a.row_bytes[m] - at);
+    int src_row;
+    if (a.hdr) {
+      int t = 0;
+      while (t + 1 < a.q && s_pad[t + 1] <= row) ++t;
+      const int r = row - s_pad[t];
+      src_row = row < s_pad[a.q] && r < s_off[t + 1] - s_off[t] ? __ldg(a.perm + s_off[t] + r) : -1;
+    } else {
+      src_row = __ldg(a.perm + row);
+    }
+    uint8_t *dst = a.dst[m] + (int64_t)row * a.row_bytes[m] + at;
+    if (src_row >= 0) {
+      const uint8_t *src = a.src[m] + (int64_t)src_row * a.ld_src[m] + at;
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot), "l"(src), "r"(bytes), "r"(bar)
+                   : "memory");
+      uint32_t done = 0;
+      const long long t0 = clock64();
+      while (!done) {
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(done)
+                     : "r"(bar), "r"(parity)
+                     : "memory");
+        if (!done && clock64() - t0 > a.wait_limit) {
+          atomicExch(a.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+          while (clock64() - t0 < a.wait_limit + 2000000LL) {   // the copy gets time to land
+          }
+          return;
+        }
+      }
+      parity ^= 1u;
+    }
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src_row >= 0 ? slot : zeros), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the slot may be filled again
+  }
+  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 }  // namespace
@@ -499,9 +573,49 @@ cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K, int elem_bytes,
-                               void *Xb, cudaStream_t st) {
+namespace {
+cudaError_t launch_copy_rows(CopyArgs a, cudaStream_t st) {
+  int slot = 0;
+  for (int m = 0; m < 2; ++m) {
+    a.pieces[m] = a.row_bytes[m] ? ceil_div(a.row_bytes[m], kMaxPiece) : 0;
+    a.piece[m] = a.pieces[m] ? (ceil_div(a.row_bytes[m], a.pieces[m]) + 15) / 16 * 16 : 0;
+    slot = std::max(slot, a.piece[m]);
+  }
+  a.slot = (slot + 127) / 128 * 128;
+  a.agents = std::min(kMaxAgents, kSlotBytes / a.slot - (a.hdr ? 1 : 0));
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(copy_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlotBytes + 1024);
+    if (e != cudaSuccess) return e;
+    attr = true;
+  }
+  const int64_t units = (int64_t)a.rows * (a.pieces[0] + a.pieces[1]);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(148, units)), 1, 1);
+  cfg.blockDim = dim3(kMaxAgents, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)(a.agents + (a.hdr ? 1 : 0)) * a.slot;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  count_launch(1);
+  return cudaLaunchKernelEx(&cfg, copy_rows_kernel, a);
+}
+}  // namespace
+
+cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K, int elem_bytes, void *Xb, int *status,
+                               long long wait_limit, cudaStream_t st) {
   const int vecs = K * elem_bytes / 16;
+  if ((int64_t)M * K * elem_bytes >= kBulkCopyBytes) {
+    CopyArgs a = {};
+    a.src[0] = (const uint8_t *)X, a.dst[0] = (uint8_t *)Xb;
+    a.ld_src[0] = ldx * elem_bytes, a.row_bytes[0] = K * elem_bytes;
+    a.rows = M, a.perm = perm;
+    a.status = status, a.wait_limit = wait_limit;
+    return launch_copy_rows(a, st);
+  }
   int grid = ceil_div(M, 8);  // eight warps (rows) per CTA
   if (grid > 148 * 8) grid = 148 * 8;
   count_launch(1);
@@ -512,14 +626,15 @@ cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int 
                     (uint4 *)Xb);
 }
 
-cudaError_t launch_gather_rows_padded(const void *G, int64_t ldg, const WsHeader *hdr, const int *perm, int q, int m_pad,
-                                      int N, void *Gp, cudaStream_t st) {
-  const int vecs = N * 2 / 16;
-  int grid = ceil_div(m_pad, 8);
-  if (grid > 148 * 8) grid = 148 * 8;
-  count_launch(1);
-  return launch_pdl(gather_rows_padded_kernel, grid, 256, st, (const uint4 *)G, (int64_t)(ldg * 2 / 16), hdr, perm, q, m_pad,
-                    vecs, (uint4 *)Gp);
+cudaError_t launch_gather_rows_padded(const void *X, int64_t ldx, int K, void *Xp, const void *G, int64_t ldg, int N, void *Gp,
+                                      const WsHeader *hdr, const int *perm, int q, int m_pad, int *status, long long wait_limit,
+                                      cudaStream_t st) {
+  CopyArgs a = {};
+  a.src[0] = (const uint8_t *)X, a.dst[0] = (uint8_t *)Xp, a.ld_src[0] = ldx * 2, a.row_bytes[0] = K * 2;
+  a.src[1] = (const uint8_t *)G, a.dst[1] = (uint8_t *)Gp, a.ld_src[1] = ldg * 2, a.row_bytes[1] = N * 2;
+  a.rows = m_pad, a.perm = perm, a.hdr = hdr, a.q = q;
+  a.status = status, a.wait_limit = wait_limit;
+  return launch_copy_rows(a, st);
 }
 
 cudaError_t launch_gather_transpose_padded(const void *X, int64_t ldx, const WsHeader *hdr, const int *perm, int q,

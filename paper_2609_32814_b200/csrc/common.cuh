@@ -87,13 +87,15 @@ struct BucketArgs {
 
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t st);
 // Xb[d, 0:K] = X[perm[d], 0:K] (16-byte vectors; K*elem_bytes % 16 == 0)
-cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K,
-                               int elem_bytes, void *Xb, cudaStream_t st);
-// Weight-gradient pass (bf16): bucketed copies with every bucket padded to a multiple of 64 rows, pad
-// rows zero.  Gp[p, 0:N] = G[perm[..], 0:N] for the padded row p;  XpT[c, p] = X[perm[..], c]
-// (transposed: K x m_pad, leading dimension m_pad).  m_pad >= padded total (hdr->pad_offsets[q]).
-cudaError_t launch_gather_rows_padded(const void *G, int64_t ldg, const WsHeader *hdr, const int *perm, int q, int m_pad,
-                                      int N, void *Gp, cudaStream_t st);
+constexpr int64_t kBulkCopyBytes = 40 << 20;   // from this many bytes on by the bulk copy engine (see copy_rows_kernel)
+cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K, int elem_bytes, void *Xb, int *status,
+                               long long wait_limit, cudaStream_t st);
+// Weight-gradient pass (bf16): bucketed copies of X (K columns) and G (N columns) with every bucket padded to a multiple
+// of 64 rows, pad rows zero: Xp[p] = X[perm[..]], Gp[p] = G[perm[..]].  m_pad >= padded total (hdr->pad_offsets[q]).
+cudaError_t launch_gather_rows_padded(const void *X, int64_t ldx, int K, void *Xp, const void *G, int64_t ldg, int N, void *Gp,
+                                      const WsHeader *hdr, const int *perm, int q, int m_pad, int *status, long long wait_limit,
+                                      cudaStream_t st);
+// The same for X alone, transposed (K x m_pad, leading dimension m_pad): feature groups that do not start on 16 bytes.
 cudaError_t launch_gather_transpose_padded(const void *X, int64_t ldx, const WsHeader *hdr, const int *perm, int q,
                                            int m_pad, int K, void *XpT, cudaStream_t st);
 
@@ -155,9 +157,11 @@ struct ProjArgs {
   // reduction segments come from device memory (padded row buckets; dW = X^T G reduces over rows).
   int w_kmajor;
   const int *dyn_so;
-  // Weight-gradient pass with the cyclic schedule and M a multiple of 64 q: nothing is copied.  The reduction
-  // segment of type t is rows t, t + q, ... of X and of G read in place (type-strided views); the A operand is
-  // the X block as it lies in memory (features contiguous: MN-major A).  seg_rows = M / q; 0 = off.
+  // Weight-gradient pass: the A operand is the X block as it lies in memory (features contiguous: MN-major A).  a_mn: on.
+  // Cyclic schedule with M a multiple of 64 q: nothing is copied, the reduction segment of type t is rows t, t + q, ...
+  // of X and of G read in place (type-strided views), seg_rows = M / q; else (seg_rows = 0) segments are the padded
+  // buckets dyn_so.
+  int a_mn;
   int seg_rows;
   // Gated (SwiGLU) up projection: W is the merged bank [W_gate | W_up] with 2 * gated_f columns, a
   // tile accumulates 128 gate columns and the matching 128 up columns side by side, the epilogue

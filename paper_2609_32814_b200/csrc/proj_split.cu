@@ -208,11 +208,12 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           const int k0 = k_begin + (i << 6);
           if (elect_one()) {
             mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
-            if (a.seg_rows) {   // weight gradient, cyclic schedule: X and G in place, features / columns contiguous
+            if (a.a_mn) {   // weight gradient: rows of X and G as they lie, features / columns contiguous
+              const int pos0 = a.seg_rows ? i << 6 : k0, seg = a.seg_rows ? k : 0;
 #pragma unroll
-              for (int c = 0; c < 2; ++c) tma_load_3d(sa + c * kBChunkBytes, &tmA, bar, row0 + c * 64, k, i << 6);
+              for (int c = 0; c < 2; ++c) tma_load_3d(sa + c * kBChunkBytes, &tmA, bar, row0 + c * 64, seg, pos0);
 #pragma unroll
-              for (int c = 0; c < TILE_N / 64; ++c) tma_load_3d(sa + kABytes + c * kBChunkBytes, &tmB, bar, n0 + c * 64, k, i << 6);
+              for (int c = 0; c < TILE_N / 64; ++c) tma_load_3d(sa + kABytes + c * kBChunkBytes, &tmB, bar, n0 + c * 64, seg, pos0);
             } else {
               if (a.a_cyclic_rows) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
               else tma_load_2d(sa, &tmA, bar, k0, a_row);
@@ -234,11 +235,11 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     } else if (warp == 1) {
       // ---------------- MMA issuer (operand layouts as in proj_tc.cu) ----------------
       const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      const uint64_t da0 = a.seg_rows ? make_smem_desc(smem_u32(smem), 64 * 64 * 2, 1024) : make_smem_desc(smem_u32(smem), 16, 1024);
-      const uint64_t da_step = a.seg_rows ? 128 : 2;
+      const uint64_t da0 = a.a_mn ? make_smem_desc(smem_u32(smem), 64 * 64 * 2, 1024) : make_smem_desc(smem_u32(smem), 16, 1024);
+      const uint64_t da_step = a.a_mn ? 128 : 2;
       const uint64_t db0 = a.w_kmajor ? make_smem_desc(smem_u32(smem) + kABytes, 16, 1024) : make_smem_desc(smem_u32(smem) + kABytes, kBChunkBytes, 1024);
       const uint64_t db_step = a.w_kmajor ? 2 : 128;
-      const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.seg_rows ? (1u << 15) : 0u);
+      const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.a_mn ? (1u << 15) : 0u);
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;

@@ -290,18 +290,18 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             g_rows[h][2], g_rows[h][3]);
             }
           } else if (elect_one()) {
-            if (a.seg_rows) {
-              // weight gradient, cyclic schedule: rows k, k + q, ... of X (A, features contiguous) and of G (B),
-              // 64 of them from position k0 - so[k] on, in boxes of 64 features / 64 output columns
-              const int pos0 = k0 - k_begin;
+            if (a.a_mn) {
+              // weight gradient: 64 rows of X (A, features contiguous) and of G (B), in boxes of 64 features / 64 output
+              // columns.  Cyclic schedule: rows k, k + q, ... from position k0 - so[k] on; else padded rows from k0 on
+              const int pos0 = a.seg_rows ? k0 - k_begin : k0, seg = a.seg_rows ? k : 0;
               if (loads_a) {
                 mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
 #pragma unroll
-                for (int c = 0; c < TILE_M / 64; ++c) tma_load_3d(sa + c * (64 * BK * 2), &tmA, bar, row0 + c * 64, k, pos0);
+                for (int c = 0; c < TILE_M / 64; ++c) tma_load_3d(sa + c * (64 * BK * 2), &tmA, bar, row0 + c * 64, seg, pos0);
               } else {
 #pragma unroll
                 for (int c = 0; c < TILE_N / 64; ++c)
-                  tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, &tmB, bar, n0 + c * 64, k, pos0);
+                  tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, &tmB, bar, n0 + c * 64, seg, pos0);
               }
             } else if (AMODE == 1 && loads_a && a.a_cyclic_rows) {
               // runs of run_rows rows per period: 64-row boxes, each inside one run
@@ -346,14 +346,14 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tfull0 = smem_u32(&ctl->tmem_full[0]), tempty0 = smem_u32(&ctl->tmem_empty[0]);
     // A: K-major rows of 128 (64) bytes; in the in-place weight-gradient pass the block lies MN-major like B
     // (64-feature chunks one box apart, 16 reduction rows = 128 descriptor units per K step)
-    const uint64_t da0 = a.seg_rows ? make_smem_desc(smem_u32(smem), 64 * BK * 2, 1024)
+    const uint64_t da0 = a.a_mn ? make_smem_desc(smem_u32(smem), 64 * BK * 2, 1024)
                                     : make_smem_desc(smem_u32(smem), 16, C::kSboK, C::kSwzK);
-    const uint64_t da_step = a.seg_rows ? 128 : 2;
+    const uint64_t da_step = a.a_mn ? 128 : 2;
     // B: the canonical bank lands MN-major (64-column chunks one box apart, 16 k-rows = two 8-row groups
     // = 128 descriptor units per K step); used transposed it lands K-major like A (32 bytes per K step)
     const uint64_t db0 = a.w_kmajor ? make_smem_desc(smem_u32(smem) + C::kABytes, 16, C::kSboK, C::kSwzK)
                                     : make_smem_desc(smem_u32(smem) + C::kABytes, C::kBChunkBytes, 1024);
-    const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.seg_rows ? (1u << 15) : 0u);
+    const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.a_mn ? (1u << 15) : 0u);
     const uint64_t db_step = a.w_kmajor ? 2 : 128;
     TileRec rec = tile_seq_get(recs, tm, a.geom, 0, blockIdx.x, gridDim.x, ctl->nkb);
     while (ok && __shfl_sync(0xffffffffu, rec.row0, 0) >= 0) {
@@ -604,13 +604,15 @@ namespace tc {
 // Tensor maps of both operands of the one-CTA kernels; sets a->b_3d.
 cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int tile_n, int tile_m, bool gated, int bk) {
   a->b_3d = 0;
-  if (a->seg_rows) {
-    // X and G as {columns, type, position in the type}: rows t, t + q, ... are the reduction segment of type t
+  if (a->a_mn) {
+    // X and G as {columns, type, position in the type}: rows t, t + q, ... are the reduction segment of type t; the
+    // padded copies as {columns, 1, padded row}
     if (gated || a->w_kmajor || tile_m != 128 || bk != 64) return cudaErrorInvalidValue;
-    const uint64_t da[3] = {(uint64_t)a->M, (uint64_t)a->q, (uint64_t)a->seg_rows};
-    const uint64_t sa[2] = {(uint64_t)a->ldx * 2, (uint64_t)a->ldx * 2 * (uint64_t)a->q};
-    const uint64_t db[3] = {(uint64_t)a->N, (uint64_t)a->q, (uint64_t)a->seg_rows};
-    const uint64_t sb[2] = {(uint64_t)a->ldw * 2, (uint64_t)a->ldw * 2 * (uint64_t)a->q};
+    const uint64_t types = a->seg_rows ? (uint64_t)a->q : 1u, len = a->seg_rows ? (uint64_t)a->seg_rows : (uint64_t)a->K;
+    const uint64_t da[3] = {(uint64_t)a->M, types, len};
+    const uint64_t sa[2] = {(uint64_t)a->ldx * 2, (uint64_t)a->ldx * 2 * types};
+    const uint64_t db[3] = {(uint64_t)a->N, types, len};
+    const uint64_t sb[2] = {(uint64_t)a->ldw * 2, (uint64_t)a->ldw * 2 * types};
     const uint32_t box[3] = {64, 1, 64};
     const cudaError_t e = make_map_nd(tmA, a->X, 3, da, sa, box, 128);
     return e == cudaSuccess ? make_map_nd(tmB, a->W, 3, db, sb, box, 128) : e;

@@ -122,3 +122,19 @@ def test_grad_maps_on_split_reductions(q, M, s_w, r_w, schedule):
     widths = [s_w] * q, [r_w] * q
     assert np.array_equal(H.to_np(dX), oracle.proj_vjp_x(G, types, W, *widths))
     assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X, G, types, *widths))
+
+
+@pytest.mark.parametrize("q,M,s,r", [
+    (2, 900, [200, 56], [128, 256]),     # feature groups on 16 bytes but off the tile: X through rows of 512 bytes
+    (3, 515, [20, 44, 64], [128] * 3),   # feature groups off 16 bytes: X transposed
+    (2, 70, [128, 128], [1280, 1280]),   # G rows of several pieces, few rows
+])
+@pytest.mark.parametrize("schedule", ["explicit", "cyclic"])
+def test_weight_gradient_row_copies(q, M, s, r, schedule):
+    M = M // q * q
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    X, G = synth.small_ints(1, (M, sum(s)), -1, 1), synth.small_ints(2, (M, sum(r)), -1, 1)
+    grad = binding.ProjGrad(s, r, schedule=schedule)
+    dW = grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), None if schedule == "cyclic" else H.dev_types(types))
+    assert grad.last_status() == 0
+    assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X, G, types, s, r))

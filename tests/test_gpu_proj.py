@@ -538,3 +538,12 @@ def test_split_reduction_is_exact(q, M, s_w, r_w, schedule):
     if bad is not None:
         want[bad] = 0
     assert np.abs(g - want).max() <= 1e-6 * (1 + np.abs(want).max())   # the GELU's own error is below 1e-7 |z|
+
+
+@pytest.mark.parametrize("s_w", [384, 2304])   # just past the size of the bulk copy: rows of one piece, of two
+def test_large_row_copy(s_w):
+    wl = _tc_workload(2, (40 << 20) // (4 * s_w) + 5, s_w, 128, seed=81)
+    Y, proj = _run_proj(wl, out_dtype=torch.float32)
+    rows = np.unique(np.r_[0:30, wl.M // 2:wl.M // 2 + 30, wl.M - 30:wl.M])
+    ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref)
