@@ -430,32 +430,36 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!ok) break;
       if (e == 0 && lane == 0) ALG_TRACE(2, 1);
       tc_fence_after();
+      // columns of this warp: its share of the accumulator, or GATED 64 output columns -- gate values sit in accumulator
+      // columns [0, 128), the matching up values 128 columns further
+      constexpr int kCols = GATED ? 64 : C::kHalf;
       const uint32_t taddr =
-          tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::kAccStride + half * C::kHalf);
-      const int col_base = rec.n0 + (C::kHalves == 2 ? 0 : half * C::kHalf);
-      if (GATED) {
-        // this warp: 32 rows x 64 output columns; gate values sit in accumulator columns [0, 128),
-        // the matching up values 128 columns further
-        const uint32_t tg = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::kAccStride + half * 64);
-#pragma unroll 1
-        for (int c0 = 0; c0 < 64; c0 += 32) {
-          uint32_t vg[32], vu[32];
-          tc_ld_32x32(tg + (uint32_t)c0, vg);
-          tc_ld_32x32(tg + (uint32_t)(128 + c0), vu);
+          tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * C::kAccStride + half * kCols);
+      const int col_base = rec.n0 + (C::kHalves == 2 ? 0 : half * kCols);
+      auto load_32 = [&](float(&f)[32], int c0) {   // whole warp
+        uint32_t v[32];
+        tc_ld_32x32(taddr + (uint32_t)c0, v);
+        if (GATED) {
+          uint32_t vu[32];
+          tc_ld_32x32(taddr + (uint32_t)(128 + c0), vu);
           tc_wait_ld();
-          if (out_row >= 0) {
-            float f[32];
 #pragma unroll
-            for (int x = 0; x < 32; ++x) {
-              const float g = __uint_as_float(vg[x]);
-              float th;
-              asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * g));
-              f[x] = g * fmaf(0.5f, th, 0.5f) * __uint_as_float(vu[x]);   // silu(g) * u, sigmoid(g) = (1 + tanh(g/2)) / 2
-            }
-            finish_and_store_32(f, a, out_row, rec.n0 + half * 64 + c0);
+          for (int x = 0; x < 32; ++x) {
+            const float g = __uint_as_float(v[x]);
+            float th;
+            asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * g));
+            f[x] = g * fmaf(0.5f, th, 0.5f) * __uint_as_float(vu[x]);   // silu(g) * u, sigmoid(g) = (1 + tanh(g/2)) / 2
+          }
+        } else {
+          tc_wait_ld();
+#pragma unroll
+          for (int x = 0; x < 32; ++x) f[x] = __uint_as_float(v[x]);
+          if (empty_tile) {   // (rare and the same for the whole tile: a branch, not 32 selects per chunk)
+#pragma unroll
+            for (int x = 0; x < 32; ++x) f[x] = 0.f;
           }
         }
-      } else
+      };
       // bf16 outputs are transposed through a 2 KB staging buffer per warp: every lane writes its
       // own row segment (64 bytes, 16-byte pieces XOR-swizzled so that the writes and the reads
       // below are bank-conflict free), then four lanes together store one row segment, so one
@@ -473,17 +477,9 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int g = 0; g < 4; ++g) dst_row[g] = __shfl_sync(0xffffffffu, out_row, g * 8 + sub);
         const uint32_t rd_base = smem_u32(buf) + (uint32_t)sub * 64u;
 #pragma unroll 1
-        for (int c0 = 0; c0 < C::kHalf; c0 += 32) {
-          uint32_t v[32];
-          tc_ld_32x32(taddr + (uint32_t)c0, v);
-          tc_wait_ld();
+        for (int c0 = 0; c0 < kCols; c0 += 32) {
           float f[32];
-#pragma unroll
-          for (int x = 0; x < 32; ++x) f[x] = __uint_as_float(v[x]);
-          if (empty_tile) {   // (rare and the same for the whole tile: a branch, not 32 selects per chunk)
-#pragma unroll
-            for (int x = 0; x < 32; ++x) f[x] = 0.f;
-          }
+          load_32(f, c0);
           finish_32(f, a, col_base + c0);
           uint32_t w[16];
           pack_bf16_32(f, w);
@@ -508,21 +504,11 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       } else {
 #pragma unroll 1
-      for (int c0 = 0; c0 < C::kHalf; c0 += 32) {
-        uint32_t v[32];
-        tc_ld_32x32(taddr + (uint32_t)c0, v);
-        tc_wait_ld();
-        if (out_row >= 0) {
+        for (int c0 = 0; c0 < kCols; c0 += 32) {
           float f[32];
-#pragma unroll
-          for (int x = 0; x < 32; ++x) f[x] = __uint_as_float(v[x]);
-          if (empty_tile) {
-#pragma unroll
-            for (int x = 0; x < 32; ++x) f[x] = 0.f;
-          }
-          finish_and_store_32(f, a, out_row, col_base + c0);
+          load_32(f, c0);
+          if (out_row >= 0) finish_and_store_32(f, a, out_row, col_base + c0);
         }
-      }
       }
       tc_fence_before();
       __syncwarp();
@@ -569,7 +555,7 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   cudaError_t e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
   if (e != cudaSuccess) return e;
   // staging buffers for the transposing epilogue, when they fit and the output rows are 16-byte aligned
-  b.y_staged = !GATED && a.y_bf16 && smem_bytes + kEpiWarps * C::kStoreBufBytes <= 227 * 1024 && ((uintptr_t)a.Y & 15u) == 0 &&
+  b.y_staged = a.y_bf16 && smem_bytes + kEpiWarps * C::kStoreBufBytes <= 227 * 1024 && ((uintptr_t)a.Y & 15u) == 0 &&
                (a.ldy * 2) % 16 == 0;
   if (b.y_staged) smem_bytes += kEpiWarps * C::kStoreBufBytes;
   cudaLaunchConfig_t cfg = {};
