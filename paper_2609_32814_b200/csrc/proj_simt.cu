@@ -35,7 +35,8 @@ __global__ void __launch_bounds__(256) proj_simt_kernel(const ProjArgs a) {
   TileMap *tm = reinterpret_cast<TileMap *>(s_map);
   const DevTable *__restrict__ tab = a.tab;
   const int q = a.q;
-  tile_map_build(tm, tab, a.st, a.q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom);
+  tile_map_classes(tm, tab, a.st, q, a.n_classes, threadIdx.x, 256);
+  tile_map_build(tm, q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom);
   const int n_tiles = tm->total;
   const T *__restrict__ X = (const T *)a.X;
   const T *__restrict__ W = (const T *)a.W;
@@ -226,9 +227,10 @@ __global__ void __launch_bounds__(256, TM_ == 64 ? 2 : 1) proj_f32_kernel(const 
   const DevTable *__restrict__ tab = a.tab;
   const int q = a.q, tid = threadIdx.x;
   const int grp = tid / C::kGroupThreads, tx = tid & 7, ty = (tid % C::kGroupThreads) >> 3;
+  tile_map_classes(tm, tab, a.st, q, a.n_classes, tid, 256);
   asm volatile("griddepcontrol.wait;" ::: "memory");   // the bucket offsets come from the previous kernel
   if (a.count_rows) count_rows(a, s_count);
-  tile_map_build(tm, tab, a.st, q, a.n_classes, a.count_rows ? s_count.off : a.offsets, a.cyclic_rows, a.M, a.geom);
+  tile_map_build(tm, q, a.n_classes, a.count_rows ? s_count.off : a.offsets, a.cyclic_rows, a.M, a.geom);
   const int n_tiles = tm->total;
   const float *__restrict__ X = (const float *)a.X;
   const float *__restrict__ W = (const float *)a.W;

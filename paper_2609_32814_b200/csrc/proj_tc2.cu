@@ -172,6 +172,7 @@ proj_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       if ((mask >> k) & 1u) n += (a.st.valid ? a.st.so[k + 1] - a.st.so[k] : tab->so[k + 1] - tab->so[k]) / kTcBlockK;
     nkb[e] = (uint16_t)n;
   }
+  tile_map_classes(tm, tab, a.st, q, a.n_classes, threadIdx.x, kThreads);
   if (warp == 1) {  // both CTAs of the pair allocate together, same shared-memory slot
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&ctl->tmem_base)),
                  "r"((uint32_t)kTmemCols)
@@ -181,7 +182,7 @@ proj_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   // Programmatic dependent launch: everything above touches only this CTA's own state.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  tile_map_build(tm, tab, a.st, a.q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom);
+  tile_map_build(tm, q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom);
   tile_seq_build(recs, kSeqCap, tm, a.geom, blockIdx.x >> 1, gridDim.x >> 1, nkb);
   tc_fence_before();
   __syncthreads();

@@ -31,19 +31,26 @@ __host__ __device__ inline size_t tile_map_bytes(int n_classes) {
   return sizeof(TileMap) + (size_t)n_classes * sizeof(ClassRec) + (size_t)(n_classes + 1) * sizeof(int);
 }
 
-// Called by all threads of the CTA (blockDim.x >= 32).  `offsets` = device bucket offsets, or
-// nullptr for the cyclic schedule with equal buckets of cyclic_rows rows.  Ends with a barrier.
-__device__ inline void tile_map_build(TileMap *tm, const DevTable *tab, const SmallTable &st, int q, int nc,
-                                      const int *offsets, int cyclic_rows, int M, const TileGeom &g) {
-  if (threadIdx.x == 0) tm->n_classes = nc, tm->q = q;
+// Class records into shared memory, by `threads` threads.  They are the handle's, so this runs before the wait for the
+// previous kernel: read after it, from the table in global memory, they and the K-block counts kept the planning of an
+// explicit batch with 8 types at 4.3 us per launch.
+__device__ __forceinline__ void tile_map_classes(TileMap *tm, const DevTable *tab, const SmallTable &st, int q, int nc,
+                                                 int thread, int threads) {
+  if (thread == 0) tm->n_classes = nc, tm->q = q;
+  ClassRec *cls = reinterpret_cast<ClassRec *>(tm + 1);
+  for (int c = thread; c < nc; c += threads) cls[c] = st.valid ? st.cls[c] : tab->cls[c];
+}
+
+// Called by all threads of the CTA (blockDim.x >= 32) behind tile_map_classes and a barrier.  `offsets` = device bucket
+// offsets, or nullptr for the cyclic schedule with equal buckets of cyclic_rows rows.  Ends with a barrier.
+__device__ inline void tile_map_build(TileMap *tm, int q, int nc, const int *offsets, int cyclic_rows, int M, const TileGeom &g) {
   for (int t = threadIdx.x; t <= q + 1; t += blockDim.x)
     tm->offsets[t] = offsets ? offsets[t] : (t <= q ? t * cyclic_rows : M);
   __syncthreads();
-  ClassRec *cls = tm->cls();
+  const ClassRec *cls = tm->cls();
   int *prefix = tm->prefix();
   for (int c = threadIdx.x; c < nc; c += blockDim.x) {
-    const ClassRec r = st.valid ? st.cls[c] : tab->cls[c];
-    cls[c] = r;
+    const ClassRec r = cls[c];
     const int rows = tm->offsets[r.i + 1] - tm->offsets[r.i];
     prefix[c] = ((rows + g.tile_m - 1) >> g.tile_m_log2) * (int)r.n_tiles;
   }
@@ -138,29 +145,23 @@ __device__ __forceinline__ TileRec tile_seq_get(const TileRec *recs, TileMap *tm
   return tile_seq_decode(tm, g, round, worker, n_workers, nkb_of_pair);
 }
 
-// The whole plan of one worker -- class prefix table and its own tile sequence, K-block counts
-// included -- built by ONE warp with warp-level synchronisation only, so that the other warps of
-// the CTA can set up barriers and tensor memory meanwhile and a single CTA barrier ends the
-// prologue.  `keep` / `so` are read from the by-value table when it is valid, else from `tab`.
-// `seg_rows` (optional): every reduction segment has this many rows (weight-gradient pass, cyclic schedule).
-// `dyn_so` (optional, device memory): offsets of the reduction segments when they are not the
-// table's (weight-gradient pass: padded row buckets).
-__device__ inline void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, const DevTable *tab, const SmallTable &st,
-                                      int q, int nc, const int *offsets, int cyclic_rows, int M, const TileGeom &g,
-                                      int worker, int n_workers, int k_block, const int *dyn_so = nullptr, int seg_rows = 0) {
+// The plan of one worker -- class prefix table and its own tile sequence, K-block counts included -- built by ONE warp
+// with warp-level synchronisation only, so that the other warps of the CTA can set up barriers and tensor memory
+// meanwhile and a single CTA barrier ends the prologue.  The warp has run tile_map_classes and written the K blocks
+// per pair (`nkb_of_pair`) before; only the bucket offsets come from the previous kernel.
+__device__ inline void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, int q, int nc, const int *offsets, int cyclic_rows,
+                                      int M, const TileGeom &g, int worker, int n_workers, const uint16_t *nkb_of_pair) {
   const int lane = threadIdx.x & 31;
-  if (lane == 0) tm->n_classes = nc, tm->q = q;
   for (int t = lane; t <= q + 1; t += 32) tm->offsets[t] = offsets ? offsets[t] : (t <= q ? t * cyclic_rows : M);
   __syncwarp();
-  ClassRec *cls = tm->cls();
+  const ClassRec *cls = tm->cls();
   int *prefix = tm->prefix();
   int carry = 0;
   for (int c0 = 0; c0 < nc; c0 += 32) {
     const int c = c0 + lane;
     int v = 0;
     if (c < nc) {
-      const ClassRec r = st.valid ? st.cls[c] : tab->cls[c];
-      cls[c] = r;
+      const ClassRec r = cls[c];
       const int rows = tm->offsets[r.i + 1] - tm->offsets[r.i];
       v = ((rows + g.tile_m - 1) >> g.tile_m_log2) * (int)r.n_tiles;
     }
@@ -179,19 +180,7 @@ __device__ inline void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, const
   const int rounds = min(cap, valid + 1);
   if (lane == 0) prefix[nc] = total, tm->total = total, tm->seq_rounds = rounds, tm->seq_valid = valid;
   __syncwarp();
-  for (int r = lane; r < rounds; r += 32) {
-    TileRec rec = tile_seq_decode(tm, g, r, worker, n_workers, nullptr);
-    if (rec.row0 >= 0) {
-      const int pr = rec.pair & 0xFFFF;
-      const uint32_t mask = st.valid ? st.keep[pr] : tab->keep[pr];
-      int n = 0;
-      for (int k = 0; k < q; ++k)
-        if ((mask >> k) & 1u)
-          n += (seg_rows ? seg_rows : dyn_so ? dyn_so[k + 1] - dyn_so[k] : st.valid ? st.so[k + 1] - st.so[k] : tab->so[k + 1] - tab->so[k]) / k_block;
-      rec.rows |= n << 16;
-    }
-    recs[r] = rec;
-  }
+  for (int r = lane; r < rounds; r += 32) recs[r] = tile_seq_decode(tm, g, r, worker, n_workers, nkb_of_pair);
 }
 
 }  // namespace algproj
