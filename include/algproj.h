@@ -116,8 +116,9 @@ typedef enum {
  *   ROW_GATHER        explicit row types on the one-CTA GEMM kernel: how the rows of a type reach the kernel.
  *                     1 = a copy pass writes the type-bucketed copy of X into the workspace; 2 = the kernel's
  *                     producer warps fetch the rows through the permutation themselves (four rows per copy
- *                     instruction, X read in place, one launch fewer); 0 (default) = 1, which measures faster or
- *                     equal on every benchmark step.  Results are identical.  Ignored by the other kernels.
+ *                     instruction, X read in place, one launch fewer); 0 (default) = the library's choice: the
+ *                     bucketed copy, written by the bucketing launch for up to 8192 rows and by a pass of its own
+ *                     beyond.  Results are identical.  2 is ignored by the other kernels.
  *   WEIGHT_PACKED     1: the W given to alg_proj_forward is the padded bank alg_proj_pack_weight wrote (ldw is
  *                     ignored); 0 (default): the caller's K x N bank.  Only handles whose
  *                     alg_proj_packed_weight_bytes is not 0 take 1 (else ALG_ERR_UNSUPPORTED_SHAPE).

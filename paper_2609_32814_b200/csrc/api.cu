@@ -797,6 +797,12 @@ bool use_row_decode(const alg_proj_s &p, int64_t M) {
          !p.w_kmajor && !p.dyn_segments && p.sched != ALG_SCHED_INTERVAL && row_decode_fits(p.q, p.K, p.N);
 }
 
+// Explicit types on the tensor-core kernels: are the buckets counted and X copied into them by one launch?  (A call
+// whose kernel or row gather was chosen by an option keeps one launch for each.)
+bool copies_with_buckets(const alg_proj_s &p, int64_t M) {
+  return p.opt_kernel == 0 && p.opt_row_gather == 0 && (use_tc(p) || use_big_counted(p, M)) && bucket_copy_takes(p.q, M, (int64_t)p.K * 2);
+}
+
 // Forward call on the large-algebra path.  Equal buckets (cyclic or interval schedule, q | M) need no
 // pre-kernel at all; explicit types (q <= kMaxQ) go through bucketing and the row gather first.
 alg_status_t run_big(alg_proj_s &p, const WsLayout &L, char *ws, const void *X, int64_t ldx, const int32_t *types,
@@ -845,10 +851,12 @@ alg_status_t run_big(alg_proj_s &p, const WsLayout &L, char *ws, const void *X, 
     b.ldy = ldy;
     b.N = p.N;
     b.y_elem_bytes = elem_bytes(y_dtype);
-    if (launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
+    const bool copied = copies_with_buckets(p, M);
+    if (copied && launch_bucket_copy(b, X, ldx, p.K, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
+    if (!copied && launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
     a.sched = 0;
     if (!p.big.repack) {   // (the repacking pass below gathers the rows itself)
-      if (launch_gather_rows(X, ldx, b.perm, (int)M, p.K, 2, ws + L.xb, p.d_status, p.wait_limit, st) != cudaSuccess) return ALG_ERR_CUDA;
+      if (!copied && launch_gather_rows(X, ldx, b.perm, (int)M, p.K, 2, ws + L.xb, p.d_status, p.wait_limit, st) != cudaSuccess) return ALG_ERR_CUDA;
       a.X = ws + L.xb, a.ldx = p.K;
     }
     a.offsets = (const int *)(ws + L.hdr);   // WsHeader starts with its offsets
@@ -1108,6 +1116,10 @@ alg_status_t alg_proj_forward(alg_proj_t h, const void *X, int64_t ldx, const in
   // (320 -> 640, q = 2: M = 1500 30.6 -> 28.4 us, M = 4096 66.0 -> 65.6).
   if (h->dtype == ALG_F32 && M <= kCountRows && h->q <= kParamQ)
     return run_proj(*h, L, ws, X, ldx, false, W, ldw, bias, act, Y, ldy, y_dtype, false, M, st, nullptr, false, 0, 0, b.types, true);
+  if (!cyc && copies_with_buckets(*h, M)) {
+    if (launch_bucket_copy(b, X, ldx, h->K, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
+    return run_proj(*h, L, ws, ws + L.xb, h->K, true, W, ldw, bias, act, Y, ldy, y_dtype, false, M, st);
+  }
   if (!cyc && launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
   return run_proj(*h, L, ws, X, ldx, false, W, ldw, bias, act, Y, ldy, y_dtype, false, M, st, nullptr, cyc);
 }
@@ -1622,11 +1634,13 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
   const bool cyc = run_rows > 0 ||
                    (h->up.sched == ALG_SCHED_CYCLIC && M % h->up.q == 0 &&
                     ((use_tc(h->up) && use_tc(h->down)) || (use_big_equal(h->up, M) && use_big_equal(h->down, M))));
-  if (!cyc && launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
+  const bool copied = !cyc && copies_with_buckets(h->up, M);
+  if (copied && launch_bucket_copy(b, X, h->D, h->D, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
+  if (!cyc && !copied && launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
   if (tm) cudaEventRecord(h->ev[1], st);
   void *H = ws + L.h;
   if (h->gated && (b_up || b_down || act != ALG_ACT_NONE)) return ALG_ERR_INVALID_ARG;   // bias-free, silu(gate) * up
-  alg_status_t s = run_proj(h->up, L, ws, X, h->D, false, W_up, h->gated ? 2 * (int64_t)h->F : h->F, b_up, act, H, h->F,
+  alg_status_t s = run_proj(h->up, L, ws, copied ? ws + L.xb : X, h->D, copied, W_up, h->gated ? 2 * (int64_t)h->F : h->F, b_up, act, H, h->F,
                             h->up.dtype, true, M, st, tm ? h->ev[2] : nullptr, cyc, run_rows, run_period);
   if (s != ALG_OK) return s;
   if (tm) cudaEventRecord(h->ev[3], st);

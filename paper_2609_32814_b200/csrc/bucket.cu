@@ -10,6 +10,7 @@
 //                       then perm[offset[t] + base[t] + rank_in_chunk] = row  (stable); CTA 0
 //                       publishes the bucket offsets.
 //   kernel 3 (gather):  Xb[d,:] = X[perm[d],:]  -- every type becomes a contiguous M-slab.
+//   M <= 8192 with a copy of X to write: one kernel for all of it (bucket_copy_kernel).
 #include <algorithm>
 
 #include "common.cuh"
@@ -323,6 +324,139 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint4 *__restric
   if (threadIdx.x == 0) ALG_TRACE(1, 3);
 }
 
+// Bucketing and the bucketed copy of X in one launch, for batches whose types every CTA can afford to read (M <=
+// kCopyCountRows).  A CTA owns `rows` consecutive rows of the batch: it requests the first of them, counts the types of
+// the whole batch meanwhile -- all rows, and those before its own -- ranks its rows and scatters them to their places.
+// As two kernels the copy waits for the last CTA of the count, one launch boundary and its own first loads; as one, the
+// first rows are on their way while the types are counted (FFN 768 -> 3072, q = 2: M = 100 22.5 -> 20.7 us, 1777 35.9 ->
+// 34.1, 8003 69.7 -> 68.6; gated 2048 -> 6144, q = 32, M = 600 71.6 -> 68.2).  Every CTA reads all types, and past its
+// first row a warp waits for one load at a time: beyond 8192 rows the two kernels are the faster ones (768 -> 3072, q = 4,
+// M = 12000: 74.1 there, 74.9 here; 1024 -> 4096, q = 8, M = 16384: 116.0 there, 117.7 here).
+//
+// PACKED (q <= 8): counts in four registers of four 16-bit fields, summed by warp reductions.  Otherwise one shared-memory
+// histogram per warp (with two types 16 lanes would queue for one counter; with 9 and more it is 3 or 4).
+constexpr int kCopyThreads = 1024, kCopyWarps = kCopyThreads / 32, kCopyUnit = 128;   // 16-byte pieces a warp moves at a time
+constexpr int kCopyCountRows = 8192, kCopyRows = 64;                                // largest batch, rows of a CTA
+template <bool PACKED>
+__global__ void __launch_bounds__(kCopyThreads) bucket_copy_kernel(const BucketArgs a, const uint4 *__restrict__ X, int64_t ldx_v, int vecs,
+                                                                   uint4 *__restrict__ Xb, int rows) {
+  __shared__ uint32_t s_part[PACKED ? kCopyWarps : 1][9];   // (one word of padding: a lane per warp reads a column)
+  __shared__ int s_hist[PACKED ? 1 : kCopyWarps][kMaxQ + 1];     // rows of a type, and 2^16 times those before this CTA's
+  __shared__ int s_wcnt[kCopyRows / 32][kMaxQ + 1];
+  __shared__ int s_off[kMaxQ + 2], s_base[kMaxQ + 1], s_dst[kCopyRows];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = a.q + 1;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // types and X may come from the previous kernel
+  const int r0 = blockIdx.x * rows, n = min(rows, a.M - r0);
+  const int chunks = (vecs + kCopyUnit - 1) / kCopyUnit, units = n * chunks;
+  uint4 w[4];
+  auto load = [&](int u) {
+    const int row = u / chunks, v0 = (u - row * chunks) * kCopyUnit + lane;
+    const uint4 *src = X + (int64_t)(r0 + row) * ldx_v;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (v0 + e * 32 < vecs) w[e] = __ldg(src + v0 + e * 32);
+  };
+  if (warp < units) load(warp);
+  const int t_own = tid < n ? row_type(a, r0 + tid) : -1 - lane;   // (idle lanes never match each other)
+
+  if (PACKED) {
+    uint64_t lo = 0, hi = 0, lo_b = 0, hi_b = 0;
+#pragma unroll 4
+    for (int row = tid; row < a.M; row += kCopyThreads) {
+      const int t = row_type(a, row);
+      const uint64_t one = t < a.q ? 1ull << (16 * (t & 3)) : 0ull;
+      if (t < 4) {
+        lo += one;
+        if (row < r0) lo_b += one;
+      } else {
+        hi += one;
+        if (row < r0) hi_b += one;
+      }
+    }
+    const uint64_t own[4] = {lo, hi, lo_b, hi_b};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {   // (no field overflows, so the halves add up by themselves)
+      const uint32_t v = __reduce_add_sync(0xffffffffu, (uint32_t)(own[e >> 1] >> (32 * (e & 1))));
+      if (lane == e) s_part[warp][e] = v;
+    }
+  } else {
+    for (int t = lane; t < nt; t += 32) s_hist[warp][t] = 0;
+    __syncwarp();
+#pragma unroll 4
+    for (int row = tid; row < a.M; row += kCopyThreads) atomicAdd(&s_hist[warp][row_type(a, row)], row < r0 ? 0x10001 : 1);
+  }
+  const unsigned peers = __match_any_sync(0xffffffffu, t_own);
+  const int rank = __popc(peers & ((1u << lane) - 1u));
+  if (warp < kCopyRows / 32) {
+    for (int t = lane; t < nt; t += 32) s_wcnt[warp][t] = 0;
+    __syncwarp();
+    if (tid < n && rank == 0) s_wcnt[warp][t_own] = __popc(peers);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int tot = 0, bef = 0, tot_last = 0, bef_last = 0;   // of type `lane`; of type 32 (lane 0)
+    if (PACKED) {
+      // lane e of every eight holds types 2e, 2e + 1 of the batch (e < 4) and of the rows before this CTA's
+      uint32_t v = 0;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, s_part[lane][e]);
+        if ((lane & 7) == e) v = sum;
+      }
+      const uint32_t v_tot = __shfl_sync(0xffffffffu, v, lane >> 1), v_bef = __shfl_sync(0xffffffffu, v, 4 + (lane >> 1));
+      if (lane < a.q) tot = (int)((v_tot >> (16 * (lane & 1))) & 0xFFFFu), bef = (int)((v_bef >> (16 * (lane & 1))) & 0xFFFFu);
+      const int all = __reduce_add_sync(0xffffffffu, tot), all_b = __reduce_add_sync(0xffffffffu, bef);
+      if (lane == a.q) tot = a.M - all, bef = r0 - all_b;
+    } else {
+      for (int x = 0; x < kCopyWarps; ++x) {
+        const int v = lane < nt ? s_hist[x][lane] : 0;
+        tot += v & 0xFFFF, bef += v >> 16;
+        if (nt > 32 && lane == 0) tot_last += s_hist[x][32] & 0xFFFF, bef_last += s_hist[x][32] >> 16;
+      }
+    }
+    int incl = tot;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    const int total32 = __shfl_sync(0xffffffffu, incl, 31);
+    if (lane < nt) s_off[lane] = incl - tot, s_base[lane] = incl - tot + bef;
+    if (lane == 0) {
+      if (nt > 32) s_off[32] = total32, s_base[32] = total32 + bef_last, s_off[33] = total32 + tot_last;
+      else s_off[nt] = total32;   // == M
+    }
+  }
+  __syncthreads();
+  if (tid < n) {
+    int d = s_base[t_own] + rank;
+    for (int x = 0; x < warp; ++x) d += s_wcnt[x][t_own];
+    s_dst[tid] = d;
+    a.perm[d] = r0 + tid;
+    if (t_own == a.q) {
+      atomicExch(a.status, (int)ALG_ERR_BAD_TYPE);
+      if (a.Y) {   // out-of-range type: the row's output is defined to be zero
+        char *y = (char *)a.Y + (size_t)(r0 + tid) * a.ldy * a.y_elem_bytes;
+        for (int e = 0; e < a.N * a.y_elem_bytes; ++e) y[e] = 0;
+      }
+    }
+  }
+  __syncthreads();
+  for (int u = warp; u < units; u += kCopyWarps) {
+    if (u != warp) load(u);
+    const int row = u / chunks, v0 = (u - row * chunks) * kCopyUnit + lane;
+    uint4 *dst = Xb + (int64_t)s_dst[row] * vecs;
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (v0 + e * 32 < vecs) dst[v0 + e * 32] = w[e];
+  }
+  if (blockIdx.x == 0) {
+    for (int t = tid; t <= nt; t += kCopyThreads) a.hdr->offsets[t] = s_off[t];
+    if (tid == 0) write_pad_offsets(a.hdr, s_off, a.q);
+  }
+}
+
 // padded row p -> original row (or -1 for a pad row / beyond the last bucket)
 __device__ __forceinline__ int padded_source_row(const WsHeader *hdr, const int *perm, int q, int p) {
   int t = 0;
@@ -604,6 +738,19 @@ cudaError_t launch_copy_rows(CopyArgs a, cudaStream_t st) {
   return cudaLaunchKernelEx(&cfg, copy_rows_kernel, a);
 }
 }  // namespace
+
+bool bucket_copy_takes(int q, int64_t M, int64_t row_bytes) {
+  return q <= kMaxQ && M <= kCopyCountRows && M * row_bytes < kBulkCopyBytes && row_bytes % 16 == 0;
+}
+
+cudaError_t launch_bucket_copy(const BucketArgs &a, const void *X, int64_t ldx, int K, int elem_bytes, void *Xb, cudaStream_t st) {
+  const int64_t row_bytes = (int64_t)K * elem_bytes;
+  if (!bucket_copy_takes(a.q, a.M, row_bytes)) return cudaErrorInvalidValue;
+  const int rows = ceil_div(a.M, 148), grid = ceil_div(a.M, rows);
+  count_launch(1);
+  return launch_pdl(a.q <= 8 ? bucket_copy_kernel<true> : bucket_copy_kernel<false>, grid, kCopyThreads, st, a, (const uint4 *)X,
+                    (int64_t)(ldx * elem_bytes / 16), (int)(row_bytes / 16), (uint4 *)Xb, rows);
+}
 
 cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K, int elem_bytes, void *Xb, int *status,
                                long long wait_limit, cudaStream_t st) {

@@ -88,6 +88,9 @@ struct BucketArgs {
 cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t st);
 // Xb[d, 0:K] = X[perm[d], 0:K] (16-byte vectors; K*elem_bytes % 16 == 0)
 constexpr int64_t kBulkCopyBytes = 40 << 20;   // from this many bytes on by the bulk copy engine (see copy_rows_kernel)
+// Bucketing and the bucketed copy of X in one launch; only where bucket_copy_takes says so.
+bool bucket_copy_takes(int q, int64_t M, int64_t row_bytes);
+cudaError_t launch_bucket_copy(const BucketArgs &a, const void *X, int64_t ldx, int K, int elem_bytes, void *Xb, cudaStream_t st);
 cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int M, int K, int elem_bytes, void *Xb, int *status,
                                long long wait_limit, cudaStream_t st);
 // Weight-gradient pass (bf16): bucketed copies of X (K columns) and G (N columns) with every bucket padded to a multiple

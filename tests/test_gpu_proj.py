@@ -547,3 +547,38 @@ def test_large_row_copy(s_w):
     rows = np.unique(np.r_[0:30, wl.M // 2:wl.M // 2 + 30, wl.M - 30:wl.M])
     ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
     assert np.array_equal(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref)
+
+
+# ---- buckets and the bucketed copy of X in one launch: one row per CTA, several, the last batch it takes and the first it
+# does not, counters in registers (q <= 8) and in shared memory (more), rows of less than one unit of a warp and of several,
+# an absent type, out-of-range types, rows with a gap between them -----------------------------------------------------
+
+@pytest.mark.parametrize("q,M", [(1, 65), (2, 148), (3, 149), (8, 1025), (9, 1777), (32, 2100), (8, 8192), (32, 8192), (8, 8193)])
+@pytest.mark.parametrize("s_w", [64, 1088])
+def test_buckets_and_copy_in_one_launch(q, M, s_w):
+    if q * s_w * M > 1 << 24:
+        s_w = 64
+    types = synth.uniform_types(5 * q + M, M, q)
+    if q > 2:
+        types[types == 1] = 2
+    wl = _tc_workload(q, M, s_w, 128, types=types, seed=91)
+    t2 = types.copy()
+    t2[M // 2], t2[M - 1] = -1, q                 # outside [0, q): those rows of Y are zero
+    X = torch.zeros((M, q * s_w + 8), dtype=torch.bfloat16, device="cuda")
+    X[:, :q * s_w] = H.to_dev(wl.X, "bf16")
+    X = X[:, :q * s_w]
+    W, tt = H.to_dev(wl.W_up, "bf16"), H.dev_types(t2)
+    proj = binding.Proj(wl.d_widths, wl.f_widths)
+    n0 = binding.launch_count()
+    got = proj.forward(X, tt, W, out_dtype=torch.float32)
+    one_launch = binding.launch_count() - n0 == 2
+    assert one_launch == (M <= 8192)
+    assert proj.last_status() == 5
+    assert not got[M // 2].any() and not got[M - 1].any()
+    rows = np.unique(np.r_[np.arange(0, M, max(1, M // 300)), M - 2])
+    rows = rows[(rows != M // 2) & (rows != M - 1)]
+    ref = oracle.proj(wl.X[rows], types[rows], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(got[torch.from_numpy(rows).cuda()]), ref)
+    apart = binding.Proj(wl.d_widths, wl.f_widths)
+    apart.set_option("row_gather", 1)             # a copy pass of its own: every row, bit for bit
+    assert torch.equal(apart.forward(X, tt, W, out_dtype=torch.float32), got)
