@@ -69,6 +69,8 @@ constexpr int kEpiWarps = 8;
 constexpr int kProducerWarpB = 10;
 constexpr int kStoreBufBytes = 32 * 64;   // per epilogue warp: 32 rows x 32 bf16 columns
 
+constexpr int kBigSeq = 64;   // tiles of a CTA decoded in the prologue
+
 struct Ctl {
   uint64_t full[12];
   uint64_t empty[12];
@@ -78,6 +80,7 @@ struct Ctl {
   volatile int abort_flag;
   long long wait_limit;
   int total;                    // tiles of the launch
+  int4 recs[kBigSeq];           // this CTA's first tiles (pack_tile)
   int off[kBigMaxQ + 1];        // sched 0: first bucketed row of every type
   int pre[kBigMaxQ + 1];        // sched 0: tiles before type i
 };
@@ -137,7 +140,7 @@ __device__ __forceinline__ int fast_div(int t, int d, float inv_d) {
 
 // Tile t of the launch (uniform across the warp).  Type-major; inside a type: m-tile fastest, then
 // the column tile, then the output group.
-__device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
+__device__ __noinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
   Tile o;
   o.row0 = -1, o.rows = 0, o.i = 0, o.j = 0, o.n0 = 0, o.cols = 0, o.n0_w = 0, o.np = 1, o.ng = 1;
   if (t >= ctl->total) return o;
@@ -220,10 +223,40 @@ __device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, in
   return o;
 }
 
+// The tiles of a CTA are decoded once, a tile per lane, into 16-byte records.  Decoded by every role for every tile (a
+// search over the types and divisions, in code of its own per role) a tile cost the MMA warp 2.4 k of the 4 k cycles it
+// took at 64 rows per type and reductions of 128, and no wait showed it.  (Gated FFN 2048 -> 6144, q = 32, M = 2048: 73.2 ->
+// 67.2 us, M = 4096 106.1 -> 94.5; 25600 -> 5120, q = 128, M = 2048: 114.5 -> 109; 2048 -> 768, q = 16: 9.1 -> 7.8.)
+__device__ __forceinline__ int4 pack_tile(const Tile &o) {
+  return make_int4(o.row0, o.n0, o.rows | (o.cols << 8) | (o.np << 20), o.i | (o.j << 8) | (o.ng << 16));
+}
+// record `round` of this CTA, uniform across the warp; tiles past the records are decoded where they are needed
+__device__ __forceinline__ Tile get_tile(const BigArgs &a, const Ctl *ctl, int round) {
+  if (round >= kBigSeq) return decode_tile(a, ctl, blockIdx.x + round * gridDim.x);
+  const int4 v = ctl->recs[round];
+  const int w = __shfl_sync(0xffffffffu, v.z, 0), x = __shfl_sync(0xffffffffu, v.w, 0);
+  Tile o;
+  o.row0 = __shfl_sync(0xffffffffu, v.x, 0), o.n0 = __shfl_sync(0xffffffffu, v.y, 0);
+  o.rows = w & 0xFF, o.cols = (w >> 8) & 0xFFF, o.np = (w >> 20) & 0xFF;
+  o.i = x & 0xFF, o.j = (x >> 8) & 0xFF, o.ng = x >> 16;
+  o.n0_w = o.n0 + o.j * (a.r - a.r_out);
+  return o;
+}
+__device__ __forceinline__ void decode_tiles(const BigArgs &a, Ctl *ctl) {   // one warp
+  __syncwarp();
+  const int lane = threadIdx.x & 31;
+  for (int round = lane; round < kBigSeq; round += 32) {
+    const Tile o = decode_tile(a, ctl, blockIdx.x + round * gridDim.x);
+    ctl->recs[round] = pack_tile(o);
+    if (!__any_sync(0xffffffffu, o.row0 >= 0)) break;
+  }
+}
+
 template <int TILE_N, int BK>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2, const BigArgs a) {
+                const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2,
+                const __grid_constant__ BigArgs a) {
   using C = Cfg<TILE_N, BK>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -260,9 +293,10 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   }
   // Everything above touches only this CTA's own state and may overlap the previous kernel of the stream.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.sched == 0 || warp != 2) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 2) {
-    // tile counts: one warp turns the bucket offsets into "tiles before type i"
+    // tile counts (counted buckets: one warp turns the bucket offsets into "tiles before type i"), then this CTA's tiles;
+    // with equal buckets nothing of it comes from the previous kernel
     if (a.pack > 1 && a.gpack > 1) {
       // tiles before every type group (see decode_tile)
       const int n_tg = (q + a.pack - 1) / a.pack, g = a.gpack, n_units = (q + g - 1) / g;
@@ -310,6 +344,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
       if (lane == 0) ctl->pre[q] = carry, ctl->total = carry;
     }
+    decode_tiles(a, ctl);
+    if (a.sched != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -328,8 +364,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t smem0 = smem_u32(smem);
     const int b_chunks = a.gated_f ? 2 * a.n_chunks : a.n_chunks;   // 64-column boxes of the bank per stage
     const uint32_t stage_tx = (uint32_t)(a.a_box_rows * BK * 2 + b_chunks * C::kBChunkBytes);   // bytes the copies of a stage deliver
-    for (int t = blockIdx.x; ok; t += gridDim.x) {
-      const Tile tl = decode_tile(a, ctl, t);
+    for (int round = 0; ok; ++round) {
+      const Tile tl = get_tile(a, ctl, round);
       if (tl.row0 < 0) break;
       if (loads_a && lane == 0) ALG_TRACE(0, 1);
       const bool packed = a.pack > 1;
@@ -414,8 +450,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int mma_n = a.gated_f ? 2 * a.n_chunks * 64 : a.tile_n;   // gated: gate chunks and up chunks side by side
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(mma_n >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
-    for (int t = blockIdx.x; ok; t += gridDim.x) {
-      const Tile tl = decode_tile(a, ctl, t);
+    for (int round = 0; ok; ++round) {
+      const Tile tl = get_tile(a, ctl, round);
       if (tl.row0 < 0) break;
       const int j_in_t = tl.ng == 1 && tl.j >= tl.i && tl.j < tl.i + tl.np ? 1 : 0;
       const bool pg = a.pack > 1 && a.gpack > 1;
@@ -484,8 +520,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t wr_sw = (uint32_t)(lane & 7);
     const int rd_r = lane >> 3, rd_p = lane & 7;     // row within a group of four, 16-byte piece of the row
     const bool store8 = (a.r_out & 7) != 0;
-    for (int t = blockIdx.x;; t += gridDim.x) {
-      const Tile tl = decode_tile(a, ctl, t);
+    for (int round = 0;; ++round) {
+      const Tile tl = get_tile(a, ctl, round);
       if (tl.row0 < 0) break;
       const int r = quad * 32 + lane;
       int64_t out_row = -1;

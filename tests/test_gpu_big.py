@@ -267,3 +267,22 @@ def test_big_many_small_types_and_narrow_groups_random(k):
     if out_dtype == torch.bfloat16:
         ref = H.bf16_rne(ref)
     assert np.array_equal(H.to_np(Y), ref), (q, rows, s_w, r_w, schedule)
+
+
+@pytest.mark.parametrize("q,M,s_w,r_w,schedule", [
+    (64, 64 * 130, 8, 264, "interval"),       # 16384 tiles: more per SM than the 64 a CTA decodes in its prologue
+    (64, 64 * 130, 8, 264, "cyclic"),
+    (32, 32 * 560, 8, 264, "explicit"),       # the same on counted buckets, with an absent type
+])
+def test_more_tiles_than_records(q, M, s_w, r_w, schedule):
+    wl = _workload(q, M, s_w, r_w, schedule, seed=61)
+    if schedule == "explicit":
+        wl.types[wl.types == 3] = 4
+    proj = binding.Proj(wl.d_widths, wl.f_widths, dtype="bf16", schedule=schedule)
+    proj.set_option("gemm_kernel", 4)
+    Y = proj.forward(H.to_dev(wl.X, "bf16"), H.dev_types(wl.types) if schedule == "explicit" else None, H.to_dev(wl.W_up, "bf16"),
+                     out_dtype=torch.float32)
+    assert proj.last_status() == 0
+    rows = np.unique(np.r_[np.arange(0, M, 61), M - 1])
+    ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref)
