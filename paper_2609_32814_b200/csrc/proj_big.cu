@@ -264,6 +264,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   Ctl *ctl = (Ctl *)(store_buf + kEpiWarps * kStoreBufBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = a.q;
+  const int nkb_seg = (a.s + BK - 1) / BK;   // pipeline stages per reduction segment (the last one zero-padded)
   ALG_TRACE_VARS;
   ALG_TRACE_CTA(0, 0);
   if (threadIdx.x == 0) ALG_TRACE(0, 20);
@@ -290,6 +291,18 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
     if (a.pack > 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA2) : "memory");
     if (a.gpack > 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB2) : "memory");
+  }
+  // Groups narrower than a stage: only their rows of W are fetched (a row costs the copy engine the same whether it holds
+  // data or fill).  The rows below them are zeroed here and never written again -- X is zero there, but zero times what
+  // the memory held may be NaN.  5120 -> 25600, q = 128 (groups of 40): M = 2048 92.0 -> 88.5 us, 8192 224 -> 214; q = 256
+  // 161.8 -> 158.
+  if (a.b_box_rows < BK) {
+    const int pieces = (BK - a.b_box_rows) * 8;   // 16-byte pieces of a 64-column box
+    for (int e = threadIdx.x; e < C::kStages * C::kChunks * pieces; e += kThreads) {
+      const int box = e / pieces, st = box / C::kChunks, c = box - st * C::kChunks;
+      *(uint4 *)(smem + st * C::kStageBytes + C::kABytes + c * C::kBChunkBytes + a.b_box_rows * 128 + (e - box * pieces) * 16) = make_uint4(0, 0, 0, 0);
+    }
+    fence_async_smem();
   }
   // Everything above touches only this CTA's own state and may overlap the previous kernel of the stream.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -352,7 +365,6 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   tc_fence_after();
   const uint32_t tmem_base = ctl->tmem_base;
   if (threadIdx.x == 0) ALG_TRACE(0, 24);
-  const int nkb_seg = (a.s + BK - 1) / BK;   // pipeline stages per reduction segment (the last one zero-padded)
 
   if (warp == 0 || warp == kProducerWarpB) {
     // ---------------- TMA producers (warp-uniform loops, one elected lane issues) ----------------
@@ -363,7 +375,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t smem0 = smem_u32(smem);
     const int b_chunks = a.gated_f ? 2 * a.n_chunks : a.n_chunks;   // 64-column boxes of the bank per stage
-    const uint32_t stage_tx = (uint32_t)(a.a_box_rows * BK * 2 + b_chunks * C::kBChunkBytes);   // bytes the copies of a stage deliver
+    const int box_bytes = a.b_box_rows * 128;                        // of such a box
+    const uint32_t stage_tx = (uint32_t)(a.a_box_rows * BK * 2 + b_chunks * box_bytes);   // bytes the copies of a stage deliver
     for (int round = 0; ok; ++round) {
       const Tile tl = get_tile(a, ctl, round);
       if (tl.row0 < 0) break;
@@ -406,17 +419,17 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
               if (diag_seg) {   // all rows of the tile: np types x rows_per_type rows, type-major
                 const int goff = (k - tl.j) * a.r;   // (with several groups only the 64-column boxes of group k are fetched)
                 const int nb = pg ? (goff + a.r - 1) / 64 - goff / 64 + 1 : b_chunks;
-                mbar_expect_tx(bar, (uint32_t)(a.pack * a.rows_per_type * BK * 2 + nb * C::kBChunkBytes));
+                mbar_expect_tx(bar, (uint32_t)(a.pack * a.rows_per_type * BK * 2 + nb * box_bytes));
                 tma_load_4d(sa, &tmA, bar, kb * BK, k, 0, tl.i);
               } else {         // the rows of type k where they sit in the tile, zeros everywhere else
-                mbar_expect_tx(bar, (uint32_t)(128 * BK * 2 + b_chunks * C::kBChunkBytes));
+                mbar_expect_tx(bar, (uint32_t)(128 * BK * 2 + b_chunks * box_bytes));
                 tma_load_4d(sa, &tmA2, bar, kb * BK, k, -(k - tl.i) * a.rows_per_type, k);
               }
             } else if (loads_a) {
               // (a diagonal segment of a multi-group tile fetches only the 64-column boxes its group touches)
               const int goff = (k - tl.j) * a.r;
               const int nb = gp && sg > 0 ? (goff + a.r - 1) / 64 - goff / 64 + 1 : b_chunks;
-              mbar_expect_tx(bar, (uint32_t)(a.a_box_rows * BK * 2 + nb * C::kBChunkBytes));
+              mbar_expect_tx(bar, (uint32_t)(a.a_box_rows * BK * 2 + nb * box_bytes));
               if (a.sched == 2) tma_load_4d(sa, &tmA, bar, kb * BK, k, tl.i, a_row);
               else tma_load_3d(sa, &tmA, bar, kb * BK, k, a_row);
             } else if (pg ? diag_seg : gp && sg > 0) {
@@ -782,7 +795,7 @@ cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
     // the bank by {column in group, column group, k in group, row group}
     const uint64_t dims[4] = {(uint64_t)a.r, (uint64_t)a.q, (uint64_t)a.s, (uint64_t)a.q};
     const uint64_t str[3] = {(uint64_t)a.r * 2, (uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
-    const uint32_t box[4] = {64, 1, (uint32_t)BK, 1};
+    const uint32_t box[4] = {64, 1, (uint32_t)a.b_box_rows, 1};
     e = make_map_nd(&tmB2, a.W, 4, dims, str, box, 128);
     if (e != cudaSuccess) return e;
   }
@@ -790,7 +803,7 @@ cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
     // the bank as {columns, k in group, group}: rows past the group's width read as zero
     const uint64_t dims[3] = {(uint64_t)a.q * (uint64_t)a.r * (a.gated_f ? 2 : 1), (uint64_t)a.s, (uint64_t)a.q};
     const uint64_t str[2] = {(uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
-    const uint32_t box[3] = {64, (uint32_t)BK, 1};
+    const uint32_t box[3] = {64, (uint32_t)a.b_box_rows, 1};
     e = make_map_nd(&tmB, a.W, 3, dims, str, box, 128);
   }
   if (e != cudaSuccess) return e;
@@ -838,6 +851,7 @@ cudaError_t launch_proj_big(const BigArgs &in, int num_sms, cudaStream_t st) {
   // several whole output groups per tile when they are narrow (one type per tile, no bias, no gate).  Measured:
   // 25600 -> 5120 at M = 32768: q = 64 (groups of 80) 0.557 -> 0.533 ms, q = 256 (24) 1.97 -> 1.57 ms; 5120 -> 25600 at
   // q = 256 (104) 1.49 -> 1.39 ms; groups of 128 lose (square product n = 8192: 0.065 -> 0.088 ms) and stay one per tile
+  a.b_box_rows = std::min(a.s, a.block_k);
   a.gpack = 1;
   a.col_units = a.q * a.nt_n;
   if (a.nt_n == 1 && !a.gated_f && !a.bias && a.r <= 112 && a.q >= 2) {
