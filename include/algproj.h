@@ -154,8 +154,8 @@ typedef enum {
 
 /* ---- projection handle ---------------------------------------------------------------------
  * alg_proj_create: build the interaction table for q groups (Eqs. q-product-diag/off, or the
- * DENSE / CUSTOM variants), pick kernels, allocate a few hundred bytes of device metadata on
- * the CURRENT device.  in_widths = s[q], out_widths = r[q] (host arrays, copied).  dtype is
+ * DENSE / CUSTOM variants), pick kernels, allocate device metadata on the CURRENT device (kilobytes; FFN handles that
+ * take the one-launch decode kernels also two buffers of hidden rows).  in_widths = s[q], out_widths = r[q] (host arrays, copied).  dtype is
  * the element type of X and W (ALG_F32: true fp32 FMAs; ALG_BF16: bf16 operands, fp32
  * accumulation).  custom_keep is read only for ALG_TABLE_CUSTOM, else pass NULL; every
  * (i,j) of a custom table must keep at least one k.  1 <= q <= ALG_MAX_Q.
@@ -334,8 +334,9 @@ alg_status_t alg_ffn_gated_forward(alg_ffn_t h, const void *X, const int32_t *ty
  *   grad_input : W is the forward bank (K x N, ldw >= N), used transposed in place.
  *   grad_weight: dW (K x N, lddw >= N) is overwritten, never accumulated into; blocks whose row
  *                types are absent from the batch come out zero.  Internally the rows are bucketed
- *                by type, X is copied transposed and G bucketed (both padded per bucket to a
- *                multiple of 64 rows with zeros), and one grouped GEMM reduces over the buckets.
+ *                by type, X and G are copied into buckets padded to a multiple of 64 rows with zeros
+ *                (X transposed where an input group is no multiple of 8 features), and one grouped
+ *                GEMM reduces over the buckets.
  * Workspace: alg_proj_grad_workspace_bytes(h, M), 256-byte aligned, no initialisation needed. */
 alg_status_t alg_proj_grad_create(alg_proj_grad_t *out, int q, const int32_t *in_widths,
                                   const int32_t *out_widths, alg_table_t table,

@@ -554,3 +554,30 @@ def test_one_launch_ffn_strip_widths_and_rows(dw, fw, M):
         assert np.array_equal(H.to_np(got), ref)
         types.fill_(int((wl.types[0] + 1) % q))
     assert ffn.last_status() == 0
+
+
+# ---- decode kernel: every count of 16-row fragments with its edges, X boxes of 16, 32 and 64 columns, clusters of 1 to 8
+# CTAs, 32- and 64-wide strips, groups whose k the warps do not share evenly ---------------------------------------------
+
+@pytest.mark.parametrize("q,s_w,r_w", [
+    (2, 16, 32),       # one CTA per strip, boxes of 16, one k step per group
+    (2, 48, 96),       # 32-wide strips
+    (3, 160, 64),      # boxes of 32
+    (2, 384, 1536),    # four warps, 64-wide strips
+    (2, 1536, 384),    # clusters
+    (5, 112, 160),     # seven k steps per group
+])
+@pytest.mark.parametrize("M", [9, 16, 17, 32, 33, 48, 49, 64])
+def test_decode_kernel_rows_boxes_and_splits(q, s_w, r_w, M):
+    wl = _wl(q, M, s_w, r_w, seed=500 + q)
+    types = wl.types.copy()
+    types[M // 2] = q                             # outside [0, q): that row of Y is zero
+    bias = synth.small_ints(73, (q * r_w,))
+    proj = binding.Proj(wl.d_widths, wl.f_widths, dtype="bf16")
+    assert proj.kernel_path(M) == binding.ALG_PATH_DECODE
+    Y = proj.forward(H.to_dev(wl.X, "bf16"), H.dev_types(types), H.to_dev(wl.W_up, "bf16"), bias=H.to_dev(bias, "bf16"),
+                     out_dtype=torch.float32)
+    assert proj.last_status() == 5
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths, bias=bias)
+    ref[M // 2] = 0
+    assert np.array_equal(H.to_np(Y), ref)
