@@ -581,3 +581,27 @@ def test_decode_kernel_rows_boxes_and_splits(q, s_w, r_w, M):
     ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths, bias=bias)
     ref[M // 2] = 0
     assert np.array_equal(H.to_np(Y), ref)
+
+
+def test_decode_gelu_of_every_bf16_value():
+    """GELU of the decode kernel alone: one product per output (x = 1, w = z), fp32 results.  0.5 z (1 + erff(z / sqrt 2))
+    is off by at most |z| / 2 times the error of 1 + erff: 2 ulp of erff (2^-23) + one rounding of the sum (2^-24) + a
+    rounded argument (0.48 * 2^-23), so 1.2e-7 |z|, and it is exactly zero where erff has reached -1 (gelu(-6) = -5.9e-9)."""
+    z = torch.arange(65536, dtype=torch.int32).to(torch.int16).view(torch.bfloat16).float()
+    z = z[torch.isfinite(z) & (z.abs() > 1e-3) & (z.abs() < 2e4)]
+    z = z[:z.numel() // 64 * 64]
+    n, K = z.numel(), 64
+    W = torch.zeros(K, n)
+    W[0] = z
+    z64 = z.double()
+    ref = torch.where(z64 < 0, 0.5 * z64 * torch.special.erfc(-z64 * 2 ** -0.5), 0.5 * z64 * (1 + torch.special.erf(z64 * 2 ** -0.5)))
+    bound = torch.where(z64 < -6, torch.full_like(z64, 6e-9), 1.2e-7 * z64.abs())
+    proj = binding.Proj([K], [n], dtype="bf16")
+    for M in (1, 17, 64):
+        X = torch.zeros(M, K)
+        X[:, 0] = 1
+        assert proj.kernel_path(M) == binding.ALG_PATH_DECODE
+        Y = proj.forward(X.cuda().bfloat16(), torch.zeros(M, dtype=torch.int32, device="cuda"), W.cuda().bfloat16(), act="gelu",
+                         out_dtype=torch.float32)
+        over = ((Y.double().cpu() - ref).abs() - bound).amax(0)
+        assert float(over.max()) <= 0, (M, float(z[over.argmax()]), float(over.max()))
