@@ -21,6 +21,7 @@ constexpr int kRowsUp = 4, kRowsDn = 8;   // row pairs per thread and phase: D <
 
 struct RowsCtl {
   uint64_t bar_up, bar_dn, bar_miss[2];
+  uint32_t spec_up, spec_dn;   // input groups requested for the row types as they stood early
   volatile int abort_flag;
 };
 
@@ -133,21 +134,23 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_rows_kernel(const __grid_cons
   // kept input groups of every row type for the two strips, 8 bits a type
   uint64_t keeps_up = 0, keeps_dn = 0;
   for (int t = 0; t < q; ++t) keeps_up |= (uint64_t)a.keep[t * q + ju] << (8 * t), keeps_dn |= (uint64_t)a.keep[t * q + jd] << (8 * t);
-  // speculative: the previous kernel may still be writing the types
-  uint32_t spec_up = 0, spec_dn = 0;
-#pragma unroll
-  for (int m = 0; m < MR; ++m) {
-    const int t = read_type(m);
-    if (t >= 0) spec_up |= (uint32_t)(keeps_up >> (8 * t)) & 0xFFu, spec_dn |= (uint32_t)(keeps_dn >> (8 * t)) & 0xFFu;
-  }
-  if (!has_up) spec_up = 0;
-  if (!has_dn) spec_dn = 0;
-
   if (tid == 0) {
-    request_slice(&tm_up, bar_up, wu, a.so_d, spec_up, q, col_u, NTU * 16, a.box_up, a.extra_expect_bytes);
-    request_slice(&tm_dn, bar_dn, wd, a.so_f, spec_dn, q, col_d, NTD * 16, a.box_dn, a.extra_expect_bytes);
+    // speculative: the previous kernel may still be writing the types, so one thread reads them for all -- read by every
+    // thread for itself, a warp could miss the late copies another one had asked for
+    uint32_t up = 0, dn = 0;
+#pragma unroll
+    for (int m = 0; m < MR; ++m) {
+      const int t = read_type(m);
+      if (t >= 0) up |= (uint32_t)(keeps_up >> (8 * t)) & 0xFFu, dn |= (uint32_t)(keeps_dn >> (8 * t)) & 0xFFu;
+    }
+    if (!has_up) up = 0;
+    if (!has_dn) dn = 0;
+    ctl->spec_up = up, ctl->spec_dn = dn;
+    request_slice(&tm_up, bar_up, wu, a.so_d, up, q, col_u, NTU * 16, a.box_up, a.extra_expect_bytes);
+    request_slice(&tm_dn, bar_dn, wd, a.so_f, dn, q, col_d, NTD * 16, a.box_dn, a.extra_expect_bytes);
   }
-  __syncthreads();   // the barriers are ready
+  __syncthreads();   // the barriers are ready, what was requested is known
+  const uint32_t spec_up = ctl->spec_up, spec_dn = ctl->spec_dn;
   // input group of this thread's row pairs, 4 bits each (15: past the end)
   uint32_t gid_up = 0, gid_dn = 0;
 #pragma unroll

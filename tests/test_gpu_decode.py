@@ -605,3 +605,56 @@ def test_decode_gelu_of_every_bf16_value():
                          out_dtype=torch.float32)
         over = ((Y.double().cpu() - ref).abs() - bound).amax(0)
         assert float(over.max()) <= 0, (M, float(z[over.argmax()]), float(over.max()))
+
+
+# ---- row types written by a kernel that lets its successor start before it stores them ---------------------------------
+
+class _TypeWriter:
+    """Writes row types with the fp32 projection, whose launch releases its successor before its stores: 1 x (t as a
+    denormal) has the bits of the integer t.  So the small-M kernels' early read of the types can see them old, new or
+    half written (a kernel of the framework never lets its successor start early)."""
+
+    def __init__(self, n, types):
+        self.proj = binding.Proj([4], [n], dtype="f32", schedule="cyclic")
+        self.x = torch.tensor([[1.0, 0, 0, 0]], device="cuda")
+        self.banks = []
+        for t in types:
+            bank = torch.zeros(4, n, dtype=torch.int32)
+            bank[0, :len(t)] = torch.as_tensor(t, dtype=torch.int32)
+            self.banks.append(bank.cuda().view(torch.float32))
+        self.out = torch.zeros(1, n, dtype=torch.float32, device="cuda")
+        self.types = self.out.view(torch.int32)[0, :len(types[0])]
+        self.ws = torch.empty(self.proj.workspace_bytes(1), dtype=torch.uint8, device="cuda")
+
+    def write(self, which):
+        self.proj.forward(self.x, None, self.banks[which], out=self.out, workspace=self.ws)
+
+
+@pytest.mark.parametrize("dw,fw,M", [
+    ([384, 384], [1536, 1536], 1), ([384, 384], [1536, 1536], 2),       # plain FMAs
+    ([128] * 4, [512] * 4, 1), ([128] * 4, [512] * 4, 2),
+    ([384, 384], [1536, 1536], 8), ([128] * 4, [512] * 4, 16),          # matrix path
+    ([384, 384], [1536, 1536], 40),                                     # two launches
+])
+def test_ffn_types_written_while_the_call_starts(dw, fw, M):
+    q = len(dw)
+    wl = _ffn_int_workload(q, M, sum(dw), sum(fw), seed=300 + M)
+    kinds = [np.full(M, 0, np.int32), np.full(M, q - 1, np.int32), wl.types]
+    writer = _TypeWriter(64, kinds)
+    ffn = binding.FFN(dw, fw, dtype="bf16")
+    X, Wu, Wd = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.to_dev(wl.W_down, "bf16")
+    refs = []
+    for t in kinds:
+        wl.types = t
+        refs.append(torch.from_numpy(_ffn_int_ref(wl)).float().cuda())
+    ws = torch.empty(ffn.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+    order = [0, 1, 2, 1, 0, 2] * 20
+    outs = [torch.empty(M, sum(dw), dtype=torch.float32, device="cuda") for _ in order]
+    torch.cuda.synchronize()
+    for which, out in zip(order, outs):
+        writer.write(which)
+        ffn.forward(X, writer.types, Wu, Wd, act=None, out=out, workspace=ws)
+    assert ffn.last_status() == 0
+    assert writer.types.tolist() == list(kinds[order[-1]])
+    for which, out in zip(order, outs):
+        assert torch.equal(out, refs[which])
