@@ -245,8 +245,9 @@ __device__ __forceinline__ void run_phase(const Phase &p, int type, const __nv_b
   }
 }
 
+// (row types are read twice, early and after the wait for the kernel that may write them: from L2, never a stale L1 line)
 __device__ __forceinline__ int read_type(const RowDecodeArgs &a) {
-  const int t = a.types ? a.types[0] : 0;
+  const int t = a.types ? __ldcg(a.types) : 0;
   return t < 0 || t >= a.q ? -1 : t;
 }
 
@@ -272,7 +273,7 @@ template <int MODE, int RC>
 __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(const RowDecodeArgs a) {
   constexpr bool GATED = MODE == 0, FFN = MODE != 2;
   __shared__ float partial[kWarps * 2 * 16];   // a piece has at most 2 x 8 columns
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_early;
   ALG_TRACE_VARS;
   if (threadIdx.x == 0) ALG_TRACE(0, 1);
   // phase 1 maps the D (projection: K) inputs to F (N) columns of W1; phase 2 maps F back to D through W2
@@ -285,11 +286,13 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
   __nv_bfloat16 *H = nullptr;   // hidden rows in the exchange buffer
   const int warp = threadIdx.x >> 5;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (threadIdx.x == 0) s_abort = 0;
 
   // ---- before the dependency resolves: the row type as it stands now and the first W1 loads it asks for (the type
-  // is read again after the wait) ----
-  const int t_early = read_type(a);
+  // is read again after the wait).  One thread reads it for the CTA: the previous kernel may be writing it, and warps
+  // that share a piece have to agree on what they compute and on the barriers they meet at ----
+  if (threadIdx.x == 0) s_abort = 0, s_early = read_type(a);
+  __syncthreads();
+  const int t_early = s_early;
   uint4 w[kLoads<GATED, RC>];
   {
     const int unit = unit_of(0, p1.ks);
@@ -298,7 +301,6 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
     load_chunk<GATED, RC>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
-  __syncthreads();   // s_abort is set
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 3);
   const int type = read_type(a);   // (in flight while phase 1 runs on the early value)
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
 }
 
 __device__ __forceinline__ int read_row_type(const RowDecodeArgs &a, int m) {
-  const int t = a.types ? a.types[m] : m % a.q;
+  const int t = a.types ? __ldcg(a.types + m) : m % a.q;
   return t < 0 || t >= a.q ? -1 : t;
 }
 
@@ -434,7 +436,7 @@ template <int MODE, int RC>
 __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(const RowDecodeArgs a) {
   constexpr bool GATED = MODE == 0, FFN = MODE != 2;
   __shared__ float partial[kWarps * 2 * 16];   // a piece has at most 2 x 8 columns
-  __shared__ int s_abort;
+  __shared__ int s_abort, s_early[kRowDecodeMaxM];
   ALG_TRACE_VARS;
   if (threadIdx.x == 0) ALG_TRACE(0, 1);
   // phase 1 maps the D (projection: K) inputs to F (N) columns of W1; phase 2 maps F back to D through W2
@@ -449,10 +451,12 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
   if (threadIdx.x == 0) s_abort = 0;
 
   // ---- before the dependency resolves: the type of this warp's first row as it stands now and the first W1 loads it
-  // asks for (the type is read again after the wait) ----
+  // asks for (the type is read again after the wait).  A thread per row reads it for the CTA, as above ----
+  if ((int)threadIdx.x < a.M) s_early[threadIdx.x] = read_row_type(a, threadIdx.x);
+  __syncthreads();
   const int per_row1 = a.M == 1 ? a.units1 : a.units1 / a.M;
   const int unit1 = unit_of(0, p1.ks), m1 = a.M == 1 ? 0 : min(unit1 / per_row1, a.M - 1);
-  const int t_early = read_row_type(a, m1);
+  const int t_early = s_early[m1];
   uint4 w[kLoads<GATED, RC>];
   {
     Lane l = lane_of(p1, unit1 - m1 * per_row1);
@@ -460,7 +464,6 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
     load_chunk<GATED, RC>(w, p1, l, max(t_early, 0), 0);
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
-  __syncthreads();   // s_abort is set
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 3);
   const Wait wait = {clock64(), a.wait_limit, &s_abort, a.status};
@@ -503,10 +506,10 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
       store1(a.Y, (int64_t)m * a.ldy + col, a.y_bf16 != 0, finish1(z, col, a.b2, ALG_ACT_NONE));
     });
     __syncthreads();
-  if (threadIdx.x == 0) {
-    ALG_TRACE(0, 12);
-    exch_leave(a.exch);
-  }
+    if (threadIdx.x == 0) {
+      ALG_TRACE(0, 12);
+      exch_leave(a.exch);
+    }
   }
 }
 

@@ -658,3 +658,39 @@ def test_ffn_types_written_while_the_call_starts(dw, fw, M):
     assert writer.types.tolist() == list(kinds[order[-1]])
     for which, out in zip(order, outs):
         assert torch.equal(out, refs[which])
+
+
+@pytest.mark.parametrize("kind,q,s_w,r_w,M", [
+    ("proj", 32, 64, 192, 1), ("proj", 8, 64, 128, 6), ("proj", 5, 24, 40, 2), ("proj", 2, 256, 64, 3),
+    ("ffn", 32, 64, 24, 1), ("ffn", 8, 96, 200, 4), ("gated", 32, 64, 24, 1), ("gated", 4, 256, 64, 8),
+])
+def test_row_kernel_types_written_while_the_call_starts(kind, q, s_w, r_w, M):
+    """The warps that share a piece (2, 4 or 8 of them for these shapes) must take the same type, whatever each would read."""
+    K, N = q * s_w, q * r_w
+    kinds = [np.full(M, 0, np.int32), np.full(M, q - 1, np.int32), synth.uniform_types(610 + q, M, q)]
+    writer = _TypeWriter(64, kinds)
+    wl, Wg = synth.gated_ffn("typerace", q, M, K, N, kinds[2], variant=31, integer=False)
+    X, Wd = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_down, "bf16")
+    Wu = H.to_dev(np.concatenate([Wg, wl.W_up], axis=1) if kind == "gated" else wl.W_up, "bf16")
+    h = {"proj": binding.Proj, "ffn": binding.FFN, "gated": binding.GatedFFN}[kind](wl.d_widths, wl.f_widths, dtype="bf16")
+    h.set_option("small_m_kernel", 3)
+    ws = torch.empty(h.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+
+    def call(types, out):
+        h.forward(X, types, Wu, **({} if kind == "proj" else {"W_down": Wd}), out=out, workspace=ws)
+    empty = lambda: torch.empty(M, N if kind == "proj" else K, dtype=torch.float32, device="cuda")
+    want = []
+    for t in kinds:   # types at rest; checked against the oracle by the tests above
+        want.append(empty())
+        call(H.dev_types(t), want[-1])
+        torch.cuda.synchronize()
+    order = [0, 1, 2, 1, 0, 2] * 20
+    outs = [empty() for _ in order]
+    torch.cuda.synchronize()
+    n0 = binding.launch_count()
+    for which, out in zip(order, outs):
+        writer.write(which)
+        call(writer.types, out)
+    assert binding.launch_count() - n0 == 2 * len(order) and h.last_status() == 0
+    for which, out in zip(order, outs):
+        assert torch.equal(out, want[which])
