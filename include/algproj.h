@@ -277,7 +277,7 @@ alg_status_t alg_proj_pack_weight(alg_proj_t h, const void *W, int64_t ldw, void
  * The two-map MLP (g = 1 in Eq. icml-decode-total) with both projections under the same law
  * and the same row types (the projection is row-local).  d_widths: q groups of d_model,
  * f_widths: q groups of d_ff.  X: M x D packed (ld = D), W_up: D x F packed, W_down: F x D
- * packed, Y: M x D packed.  The hidden state H = act(.) is kept in the workspace in the
+ * packed, Y: M x D packed; Y may be X (the layer in place).  The hidden state H = act(.) is kept in the workspace in the
  * handle's dtype (bf16: rounded to nearest even), rows in type-bucketed order.
  * 1 <= q <= ALG_MAX_Q, schedule EXPLICIT or CYCLIC (larger algebras and the INTERVAL schedule
  * exist for single projections only: ALG_ERR_UNSUPPORTED_SHAPE).  Which GEMM kernel runs the two

@@ -1556,6 +1556,7 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
   if (workspace_bytes < L.total) return ALG_ERR_WORKSPACE_TOO_SMALL;
   cudaStream_t st = (cudaStream_t)stream;
   char *ws = (char *)workspace;
+  const bool in_place = (uintptr_t)X < (uintptr_t)Y + (size_t)M * h->D * elem_bytes(y_dtype) && (uintptr_t)Y < (uintptr_t)X + (size_t)M * h->D * eb;
   if (h->fd_ok && (h->up.opt_small_m == 1 || h->up.opt_small_m == 2 || (h->up.opt_small_m == 3 && !h->rd_ok)) && M <= kFfnDecodeMaxM && !h->timing) {
     // decode step in one launch: both projections, H exchanged through L2 inside the kernel
     const alg_proj_s &u = h->up;
@@ -1570,6 +1571,7 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
     d.y_bf16 = y_dtype == ALG_BF16;
     d.D = h->D, d.F = h->F, d.q = u.q;
     d.exch = h->d_exch, d.exch_bytes = h->exch_bytes;
+    d.in_place = in_place;
     d.status = u.d_status;
     d.wait_limit = u.wait_limit;
     d.extra_expect_bytes = u.test_extra_expect;
@@ -1598,6 +1600,7 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
     d.y_bf16 = y_dtype == ALG_BF16;
     d.D = h->D, d.F = h->F, d.q = h->up.q;
     d.exch = h->d_exch, d.exch_bytes = h->exch_bytes;
+    d.in_place = in_place;
     d.status = h->up.d_status;
     d.wait_limit = h->up.wait_limit;
     d.test_withhold = h->up.test_extra_expect ? 1 : 0;

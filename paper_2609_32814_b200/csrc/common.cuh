@@ -321,6 +321,7 @@ struct FfnDecodeArgs {
   int kc_up, kc_dn, m_pad;                 // K-chunk lengths of the staged activations; staged rows (8 or 16)
   uint8_t *exch;                           // hidden rows between the phases (exchange.cuh), buffers of exch_bytes
   int exch_bytes;
+  int in_place;                            // Y lies over X: no CTA stores Y before every CTA has used its X
   int *status;
   long long wait_limit;
   int extra_expect_bytes;
@@ -358,6 +359,7 @@ struct RowDecodeArgs {
   int units1, units2;       // pieces x sharing warps                              (set by the launcher)
   uint8_t *exch;            // FFN modes: hidden rows between the phases (exchange.cuh), buffers of exch_bytes
   int exch_bytes;
+  int in_place;             // Y lies over X: no CTA stores Y before every CTA has used its X (FFN modes)
   int *status;
   long long wait_limit;
   int test_withhold;        // test hook: CTA 0 keeps its hidden values to itself, so that the waits for them run out

@@ -13,7 +13,9 @@
 // 768 -> 3072 -> 768, q = 2, per layer of a graph of layers: one row 7.5 (matrix path) -> 5.5 us, two rows 8.4 -> 7.1 us.
 // The products of 4 rows take longer here than there (9.4 against 7.8 us a layer).  The 16 CTAs of 128 that a row's
 // reader has yet to wait for when it starts (three quarters of the hints) save 0.1 us; with two rows waiting for all
-// hints is 0.3 us better, loads that come too early cost more there.
+// hints is 0.3 us better, loads that come too early cost more there.  Where Y lies over X a CTA with one row waits for all
+// hints too: the values it needs (those of the row's type, for the group of its type) do not say that the CTAs of the
+// other hidden groups have used X.
 #pragma once
 
 constexpr int kRowsMax = 2;          // rows of ffn_rows_kernel
@@ -245,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_rows_kernel(const __grid_cons
   if (has_dn) {
     uint32_t spins = 0;
     if (tid == 0)
-      while (!exch_hinted(a.exch, turn, MR == 1 ? a.n_up - (a.n_up >> 2) : a.n_up))
+      while (!exch_hinted(a.exch, turn, MR == 1 && !a.in_place ? a.n_up - (a.n_up >> 2) : a.n_up))
         if (give_up(spins)) break;
     __syncthreads();
     uint32_t xd[kRowsDn][MR], live = 0;

@@ -268,6 +268,24 @@ __device__ __forceinline__ void store1(void *out, int64_t at, bool out_bf16, flo
 }
 __device__ __forceinline__ float gated1(float g, float u) { return g / (1.f + __expf(-g)) * u; }   // silu(g) * u
 
+// Y lies over X (an FFN in place): a CTA says when it has used its X, and stores Y once every CTA of the grid has.  The
+// hidden values a CTA waits for tell it nothing about the CTAs whose values it does not need, and those may start late.
+__device__ __forceinline__ void used_x(const RowDecodeArgs &a, const ExchTurn &turn) {
+  __syncthreads();
+  if (threadIdx.x == 0) exch_hint(a.exch, turn);
+}
+__device__ __forceinline__ void all_used_x(const RowDecodeArgs &a, const ExchTurn &turn, const Wait &wait) {
+  if (threadIdx.x == 0) {
+    while (!exch_hinted(a.exch, turn, gridDim.x))
+      if (clock64() - wait.t0 > wait.limit) {
+        *wait.abort_flag = 1;
+        atomicExch(wait.status, (int)ALG_ERR_DEVICE_TIMEOUT);
+        break;
+      }
+  }
+  __syncthreads();
+}
+
 // MODE 0: gated FFN, 1: FFN, 2: projection (W1 only)
 template <int MODE, int RC>
 __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(const RowDecodeArgs a) {
@@ -337,6 +355,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
     return;
   }
 
+  if (a.in_place) used_x(a, turn);
   // ---- the first W_down loads go out before the hidden values are waited for ----
   uint4 w2[kLoads<false, RC>];
   {
@@ -348,6 +367,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
 
   exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, 1);
   if (threadIdx.x == 0) ALG_TRACE(0, 9);
+  if (a.in_place) all_used_x(a, turn, wait);
 
   // ---- phase 2: y = h * W_down (+ b_down) ----
   if (type >= 0) {
@@ -487,6 +507,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
   if (threadIdx.x == 0) ALG_TRACE(0, 6);
 
   if (FFN) {
+    if (a.in_place) used_x(a, turn);
     // ---- the first W_down loads go out before the hidden values are waited for ----
     uint4 w2[kLoads<false, RC>];
     const int per_row2 = a.M == 1 ? a.units2 : a.units2 / a.M;
@@ -500,6 +521,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
 
     exch_clear(a.exch, a.exch_bytes, turn, a.F * 2, a.M);
     if (threadIdx.x == 0) ALG_TRACE(0, 9);
+    if (a.in_place) all_used_x(a, turn, wait);
 
     // ---- phase 2: y = h * W_down (+ b_down) ----
     run_rows_phase<false, true, true, RC>(a, p2, H, a.F, w2, true, type2, a.units2, partial, wait, [&](int m, int col, float z, float) {

@@ -694,3 +694,38 @@ def test_row_kernel_types_written_while_the_call_starts(kind, q, s_w, r_w, M):
     assert binding.launch_count() - n0 == 2 * len(order) and h.last_status() == 0
     for which, out in zip(order, outs):
         assert torch.equal(out, want[which])
+
+
+# ---- FFN layers in place -------------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("kind,q,dw,fw,option", [
+    ("plain", 2, 384, 1536, 1), ("plain", 2, 512, 2048, 1),   # plain FMAs, matrix path; one CTA per SM
+    ("plain", 8, 96, 200, 3), ("gated", 32, 64, 192, 3),      # row kernel
+    ("plain", 2, 384, 1536, 0), ("gated", 32, 64, 192, 0),    # prefill kernels
+])
+@pytest.mark.parametrize("M", [1, 2, 8])
+def test_ffn_in_place(kind, q, dw, fw, option, M):
+    """Y over X gives the bits of Y elsewhere, also while another stream's kernels hold SMs and CTAs of a launch start
+    at different times."""
+    D, F = q * dw, q * fw
+    wl, Wg = synth.gated_ffn("inplace", q, M, D, F, synth.uniform_types(700 + q + M, M, q), variant=41, integer=False)
+    up = np.concatenate([Wg, wl.W_up], axis=1) if kind == "gated" else wl.W_up
+    X, types, Wu, Wd = H.to_dev(wl.X, "bf16"), H.dev_types(wl.types), H.to_dev(up, "bf16"), H.to_dev(wl.W_down, "bf16")
+    ffn = (binding.GatedFFN if kind == "gated" else binding.FFN)(wl.d_widths, wl.f_widths, dtype="bf16")
+    ffn.set_option("small_m_kernel", option)
+    ws = torch.empty(ffn.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+    want = torch.empty_like(X)
+    ffn.forward(X, types, Wu, Wd, out=want, workspace=ws)
+    bufs = [X.clone() for _ in range(30)]
+    big = torch.randn(4096, 4096, device="cuda", dtype=torch.bfloat16)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(10):
+            big @ big
+    for b in bufs:
+        ffn.forward(b, types, Wu, Wd, out=b, workspace=ws)
+    torch.cuda.synchronize()
+    assert ffn.last_status() == 0
+    for b in bufs:
+        assert torch.equal(b, want)
