@@ -253,6 +253,10 @@ bool device_facts(int dev, int *major, int *num_sms) {
          cudaDeviceGetAttribute(num_sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
 }
 
+// Device memory of a handle is filled on the legacy stream, and a fill returns before it is done.  A caller's stream need
+// not be ordered behind that one, so handles are given out, and a status is reported, when the fills are over.
+alg_status_t fills_done() { return cudaStreamSynchronize(cudaStreamLegacy) == cudaSuccess ? ALG_OK : ALG_ERR_CUDA; }
+
 // Handle of the large-algebra path only (q > kMaxQ or the interval schedule): no interaction table.
 alg_status_t init_big(alg_proj_s &p, int q, int s, int r, alg_schedule_t sched) {
   p.q = q;
@@ -271,7 +275,7 @@ alg_status_t init_big(alg_proj_s &p, int q, int s, int r, alg_schedule_t sched) 
   if (cudaMalloc(&p.d_status, 4 * sizeof(int)) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemset(p.d_status, 0, 4 * sizeof(int)) != cudaSuccess) return ALG_ERR_CUDA;
   if (tc_init() != cudaSuccess) return ALG_ERR_CUDA;
-  return ALG_OK;
+  return fills_done();
 }
 
 alg_status_t init_proj(alg_proj_s &p, int q, const int32_t *in_w, const int32_t *out_w, alg_dtype_t dtype,
@@ -378,7 +382,7 @@ alg_status_t init_proj(alg_proj_s &p, int q, const int32_t *in_w, const int32_t 
     // are several times faster (4096 -> 12288 at q = 32: M = 2 74 against 16 us, M = 64 377 against 46 us)
     if (q > kDecodeParamQ && (int64_t)p.K * p.N > (int64_t)4 << 20) p.decode_ok = false;
   }
-  return ALG_OK;
+  return fills_done();
 }
 
 void free_proj(alg_proj_s &p) {
@@ -1201,7 +1205,7 @@ static alg_status_t read_status(int *d_status, void *stream, alg_status_t *statu
   if (cudaStreamSynchronize(st) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemcpy(&v, d_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return ALG_ERR_CUDA;
   // a launch that gave up may have left the bucketing counters behind the status word half way
-  if (v != 0 && cudaMemset(d_status, 0, 4 * sizeof(int)) != cudaSuccess) return ALG_ERR_CUDA;
+  if (v != 0 && (cudaMemset(d_status, 0, 4 * sizeof(int)) != cudaSuccess || fills_done() != ALG_OK)) return ALG_ERR_CUDA;
   *status = (alg_status_t)v;
   return ALG_OK;
 }
@@ -1454,7 +1458,8 @@ static alg_status_t reset_exchange(alg_ffn_s &f) {
   const size_t buffers = 2 * (size_t)f.exch_bytes;
   if (!f.d_exch && cudaMalloc(&f.d_exch, kExchHeader + buffers) != cudaSuccess) return ALG_ERR_CUDA;
   if (cudaMemset(f.d_exch, 0, kExchHeader) != cudaSuccess) return ALG_ERR_CUDA;
-  return cuda_status(cudaMemset(f.d_exch + kExchHeader, 0xFF, buffers));
+  if (cudaMemset(f.d_exch + kExchHeader, 0xFF, buffers) != cudaSuccess) return ALG_ERR_CUDA;
+  return fills_done();   // (unfilled bytes would be taken for hidden values)
 }
 
 static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, const int32_t *f_widths,

@@ -729,3 +729,13 @@ def test_ffn_in_place(kind, q, dw, fw, option, M):
     assert ffn.last_status() == 0
     for b in bufs:
         assert torch.equal(b, want)
+
+
+def test_a_new_handle_has_its_buffers_filled():
+    """The exchange buffers start out filled with the empty pattern; a forward on a stream that is not ordered behind the
+    legacy stream may follow creation at once.  Half a gigabyte of them (no weights are needed for that) takes long enough to
+    fill to see whether creation waits."""
+    torch.cuda.synchronize()
+    ffn = binding.FFN([64] * 32, [524288] * 32, dtype="bf16")
+    assert torch.cuda.default_stream().query()
+    ffn.close()
