@@ -322,8 +322,17 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     if (splits > 1) send_f32x4(smem_u32(at), bar_p, (uint32_t)(m - slot * splits), z);
     else *(float4 *)at = z;
   }
-  if (splits > 1) wait_bar(bar_p, 0);   // every partial sum of my rows has arrived
-  else __syncthreads();
+  if (splits > 1) {
+    // every partial sum of my rows has arrived; where it has not, the senders may be late (each has waits of its own that
+    // can run out), so this thread -- and with it the shared memory they send to -- stays until every thread of the cluster
+    // has left or is here too
+    if (!wait_bar(bar_p, 0)) {
+      asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    }
+  } else {
+    __syncthreads();
+  }
   DTR();
 
   // ---- add the partial sums of my rows in split order, bias, activation, store ----

@@ -739,3 +739,24 @@ def test_a_new_handle_has_its_buffers_filled():
     ffn = binding.FFN([64] * 32, [524288] * 32, dtype="bf16")
     assert torch.cuda.default_stream().query()
     ffn.close()
+
+
+@pytest.mark.parametrize("s_w,r_w", [(1536, 384), (384, 1536)])   # clusters of several CTAs
+def test_decode_waits_that_run_out_at_different_times(s_w, r_w):
+    """With a limit of 1000 cycles the waits of a cluster's CTAs run out one here, one there, those for the partial sums
+    among them; the launch ends, says so, and the handle computes exactly afterwards."""
+    q, M = 2, 40
+    wl = _wl(q, M, s_w, r_w, seed=811)
+    proj = binding.Proj(wl.d_widths, wl.f_widths, dtype="bf16")
+    X, t, W = H.to_dev(wl.X, "bf16"), H.dev_types(wl.types), H.to_dev(wl.W_up, "bf16")
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths)
+    proj.set_option("test_stall_bytes", 1024)
+    for limit in (1000, 20000):
+        proj.set_option("wait_limit_cycles", limit)
+        for _ in range(3):
+            proj.forward(X, t, W, out_dtype=torch.float32)
+        assert proj.last_status() == 6
+    proj.set_option("test_stall_bytes", 0)
+    proj.set_option("wait_limit_cycles", 4_000_000_000)
+    assert np.array_equal(H.to_np(proj.forward(X, t, W, out_dtype=torch.float32)), ref)
+    assert proj.last_status() == 0
