@@ -662,10 +662,12 @@ cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t st) {
     return cudaGetLastError();
   }
   // clusters of 16 are not portable: asked for once, used where the device says one can be resident
+  static OncePerDevice wide;
   static int rows16 = -1;
+  const bool asked = wide([] { return cudaFuncSetAttribute(bucket_onepass_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1); }) == cudaSuccess;
   if (rows16 < 0) {
     rows16 = 0;
-    if (cudaFuncSetAttribute(bucket_onepass_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    if (asked) {
       cudaLaunchConfig_t probe = {};
       probe.gridDim = dim3(16, 1, 1);
       probe.blockDim = dim3(kFusedThreads, 1, 1);
@@ -679,7 +681,8 @@ cudaError_t launch_bucket(const BucketArgs &a, cudaStream_t st) {
     }
     (void)cudaGetLastError();
   }
-  if (a.M <= std::max(kClusterRows, rows16)) {   // one kernel, one cluster of 1 ... 16 CTAs (CTAs past the batch hold no row)
+  if (!asked) (void)cudaGetLastError();
+  if (a.M <= std::max(kClusterRows, asked ? rows16 : 0)) {   // one kernel, one cluster of 1 ... 16 CTAs (CTAs past the batch hold no row)
     int n_cta = 1;
     while (n_cta * kFusedThreads < a.M) n_cta *= 2;
     cudaLaunchConfig_t cfg = {};
@@ -717,12 +720,9 @@ cudaError_t launch_copy_rows(CopyArgs a, cudaStream_t st) {
   }
   a.slot = (slot + 127) / 128 * 128;
   a.agents = std::min(kMaxAgents, kSlotBytes / a.slot - (a.hdr ? 1 : 0));
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(copy_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlotBytes + 1024);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice limit;
+  const cudaError_t e = limit([] { return cudaFuncSetAttribute(copy_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlotBytes + 1024); });
+  if (e != cudaSuccess) return e;
   const int64_t units = (int64_t)a.rows * (a.pieces[0] + a.pieces[1]);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, std::min<int64_t>(148, units)), 1, 1);

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "algproj.h"
+#include "per_device.h"
 
 namespace algproj {
 

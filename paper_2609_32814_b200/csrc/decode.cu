@@ -378,14 +378,11 @@ decode_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
 
 template <int SN, int MT>
 cudaError_t launch_t(const DecodeArgs &a, size_t smem_bytes, cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(decode_kernel<SN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static OncePerDevice limit;
+  cudaError_t e = limit([] { return cudaFuncSetAttribute(decode_kernel<SN, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); });
+  if (e != cudaSuccess) return e;
   CUtensorMap tmW, tmX;
-  cudaError_t e = make_map_2d_sw(&tmW, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.ldw * 2, SN, (uint32_t)a.box_rows,
+  e = make_map_2d_sw(&tmW, a.W, (uint64_t)a.N, (uint64_t)a.K, (uint64_t)a.ldw * 2, SN, (uint32_t)a.box_rows,
                                  SN * 2);
   if (e != cudaSuccess) return e;
   e = make_map_2d_sw(&tmX, a.X, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.ldx * 2, (uint32_t)a.x_box, 16 * MT, a.x_box * 2);

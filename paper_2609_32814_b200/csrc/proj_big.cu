@@ -760,15 +760,11 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 template <int TILE_N, int BK>
 cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
   using C = Cfg<TILE_N, BK>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static OncePerDevice limit;
+  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
+  if (e != cudaSuccess) return e;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
   CUtensorMap tmA, tmA2, tmB;
-  cudaError_t e;
   const BigArgs &b = a;
   if (b.pack > 1) {
     // X as {k in group, group, row in type, type}: interval rows of a type are consecutive, cyclic ones q apart

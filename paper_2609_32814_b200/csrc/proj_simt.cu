@@ -4,7 +4,6 @@
 //   proj_f32_kernel   fp32 operands: asynchronous copies into a three-stage ring, register tiles.
 //   proj_simt_kernel  bf16 operands of the shapes the tensor-core paths do not cover (and their input gradient).
 #include <algorithm>
-#include <atomic>
 
 #include "tile_map.cuh"
 
@@ -374,16 +373,12 @@ __global__ void __launch_bounds__(256, TM_ == 64 ? 2 : 1) proj_f32_kernel(const 
 template <int TM_, int VEC>
 cudaError_t launch_f32(const ProjArgs &a, int grid, cudaStream_t st) {
   const size_t smem = F32Cfg<TM_>::kRingBytes + tile_map_bytes(a.n_classes);
-  static std::atomic<uint64_t> done{0};   // devices whose limit is raised, a bit each
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  static OncePerDevice limit;
+  const cudaError_t e = limit([] {
+    return cudaFuncSetAttribute(proj_f32_kernel<TM_, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                F32Cfg<TM_>::kRingBytes + (int)tile_map_bytes(kMaxClasses));
+  });
   if (e != cudaSuccess) return e;
-  if (dev > 63 || !(done.load(std::memory_order_acquire) >> dev & 1)) {
-    e = cudaFuncSetAttribute(proj_f32_kernel<TM_, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             F32Cfg<TM_>::kRingBytes + (int)tile_map_bytes(kMaxClasses));
-    if (e != cudaSuccess) return e;
-    if (dev <= 63) done.fetch_or(1ull << dev, std::memory_order_release);
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(256, 1, 1);
@@ -426,11 +421,9 @@ cudaError_t launch_proj_simt(const ProjArgs &a, bool in_bf16, bool widths4, cuda
   }
   const int grid = 148 * 4;
   const size_t map_bytes = tile_map_bytes(a.n_classes);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(proj_simt_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    attr = true;
-  }
+  static OncePerDevice limit;
+  const cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_simt_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024); });
+  if (e != cudaSuccess) return e;
   proj_simt_kernel<__nv_bfloat16><<<grid, 256, map_bytes, st>>>(a);
   count_launch(1);
   return cudaGetLastError();

@@ -543,17 +543,14 @@ PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE = 0>
 cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   using C = Cfg<TILE_N, TILE_M, BK>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    if (e != cudaSuccess) return e;
-    attr_set = true;
-  }
+  static OncePerDevice limit;
+  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
+  if (e != cudaSuccess) return e;
   int smem_bytes = C::kFixedSmemBytes + (int)tile_map_bytes(a.n_classes);
   if (smem_bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
   CUtensorMap tmA, tmB;
   ProjArgs b = a;
-  cudaError_t e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
+  e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
   if (e != cudaSuccess) return e;
   // staging buffers for the transposing epilogue, when they fit and the output rows are 16-byte aligned
   b.y_staged = a.y_bf16 && smem_bytes + kEpiWarps * C::kStoreBufBytes <= 227 * 1024 && ((uintptr_t)a.Y & 15u) == 0 &&

@@ -368,10 +368,10 @@ proj_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 }  // namespace
 
 int tc2_max_pairs(int num_sms) {
+  static OncePerDevice limit;
+  if (limit([] { return cudaFuncSetAttribute(proj_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem); }) != cudaSuccess) return 0;
   static int max_pairs = -1;
   if (max_pairs >= 0) return max_pairs;
-  if (cudaFuncSetAttribute(proj_tc2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem) != cudaSuccess)
-    return 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * (num_sms / 2));
   cfg.blockDim = dim3(kThreads);
