@@ -140,7 +140,7 @@ __device__ __forceinline__ int fast_div(int t, int d, float inv_d) {
 
 // Tile t of the launch (uniform across the warp).  Type-major; inside a type: m-tile fastest, then
 // the column tile, then the output group.
-__device__ __noinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
+__device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
   Tile o;
   o.row0 = -1, o.rows = 0, o.i = 0, o.j = 0, o.n0 = 0, o.cols = 0, o.n0_w = 0, o.np = 1, o.ng = 1;
   if (t >= ctl->total) return o;
@@ -230,9 +230,11 @@ __device__ __noinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t
 __device__ __forceinline__ int4 pack_tile(const Tile &o) {
   return make_int4(o.row0, o.n0, o.rows | (o.cols << 8) | (o.np << 20), o.i | (o.j << 8) | (o.ng << 16));
 }
+// (out of line: three roles call it, for tiles past the records only)
+__device__ __noinline__ Tile decode_tile_late(const BigArgs &a, const Ctl *ctl, int t) { return decode_tile(a, ctl, t); }
 // record `round` of this CTA, uniform across the warp; tiles past the records are decoded where they are needed
 __device__ __forceinline__ Tile get_tile(const BigArgs &a, const Ctl *ctl, int round) {
-  if (round >= kBigSeq) return decode_tile(a, ctl, blockIdx.x + round * gridDim.x);
+  if (round >= kBigSeq) return decode_tile_late(a, ctl, blockIdx.x + round * gridDim.x);
   const int4 v = ctl->recs[round];
   const int w = __shfl_sync(0xffffffffu, v.z, 0), x = __shfl_sync(0xffffffffu, v.w, 0);
   Tile o;
