@@ -162,6 +162,24 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (a.dyn_so) asm volatile("griddepcontrol.wait;" ::: "memory");   // segment offsets written by the bucketing kernel
     for (int e = lane; e <= q; e += 32)
       ctl->so[e] = a.seg_rows ? e * a.seg_rows : a.dyn_so ? a.dyn_so[e] : a.st.valid ? a.st.so[e] : tab->so[e];
+  } else if (warp == 5) {
+    // K blocks per tile of a pair, for the planner's records (warp 2 meets this warp at barrier 1).  By the planner itself
+    // they were in its way where it has nothing to wait for: cyclic 2048 -> 4096 at q = 16, M = 4096 24.6 -> 21.0 us,
+    // 512 -> 2048 at q = 8, M = 2048 8.65 -> 7.89; explicit types, FFN 2048 -> 4096 at q = 16, M = 8000 89.9 -> 83.3
+    if (a.dyn_so) asm volatile("griddepcontrol.wait;" ::: "memory");
+    for (int e = lane; e < q * q; e += 32) {
+      const uint32_t mask = a.st.valid ? a.st.keep[e] : tab->keep[e];
+      int n = 0;
+      for (int k = 0; k < q; ++k)
+        if ((mask >> k) & 1u)
+          n += (a.seg_rows ? a.seg_rows
+                : a.dyn_so   ? a.dyn_so[k + 1] - a.dyn_so[k]
+                : a.st.valid ? a.st.so[k + 1] - a.st.so[k]
+                             : tab->so[k + 1] - tab->so[k]) /
+               BK;
+      ctl->nkb[e] = (uint16_t)n;
+    }
+    asm volatile("bar.arrive 1, 64;" ::: "memory");
   }
   if (threadIdx.x == 0) ALG_TRACE(0, 21);
   if (warp == 1) {
@@ -187,25 +205,13 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (int r = lane; r < a.plan_rounds; r += 32) recs[r] = a.plan[1 + (size_t)blockIdx.x * a.plan_stride + r];
       if (lane == 0) tm->seq_rounds = a.plan_rounds, tm->seq_valid = a.plan_rounds, tm->total = 0;
     } else {
-      // what the planner needs of the handle: class records and K blocks per tile of a pair
       tile_map_classes(tm, tab, a.st, q, a.n_classes, lane, 32);
-      if (a.dyn_so) asm volatile("griddepcontrol.wait;" ::: "memory");   // (segment lengths from the bucketing kernel)
-      for (int e = lane; e < q * q; e += 32) {
-        const uint32_t mask = a.st.valid ? a.st.keep[e] : tab->keep[e];
-        int n = 0;
-        for (int k = 0; k < q; ++k)
-          if ((mask >> k) & 1u)
-            n += (a.seg_rows ? a.seg_rows
-                  : a.dyn_so   ? a.dyn_so[k + 1] - a.dyn_so[k]
-                  : a.st.valid ? a.st.so[k + 1] - a.st.so[k]
-                               : tab->so[k + 1] - tab->so[k]) /
-                 BK;
-        ctl->nkb[e] = (uint16_t)n;
-      }
       __syncwarp();
       if (a.offsets) asm volatile("griddepcontrol.wait;" ::: "memory");  // bucket offsets come from the previous kernel
-      tile_plan_warp(tm, recs, kSeqCap, q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom, blockIdx.x, gridDim.x, ctl->nkb);
+      tile_plan_warp(tm, recs, kSeqCap, q, a.n_classes, a.offsets, a.cyclic_rows, a.M, a.geom, blockIdx.x, gridDim.x, ctl->nkb,
+                     [] { asm volatile("bar.sync 1, 64;" ::: "memory"); });   // the K blocks (warp 5)
     }
+    if (planned) asm volatile("bar.sync 1, 64;" ::: "memory");
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 24);

@@ -147,10 +147,12 @@ __device__ __forceinline__ TileRec tile_seq_get(const TileRec *recs, TileMap *tm
 
 // The plan of one worker -- class prefix table and its own tile sequence, K-block counts included -- built by ONE warp
 // with warp-level synchronisation only, so that the other warps of the CTA can set up barriers and tensor memory
-// meanwhile and a single CTA barrier ends the prologue.  The warp has run tile_map_classes and written the K blocks
-// per pair (`nkb_of_pair`) before; only the bucket offsets come from the previous kernel.
-__device__ inline void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, int q, int nc, const int *offsets, int cyclic_rows,
-                                      int M, const TileGeom &g, int worker, int n_workers, const uint16_t *nkb_of_pair) {
+// meanwhile and a single CTA barrier ends the prologue.  The warp has run tile_map_classes before; another one writes the
+// K blocks per pair (`nkb_of_pair`), and `nkb_ready()` waits for them; only the bucket offsets come from the previous kernel.
+template <typename Ready>
+__device__ __forceinline__ void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, int q, int nc, const int *offsets, int cyclic_rows,
+                                               int M, const TileGeom &g, int worker, int n_workers, const uint16_t *nkb_of_pair,
+                                               Ready nkb_ready) {
   const int lane = threadIdx.x & 31;
   for (int t = lane; t <= q + 1; t += 32) tm->offsets[t] = offsets ? offsets[t] : (t <= q ? t * cyclic_rows : M);
   __syncwarp();
@@ -179,6 +181,7 @@ __device__ inline void tile_plan_warp(TileMap *tm, TileRec *recs, int cap, int q
   const int valid = all_rounds == 0 ? 0 : all_rounds - 1 + (snake_index(all_rounds - 1, worker, n_workers) < total);
   const int rounds = min(cap, valid + 1);
   if (lane == 0) prefix[nc] = total, tm->total = total, tm->seq_rounds = rounds, tm->seq_valid = valid;
+  nkb_ready();
   __syncwarp();
   for (int r = lane; r < rounds; r += 32) recs[r] = tile_seq_decode(tm, g, r, worker, n_workers, nkb_of_pair);
 }
