@@ -802,9 +802,15 @@ bool use_row_decode(const alg_proj_s &p, int64_t M) {
 }
 
 // Explicit types on the tensor-core kernels: are the buckets counted and X copied into them by one launch?  (A call
-// whose kernel or row gather was chosen by an option keeps one launch for each.)
+// whose kernel or row gather was chosen by an option keeps one launch for each.)  Rows under 1 KB before the large-algebra
+// kernel keep two launches: there is little to copy, and two small kernels whose prologues overlap are ahead of one that
+// fills the GPU with CTAs.  FFN, one launch / two, us: 384 -> 1024 at q = 4, M = 512 25.7 / 23.6; 80 -> 400 at q = 2, M = 1000
+// 25.2 / 23.1; 256 -> 1024 at q = 16, M = 1000 21.9 / 21.2; 320 -> 1600 at q = 8 24.6 / 26.2 is the exception, and rows of
+// 640 columns (q = 16) are even: 29.6 / 29.9.
 bool copies_with_buckets(const alg_proj_s &p, int64_t M) {
-  return p.opt_kernel == 0 && p.opt_row_gather == 0 && (use_tc(p) || use_big_counted(p, M)) && bucket_copy_takes(p.q, M, (int64_t)p.K * 2);
+  const bool big = use_big_counted(p, M);
+  if (p.opt_kernel != 0 || p.opt_row_gather != 0 || !(big || use_tc(p)) || (big && p.K < 512)) return false;
+  return bucket_copy_takes(p.q, M, (int64_t)p.K * 2);
 }
 
 // Forward call on the large-algebra path.  Equal buckets (cyclic or interval schedule, q | M) need no

@@ -582,3 +582,16 @@ def test_buckets_and_copy_in_one_launch(q, M, s_w):
     apart = binding.Proj(wl.d_widths, wl.f_widths)
     apart.set_option("row_gather", 1)             # a copy pass of its own: every row, bit for bit
     assert torch.equal(apart.forward(X, tt, W, out_dtype=torch.float32), got)
+
+
+@pytest.mark.parametrize("q,s_w", [(2, 40), (3, 168), (2, 256), (5, 104)])   # 160, 1008, 1024 and 1040 bytes a row
+def test_narrow_rows_before_the_large_algebra_kernel_are_copied_apart(q, s_w):
+    """Buckets and copy in one launch from rows of 1 KB on; same bits either way."""
+    M = 300
+    wl = _tc_workload(q, M, s_w, 40, types=synth.uniform_types(7 * q, M, q), seed=95)
+    X, W, t = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.dev_types(wl.types)
+    proj = binding.Proj(wl.d_widths, wl.f_widths)
+    n0 = binding.launch_count()
+    Y = proj.forward(X, t, W, out_dtype=torch.float32)
+    assert binding.launch_count() - n0 == (2 if q * s_w >= 512 else 3) and proj.last_status() == 0
+    assert np.array_equal(H.to_np(Y), oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths))
