@@ -50,6 +50,7 @@ struct alg_proj_s {
   int *d_status = nullptr;  // owned unless `shared_status`; followed by the two counters of the bucketing kernel
   bool shared_status = false;
   bool tc_ok = false;
+  bool mixed_ffn = false;   // of an FFN only one of whose projections fits the table-driven tensor-core kernels
   bool pair_kernel = false; // cta_group::2 kernel (256-row tiles)
   int tile_n = 0;           // tensor-core tile width of the one-CTA kernel
   // one-CTA kernel with 256-row x 128-column tiles (two accumulators per tile): taken when every
@@ -595,18 +596,22 @@ bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 // while with large buckets its tuned main loop and epilogue win (q = 8, M = 16384 FFN: 125.9 against 138.3 us).
 // With up to 8 groups the table-driven kernels are the better ones for small batches too, now that clusters split the
 // few tiles' reductions: FFN 768 -> 3072 at q = 2, M = 100 / 300 / 500: 38.3 / 39.4 / 39.1 us here, 22.3 / 27.2 / 27.8 there;
-// 1024 -> 4096 at q = 8, M = 300 / 1900: 30.7 / 40.5 here, 27.5 / 36.7 there.
+// 1024 -> 4096 at q = 8, M = 300 / 1900: 30.7 / 40.5 here, 27.5 / 36.7 there.  In an FFN whose other projection does not fit
+// them (`mixed_ffn`), up to 8 groups of at most 128 hidden columns stay here as well: 512 -> 1024 at q = 8, M = 512 17.0 here,
+// 20.2 there; groups of 256 do not (512 -> 2048 at q = 8 23.3 / 22.5, 256 -> 1024 at q = 4 22.8 / 19.8).
 bool use_big_counted(const alg_proj_s &p, int64_t M) {
   if (p.big.repack) return false;
-  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok) && M <= 256 * (int64_t)p.q);
+  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok || (p.mixed_ffn && p.big.r <= 128)) && M <= 256 * (int64_t)p.q);
 }
 // Equal buckets (cyclic schedule, q | M): by the library's choice when a type has at most 128 rows -- the
 // large-algebra kernel then packs several types into a tile (FFN 4096 -> 12288 -> 4096 at q = 32, M = 2048:
 // 128.6 -> 71.1 us); with fuller buckets the table-driven kernel is faster (58.6 against 63.2 us on the q = 2
-// FFN at M = 8192).
+// FFN at M = 8192).  An FFN reads its rows in place where both projections can, so where only one of them fits the
+// table-driven kernels the other one is here whatever the number of groups: in place / through buckets and a copy, us:
+// 512 -> 2048 at q = 8, M = 1024 16.2 / 23.3; 256 -> 1024 at q = 4, M = 256 16.4 / 19.7; 128 -> 512 at q = 2, M = 128 15.2 / 19.5.
 bool use_big_equal(const alg_proj_s &p, int64_t M) {
   if (p.big.repack) return false;
-  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok) && M <= 128 * (int64_t)p.q);
+  return p.big.on || (p.big.eligible && p.opt_kernel == 0 && (p.q > 8 || !p.tc_ok || p.mixed_ffn) && M <= 128 * (int64_t)p.q);
 }
 
 
@@ -1491,6 +1496,7 @@ static alg_status_t ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths, c
     delete f;
     return s;
   }
+  f->up.mixed_ffn = f->down.mixed_ffn = f->up.tc_ok != f->down.tc_ok;
   f->D = f->up.K;
   f->F = f->up.N;
   f->fd_ok = dtype == ALG_BF16 && !gated && schedule != ALG_SCHED_INTERVAL &&

@@ -377,3 +377,24 @@ def test_ffn_random_shapes_integer_bit_exact(k):
                     out_dtype=torch.float32)
     assert ffn.last_status() == 0
     assert np.array_equal(H.to_np(Y), oracle.proj(Hh, wl.types, wl.W_down, wl.f_widths, wl.d_widths)), (q, M, dw, fw, schedule, kernel)
+
+
+@pytest.mark.parametrize("q,dw,fw", [(8, 64, 256), (4, 64, 256), (2, 64, 256), (8, 64, 128)])
+@pytest.mark.parametrize("rows", [33, 64, 128, 129])   # of a type
+def test_small_cyclic_batch_in_place_where_one_projection_fits_the_table(q, dw, fw, rows):
+    """d groups of 64: the up projection fits the table-driven kernels, the down projection does not.  Up to 128 rows of a
+    type the FFN reads and writes its rows in place, two launches; either way and with explicit types within tolerance."""
+    M = q * rows
+    if M <= 64:
+        pytest.skip("a decode batch")
+    wl = synth.make_workload("mixed", config=7, variant=q + rows, dtype="bf16", q=q, M=M, D=q * dw, F=q * fw, types=synth.cyclic_types(M, q))
+    args = (H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.to_dev(wl.W_down, "bf16"))
+    ref = oracle.ffn(wl.X, wl.types, wl.W_up, wl.W_down, wl.d_widths, wl.f_widths)
+    for schedule, t in (("cyclic", None), ("explicit", H.dev_types(wl.types))):
+        ffn = _ffn(wl, schedule=schedule)
+        launches = binding.launch_count()
+        Y = ffn.forward(args[0], t, args[1], args[2], act="gelu", out_dtype=torch.float32)
+        assert ffn.last_status() == 0
+        if schedule == "cyclic" and rows <= 128:
+            assert binding.launch_count() - launches == 2
+        H.assert_bf16_close(H.to_np(Y), ref, False, f"{schedule} q={q} rows={rows}")
