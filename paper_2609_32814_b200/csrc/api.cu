@@ -2,6 +2,7 @@
 // validation, workspace layout and the launch sequence of one forward pass.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -468,14 +469,33 @@ struct SplitChoice {
   int splits = 1, tile_n = 0;
   const DevTable *tab = nullptr, *d_tab = nullptr;
 };
-// m_tiles = expected 128-row tiles of the launch over all row types, stages = 64-deep stages of its longest reduction.
+// 128-row tiles of a launch over all row types: `tiles`, or `more` with probability p_more.
+struct TileCount {
+  int64_t tiles, more;
+  double p_more;
+};
+// With explicit types a type has M / q rows give or take a binomial spread (the batch's types taken as an even mix), so where
+// M / q is just below whole tiles some types need one more.  Clusters chosen for the even count alone then come in two
+// rounds: FFN 768 -> 3072 at q = 2, M = 253 32.7 us, 24.9 with the spread counted; 1024 -> 4096 at q = 4, M = 1000 34.3 / 29.5.
+TileCount count_tiles(int q, int64_t M, bool even) {
+  const double rows = (double)M / q, spread = std::sqrt(rows * (1.0 - 1.0 / q));
+  const int64_t per_type = (M + 128 * (int64_t)q - 1) / (128 * (int64_t)q);
+  TileCount t = {q * per_type, q * per_type, 0.0};
+  if (!even && q > 1) {
+    const double over = 0.5 * std::erfc((per_type * 128.0 + 0.5 - rows) / (spread * 1.41421356));   // one type needs another tile
+    t.p_more = 1.0 - std::pow(1.0 - over, q);
+    t.more = t.tiles + std::max<int64_t>(1, (int64_t)(q * over + 0.5));
+  }
+  return t;
+}
+// m_tiles = 128-row tiles of the launch over all row types, stages = 64-deep stages of its longest reduction.
 // Compares the cycles of the longest chain, (stages of a CTA) x (cycles of a stage) + epilogue + the exchange, over tile
 // widths and 1, 2, 4 or 8 CTAs per tile; a choice needs its clusters resident at once (one CTA per SM, clusters of 4 and 8
 // leave some SMs of a GPC over).  Stage cycles are what the copy engine takes for the rows of a stage (about 1.75 a row).
 // Measured, whole FFN, one CTA per tile / split, us: 768 -> 3072 at q = 2, M = 700 35.4 / 29.0, M = 1777 40.8 / 36.5;
 // 1024 -> 4096 at q = 2, M = 1000 48.5 / 42.2, M = 2000 53.1 / 48.2; forward and both gradients 768 -> 3072 at q = 2,
 // M = 8003 174.0 / 168.5.
-SplitChoice choose_split(const alg_proj_s &p, int64_t m_tiles, int64_t stages, bool act) {
+SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t stages, bool act) {
   SplitChoice best;
   if (!use_tc(p) || p.gated || p.pair_kernel || p.opt_kernel != 0 || p.sched == ALG_SCHED_INTERVAL || p.opt_stage_k == 32 ||
       (p.opt_tile_n != 0 && !p.dyn_segments) || p.opt_row_gather == 2)
@@ -485,14 +505,19 @@ SplitChoice choose_split(const alg_proj_s &p, int64_t m_tiles, int64_t stages, b
   double best_cost = 1e30;
   for (const auto &w : width) {
     if (!w.on) continue;
-    const int64_t tiles = m_tiles * (p.N / w.tile_n);
+    const int64_t columns = p.N / w.tile_n;
     for (int s = 1; s <= 8; s *= 2) {
       const int resident = s == 1 ? 148 : s == 2 ? 74 : s == 4 ? 33 : 15;
       if (s == 8 && w.tile_n == 192) continue;
-      if (s > 1 && (tiles > resident || stages < 2 * s)) continue;
-      const int64_t rounds = (tiles + resident - 1) / resident;
+      if (s > 1 && (m_tiles.tiles * columns > resident || stages < 2 * s)) continue;
       const double stage = w.tile_n == 256 ? 672 : w.tile_n == 192 ? 560 : 450;
-      const double cost = rounds * ((double)((stages + s - 1) / s) * stage) + w.tile_n * (act ? 16.0 : 8.0) / s + (s > 1 ? 2000 : 0);
+      const double chain = (double)((stages + s - 1) / s) * stage, rest = w.tile_n * (act ? 16.0 : 8.0) / s + (s > 1 ? 2000 : 0);
+      // (a cluster goes through everything for its one tile, the persistent kernel overlaps all but the last epilogue)
+      auto cycles = [&](int64_t m) {
+        const double rounds = (double)((m * columns + resident - 1) / resident);
+        return s > 1 ? rounds * (chain + rest) : rounds * chain + rest;
+      };
+      const double cost = (1.0 - m_tiles.p_more) * cycles(m_tiles.tiles) + m_tiles.p_more * cycles(m_tiles.more);
       if (cost < best_cost * 0.97) {
         best_cost = cost;
         best.splits = s, best.tile_n = w.tile_n, best.tab = w.tab, best.d_tab = w.d_tab;
@@ -681,7 +706,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
   TcChoice tc = choose_tiling(p, M);
   SplitChoice sp;
   if (!tc.pair && !run_rows) {
-    sp = choose_split(p, (int64_t)p.q * ((M + (int64_t)p.q * 128 - 1) / ((int64_t)p.q * 128)), p.max_klen / 64, act != ALG_ACT_NONE);
+    sp = choose_split(p, count_tiles(p.q, M, cyclic), p.max_klen / 64, act != ALG_ACT_NONE);
     if (sp.splits > 1) tc = {128, sp.tile_n, sp.tab, sp.d_tab, false};
   }
   const DevTable &tab = *tc.tab;
@@ -1410,7 +1435,7 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   TcChoice tc = {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, false};
   int64_t m_tiles = 0;   // 128-row tiles of the feature groups
   for (int e = 0; e < p.q; ++e) m_tiles += (h->dx.r[e] + 127) / 128;
-  const SplitChoice sp = choose_split(p, m_tiles, p.max_groups * ((M / p.q + 63) / 64), false);
+  const SplitChoice sp = choose_split(p, {m_tiles, m_tiles, 0.0}, p.max_groups * ((M / p.q + 63) / 64), false);
   if (sp.splits > 1) tc = {128, sp.tile_n, sp.tab, sp.d_tab, false};
   const DevTable &tab = *tc.tab;
   a.tab = tc.d_tab;

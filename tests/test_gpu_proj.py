@@ -595,3 +595,16 @@ def test_narrow_rows_before_the_large_algebra_kernel_are_copied_apart(q, s_w):
     Y = proj.forward(X, t, W, out_dtype=torch.float32)
     assert binding.launch_count() - n0 == (2 if q * s_w >= 512 else 3) and proj.last_status() == 0
     assert np.array_equal(H.to_np(Y), oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths))
+
+
+@pytest.mark.parametrize("q,M,s_w,r_w", [(2, 253, 384, 1536), (2, 509, 256, 1024), (4, 1000, 256, 1024), (8, 1021, 384, 128)])
+@pytest.mark.parametrize("shift", [0, 5, 40])
+def test_buckets_just_below_and_above_whole_tiles(q, M, s_w, r_w, shift):
+    """M / q just below whole 128-row tiles: even buckets, and buckets of which some need a tile more (the tiles of a launch
+    are estimated on the host, its clusters and rounds follow from the buckets)."""
+    types = np.arange(M, dtype=np.int32) % q
+    types[np.flatnonzero(types == q - 1)[:shift]] = 0
+    wl = _tc_workload(q, M, s_w, r_w, types=types, seed=97)
+    Y, proj = _run_proj(wl, out_dtype=torch.float32)
+    assert proj.last_status() == 0
+    assert np.array_equal(H.to_np(Y), oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths))
