@@ -526,9 +526,33 @@ SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t 
   }
   return best;
 }
+// Groups off the 256-column grid with reductions of 4096 and more: pairs against 256 x 128 one-CTA tiles (the same
+// arithmetic on two SMs and on one), for the batches that fill either.  Pairs are the faster ones per stage; their last,
+// 128-wide tile of a group takes about three quarters of a full one.  So: pairs where their tiles, weighted by width and
+// length, fit the GPU at once, and where that rest is a small part of a group and one-CTA tiles do not fit either.  Cyclic
+// types, pairs / one CTA, us: 8192 -> 2304 at q = 2, M = 2048 49.4 / 60.6, M = 8192 164 / 176; 4096 -> 640 at q = 1, M = 8192
+// 43.0 / 59.8; 16384 -> 4608 at q = 4, M = 32768 1497 / 1768; the other side: 8192 -> 768 at q = 2, M = 8192 72.0 / 63.5;
+// 4096 -> 1152 at q = 1, M = 4096 40.0 / 36.1.
+bool use_long_pairs(const alg_proj_s &p, int64_t M) {
+  if (p.pair_min_klen < 4096 || p.all256 || M / p.q < 1024) return false;
+  double pairs = 0, single = 0;   // tiles of the longest reduction, per 256 rows of every type
+  int narrowest = p.r[0];
+  for (int pr = 0; pr < p.q * p.q; ++pr) {
+    const int r = p.r[pr % p.q];
+    double len = 0;
+    for (int k = 0; k < p.q; ++k)
+      if ((p.tab.keep[pr] >> k) & 1u) len += p.s[k];
+    len /= p.max_klen;
+    pairs += len * (r / kTc2TileN + (r % kTc2TileN ? 0.75 : 0.0)), single += len * (r / 128);
+    narrowest = std::min(narrowest, r);
+  }
+  const double m_tiles = (double)M / kTc2TileM / p.q;   // of a type
+  return m_tiles * pairs <= p.num_sms / 2 || (narrowest >= 640 && m_tiles * single > p.num_sms);
+}
 // 256-row tiles pay when every row type fills several of them (a ragged last tile then wastes
 // little); with explicit types the rows per type are not known on the host: assume an even mix.
 TcChoice choose_tiling(const alg_proj_s &p, int64_t M) {
+  if (p.opt_kernel != 3 && use_long_pairs(p, M)) return {kTc2TileM, kTc2TileN, &p.tab_pair, p.d_tab_pair, true};
   if (p.tall_ok && (p.opt_kernel == 3 || M / p.q >= 1024)) return {256, 128, &p.tab_tall, p.d_tab_tall, false};
   if (use_pairs(p, M)) return {kTc2TileM, kTc2TileN, &p.tab_pair, p.d_tab_pair, true};
   return {tile_m_of(p), tile_n_of(p), &p.tab, p.d_tab, p.pair_kernel};
@@ -705,7 +729,7 @@ alg_status_t run_proj(alg_proj_s &p, const WsLayout &L, char *ws, const void *X,
   ProjArgs a;
   TcChoice tc = choose_tiling(p, M);
   SplitChoice sp;
-  if (!tc.pair && !run_rows) {
+  if (!run_rows) {   // (batches that fill CTA pairs on the 256-column grid have too many tiles for it)
     sp = choose_split(p, count_tiles(p.q, M, cyclic), p.max_klen / 64, act != ALG_ACT_NONE);
     if (sp.splits > 1) tc = {128, sp.tile_n, sp.tab, sp.d_tab, false};
   }
