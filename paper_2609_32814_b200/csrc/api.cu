@@ -65,7 +65,7 @@ struct alg_proj_s {
   DevTable tab_tall;
   DevTable *d_tab_tall = nullptr;
   // CTA pairs (256-row x 256-column tiles) by the library's choice, for batches that fill them; their tile classes
-  int max_klen = 0, max_groups = 0;   // longest reduction of a tile: columns, input groups
+  int max_klen = 0, min_klen = 0, max_groups = 0;   // longest and shortest reduction of a tile: columns, input groups
   int pair_min_klen = 0;    // shortest reduction of a tile where the shape allows them, else 0
   DevTable tab_pair;
   DevTable *d_tab_pair = nullptr;
@@ -178,6 +178,7 @@ alg_status_t configure_kernels(alg_proj_s &p) {
     min_klen = std::min(min_klen, len);
     p.max_klen = std::max(p.max_klen, len), p.max_groups = std::max(p.max_groups, __builtin_popcount(p.tab.keep[pr]));
   }
+  p.min_klen = min_klen;
   p.pair_kernel = false;
   if (p.gated && !(p.tc_ok && all128)) {
     // hidden groups off the 128-column grid: only the large-algebra kernel has a gated form for them (the caller
@@ -512,10 +513,15 @@ SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t 
       if (s > 1 && (m_tiles.tiles * columns > resident || stages < 2 * s)) continue;
       const double stage = w.tile_n == 256 ? 672 : w.tile_n == 192 ? 560 : 450;
       const double chain = (double)((stages + s - 1) / s) * stage, rest = w.tile_n * (act ? 16.0 : 8.0) / s + (s > 1 ? 2000 : 0);
-      // (a cluster goes through everything for its one tile, the persistent kernel overlaps all but the last epilogue)
       auto cycles = [&](int64_t m) {
-        const double rounds = (double)((m * columns + resident - 1) / resident);
-        return s > 1 ? rounds * (chain + rest) : rounds * chain + rest;
+        const int64_t tiles = m * columns;
+        if (s == 1) return (double)((tiles + resident - 1) / resident) * chain + rest;   // (all epilogues but the last overlap)
+        if (tiles <= resident) return chain + rest;
+        // a cluster goes through everything for its one tile, and starting in a second round costs it about 5 us.  The
+        // longest tiles come first, so a few too many wait for the shortest ones to leave and are short themselves (8192 -> 768
+        // at q = 2, M = 1024: 26.5 us in clusters of 4 although 36 tiles exceed the 33 resident ones, 34.0 in pairs)
+        const double late = 9000 + 2 * rest, shorter = chain * p.min_klen / p.max_klen;
+        return (tiles - resident) * p.q <= tiles ? std::max(chain + rest, 2 * shorter + late) : 2 * chain + late;
       };
       const double cost = (1.0 - m_tiles.p_more) * cycles(m_tiles.tiles) + m_tiles.p_more * cycles(m_tiles.more);
       if (cost < best_cost * 0.97) {
