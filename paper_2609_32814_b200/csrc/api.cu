@@ -459,7 +459,7 @@ struct TcChoice {
 // 280.7 / 290.6.  With explicit types every type ends in a ragged tile, half of 256 rows on average, which eats the gain
 // at 1024 rows a type (FFN 4096 -> 16384 at q = 16, M = 16384: 605 / 616).
 bool use_pairs(const alg_proj_s &p, int64_t M) {
-  if (!p.pair_min_klen) return false;
+  if (!p.pair_min_klen || p.opt_stage_k == 32 || p.opt_row_gather == 2) return false;   // (options of the one-CTA kernel)
   const int64_t tiles = ceil_div((int)M, kTc2TileM) * (int64_t)ceil_div(p.N, kTc2TileN);
   const bool ragged = p.sched == ALG_SCHED_EXPLICIT;
   if (p.pair_min_klen >= 1024) return tiles >= 96 && M / p.q >= (ragged ? 2048 : 256);

@@ -608,3 +608,24 @@ def test_buckets_just_below_and_above_whole_tiles(q, M, s_w, r_w, shift):
     Y, proj = _run_proj(wl, out_dtype=torch.float32)
     assert proj.last_status() == 0
     assert np.array_equal(H.to_np(Y), oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths))
+
+
+def test_options_of_the_one_cta_kernel_hold_for_batches_that_fill_pairs():
+    """1024 -> 2048 at q = 2, M = 8192 runs on CTA pairs by the library's choice; ROW_GATHER = 2 (two launches: the kernel
+    fetches the rows itself) and STAGE_K = 32 ask for the one-CTA kernel.  Same sums in the same order, integers exact."""
+    q, M, s_w, r_w = 2, 8192, 512, 1024
+    wl = _tc_workload(q, M, s_w, r_w, types=synth.uniform_types(17, M, q), seed=99)
+    X, W, t = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.dev_types(wl.types)
+    plain = binding.Proj(wl.d_widths, wl.f_widths)
+    want = plain.forward(X, t, W, out_dtype=torch.float32)
+    gather = binding.Proj(wl.d_widths, wl.f_widths)
+    gather.set_option("row_gather", 2)
+    n0 = binding.launch_count()
+    assert torch.equal(gather.forward(X, t, W, out_dtype=torch.float32), want)
+    assert binding.launch_count() - n0 == 2 and gather.last_status() == 0
+    short = binding.Proj(wl.d_widths, wl.f_widths)
+    short.set_option("stage_k", 32)
+    assert torch.equal(short.forward(X, t, W, out_dtype=torch.float32), want) and short.last_status() == 0
+    rows = np.arange(0, M, 41)
+    ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(want[torch.from_numpy(rows).cuda()]), ref)
