@@ -507,6 +507,9 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) rows_decode_kernel(
   if (threadIdx.x == 0) ALG_TRACE(0, 6);
 
   if (FFN) {
+    // the phases share the barriers of the pieces' warps: where those are groups of different sizes, no warp may come to a
+    // barrier of phase 2 while others still meet at the one of that number in phase 1
+    if (p1.ks != p2.ks && p1.ks > 1 && p2.ks > 1) __syncthreads();
     if (a.in_place) used_x(a, turn);
     // ---- the first W_down loads go out before the hidden values are waited for ----
     uint4 w2[kLoads<false, RC>];

@@ -761,3 +761,31 @@ def test_decode_waits_that_run_out_at_different_times(s_w, r_w):
     proj.set_option("wait_limit_cycles", 4_000_000_000)
     assert np.array_equal(H.to_np(proj.forward(X, t, W, out_dtype=torch.float32)), ref)
     assert proj.last_status() == 0
+
+
+@pytest.mark.parametrize("kind,q,dw,fw,M", [
+    ("gated", 32, 64, 24, 3), ("ffn", 4, 256, 64, 3), ("ffn", 4, 256, 64, 5), ("ffn", 2, 512, 2048, 2), ("ffn", 8, 96, 200, 2),
+])
+def test_row_kernel_phases_with_different_groups_of_warps(kind, q, dw, fw, M):
+    """4 and 2 (or 8 and 2, ...) warps share a piece in the two phases; many calls in a row, all the same bits."""
+    def warps(pieces):
+        k = 1
+        while k < 8 and pieces * k * 2 <= 148 * 8:
+            k *= 2
+        return k
+    D, F = q * dw, q * fw
+    sizes = [warps(M * (n * q // (16 if n % 16 == 0 else 8))) for n in (fw, dw)]
+    assert sizes[0] != sizes[1] and min(sizes) > 1, sizes
+    wl, Wg = synth.gated_ffn("groups", q, M, D, F, synth.uniform_types(21 + M, M, q), variant=51, integer=False)
+    X, types, Wd = H.to_dev(wl.X, "bf16"), H.dev_types(wl.types), H.to_dev(wl.W_down, "bf16")
+    Wu = H.to_dev(np.concatenate([Wg, wl.W_up], axis=1) if kind == "gated" else wl.W_up, "bf16")
+    ffn = (binding.GatedFFN if kind == "gated" else binding.FFN)(wl.d_widths, wl.f_widths, dtype="bf16")
+    ffn.set_option("small_m_kernel", 3)
+    if kind == "gated":
+        ref = oracle.ffn_swiglu(wl.X, wl.types, Wg, wl.W_up, wl.W_down, wl.d_widths, wl.f_widths)
+    else:
+        ref = oracle.ffn(wl.X, wl.types, wl.W_up, wl.W_down, wl.d_widths, wl.f_widths)
+    outs = [ffn.forward(X, types, Wu, Wd, out_dtype=torch.float32) for _ in range(60)]
+    assert ffn.last_status() == 0
+    H.assert_bf16_close(H.to_np(outs[0]), ref, False, kind)
+    assert all(torch.equal(o, outs[0]) for o in outs)
