@@ -282,7 +282,13 @@ alg_status_t alg_proj_pack_weight(alg_proj_t h, const void *W, int64_t ldw, void
  * 1 <= q <= ALG_MAX_Q, schedule EXPLICIT or CYCLIC (larger algebras and the INTERVAL schedule
  * exist for single projections only: ALG_ERR_UNSUPPORTED_SHAPE).  Which GEMM kernel runs the two
  * projections is the library's choice per call (alg_ffn_set_option(GEMM_KERNEL) overrides it);
- * kernels differ in the order of their fp32 sums, so results agree to rounding between them. */
+ * kernels differ in the order of their fp32 sums, so results agree to rounding between them.
+ * Forward calls on one handle must be ordered on the GPU, with a workspace each or not: the one-launch decode steps pass
+ * hidden values through memory of the handle.  Inside such a launch CTAs wait for values of others.  Calls of different
+ * handles may overlap on two streams; with more of them, or with the row kernel at widths where it fills an SM (4096 ->
+ * 12288 at q = 32), launches that are each placed in part can wait for one another until the wait limit runs out
+ * (ALG_ERR_DEVICE_TIMEOUT): order those, or set SMALL_M_KERNEL = 0.  Steps whose weight slices do not fit half an SM's
+ * shared memory (1024 -> 4096 at q = 2) place the CTAs that are waited for first and overlap freely. */
 alg_status_t alg_ffn_create(alg_ffn_t *out, int q, const int32_t *d_widths,
                             const int32_t *f_widths, alg_dtype_t dtype, alg_table_t table,
                             const uint8_t *custom_keep, alg_schedule_t schedule);

@@ -304,8 +304,9 @@ constexpr int kFfnDecodeMaxM = 16;
 struct FfnDecodePlan {
   int su, sd;          // columns of the hidden state / of the output one CTA owns (multiples of 8)
   int n_up, n_dn;      // CTAs with an up strip / a down strip
+  bool apart;          // a CTA has one of the two, up strips first
   int box_up, box_dn;  // weight rows per tiled copy (divide every d / f width, <= 256)
-  int wd_bytes, wu_bytes, stage_bytes, p_bytes, ctl_bytes;  // shared-memory regions
+  int wd_bytes, wu_bytes, w_bytes, stage_bytes, p_bytes, ctl_bytes;  // shared-memory regions (w_bytes: slices of a CTA)
 };
 struct FfnDecodeArgs {
   const void *X;          // [M][D] bf16, packed
@@ -318,7 +319,9 @@ struct FfnDecodeArgs {
   int y_bf16;
   int D, F, q;
   int su, sd, n_up, n_dn, box_up, box_dn;
+  int apart;                               // CTA c < n_up has up strip c, CTA n_up + c down strip c; else CTA c has both
   int off_wu, off_stage, off_p, off_ctl;   // shared-memory offsets (the W_down slice sits at 0)
+  int off_hidden;                          // staged hidden values
   int kc_up, kc_dn, m_pad;                 // K-chunk lengths of the staged activations; staged rows (8 or 16)
   uint8_t *exch;                           // hidden rows between the phases (exchange.cuh), buffers of exch_bytes
   int exch_bytes;

@@ -42,9 +42,14 @@ ALG_TRACE_DEFINE(ffn_decode)
 namespace {
 
 constexpr int kThreads = 256, kWarps = 8;
-// Two CTAs (this launch and the next layer's) per SM where the weight slices leave room for that, else one: the next
-// layer's weights then come after this layer's, still in one launch (1024 -> 4096 -> 1024, q = 2, per layer of a graph:
-// M = 1 19.7 -> 7.8 us, M = 8 16.5 -> 11.5 us against two launches).
+// Two CTAs (this launch and the next layer's) per SM.  Where both weight slices of a CTA do not fit that, a CTA has one of
+// them (`apart`), still in one launch (1024 -> 4096 -> 1024, q = 2, per layer of a graph, two launches / both strips in a CTA
+// that fills an SM / apart: M = 1 18.8 / 8.1 / 6.8 us, M = 2 25.2 / 10.0 / 8.5, M = 8 16.2 / 11.3 / 11.7, M = 16 15.0 / 12.9 / 15.1).
+// A CTA waits for values of others of its launch, so a launch ends only if those get a place.  The CTAs of a launch take
+// their places in the order of their indexes: apart, the CTAs with up strips come first, wait for nobody but their own
+// copies and the previous kernel, and leave; the others find every CTA they wait for placed before them, whatever else runs
+// on the GPU.  With one CTA per SM for both strips (and all of its shared memory) two such launches of two streams could
+// hold half of the GPU each and wait for the other's half until the limit.
 constexpr int kSmemBudget = 112 * 1024, kSmemBudgetOne = 220 * 1024;
 
 constexpr int kStagers = 128;   // warps 4-7 stage the activations
@@ -355,12 +360,13 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const __grid_co
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 127) & ~(uintptr_t)127);
   uint8_t *wd_sm = smem;                        // W_down slice  [F][sd]
   uint8_t *wu_sm = smem + a.off_wu;             // W_up slice    [D][su]; later part of the H stage
-  uint8_t *st_sm = smem + a.off_stage;          // X stage; the H stage starts at wu_sm and runs through here
+  uint8_t *st_sm = smem + a.off_stage;          // X stage; the H stage (off_hidden) starts at wu_sm and runs through here
   Ctl *ctl = (Ctl *)(smem + a.off_ctl);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c = blockIdx.x, q = a.q, M = a.M;
-  const bool has_up = c < a.n_up, has_dn = c < a.n_dn;
-  const int col_u = c * a.su, col_d = c * a.sd;
+  const int c_dn = a.apart ? c - a.n_up : c;
+  const bool has_up = c < a.n_up, has_dn = c_dn >= 0 && c_dn < a.n_dn;
+  const int col_u = c * a.su, col_d = c_dn * a.sd;
   const int D = a.D, F = a.F;
   ALG_TRACE_VARS;
 #define TR(tag) do { if (tid == 0) ALG_TRACE(0, tag); ALG_TRACE_SEQ(tag); } while (0)
@@ -479,7 +485,7 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const __grid_co
     if (ok) {
       Phase dn;
       dn.src = (const __nv_bfloat16 *)hidden, dn.ld = F, dn.K = F, dn.kc = a.kc_dn, dn.pitch_bytes = a.kc_dn * 2;
-      dn.stage_base = smem_u32(wu_sm), dn.w_base = smem_u32(wd_sm), dn.cols = a.sd, dn.col0 = col_d;
+      dn.stage_base = smem_u32(smem + a.off_hidden), dn.w_base = smem_u32(wd_sm), dn.cols = a.sd, dn.col0 = col_d;
       dn.so = ctl->so_f, dn.rows_k = ctl->rows_dn, dn.need = ctl->need_dn, dn.bias = a.b_down, dn.act = ALG_ACT_NONE;
       dn.out = a.Y, dn.out_ld = D, dn.out_bf16 = a.y_bf16;
       ok = wait_bar(sh, bar_dn, 0);
@@ -557,8 +563,10 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
   p.wu_bytes = D * p.su * 2;
   p.p_bytes = kWarps * 16 * (p.su > p.sd ? p.su : p.sd) * 4;   // for 16 staged rows; half of it for 8
   p.ctl_bytes = ((int)sizeof(Ctl) + 127) & ~127;
-  for (int budget : {kSmemBudget, kSmemBudgetOne}) {
-    p.stage_bytes = (budget - 128 - p.wd_bytes - p.wu_bytes - p.p_bytes - p.ctl_bytes) & ~127;
+  for (bool apart : {false, true}) {
+    p.apart = apart;
+    p.w_bytes = apart ? std::max(p.wd_bytes, p.wu_bytes) : p.wd_bytes + p.wu_bytes;
+    p.stage_bytes = (kSmemBudget - 128 - p.w_bytes - p.p_bytes - p.ctl_bytes) & ~127;
     if (p.stage_bytes >= 16 * 64 * 2) break;
   }
   if (p.stage_bytes < 16 * 64 * 2) return false;   // at least one 64-deep chunk of 16 rows
@@ -568,6 +576,7 @@ bool ffn_decode_plan(int q, const int *dw, const int *fw, int D, int F, int num_
 
 cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p, cudaStream_t st) {
   FfnDecodeArgs a = args;
+  a.apart = p.apart;
   a.su = p.su, a.sd = p.sd, a.n_up = p.n_up, a.n_dn = p.n_dn, a.box_up = p.box_up, a.box_dn = p.box_dn;
   // up to kRowsMax rows on plain FMAs (tables in the kernel parameters only)
   const bool rows = a.M <= kRowsMax && a.small_q && a.D <= 512 * kRowsUp && a.F <= 512 * kRowsDn;
@@ -576,26 +585,29 @@ cudaError_t launch_ffn_decode(const FfnDecodeArgs &args, const FfnDecodePlan &p,
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudgetOne);
   if (e != cudaSuccess) return e;
   int ctl_bytes = p.ctl_bytes;
-  a.off_wu = p.wd_bytes;
+  a.off_wu = p.apart ? 0 : p.wd_bytes;
   if (rows) {
-        a.off_p = a.off_wu + p.wu_bytes;
+    a.off_p = p.w_bytes;
     a.off_ctl = (a.off_p + kWarps * (p.su + p.sd) * a.M * 4 + 127) & ~127;
     ctl_bytes = (int)sizeof(RowsCtl);
   } else {
     a.m_pad = a.M <= 8 ? 8 : 16;
     // the partial-sum buffer shrinks with the staged rows; what it gives up goes to the activation stage
     const int p_bytes = p.p_bytes * a.m_pad / 16;
-    const int stage_bytes = p.stage_bytes + (p.p_bytes - p_bytes);
-    a.off_stage = a.off_wu + p.wu_bytes;
+    int stage_bytes = p.stage_bytes + (p.p_bytes - p_bytes);
+    // apart, hidden rows in more than three chunks: one CTA per SM (1024 -> 4096 at M = 9 14.7 us, two per SM 16.6)
+    if (p.apart && stage_bytes / (a.m_pad * 2) < a.F / 3) stage_bytes += kSmemBudgetOne - kSmemBudget;
+    a.off_stage = p.w_bytes;
+    a.off_hidden = p.apart ? a.off_stage : a.off_wu;   // (over the slice of W_up, which the CTA has used up by then)
     a.off_p = a.off_stage + stage_bytes;
     a.off_ctl = a.off_p + p_bytes;
     auto round64 = [](int v) { return (v + 63) & ~63; };
     a.kc_up = std::min(round64(a.D), (stage_bytes / (a.m_pad * 2)) & ~63);
-    a.kc_dn = std::min(round64(a.F), ((p.wu_bytes + stage_bytes) / (a.m_pad * 2)) & ~63);
+    a.kc_dn = std::min(round64(a.F), ((a.off_p - a.off_hidden) / (a.m_pad * 2)) & ~63);
     if (a.kc_up < 64 || a.kc_dn < 64) return cudaErrorInvalidConfiguration;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(std::max(a.n_up, a.n_dn), 1, 1);
+  cfg.gridDim = dim3(p.apart ? a.n_up + a.n_dn : std::max(a.n_up, a.n_dn), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = a.off_ctl + ctl_bytes + (rows ? 512 : 128);
   cfg.stream = st;

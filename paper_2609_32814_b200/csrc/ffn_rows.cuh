@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(kThreads, 2) ffn_rows_kernel(const __grid_cons
   float *part_up = (float *)(smem + a.off_p), *part_dn = part_up + kWarps * NTU * 8 * MR;
   RowsCtl *ctl = (RowsCtl *)(smem + a.off_ctl);
   const int tid = threadIdx.x, c = blockIdx.x, q = a.q, M = a.M;
-  const bool has_up = c < a.n_up, has_dn = c < a.n_dn;
-  const int col_u = c * (8 * NTU), col_d = c * (8 * NTD), D = a.D, F = a.F;
+  const int c_dn = a.apart ? c - a.n_up : c;
+  const bool has_up = c < a.n_up, has_dn = c_dn >= 0 && c_dn < a.n_dn;
+  const int col_u = c * (8 * NTU), col_d = c_dn * (8 * NTD), D = a.D, F = a.F;
   const uint32_t bar_up = smem_u32(&ctl->bar_up), bar_dn = smem_u32(&ctl->bar_dn), bar_miss = smem_u32(&ctl->bar_miss[0]);
   if (tid == 0) {
     mbar_init(bar_up, 1);

@@ -789,3 +789,62 @@ def test_row_kernel_phases_with_different_groups_of_warps(kind, q, dw, fw, M):
     assert ffn.last_status() == 0
     H.assert_bf16_close(H.to_np(outs[0]), ref, False, kind)
     assert all(torch.equal(o, outs[0]) for o in outs)
+
+
+# ---- slices too large for two CTAs with both strips per SM: CTAs with one strip each, up strips first --------------------
+
+@pytest.mark.parametrize("dw,fw,M", [([512, 512], [2048, 2048], 1), ([512, 512], [2048, 2048], 8), ([448, 448], [1792, 1792], 16)])
+def test_one_launch_ffn_strips_apart_types_stall_and_streams(dw, fw, M):
+    """Types written while the call starts; a stall that runs out and the calls after it; three handles on three streams at
+    once, each a chain of dependent layers (no launch waits for CTAs that have no place yet)."""
+    q, D, F = len(dw), sum(dw), sum(fw)
+    wl = _ffn_int_workload(q, M, D, F, seed=900 + M)
+    kinds = [np.full(M, 0, np.int32), np.full(M, q - 1, np.int32), wl.types]
+    X, Wu, Wd = H.to_dev(wl.X, "bf16"), H.to_dev(wl.W_up, "bf16"), H.to_dev(wl.W_down, "bf16")
+    refs = []
+    for t in kinds:
+        wl.types = t
+        refs.append(torch.from_numpy(_ffn_int_ref(wl)).float().cuda())
+    writer = _TypeWriter(64, kinds)
+    ffn = binding.FFN(dw, fw, dtype="bf16")
+    order = [0, 1, 2, 1, 0, 2] * 10
+    outs = [torch.empty(M, D, dtype=torch.float32, device="cuda") for _ in order]
+    n0 = binding.launch_count()
+    for which, out in zip(order, outs):
+        writer.write(which)
+        ffn.forward(X, writer.types, Wu, Wd, act=None, out=out)
+    assert binding.launch_count() - n0 == 2 * len(order) and ffn.last_status() == 0
+    for which, out in zip(order, outs):
+        assert torch.equal(out, refs[which])
+
+    t2 = H.dev_types(kinds[2])
+    ffn.set_option("wait_limit_cycles", 6_000_000)
+    ffn.set_option("test_stall_bytes", 512)
+    ffn.forward(X, t2, Wu, Wd, act=None, out_dtype=torch.float32)
+    assert ffn.last_status() == 6
+    ffn.set_option("test_stall_bytes", 0)
+    ffn.set_option("wait_limit_cycles", 4_000_000_000)
+    for _ in range(3):
+        assert torch.equal(ffn.forward(X, t2, Wu, Wd, act=None, out_dtype=torch.float32), refs[2])
+    assert ffn.last_status() == 0
+
+    # chains of real-valued layers, kept small
+    Wu, Wd = (torch.from_numpy(synth.bf16_round(synth.normal(seed, shape, 0.02))).cuda().bfloat16() for seed, shape in ((5, (D, F)), (6, (F, D))))
+    chains = []
+    for _ in range(3):
+        handle = binding.FFN(dw, fw, dtype="bf16")
+        ws = torch.empty(handle.workspace_bytes(M), dtype=torch.uint8, device="cuda")
+        chains.append((handle, [X] + [torch.empty_like(X) for _ in range(40)], ws, torch.cuda.Stream()))
+    alone = binding.FFN(dw, fw, dtype="bf16")
+    want = [X]
+    for _ in range(40):
+        want.append(alone.forward(want[-1], t2, Wu, Wd, act="gelu"))
+    torch.cuda.synchronize()
+    for i in range(40):
+        for handle, acts, ws, stream in chains:
+            handle.forward(acts[i], t2, Wu, Wd, act="gelu", out=acts[i + 1], workspace=ws, stream=stream)
+    torch.cuda.synchronize()
+    for handle, acts, ws, stream in chains:
+        assert handle.last_status() == 0
+        assert all(torch.equal(a, b) for a, b in zip(acts, want))
+    assert bool(torch.isfinite(want[1]).all()) and bool(want[1].any())
