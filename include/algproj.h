@@ -384,6 +384,7 @@ alg_status_t alg_ffn_forward_host(alg_ffn_t h, const void *X_host, const int32_t
                                   size_t workspace_bytes, void *stream);
 /* Benchmark aid: when enabled, every alg_ffn_forward on this handle records CUDA events on the
  * call's stream between its kernels (do not enable while capturing a graph).
+ * Timed calls run bucketing and row gather as launches of their own, also where an untimed call has one for both.
  * alg_ffn_get_timing waits for the most recent call and returns four durations in
  * milliseconds: [0] row-type bucketing, [1] row gather, [2] up projection (with activation),
  * [3] down projection. */

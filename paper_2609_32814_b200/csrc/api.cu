@@ -842,11 +842,13 @@ bool interval_runs(const alg_proj_s &p, int64_t M, int *run_rows, int64_t *perio
 
 bool use_decode(const alg_proj_s &p, int64_t M) { return p.decode_ok && p.opt_small_m != 0 && M <= kDecodeMaxM; }
 // a few rows under the complete-graph law with equal groups: the one-launch FMA kernel of row_decode.cu
-// Rows up to which the row kernel is the library's choice.  It reads the diagonal block and the panel block of every
-// row (2 M segments; repeats come from L2) and runs at about 2.5 us + 0.65 us per MB read, so it wins while that stays
-// below what the prefill kernels need for a handful of rows: measured break-even near 20 MB for a projection (15-19 us
-// through bucketing, gather and the GEMM) and 45 MB for an FFN (27-37 us).  Handles with a weight-streaming kernel
-// (few groups, small banks) keep that one: 768 -> 3072 at q = 2 takes 4.9 us there against 6.3 us here at M = 1.
+// Rows up to which the row kernel is the library's choice.  It reads the diagonal block and the panel block of every row
+// (2 M segments; repeats come from L2), so its time goes with the bytes read; the prefill kernels take much the same for any
+// handful of rows.  Row kernel / prefill, us, q = 32: projections, line at 20 MB: 4096 -> 12288 M = 3 (19 MB) 12.0 / 13.8,
+// M = 4 (25 MB) 15.8 / 14.2; 2560 -> 9728 M = 6 (19 MB) 15.6 / 16.1, M = 8 19.6 / 16.1.  FFNs, line at 45 MB: gated 4096 -> 12288
+// M = 2 (38 MB) 22.8 / 25.8, M = 3 (57 MB) 31.3 / 26.6; gated 2560 -> 9728 M = 4 (37 MB) 29.3 / 28.5; plain M = 6 (37 MB) 31.3 /
+// 36.6, M = 8 46.4 / 36.6; gated 7168 -> 2048 M = 6 (33 MB) 25.6 / 25.0, M = 8 (44 MB) 29.7 / 25.8.  Handles with a
+// weight-streaming kernel (few groups, small banks) keep that one: 768 -> 3072 at q = 2 took 4.9 us there, 6.3 here at M = 1.
 int row_decode_rows(const alg_proj_s &p) {
   if (p.decode_ok) return 0;
   const double per_row = 4.0 * p.K * (double)p.N / p.q;   // bytes: two segments of K / q rows of the bank
@@ -1709,7 +1711,7 @@ alg_status_t alg_ffn_forward(alg_ffn_t h, const void *X, const int32_t *types, i
   const bool cyc = run_rows > 0 ||
                    (h->up.sched == ALG_SCHED_CYCLIC && M % h->up.q == 0 &&
                     ((use_tc(h->up) && use_tc(h->down)) || (use_big_equal(h->up, M) && use_big_equal(h->down, M))));
-  const bool copied = !cyc && copies_with_buckets(h->up, M);
+  const bool copied = !cyc && !tm && copies_with_buckets(h->up, M);   // (timed calls keep the two passes apart, to time them)
   if (copied && launch_bucket_copy(b, X, h->D, h->D, 2, ws + L.xb, st) != cudaSuccess) return ALG_ERR_CUDA;
   if (!cyc && !copied && launch_bucket(b, st) != cudaSuccess) return ALG_ERR_CUDA;
   if (tm) cudaEventRecord(h->ev[1], st);

@@ -398,3 +398,20 @@ def test_small_cyclic_batch_in_place_where_one_projection_fits_the_table(q, dw, 
         if schedule == "cyclic" and rows <= 128:
             assert binding.launch_count() - launches == 2
         H.assert_bf16_close(H.to_np(Y), ref, False, f"{schedule} q={q} rows={rows}")
+
+
+def test_timed_calls_time_bucketing_and_gather_apart():
+    wl = synth.make_workload("timed", config=7, variant=3, dtype="bf16", q=2, M=4096, D=512, F=1024, types=synth.uniform_types(3, 4096, 2))
+    args = (H.to_dev(wl.X, "bf16"), H.dev_types(wl.types), H.to_dev(wl.W_up, "bf16"), H.to_dev(wl.W_down, "bf16"))
+    ffn = _ffn(wl)
+    want = ffn.forward(*args)
+    ffn.set_timing(True)
+    n0 = binding.launch_count()
+    got = ffn.forward(*args)
+    assert binding.launch_count() - n0 == 4               # bucketing, gather, two projections
+    ms = ffn.get_timing()
+    assert torch.equal(got, want) and min(ms) > 1e-3      # (an interval without a kernel between its events is shorter)
+    ffn.set_timing(False)
+    n0 = binding.launch_count()
+    assert torch.equal(ffn.forward(*args), want)
+    assert binding.launch_count() - n0 == 3
