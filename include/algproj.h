@@ -228,8 +228,8 @@ alg_status_t alg_proj_forward(alg_proj_t h, const void *X, int64_t ldx, const in
  * there until the process exits.
  *
  * Limits and rules
- *   - The handle must exist already: create it once at start-up (creation does allocate a few
- *     hundred bytes).  This call itself performs no cudaMalloc, cudaFree or other allocation.
+ *   - The handle must exist already: create it once at start-up (creation does allocate,
+ *     kilobytes).  This call itself performs no cudaMalloc, cudaFree or other allocation.
  *   - Problems whose scratch need, alg_proj_workspace_bytes(h, M), exceeds
  *     ALG_STATIC_SCRATCH_BYTES are refused with ALG_ERR_WORKSPACE_TOO_SMALL and nothing is
  *     launched; use alg_proj_forward with your own workspace for those.

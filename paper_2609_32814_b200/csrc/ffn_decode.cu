@@ -350,7 +350,7 @@ __device__ __forceinline__ bool run_phase_t(const Shared &sh, const Phase &ph, u
   return true;
 }
 // NTU / NTD: 8-column tiles of the up / down strip (compile-time, so that every kernel gets the
-// registers its own shape needs).  ONE: one row, and the hidden row travels through the exchange buffer.
+// registers its own shape needs).
 template <int NTU, int NTD, int MP>
 __global__ void __launch_bounds__(kThreads, 2) ffn_decode_kernel(const __grid_constant__ CUtensorMap tm_up, const __grid_constant__ CUtensorMap tm_dn, const FfnDecodeArgs a) {
   // the next launch of the stream may start now: it only requests its own weights before it waits

@@ -118,8 +118,8 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, uint32_t lbo_b
 
 // GELU with the exact (erf) definition, gelu(z) = z * Phi(z) = max(z, 0) - |z| * Phi(-|z|).  The
 // lower tail Phi(-u), u >= 0, is evaluated as 2^p(u) with a degree-6 polynomial p fitted to
-// log2(Phi(-u)) on [0, 6] (one ex2, no branches); |gelu error| < 1e-7 over the whole real line,
-// i.e. fp32 rounding level.  Two values are processed at once with the packed fp32x2 FMA of
+// log2(Phi(-u)) on [0, 6] (one ex2, no branches); |gelu error| < 1e-7 for |z| <= 100, fp32
+// rounding level (below -6 the value is 1e-9 z).  Two values are processed at once with the packed fp32x2 FMA of
 // sm_100, which halves the issue slots the epilogue takes from the producer and MMA threads.
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   return (uint64_t)__float_as_uint(lo) | ((uint64_t)__float_as_uint(hi) << 32);

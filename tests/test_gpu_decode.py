@@ -476,7 +476,7 @@ def test_few_rows_one_type_out_of_range_and_types_written_just_before():
 # predecessor wrote, whatever the row counts -------------------------------------------------------------------------
 
 @pytest.mark.parametrize("kind,q,dw,fw,rows", [
-    ("plain", 2, 384, 1536, [1, 5, 1, 1, 16, 1]),     # the staged kernel; more than one row does not use the buffers
+    ("plain", 2, 384, 1536, [1, 5, 1, 1, 16, 1]),     # plain FMAs and the matrix path in turn
     ("plain", 8, 96, 200, [1, 8, 1, 2, 7, 1, 1, 3]),  # the row kernel
     ("gated", 32, 64, 24, [8, 1, 1, 4, 8, 2, 1]),
 ])
