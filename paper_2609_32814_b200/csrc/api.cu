@@ -490,12 +490,14 @@ TileCount count_tiles(int q, int64_t M, bool even) {
   return t;
 }
 // m_tiles = 128-row tiles of the launch over all row types, stages = 64-deep stages of its longest reduction.
-// Compares the cycles of the longest chain, (stages of a CTA) x (cycles of a stage) + epilogue + the exchange, over tile
-// widths and 1, 2, 4 or 8 CTAs per tile; a choice needs its clusters resident at once (one CTA per SM, clusters of 4 and 8
-// leave some SMs of a GPC over).  Stage cycles are what the copy engine takes for the rows of a stage (about 1.75 a row).
-// Measured, whole FFN, one CTA per tile / split, us: 768 -> 3072 at q = 2, M = 700 35.4 / 29.0, M = 1777 40.8 / 36.5;
-// 1024 -> 4096 at q = 2, M = 1000 48.5 / 42.2, M = 2000 53.1 / 48.2; forward and both gradients 768 -> 3072 at q = 2,
-// M = 8003 174.0 / 168.5.
+// Compares the time of a launch in a chain of launches, in us, over tile widths and 1, 2, 4 or 8 CTAs per tile; a choice
+// needs its clusters resident at once (one CTA per SM; 74, 33 and 15 clusters of 2, 4 and 8 are).  The constants are a
+// least-squares fit over 1200 FFN steps of 170 shapes and batches with every choice forced in turn (6 % off; the choices it
+// makes cost 1.1 % over the best ones found, where counting stages and epilogue alone had cost 4.2 %, at most 45 %): per
+// launch, per stage of a CTA, per column of the epilogue, and for the SMs taken, since a launch that leaves few of them to
+// the next one delays its prologue.  Whole FFN, one CTA per tile / split: 768 -> 3072 at q = 2, M = 700 35.4 / 29.0, M = 1777
+// 40.8 / 36.5; 1024 -> 4096 at q = 2, M = 1000 48.5 / 42.2; short reductions over many tiles lose: cyclic 512 -> 512 at q = 2,
+// M = 2048 14.7 / 19.9; 768 -> 768, M = 4096 16.8 / 20.6.
 SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t stages, bool act) {
   SplitChoice best;
   if (!use_tc(p) || p.gated || p.pair_kernel || p.opt_kernel != 0 || p.sched == ALG_SCHED_INTERVAL || p.opt_stage_k == 32 ||
@@ -511,19 +513,23 @@ SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t 
       const int resident = s == 1 ? 148 : s == 2 ? 74 : s == 4 ? 33 : 15;
       if (s == 8 && w.tile_n == 192) continue;
       if (s > 1 && (m_tiles.tiles * columns > resident || stages < 2 * s)) continue;
-      const double stage = w.tile_n == 256 ? 672 : w.tile_n == 192 ? 560 : 450;
-      const double chain = (double)((stages + s - 1) / s) * stage, rest = w.tile_n * (act ? 16.0 : 8.0) / s + (s > 1 ? 2000 : 0);
-      auto cycles = [&](int64_t m) {
+      const bool wide = w.tile_n == 256, narrow = w.tile_n == 128;
+      const double columns_us = w.tile_n * (act ? 0.02 : 0.01);
+      const double chain = (double)((stages + s - 1) / s) * (s == 1 ? (wide ? 0.31 : narrow ? 0.24 : 0.25) : wide ? 0.40 : narrow ? 0.235 : 0.305);
+      auto us = [&](int64_t m) {
         const int64_t tiles = m * columns;
-        if (s == 1) return (double)((tiles + resident - 1) / resident) * chain + rest;   // (all epilogues but the last overlap)
-        if (tiles <= resident) return chain + rest;
+        if (s == 1)   // (all epilogues but the last overlap; the planner waits for the buckets of explicit types)
+          return 1.8 + (p.sched == ALG_SCHED_EXPLICIT ? 0.4 : 0.0) + (double)((tiles + resident - 1) / resident) * chain + 0.45 * columns_us +
+                 2.5 * std::min<int64_t>(tiles, resident) / resident;
+        const double start = 2.9 + 0.23 * s + 1.65 * std::min<int64_t>(tiles, resident) * s / 148, rest = 0.88 * columns_us / s;
+        if (tiles <= resident) return start + chain + rest;
         // a cluster goes through everything for its one tile, and starting in a second round costs it about 5 us.  The
         // longest tiles come first, so a few too many wait for the shortest ones to leave and are short themselves (8192 -> 768
         // at q = 2, M = 1024: 26.5 us in clusters of 4 although 36 tiles exceed the 33 resident ones, 34.0 in pairs)
-        const double late = 9000 + 2 * rest, shorter = chain * p.min_klen / p.max_klen;
-        return (tiles - resident) * p.q <= tiles ? std::max(chain + rest, 2 * shorter + late) : 2 * chain + late;
+        const double shorter = chain * p.min_klen / p.max_klen;
+        return start + ((tiles - resident) * p.q <= tiles ? std::max(chain + rest, 2 * (shorter + rest) + 5) : 2 * (chain + rest) + 5);
       };
-      const double cost = (1.0 - m_tiles.p_more) * cycles(m_tiles.tiles) + m_tiles.p_more * cycles(m_tiles.more);
+      const double cost = (1.0 - m_tiles.p_more) * us(m_tiles.tiles) + m_tiles.p_more * us(m_tiles.more);
       if (cost < best_cost * 0.97) {
         best_cost = cost;
         best.splits = s, best.tile_n = w.tile_n, best.tab = w.tab, best.d_tab = w.d_tab;
