@@ -515,9 +515,12 @@ SplitChoice choose_split(const alg_proj_s &p, const TileCount &m_tiles, int64_t 
       if (s > 1 && (m_tiles.tiles * columns > resident || stages < 2 * s)) continue;
       const bool wide = w.tile_n == 256, narrow = w.tile_n == 128;
       const double columns_us = w.tile_n * (act ? 0.02 : 0.01);
-      const double chain = (double)((stages + s - 1) / s) * (s == 1 ? (wide ? 0.31 : narrow ? 0.24 : 0.25) : wide ? 0.40 : narrow ? 0.235 : 0.305);
+      const double stage = s == 1 ? (wide ? 0.31 : narrow ? 0.24 : 0.25) : wide ? 0.40 : narrow ? 0.235 : 0.305;
+      const bool tall = s == 1 && narrow && p.tall_ok && m_tiles.tiles / p.q >= 8;   // (256-row tiles then, see choose_tiling)
       auto us = [&](int64_t m) {
-        const int64_t tiles = m * columns;
+        const int64_t tiles = tall ? m / 2 * columns : m * columns;
+        // (weights come from HBM: a few SMs alone do not get a stage in that time)
+        const double few = std::max(0.0, 1.0 - (double)tiles * s / 64), chain = (double)((stages + s - 1) / s) * (tall ? 0.36 : stage) * (1.0 + 0.5 * few);
         if (s == 1)   // (all epilogues but the last overlap; the planner waits for the buckets of explicit types)
           return 1.8 + (p.sched == ALG_SCHED_EXPLICIT ? 0.4 : 0.0) + (double)((tiles + resident - 1) / resident) * chain + 0.45 * columns_us +
                  2.5 * std::min<int64_t>(tiles, resident) / resident;
