@@ -521,6 +521,12 @@ struct CopyArgs {
   const int *perm;
   const WsHeader *hdr;  // padded buckets; nullptr: rows through perm as they are
   int q;
+  int64_t ld_dst[2];    // bytes
+  // Weight gradient under the complete-graph law (part = rows of the batch, 0 = off): a row of type t is needed for the
+  // blocks (t, j != t) alone, that is its columns S_t of X (matrix 0) and those outside R_t of G (matrix 1); row_bytes is
+  // the longest such part of a row.  In a batch with rows without a type whole rows are copied.
+  int part;
+  int cut[2][kMaxQ + 1];   // first byte of the column groups of X and of G
   int *status;
   long long wait_limit;
 };
@@ -543,28 +549,45 @@ __global__ void __launch_bounds__(kMaxAgents) copy_rows_kernel(const CopyArgs a)
   __syncthreads();
   if (tid >= a.agents) return;
   const uint32_t slot = base + (uint32_t)(tid * a.slot), zeros = base + (uint32_t)(a.agents * a.slot);
-  const int per_row = a.pieces[0] + a.pieces[1];
+  const bool part = a.part && s_off[a.q] == a.part;
+  const int pieces0 = a.part && !part ? (int)((a.ld_dst[0] + a.piece[0] - 1) / a.piece[0]) : a.pieces[0];
+  const int pieces1 = a.part && !part ? (int)((a.ld_dst[1] + a.piece[1] - 1) / a.piece[1]) : a.pieces[1];
+  const int per_row = pieces0 + pieces1;
   const int64_t units = (int64_t)a.rows * per_row;
   uint32_t parity = 0;
   for (int64_t u = blockIdx.x + (int64_t)gridDim.x * tid; u < units; u += (int64_t)gridDim.x * a.agents) {
     const int row = (int)(u / per_row), c = (int)(u - (int64_t)row * per_row);
-    const int m = c >= a.pieces[0], at = (m ? c - a.pieces[0] : c) * a.piece[m];
-    const uint32_t bytes = (uint32_t)min(a.piece[m], a.row_bytes[m] - at);
+    const int m = c >= pieces0;
+    int at = (m ? c - pieces0 : c) * a.piece[m], length = a.part && !part ? (int)a.ld_dst[m] : a.row_bytes[m], gap_at = 1 << 30, gap = 0;
     int src_row;
     if (a.hdr) {
       int t = 0;
       while (t + 1 < a.q && s_pad[t + 1] <= row) ++t;
       const int r = row - s_pad[t];
       src_row = row < s_pad[a.q] && r < s_off[t + 1] - s_off[t] ? __ldg(a.perm + s_off[t] + r) : -1;
+      if (part) {
+        const int own = a.cut[m][t + 1] - a.cut[m][t];
+        if (m) length = (int)a.ld_dst[1] - own, gap_at = a.cut[1][t], gap = own;   // all but R_t
+        else length = own, gap_at = 0, gap = a.cut[0][t];                          // S_t
+      }
     } else {
       src_row = __ldg(a.perm + row);
     }
-    uint8_t *dst = a.dst[m] + (int64_t)row * a.row_bytes[m] + at;
+    if (at >= length) continue;
+    const uint32_t bytes = (uint32_t)min(a.piece[m], length - at);
+    // bytes [at, at + bytes) of what is taken of the row: `first` of them before the gap, the rest behind it
+    const uint32_t first = (uint32_t)min(max(gap_at - at, 0), (int)bytes);
+    uint8_t *dst = a.dst[m] + (int64_t)row * a.ld_dst[m] + at;
     if (src_row >= 0) {
       const uint8_t *src = a.src[m] + (int64_t)src_row * a.ld_src[m] + at;
       asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot), "l"(src), "r"(bytes), "r"(bar)
-                   : "memory");
+      if (first)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot), "l"(src), "r"(first), "r"(bar)
+                     : "memory");
+      if (first < bytes)
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(slot + first), "l"(src + first + gap),
+                     "r"(bytes - first), "r"(bar)
+                     : "memory");
       uint32_t done = 0;
       const long long t0 = clock64();
       while (!done) {
@@ -581,7 +604,10 @@ __global__ void __launch_bounds__(kMaxAgents) copy_rows_kernel(const CopyArgs a)
       }
       parity ^= 1u;
     }
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src_row >= 0 ? slot : zeros), "r"(bytes) : "memory");
+    const uint32_t from = src_row >= 0 ? slot : zeros;
+    if (first) asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(from), "r"(first) : "memory");
+    if (first < bytes)
+      asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst + first + gap), "r"(from + first), "r"(bytes - first) : "memory");
     asm volatile("cp.async.bulk.commit_group;" ::: "memory");
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the slot may be filled again
   }
@@ -758,7 +784,7 @@ cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int 
   if ((int64_t)M * K * elem_bytes >= kBulkCopyBytes) {
     CopyArgs a = {};
     a.src[0] = (const uint8_t *)X, a.dst[0] = (uint8_t *)Xb;
-    a.ld_src[0] = ldx * elem_bytes, a.row_bytes[0] = K * elem_bytes;
+    a.ld_src[0] = ldx * elem_bytes, a.row_bytes[0] = K * elem_bytes, a.ld_dst[0] = a.row_bytes[0];
     a.rows = M, a.perm = perm;
     a.status = status, a.wait_limit = wait_limit;
     return launch_copy_rows(a, st);
@@ -774,11 +800,20 @@ cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int 
 }
 
 cudaError_t launch_gather_rows_padded(const void *X, int64_t ldx, int K, void *Xp, const void *G, int64_t ldg, int N, void *Gp,
-                                      const WsHeader *hdr, const int *perm, int q, int m_pad, int *status, long long wait_limit,
-                                      cudaStream_t st) {
+                                      const WsHeader *hdr, const int *perm, int q, int M, int m_pad, const int *s, const int *r,
+                                      int *status, long long wait_limit, cudaStream_t st) {
   CopyArgs a = {};
   a.src[0] = (const uint8_t *)X, a.dst[0] = (uint8_t *)Xp, a.ld_src[0] = ldx * 2, a.row_bytes[0] = K * 2;
   a.src[1] = (const uint8_t *)G, a.dst[1] = (uint8_t *)Gp, a.ld_src[1] = ldg * 2, a.row_bytes[1] = N * 2;
+  a.ld_dst[0] = a.row_bytes[0], a.ld_dst[1] = a.row_bytes[1];
+  if (s && r) {
+    a.part = M;
+    a.row_bytes[0] = a.row_bytes[1] = 0;
+    for (int t = 0; t < q; ++t) {
+      a.cut[0][t + 1] = a.cut[0][t] + s[t] * 2, a.cut[1][t + 1] = a.cut[1][t] + r[t] * 2;
+      a.row_bytes[0] = std::max(a.row_bytes[0], s[t] * 2), a.row_bytes[1] = std::max(a.row_bytes[1], (N - r[t]) * 2);
+    }
+  }
   a.rows = m_pad, a.perm = perm, a.hdr = hdr, a.q = q;
   a.status = status, a.wait_limit = wait_limit;
   return launch_copy_rows(a, st);

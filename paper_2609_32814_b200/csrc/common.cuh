@@ -96,9 +96,11 @@ cudaError_t launch_gather_rows(const void *X, int64_t ldx, const int *perm, int 
                                long long wait_limit, cudaStream_t st);
 // Weight-gradient pass (bf16): bucketed copies of X (K columns) and G (N columns) with every bucket padded to a multiple
 // of 64 rows, pad rows zero: Xp[p] = X[perm[..]], Gp[p] = G[perm[..]].  m_pad >= padded total (hdr->pad_offsets[q]).
+// With s and r (widths of the q column groups of X and of G; q > 1): a row of type t only brings its columns S_t of X and
+// those outside R_t of G, unless the batch has rows without a type.
 cudaError_t launch_gather_rows_padded(const void *X, int64_t ldx, int K, void *Xp, const void *G, int64_t ldg, int N, void *Gp,
-                                      const WsHeader *hdr, const int *perm, int q, int m_pad, int *status, long long wait_limit,
-                                      cudaStream_t st);
+                                      const WsHeader *hdr, const int *perm, int q, int M, int m_pad, const int *s, const int *r,
+                                      int *status, long long wait_limit, cudaStream_t st);
 // The same for X alone, transposed (K x m_pad, leading dimension m_pad): feature groups that do not start on 16 bytes.
 cudaError_t launch_gather_transpose_padded(const void *X, int64_t ldx, const WsHeader *hdr, const int *perm, int q,
                                            int m_pad, int K, void *XpT, cudaStream_t st);
@@ -167,6 +169,14 @@ struct ProjArgs {
   // buckets dyn_so.
   int a_mn;
   int seg_rows;
+  // Weight gradient under the complete-graph law: a block (k, k) takes every row of the batch whatever its type, so its
+  // reduction runs over X and G as they lie (whole_rows = rows of the batch, 0 = off) and only the rows of the blocks
+  // (k, j != k), which take type k alone, come from the padded buckets.  A batch with out-of-range types
+  // (*whole_valid, the rows that have a type, != whole_rows) takes everything from the buckets.
+  int whole_rows = 0;
+  const int *whole_valid = nullptr;
+  const void *whole_x = nullptr, *whole_g = nullptr;
+  int64_t whole_ldx = 0, whole_ldg = 0;
   // Gated (SwiGLU) up projection: W is the merged bank [W_gate | W_up] with 2 * gated_f columns, a
   // tile accumulates 128 gate columns and the matching 128 up columns side by side, the epilogue
   // stores silu(gate) * up; N = gated_f is the width of the output.  0 = ordinary projection.

@@ -35,6 +35,7 @@ struct CtlS {
   uint32_t tmem_base;
   volatile int abort_flag;
   int row0, rows, pair, n0, n_kb;   // the tile; row0 < 0: none
+  int whole;                        // the blocks (k, k) of a weight gradient take X and G as they lie
   int so[kMaxQ + 1];
   uint32_t keep[kMaxPairs];
 };
@@ -100,9 +101,18 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t addr, uint32_t rank) {
   return r;
 }
 
-template <int TILE_N, int S>
+// WHOLE: weight gradient whose blocks (k, k) are reduced over X and G as they lie (ProjArgs::whole_rows): their maps.
+template <bool WHOLE>
+struct MoreMaps {};
+template <>
+struct MoreMaps<true> {
+  CUtensorMap A, B;
+};
+
+template <int TILE_N, int S, bool WHOLE>
 __global__ void __launch_bounds__(kThreads, 1)
-proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a) {
+proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a,
+                  const __grid_constant__ MoreMaps<WHOLE> more) {
   using C = CfgS<TILE_N, S>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -147,6 +157,7 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (warp == 4 && a.dyn_so) {
     for (int e = lane; e <= q; e += 32) ctl->so[e] = __ldcg(a.dyn_so + e);
+    if (WHOLE && lane == 0) ctl->whole = __ldcg(a.whole_valid) == a.whole_rows;
   } else if (warp == 2) {
     // tile -> (class, m-tile, n-tile): tiles are enumerated class by class, the n-tile fastest
     int before = 0, row0 = -1;
@@ -187,8 +198,9 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   if (ctl->row0 >= 0) {
     const int row0 = ctl->row0, rows = ctl->rows, pair = ctl->pair, n0 = ctl->n0, type_i = pair / q;
     const uint32_t mask = ctl->keep[pair];
-    int n_kb = 0;
-    for (int k = 0; k < q; ++k)
+    const bool whole = WHOLE && ctl->whole && pair % (q + 1) == 0;   // a block (k, k): one segment, all rows
+    int n_kb = whole ? (a.whole_rows + 63) >> 6 : 0;
+    for (int k = 0; k < q && !whole; ++k)
       if ((mask >> k) & 1u) n_kb += (ctl->so[k + 1] - ctl->so[k]) >> 6;
     const int b0 = n_kb * rank / S, b1 = n_kb * (rank + 1) / S;   // this CTA's stages of the reduction
     if (warp == 0) {
@@ -198,9 +210,9 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       int stage = 0, blk = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int k = 0; k < q && ok; ++k) {
-        if (!((mask >> k) & 1u)) continue;
-        const int k_begin = ctl->so[k], n = (ctl->so[k + 1] - k_begin) >> 6;
+      for (int k = 0; k < (whole ? 1 : q) && ok; ++k) {
+        if (!whole && !((mask >> k) & 1u)) continue;
+        const int k_begin = whole ? 0 : ctl->so[k], n = whole ? n_kb : (ctl->so[k + 1] - k_begin) >> 6;
         for (int i = max(0, b0 - blk); i < min(n, b1 - blk); ++i) {
           ok = __all_sync(0xffffffffu, mbar_try_wait(empty0 + 8u * stage, phase ^ 1u) || wait_s(empty0 + 8u * stage, phase ^ 1u, ctl, a.wait_limit, a.status));
           if (!ok) break;
@@ -210,10 +222,14 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
             if (a.a_mn) {   // weight gradient: rows of X and G as they lie, features / columns contiguous
               const int pos0 = a.seg_rows ? i << 6 : k0, seg = a.seg_rows ? k : 0;
+              const CUtensorMap *map_a = &tmA, *map_b = &tmB;
+              if constexpr (WHOLE) {
+                if (whole) map_a = &more.A, map_b = &more.B;
+              }
 #pragma unroll
-              for (int c = 0; c < 2; ++c) tma_load_3d(sa + c * kBChunkBytes, &tmA, bar, row0 + c * 64, seg, pos0);
+              for (int c = 0; c < 2; ++c) tma_load_3d(sa + c * kBChunkBytes, map_a, bar, row0 + c * 64, seg, pos0);
 #pragma unroll
-              for (int c = 0; c < TILE_N / 64; ++c) tma_load_3d(sa + kABytes + c * kBChunkBytes, &tmB, bar, n0 + c * 64, seg, pos0);
+              for (int c = 0; c < TILE_N / 64; ++c) tma_load_3d(sa + kABytes + c * kBChunkBytes, map_b, bar, n0 + c * 64, seg, pos0);
             } else {
               if (a.a_cyclic_rows) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
               else tma_load_2d(sa, &tmA, bar, k0, a_row);
@@ -391,16 +407,21 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   }
 }
 
-template <int TILE_N, int S>
-cudaError_t launch_s(const ProjArgs &a, int tiles, cudaStream_t st) {
+template <int TILE_N, int S, bool WHOLE>
+cudaError_t launch_w(const ProjArgs &a, int tiles, cudaStream_t st) {
   using C = CfgS<TILE_N, S>;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
-  cudaError_t e = cudaFuncSetAttribute(proj_split_kernel<TILE_N, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(proj_split_kernel<TILE_N, S, WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   if (e != cudaSuccess) return e;
   CUtensorMap tmA, tmB;
   ProjArgs b = a;
   e = make_tc_maps(&tmA, &tmB, &b, TILE_N, 128, false, 64);
   if (e != cudaSuccess) return e;
+  MoreMaps<WHOLE> more;
+  if constexpr (WHOLE) {
+    e = make_grad_maps(&more.A, &more.B, a.whole_x, a.whole_ldx, a.M, a.whole_g, a.whole_ldg, a.N, 1, a.whole_rows);
+    if (e != cudaSuccess) return e;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(tiles * S), 1, 1);
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -414,7 +435,11 @@ cudaError_t launch_s(const ProjArgs &a, int tiles, cudaStream_t st) {
   cfg.attrs = at;
   cfg.numAttrs = 2;
   count_launch(1);
-  return cudaLaunchKernelEx(&cfg, proj_split_kernel<TILE_N, S>, tmA, tmB, b);
+  return cudaLaunchKernelEx(&cfg, proj_split_kernel<TILE_N, S, WHOLE>, tmA, tmB, b, more);
+}
+template <int TILE_N, int S>
+cudaError_t launch_s(const ProjArgs &a, int tiles, cudaStream_t st) {
+  return a.whole_rows ? launch_w<TILE_N, S, true>(a, tiles, st) : launch_w<TILE_N, S, false>(a, tiles, st);
 }
 
 }  // namespace
@@ -422,7 +447,7 @@ cudaError_t launch_s(const ProjArgs &a, int tiles, cudaStream_t st) {
 cudaError_t launch_proj_split(const ProjArgs &a, int tile_n, int splits, int tiles, cudaStream_t st) {
   cudaError_t e = tc_init();
   if (e != cudaSuccess) return e;
-  if (a.geom.tile_m != 128 || a.block_k != 64 || a.gated_f || a.run_rows || a.in_perm || tiles < 1) return cudaErrorInvalidValue;
+  if (a.geom.tile_m != 128 || a.block_k != 64 || a.gated_f || a.run_rows || a.in_perm || tiles < 1 || (a.whole_rows && !a.a_mn)) return cudaErrorInvalidValue;
   if (tile_n == 256) {
     if (splits == 2) return launch_s<256, 2>(a, tiles, st);
     if (splits == 4) return launch_s<256, 4>(a, tiles, st);

@@ -42,6 +42,7 @@ struct Ctl {
   volatile int abort_flag;
   long long wait_limit;     // bound of every wait, in clock64 cycles
   // interaction table, copied once per CTA so no role waits on global metadata at a tile start
+  int whole;                // the blocks (k, k) of a weight gradient take X and G as they lie
   int so[kMaxQ + 1];
   uint32_t keep[kMaxPairs];
   uint16_t nkb[kMaxPairs];  // K blocks per tile of a pair
@@ -119,9 +120,17 @@ struct Cfg {
 // leave the chip (the merged gate/up kernel of the appendix "Kernel Benchmark Details").
 constexpr int kGatherWarps = 6;   // AMODE 2: extra warps that only issue row gathers, after the B producer
 constexpr int kGatherLanes = 32 / (2 + kGatherWarps);   // lanes of a warp that issue gathers
+// AMODE 3: weight gradient whose blocks (k, k) are reduced over X and G as they lie (ProjArgs::whole_rows): their maps.
+template <int AMODE>
+struct MoreMaps {};
+template <>
+struct MoreMaps<3> {
+  CUtensorMap A, B;
+};
 template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE>
 __global__ void __launch_bounds__(AMODE == 2 ? kThreads + 32 * kGatherWarps : kThreads, 1)
-proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a) {
+proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a,
+               const __grid_constant__ MoreMaps<AMODE> more) {
   using C = Cfg<TILE_N, TILE_M, BK>;
   static_assert(!GATED || (TILE_N == 256 && TILE_M == 128), "the gated kernel pairs two 128-column halves");
   extern __shared__ uint8_t smem_raw[];
@@ -162,6 +171,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (a.dyn_so) asm volatile("griddepcontrol.wait;" ::: "memory");   // segment offsets written by the bucketing kernel
     for (int e = lane; e <= q; e += 32)
       ctl->so[e] = a.seg_rows ? e * a.seg_rows : a.dyn_so ? a.dyn_so[e] : a.st.valid ? a.st.so[e] : tab->so[e];
+    if (AMODE == 3 && lane == 0) ctl->whole = __ldcg(a.whole_valid) == a.whole_rows;
   } else if (warp == 5) {
     // K blocks per tile of a pair, for the planner's records (warp 2 meets this warp at barrier 1).  By the planner itself
     // they were in its way where it has nothing to wait for: cyclic 2048 -> 4096 at q = 16, M = 4096 24.6 -> 21.0 us,
@@ -177,6 +187,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 : a.st.valid ? a.st.so[k + 1] - a.st.so[k]
                              : tab->so[k + 1] - tab->so[k]) /
                BK;
+      if (AMODE == 3 && e % (q + 1) == 0 && __ldcg(a.whole_valid) == a.whole_rows) n = (a.whole_rows + BK - 1) / BK;   // pair (k, k)
       ctl->nkb[e] = (uint16_t)n;
     }
     asm volatile("bar.arrive 1, 64;" ::: "memory");
@@ -262,10 +273,11 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 #pragma unroll
           for (int j = 0; j < 4; ++j) g_rows[h][j] = __ldg(a.in_perm + min(row0 + h * 128 + g_slot * 4 + j, a.M - 1));
       }
-      for (int k = 0; k < q && ok; ++k) {
-        if (!((mask >> k) & 1u)) continue;
-        const int k_begin = __shfl_sync(0xffffffffu, ctl->so[k], 0);
-        const int k_end = __shfl_sync(0xffffffffu, ctl->so[k + 1], 0);
+      const bool whole = AMODE == 3 && __shfl_sync(0xffffffffu, ctl->whole, 0) && pair % (q + 1) == 0;   // one segment: all rows
+      for (int k = 0; k < (whole ? 1 : q) && ok; ++k) {
+        if (!whole && !((mask >> k) & 1u)) continue;
+        const int k_begin = whole ? 0 : __shfl_sync(0xffffffffu, ctl->so[k], 0);
+        const int k_end = whole ? a.whole_rows : __shfl_sync(0xffffffffu, ctl->so[k + 1], 0);
         for (int k0 = k_begin; k0 < k_end; k0 += BK) {
           ok = __all_sync(0xffffffffu, wait_bar(empty0 + 8u * (uint32_t)stage, phase ^ 1u, ctl, a.status));
           if (!ok) break;
@@ -301,14 +313,18 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               // weight gradient: 64 rows of X (A, features contiguous) and of G (B), in boxes of 64 features / 64 output
               // columns.  Cyclic schedule: rows k, k + q, ... from position k0 - so[k] on; else padded rows from k0 on
               const int pos0 = a.seg_rows ? k0 - k_begin : k0, seg = a.seg_rows ? k : 0;
+              const CUtensorMap *map_a = &tmA, *map_b = &tmB;
+              if constexpr (AMODE == 3) {
+                if (whole) map_a = &more.A, map_b = &more.B;
+              }
               if (loads_a) {
                 mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
 #pragma unroll
-                for (int c = 0; c < TILE_M / 64; ++c) tma_load_3d(sa + c * (64 * BK * 2), &tmA, bar, row0 + c * 64, seg, pos0);
+                for (int c = 0; c < TILE_M / 64; ++c) tma_load_3d(sa + c * (64 * BK * 2), map_a, bar, row0 + c * 64, seg, pos0);
               } else {
 #pragma unroll
                 for (int c = 0; c < TILE_N / 64; ++c)
-                  tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, &tmB, bar, n0 + c * 64, seg, pos0);
+                  tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, map_b, bar, n0 + c * 64, seg, pos0);
               }
             } else if (AMODE == 1 && loads_a && a.a_cyclic_rows) {
               // runs of run_rows rows per period: 64-row boxes, each inside one run
@@ -558,6 +574,11 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   ProjArgs b = a;
   e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
   if (e != cudaSuccess) return e;
+  MoreMaps<AMODE> more;
+  if constexpr (AMODE == 3) {
+    e = make_grad_maps(&more.A, &more.B, a.whole_x, a.whole_ldx, a.M, a.whole_g, a.whole_ldg, a.N, 1, a.whole_rows);
+    if (e != cudaSuccess) return e;
+  }
   // staging buffers for the transposing epilogue, when they fit and the output rows are 16-byte aligned
   b.y_staged = a.y_bf16 && smem_bytes + kEpiWarps * C::kStoreBufBytes <= 227 * 1024 && ((uintptr_t)a.Y & 15u) == 0 &&
                (a.ldy * 2) % 16 == 0;
@@ -572,7 +593,7 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, tmA, tmB, b);
+  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, tmA, tmB, b, more);
   count_launch(1);
   return e;
 }
@@ -583,6 +604,10 @@ cudaError_t launch_t(const ProjArgs &a, int num_sms, cudaStream_t st) {
   if (a.run_rows) return a.block_k == 64 ? launch_bk<TILE_N, TILE_M, GATED, 64, 1>(a, num_sms, st) : cudaErrorInvalidValue;
   // so are the rows of explicit types fetched through the permutation by the A producer
   if (a.in_perm) return a.block_k == 64 && !a.w_kmajor && !a.seg_rows ? launch_bk<TILE_N, TILE_M, GATED, 64, 2>(a, num_sms, st) : cudaErrorInvalidValue;
+  if constexpr (TILE_M == 128 && !GATED) {
+    if (a.whole_rows) return a.a_mn && a.block_k == 64 ? launch_bk<TILE_N, TILE_M, GATED, 64, 3>(a, num_sms, st) : cudaErrorInvalidValue;
+  }
+  if (a.whole_rows) return cudaErrorInvalidValue;
   if (a.block_k == 32) return launch_bk<TILE_N, TILE_M, GATED, 32>(a, num_sms, st);
   if (a.block_k == 64) return launch_bk<TILE_N, TILE_M, GATED, 64>(a, num_sms, st);
   return cudaErrorInvalidValue;
@@ -599,13 +624,7 @@ cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int ti
     // padded copies as {columns, 1, padded row}
     if (gated || a->w_kmajor || tile_m != 128 || bk != 64) return cudaErrorInvalidValue;
     const uint64_t types = a->seg_rows ? (uint64_t)a->q : 1u, len = a->seg_rows ? (uint64_t)a->seg_rows : (uint64_t)a->K;
-    const uint64_t da[3] = {(uint64_t)a->M, types, len};
-    const uint64_t sa[2] = {(uint64_t)a->ldx * 2, (uint64_t)a->ldx * 2 * types};
-    const uint64_t db[3] = {(uint64_t)a->N, types, len};
-    const uint64_t sb[2] = {(uint64_t)a->ldw * 2, (uint64_t)a->ldw * 2 * types};
-    const uint32_t box[3] = {64, 1, 64};
-    const cudaError_t e = make_map_nd(tmA, a->X, 3, da, sa, box, 128);
-    return e == cudaSuccess ? make_map_nd(tmB, a->W, 3, db, sb, box, 128) : e;
+    return make_grad_maps(tmA, tmB, a->X, a->ldx, a->M, a->W, a->ldw, a->N, (int)types, (int)len);
   }
   const cudaError_t e = make_map_a(tmA, *a);
   if (e != cudaSuccess) return e;
@@ -617,6 +636,17 @@ cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int ti
   if (a->b_3d) return cudaSuccess;
   if (gated) return cudaErrorInvalidValue;
   return make_map_2d(tmB, a->W, (uint64_t)a->N, (uint64_t)a->K, (uint64_t)a->ldw * 2, 64, (uint32_t)bk);
+}
+
+cudaError_t make_grad_maps(CUtensorMap *tmA, CUtensorMap *tmB, const void *X, int64_t ldx, int K, const void *G, int64_t ldg, int N,
+                           int types, int rows) {
+  const uint64_t da[3] = {(uint64_t)K, (uint64_t)types, (uint64_t)rows};
+  const uint64_t sa[2] = {(uint64_t)ldx * 2, (uint64_t)ldx * 2 * (uint64_t)types};
+  const uint64_t db[3] = {(uint64_t)N, (uint64_t)types, (uint64_t)rows};
+  const uint64_t sb[2] = {(uint64_t)ldg * 2, (uint64_t)ldg * 2 * (uint64_t)types};
+  const uint32_t box[3] = {64, 1, 64};
+  const cudaError_t e = make_map_nd(tmA, X, 3, da, sa, box, 128);
+  return e == cudaSuccess ? make_map_nd(tmB, G, 3, db, sb, box, 128) : e;
 }
 
 cudaError_t make_map_2d_sw(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t ld_bytes,

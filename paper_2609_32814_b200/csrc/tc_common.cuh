@@ -223,6 +223,9 @@ cudaError_t make_map_nd(CUtensorMap *map, const void *base, int rank, const uint
 // {K, q, M/q} of X with strides {ld, q*ld} and a box of 64 x 1 x 128 (same shared-memory image).
 cudaError_t make_map_a(CUtensorMap *map, const ProjArgs &a);
 cudaError_t make_map_b3d(CUtensorMap *map, const ProjArgs &a, int chunks);
+// X and G of the weight gradient as {columns, type, position in the type}, boxes of 64 x 1 x 64.
+cudaError_t make_grad_maps(CUtensorMap *tmA, CUtensorMap *tmB, const void *X, int64_t ldx, int K, const void *G, int64_t ldg, int N,
+                           int types, int rows);
 cudaError_t make_tc_maps(CUtensorMap *tmA, CUtensorMap *tmB, ProjArgs *a, int tile_n, int tile_m, bool gated, int bk);
 
 }  // namespace tc

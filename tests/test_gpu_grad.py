@@ -138,3 +138,29 @@ def test_weight_gradient_row_copies(q, M, s, r, schedule):
     dW = grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), None if schedule == "cyclic" else H.dev_types(types))
     assert grad.last_status() == 0
     assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X, G, types, s, r))
+
+
+@pytest.mark.parametrize("q,M,s,r,schedule", [
+    (3, 130, [64, 136, 8], [2560, 256, 2048], "explicit"),   # parts of a G row in several pieces, one of them around the gap
+    (2, 65, [128, 384], [1536, 1536], "explicit"),           # one row past whole blocks, clusters of CTAs per tile
+    (2, 1, [128, 128], [256, 256], "explicit"),              # a single row
+    (2, 2050, [1024, 1024], [4096, 4096], "explicit"),       # more tiles than CTAs: the persistent kernel
+    (4, 3 * 100, [64, 72, 80, 200], [128] * 4, "cyclic"),    # 75 rows per type: not read in place
+])
+@pytest.mark.parametrize("bad", [False, True])
+def test_weight_gradient_blocks_that_take_every_row(q, M, s, r, schedule, bad):
+    """dW_kk is reduced over X and G as they lie, the other blocks over the parts of the rows that were copied; a batch with
+    a type out of range takes everything from whole copies."""
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    good = np.ones(M, bool)
+    if bad:
+        if schedule == "cyclic":
+            pytest.skip("the schedule's own types are never out of range")
+        types = types.copy()
+        types[M // 2], good[M // 2] = q, False
+    X, G = synth.small_ints(1, (M, sum(s)), -1, 1), synth.small_ints(2, (M, sum(r)), -1, 1)
+    grad = binding.ProjGrad(s, r, schedule=schedule)
+    ws = torch.full((grad.workspace_bytes(M),), 0xFF, dtype=torch.uint8, device="cuda")   # what is not copied is NaN
+    dW = grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), None if schedule == "cyclic" else H.dev_types(types), workspace=ws)
+    assert grad.last_status() == (5 if bad else 0)
+    assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X[good], G[good], types[good], s, r))
