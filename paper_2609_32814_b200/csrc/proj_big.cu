@@ -120,6 +120,16 @@ struct Cfg {
   static_assert(TILE_N == 128 || TILE_N == 256, "stage width");
 };
 
+// What the tiles of a launch look like is known at compile time.  The tiles are short, and with the tests of it in the loops
+// of the producers and of the MMA warp (and the index arithmetic of the forms that do not occur) the instructions of these
+// single warps, not the copies, set the pace.  Asked at run time / compiled in, us: gated FFN at q = 32, 2048 -> 6144, M = 2048
+// 61.6 / 49.7; 4096 -> 12288, M = 1500 117.6 / 105.1; 7168 -> 2048, M = 700 61.8 / 56.5; 2048 -> 768, M = 1000 37.2 / 29.1; single
+// projections 25600 -> 5120 at q = 128, M = 1280 119.5 / 110.2, 5120 -> 25600 at q = 32, M = 7584 251 / 243; at q = 64 to 256 and
+// M = 2048 even.
+constexpr int kPacked = 1;   // several row types per tile
+constexpr int kGroups = 2;   // several output groups per tile
+constexpr int kGated = 4;    // gated up projection (never with kGroups)
+
 struct Tile {
   int row0, rows;   // bucketed rows [row0, row0 + rows), all of type i; row0 < 0: no more tiles
   int i, j;         // packed tiles: i = first of np consecutive types; j = first of ng consecutive output groups
@@ -140,11 +150,13 @@ __device__ __forceinline__ int fast_div(int t, int d, float inv_d) {
 
 // Tile t of the launch (uniform across the warp).  Type-major; inside a type: m-tile fastest, then
 // the column tile, then the output group.
+template <int MODE>
 __device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
+  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups;
   Tile o;
   o.row0 = -1, o.rows = 0, o.i = 0, o.j = 0, o.n0 = 0, o.cols = 0, o.n0_w = 0, o.np = 1, o.ng = 1;
   if (t >= ctl->total) return o;
-  if (a.pack > 1 && a.gpack > 1) {
+  if (PACKED && GROUPS) {
     // several types AND several output groups per tile.  Type-group major; inside a type group first the column
     // units (a.gpack groups each) that hold none of its types, one tile each, then the groups of the other units
     // one by one (a tile never holds a type together with other groups than its own: the diagonal product of
@@ -172,7 +184,7 @@ __device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, in
     o.cols = o.ng * a.r;
     return o;
   }
-  if (a.pack > 1) {   // type-group major, then the output group, then the column tile
+  if (PACKED) {   // type-group major, then the output group, then the column tile
     const int per_group = a.q * a.nt_n;
     const int tg = fast_div(t, per_group, a.inv_per_type), rem = t - tg * per_group;
     const int j = a.nt_n == 1 ? rem : rem / a.nt_n, nt = rem - j * a.nt_n;
@@ -207,7 +219,7 @@ __device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, in
   const int u = mt_i == 1 ? rem : rem / mt_i, mt = rem - u * mt_i;
   o.row0 = base + (mt << 7);
   o.rows = min(128, rows_i - (mt << 7));
-  if (a.gpack > 1) {   // a tile of several whole output groups
+  if (GROUPS) {   // a tile of several whole output groups
     o.i = i, o.j = u * a.gpack;
     o.ng = min(a.gpack, a.q - o.j);
     o.n0 = o.j * a.r_out;
@@ -231,10 +243,12 @@ __device__ __forceinline__ int4 pack_tile(const Tile &o) {
   return make_int4(o.row0, o.n0, o.rows | (o.cols << 8) | (o.np << 20), o.i | (o.j << 8) | (o.ng << 16));
 }
 // (out of line: three roles call it, for tiles past the records only)
-__device__ __noinline__ Tile decode_tile_late(const BigArgs &a, const Ctl *ctl, int t) { return decode_tile(a, ctl, t); }
+template <int MODE>
+__device__ __noinline__ Tile decode_tile_late(const BigArgs &a, const Ctl *ctl, int t) { return decode_tile<MODE>(a, ctl, t); }
 // record `round` of this CTA, uniform across the warp; tiles past the records are decoded where they are needed
+template <int MODE>
 __device__ __forceinline__ Tile get_tile(const BigArgs &a, const Ctl *ctl, int round) {
-  if (round >= kBigSeq) return decode_tile_late(a, ctl, blockIdx.x + round * gridDim.x);
+  if (round >= kBigSeq) return decode_tile_late<MODE>(a, ctl, blockIdx.x + round * gridDim.x);
   const int4 v = ctl->recs[round];
   const int w = __shfl_sync(0xffffffffu, v.z, 0), x = __shfl_sync(0xffffffffu, v.w, 0);
   Tile o;
@@ -244,22 +258,24 @@ __device__ __forceinline__ Tile get_tile(const BigArgs &a, const Ctl *ctl, int r
   o.n0_w = o.n0 + o.j * (a.r - a.r_out);
   return o;
 }
+template <int MODE>
 __device__ __forceinline__ void decode_tiles(const BigArgs &a, Ctl *ctl) {   // one warp
   __syncwarp();
   const int lane = threadIdx.x & 31;
   for (int round = lane; round < kBigSeq; round += 32) {
-    const Tile o = decode_tile(a, ctl, blockIdx.x + round * gridDim.x);
+    const Tile o = decode_tile<MODE>(a, ctl, blockIdx.x + round * gridDim.x);
     ctl->recs[round] = pack_tile(o);
     if (!__any_sync(0xffffffffu, o.row0 >= 0)) break;
   }
 }
 
-template <int TILE_N, int BK>
+template <int TILE_N, int BK, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                 const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2,
                 const __grid_constant__ BigArgs a) {
   using C = Cfg<TILE_N, BK>;
+  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups, GATED = MODE & kGated;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *store_buf = smem + C::kStages * C::kStageBytes;
@@ -291,8 +307,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   } else if (warp == 3 && lane == 0) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
-    if (a.pack > 1 || a.sched == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA2) : "memory");
-    if (a.gpack > 1) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB2) : "memory");
+    if (PACKED || a.sched == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmA2) : "memory");
+    if (GROUPS) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB2) : "memory");
   }
   // Groups narrower than a stage: only their rows of W are fetched (a row costs the copy engine the same whether it holds
   // data or fill).  The rows below them are zeroed here and never written again -- X is zero there, but zero times what
@@ -312,7 +328,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   if (warp == 2) {
     // tile counts (counted buckets: one warp turns the bucket offsets into "tiles before type i"), then this CTA's tiles;
     // with equal buckets nothing of it comes from the previous kernel
-    if (a.pack > 1 && a.gpack > 1) {
+    if (PACKED && GROUPS) {
       // tiles before every type group (see decode_tile)
       const int n_tg = (q + a.pack - 1) / a.pack, g = a.gpack, n_units = (q + g - 1) / g;
       int carry = 0;
@@ -333,7 +349,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         carry += __shfl_sync(0xffffffffu, incl, 31);
       }
       if (lane == 0) ctl->pre[n_tg] = carry, ctl->total = carry;
-    } else if (a.pack > 1) {
+    } else if (PACKED) {
       if (lane == 0) ctl->total = ((q + a.pack - 1) / a.pack) * q * a.nt_n;
     } else if (a.sched != 0) {
       if (lane == 0) ctl->total = q * ((a.rows_per_type + 127) >> 7) * a.col_units;
@@ -359,7 +375,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       }
       if (lane == 0) ctl->pre[q] = carry, ctl->total = carry;
     }
-    decode_tiles(a, ctl);
+    decode_tiles<MODE>(a, ctl);
     if (a.sched != 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   }
   tc_fence_before();
@@ -376,17 +392,17 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     bool ok = true;
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t smem0 = smem_u32(smem);
-    const int b_chunks = a.gated_f ? 2 * a.n_chunks : a.n_chunks;   // 64-column boxes of the bank per stage
+    const int b_chunks = GATED ? 2 * a.n_chunks : a.n_chunks;   // 64-column boxes of the bank per stage
     const int box_bytes = a.b_box_rows * 128;                        // of such a box
     for (int round = 0; ok; ++round) {
-      const Tile tl = get_tile(a, ctl, round);
+      const Tile tl = get_tile<MODE>(a, ctl, round);
       if (tl.row0 < 0) break;
       if (loads_a && lane == 0) ALG_TRACE(0, 1);
-      const bool packed = a.pack > 1;
+      const bool packed = PACKED;
       // packed tile: segment 0 is the diagonal one (group j), then one panel segment per type of the tile other than j
       const int j_in = packed && tl.ng == 1 && tl.j >= tl.i && tl.j < tl.i + tl.np ? 1 : 0;
       // tile of several output groups: segment 0 is the panel product (k = i), then one diagonal product per group other than i
-      const bool gp = a.gpack > 1;
+      const bool gp = GROUPS;
       // several types and several groups: one panel segment per type, then one diagonal segment per group (all rows)
       const bool pg = packed && gp;
       const int i_in = gp && !packed && tl.i >= tl.j && tl.i < tl.j + tl.ng ? 1 : 0;
@@ -447,7 +463,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             } else {
               for (int c = 0; c < a.n_chunks; ++c)
                 tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, &tmB, bar, tl.n0_w + c * 64, kb * BK, k);
-              for (int c = 0; c < (a.gated_f ? a.n_chunks : 0); ++c)   // the matching up columns, behind the gate chunks
+              for (int c = 0; c < (GATED ? a.n_chunks : 0); ++c)   // the matching up columns, behind the gate chunks
                 tma_load_3d(sa + C::kABytes + (a.n_chunks + c) * C::kBChunkBytes, &tmB, bar, a.gated_f + tl.n0_w + c * 64, kb * BK, k);
             }
           }
@@ -466,17 +482,17 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint64_t da0 = make_smem_desc(smem_u32(smem), 16, C::kSboK, C::kSwzK);
     const uint64_t db0 = make_smem_desc(smem_u32(smem) + C::kABytes, C::kBChunkBytes, 1024);
     // instruction descriptor: D = f32, A = B = bf16, A K-major, B MN-major, N = tile_n, M = 128
-    const int mma_n = a.gated_f ? 2 * a.n_chunks * 64 : a.tile_n;   // gated: gate chunks and up chunks side by side
+    const int mma_n = GATED ? 2 * a.n_chunks * 64 : a.tile_n;   // gated: gate chunks and up chunks side by side
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(mma_n >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
     for (int round = 0; ok; ++round) {
-      const Tile tl = get_tile(a, ctl, round);
+      const Tile tl = get_tile<MODE>(a, ctl, round);
       if (tl.row0 < 0) break;
       const int j_in_t = tl.ng == 1 && tl.j >= tl.i && tl.j < tl.i + tl.np ? 1 : 0;
-      const bool pg = a.pack > 1 && a.gpack > 1;
+      const bool pg = PACKED && GROUPS;
       const int n_kb = (pg            ? tl.ng + tl.np - j_in_t
-                        : a.pack > 1  ? 1 + tl.np - j_in_t
-                        : a.gpack > 1 ? 1 + tl.ng - (tl.i >= tl.j && tl.i < tl.j + tl.ng ? 1 : 0)
+                        : PACKED  ? 1 + tl.np - j_in_t
+                        : GROUPS ? 1 + tl.ng - (tl.i >= tl.j && tl.i < tl.j + tl.ng ? 1 : 0)
                                       : (tl.i == tl.j ? 1 : 2)) *
                        nkb_seg;
       if (lane == 0) ALG_TRACE(1, 1);
@@ -485,7 +501,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       if (lane == 0) ALG_TRACE(1, 2);
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TILE_N);
-      const bool gp = a.gpack > 1 && !pg;
+      const bool gp = GROUPS && !pg;
       const int i_in = gp && tl.i >= tl.j && tl.i < tl.j + tl.ng ? 1 : 0;
       for (int kb = 0; kb < n_kb; ++kb) {
         ok = __all_sync(0xffffffffu, wait_bar(full0 + 8u * (uint32_t)stage, phase, ctl, a.status));
@@ -540,12 +556,12 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int rd_r = lane >> 3, rd_p = lane & 7;     // row within a group of four, 16-byte piece of the row
     const bool store8 = (a.r_out & 7) != 0;
     for (int round = 0;; ++round) {
-      const Tile tl = get_tile(a, ctl, round);
+      const Tile tl = get_tile<MODE>(a, ctl, round);
       if (tl.row0 < 0) break;
       const int r = quad * 32 + lane;
       int64_t out_row = -1;
       if (r < tl.rows) {
-        if (a.sched_out == 2 && a.pack > 1) {   // rows of a packed tile are type-major: type tl.i + r / rows_per_type
+        if (a.sched_out == 2 && PACKED) {   // rows of a packed tile are type-major: type tl.i + r / rows_per_type
           const int ti = fast_div(r, a.rows_per_type, a.inv_rpt);
           out_row = (int64_t)(r - ti * a.rows_per_type) * q + tl.i + ti;
         } else if (a.sched_out == 2) out_row = (int64_t)(tl.row0 + r - tl.i * a.rows_per_type) * q + tl.i;
@@ -563,7 +579,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       // Tiles of this path have short reductions, so the epilogue is the longest chain of a tile: warps
       // whose 32 rows lie past the tile's last row do nothing.
       const int c_end = quad * 32 < tl.rows ? tl.cols : 0;
-      if (a.gated_f) {
+      if (GATED) {
         // gate values sit in accumulator columns [0, cols), the matching up values n_chunks * 64 columns further;
         // silu(g) * u with sigmoid(g) = (1 + tanh(g / 2)) / 2, then the 32 x 32 chunk goes through the warp's
         // buffer as 64-byte rows (four lanes store one row segment, 8 rows per store instruction)
@@ -674,7 +690,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                            : "=r"(val.x), "=r"(val.y), "=r"(val.z), "=r"(val.w)
                            : "r"(buf0 + (uint32_t)rr * 128u + ((((uint32_t)rd_p) ^ (uint32_t)(rr & 7)) << 4)));
               const int64_t dr = dst_row[ph * 4 + g];
-              if (a.gpack > 1) {
+              if (GROUPS) {
                 // the piece's 8 accumulator columns lie in one group of the tile: group gi, column cg of it
                 const int tc = c0 + rd_p * 8, gi = fast_div(tc, a.r, a.inv_r), cg = tc - gi * a.r;
                 __nv_bfloat16 *dst = (__nv_bfloat16 *)a.Y + dr * a.ldy + tl.n0 + gi * a.r_out + cg;
@@ -719,7 +735,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
             for (int x = 0; x < 32; ++x) f[x] = gelu_tanh(f[x]);
           }
-          if (out_row >= 0 && a.gpack > 1) {
+          if (out_row >= 0 && GROUPS) {
 #pragma unroll
             for (int g = 0; g < 8; ++g) {   // four accumulator columns lie in one group of the tile
               const int tc = c0 + g * 4, gi = fast_div(tc, a.r, a.inv_r), cg = tc - gi * a.r;
@@ -759,11 +775,11 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   }
 }
 
-template <int TILE_N, int BK>
-cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
+template <int TILE_N, int BK, int MODE>
+cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   using C = Cfg<TILE_N, BK>;
   static OncePerDevice limit;
-  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
+  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
   if (e != cudaSuccess) return e;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
   CUtensorMap tmA, tmA2, tmB;
@@ -840,9 +856,21 @@ cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (b.gpack <= 1) tmB2 = tmB;
-  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK>, tmA, tmA2, tmB, tmB2, b);
+  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK, MODE>, tmA, tmA2, tmB, tmB2, b);
   count_launch(1);
   return e;
+}
+
+template <int TILE_N, int BK>
+cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
+  if (a.gated_f) {
+    if constexpr (TILE_N == 256)
+      return a.pack > 1 ? launch_m<TILE_N, BK, kGated | kPacked>(a, num_sms, st) : launch_m<TILE_N, BK, kGated>(a, num_sms, st);
+    else
+      return cudaErrorInvalidValue;
+  }
+  if (a.pack > 1) return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups>(a, num_sms, st) : launch_m<TILE_N, BK, kPacked>(a, num_sms, st);
+  return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups>(a, num_sms, st) : launch_m<TILE_N, BK, 0>(a, num_sms, st);
 }
 
 }  // namespace
