@@ -219,6 +219,7 @@ struct BigArgs {
   int block_k;            // 64 or 32: reduction depth of a pipeline stage
   int n_chunks;           // 64-column boxes of W fetched per stage = ceil(tile_n / 64)
   int b_box_rows;         // rows of W fetched per stage: block_k, or the group's width when that is less            (set by the launcher)
+  int b_tail_rows;        // the same of the last stage of a segment: no more than the group has there, in multiples of 16 (set by the launcher)
   int a_box_rows;         // rows of X fetched per stage: 128, or fewer when no type has that many rows
   int gated_f;            // > 0: SwiGLU up projection over the merged bank [W_gate | W_up] (2 * gated_f columns): a tile
                           // accumulates its gate columns and, n_chunks * 64 accumulator columns further, the matching

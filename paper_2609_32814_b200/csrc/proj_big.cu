@@ -129,6 +129,8 @@ struct Cfg {
 constexpr int kPacked = 1;   // several row types per tile
 constexpr int kGroups = 2;   // several output groups per tile
 constexpr int kGated = 4;    // gated up projection (never with kGroups)
+constexpr int kTail = 8;     // segments that end inside a stage: of their last stage only the rows of W that the group has
+                             // are fetched and multiplied, in multiples of 16
 
 struct Tile {
   int row0, rows;   // bucketed rows [row0, row0 + rows), all of type i; row0 < 0: no more tiles
@@ -273,9 +275,10 @@ template <int TILE_N, int BK, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                 const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2,
+                const __grid_constant__ CUtensorMap tmBt, const __grid_constant__ CUtensorMap tmB2t,
                 const __grid_constant__ BigArgs a) {
   using C = Cfg<TILE_N, BK>;
-  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups, GATED = MODE & kGated;
+  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups, GATED = MODE & kGated, TAIL = MODE & kTail;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *store_buf = smem + C::kStages * C::kStageBytes;
@@ -393,7 +396,6 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
     const uint32_t smem0 = smem_u32(smem);
     const int b_chunks = GATED ? 2 * a.n_chunks : a.n_chunks;   // 64-column boxes of the bank per stage
-    const int box_bytes = a.b_box_rows * 128;                        // of such a box
     for (int round = 0; ok; ++round) {
       const Tile tl = get_tile<MODE>(a, ctl, round);
       if (tl.row0 < 0) break;
@@ -434,6 +436,9 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           if (!ok) break;
           const uint32_t bar = full0 + 8u * (uint32_t)stage;
           const uint32_t sa = smem0 + (uint32_t)stage * (uint32_t)C::kStageBytes;
+          const bool last = TAIL && kb == nkb_seg - 1;
+          const int box_bytes = (last ? a.b_tail_rows : a.b_box_rows) * 128;   // of a 64-column box
+          const CUtensorMap *map_b = last ? &tmBt : &tmB, *map_b2 = last ? &tmB2t : &tmB2;
           if (elect_one()) {
             if (loads_a && packed) {
               if (diag_seg) {   // all rows of the tile: np types x rows_per_type rows, type-major
@@ -459,12 +464,12 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
               // (64 c - offset of the group in the tile) of group k is out of range on both sides of the group
               const int goff = (k - tl.j) * a.r;
               for (int c = goff / 64; c <= (goff + a.r - 1) / 64; ++c)
-                tma_load_4d(sa + C::kABytes + c * C::kBChunkBytes, &tmB2, bar, c * 64 - goff, k, kb * BK, k);
+                tma_load_4d(sa + C::kABytes + c * C::kBChunkBytes, map_b2, bar, c * 64 - goff, k, kb * BK, k);
             } else {
               for (int c = 0; c < a.n_chunks; ++c)
-                tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, &tmB, bar, tl.n0_w + c * 64, kb * BK, k);
+                tma_load_3d(sa + C::kABytes + c * C::kBChunkBytes, map_b, bar, tl.n0_w + c * 64, kb * BK, k);
               for (int c = 0; c < (GATED ? a.n_chunks : 0); ++c)   // the matching up columns, behind the gate chunks
-                tma_load_3d(sa + C::kABytes + (a.n_chunks + c) * C::kBChunkBytes, &tmB, bar, a.gated_f + tl.n0_w + c * 64, kb * BK, k);
+                tma_load_3d(sa + C::kABytes + (a.n_chunks + c) * C::kBChunkBytes, map_b, bar, a.gated_f + tl.n0_w + c * 64, kb * BK, k);
             }
           }
           __syncwarp();
@@ -485,6 +490,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const int mma_n = GATED ? 2 * a.n_chunks * 64 : a.tile_n;   // gated: gate chunks and up chunks side by side
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(mma_n >> 3) << 17) |
                            ((uint32_t)(128 >> 4) << 24);
+    // 16-deep steps of a segment's last stage (the stage's other rows of W are not there)
+    const int last_steps = a.b_tail_rows / 16;
     for (int round = 0; ok; ++round) {
       const Tile tl = get_tile<MODE>(a, ctl, round);
       if (tl.row0 < 0) break;
@@ -503,7 +510,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TILE_N);
       const bool gp = GROUPS && !pg;
       const int i_in = gp && tl.i >= tl.j && tl.i < tl.j + tl.ng ? 1 : 0;
-      for (int kb = 0; kb < n_kb; ++kb) {
+      for (int kb = 0, left = nkb_seg; kb < n_kb; ++kb) {
         ok = __all_sync(0xffffffffu, wait_bar(full0 + 8u * (uint32_t)stage, phase, ctl, a.status));
         if (!ok) break;
         if (kb == 0 && lane == 0) ALG_TRACE(1, 3);
@@ -522,10 +529,12 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           d_seg += (uint32_t)(c_lo * 64);
           idesc_seg = (idesc & ~(0x3Fu << 17)) | ((uint32_t)(((c_hi - c_lo + 1) * 64) >> 3) << 17);
         }
+        const int steps = TAIL && left == 1 ? last_steps : BK / 16;
+        if (TAIL && --left == 0) left = nkb_seg;
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
-            tc_mma_bf16(d_seg, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 128), idesc_seg, (kb | kk) ? 1u : 0u);
+            if (!TAIL || kk < steps) tc_mma_bf16(d_seg, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 128), idesc_seg, (kb | kk) ? 1u : 0u);
           tc_commit(empty0 + 8u * (uint32_t)stage);
         }
         __syncwarp();
@@ -782,7 +791,7 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
   if (e != cudaSuccess) return e;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
-  CUtensorMap tmA, tmA2, tmB;
+  CUtensorMap tmA, tmA2, tmB, tmBt, tmB2t;
   const BigArgs &b = a;
   if (b.pack > 1) {
     // X as {k in group, group, row in type, type}: interval rows of a type are consecutive, cyclic ones q apart
@@ -821,16 +830,18 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
     // the bank by {column in group, column group, k in group, row group}
     const uint64_t dims[4] = {(uint64_t)a.r, (uint64_t)a.q, (uint64_t)a.s, (uint64_t)a.q};
     const uint64_t str[3] = {(uint64_t)a.r * 2, (uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
-    const uint32_t box[4] = {64, 1, (uint32_t)a.b_box_rows, 1};
+    const uint32_t box[4] = {64, 1, (uint32_t)a.b_box_rows, 1}, box_t[4] = {64, 1, (uint32_t)a.b_tail_rows, 1};
     e = make_map_nd(&tmB2, a.W, 4, dims, str, box, 128);
+    if (e == cudaSuccess) e = make_map_nd(&tmB2t, a.W, 4, dims, str, box_t, 128);
     if (e != cudaSuccess) return e;
   }
   {
     // the bank as {columns, k in group, group}: rows past the group's width read as zero
     const uint64_t dims[3] = {(uint64_t)a.q * (uint64_t)a.r * (a.gated_f ? 2 : 1), (uint64_t)a.s, (uint64_t)a.q};
     const uint64_t str[2] = {(uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
-    const uint32_t box[3] = {64, (uint32_t)a.b_box_rows, 1};
+    const uint32_t box[3] = {64, (uint32_t)a.b_box_rows, 1}, box_t[3] = {64, (uint32_t)a.b_tail_rows, 1};
     e = make_map_nd(&tmB, a.W, 3, dims, str, box, 128);
+    if (e == cudaSuccess) e = make_map_nd(&tmBt, a.W, 3, dims, str, box_t, 128);
   }
   if (e != cudaSuccess) return e;
   long long tiles;
@@ -855,22 +866,30 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (b.gpack <= 1) tmB2 = tmB;
-  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK, MODE>, tmA, tmA2, tmB, tmB2, b);
+  if (b.gpack <= 1) tmB2 = tmB, tmB2t = tmBt;
+  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK, MODE>, tmA, tmA2, tmB, tmB2, tmBt, tmB2t, b);
   count_launch(1);
   return e;
 }
 
-template <int TILE_N, int BK>
-cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
+template <int TILE_N, int BK, int TAIL>
+cudaError_t launch_s(const BigArgs &a, int num_sms, cudaStream_t st) {
   if (a.gated_f) {
     if constexpr (TILE_N == 256)
-      return a.pack > 1 ? launch_m<TILE_N, BK, kGated | kPacked>(a, num_sms, st) : launch_m<TILE_N, BK, kGated>(a, num_sms, st);
+      return a.pack > 1 ? launch_m<TILE_N, BK, kGated | kPacked | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, kGated | TAIL>(a, num_sms, st);
     else
       return cudaErrorInvalidValue;
   }
-  if (a.pack > 1) return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups>(a, num_sms, st) : launch_m<TILE_N, BK, kPacked>(a, num_sms, st);
-  return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups>(a, num_sms, st) : launch_m<TILE_N, BK, 0>(a, num_sms, st);
+  if (a.pack > 1)
+    return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, kPacked | TAIL>(a, num_sms, st);
+  return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, TAIL>(a, num_sms, st);
+}
+template <int TILE_N, int BK>
+cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
+  if constexpr (BK == 64) {
+    if (a.b_tail_rows < a.b_box_rows) return launch_s<TILE_N, BK, kTail>(a, num_sms, st);
+  }
+  return launch_s<TILE_N, BK, 0>(a, num_sms, st);
 }
 
 }  // namespace
@@ -890,6 +909,9 @@ cudaError_t launch_proj_big(const BigArgs &in, int num_sms, cudaStream_t st) {
   // 25600 -> 5120 at M = 32768: q = 64 (groups of 80) 0.557 -> 0.533 ms, q = 256 (24) 1.97 -> 1.57 ms; 5120 -> 25600 at
   // q = 256 (104) 1.49 -> 1.39 ms; groups of 128 lose (square product n = 8192: 0.065 -> 0.088 ms) and stay one per tile
   a.b_box_rows = std::min(a.s, a.block_k);
+  // (5120 -> 25600: q = 64, groups of 80 = 64 + 16, M = 2048 95.2 -> 85.3 us, q = 32, groups of 160, M = 7584 243.5 -> 233.1; gated
+  // 2560 -> 9728 at q = 32, M = 3000 102.9 -> 98.7)
+  a.b_tail_rows = a.s <= a.block_k ? a.b_box_rows : a.s % a.block_k ? (a.s % a.block_k + 15) / 16 * 16 : a.block_k;
   a.gpack = 1;
   a.col_units = a.q * a.nt_n;
   if (a.nt_n == 1 && !a.gated_f && !a.bias && a.r <= 112 && a.q >= 2) {

@@ -286,3 +286,13 @@ def test_more_tiles_than_records(q, M, s_w, r_w, schedule):
     rows = np.unique(np.r_[np.arange(0, M, 61), M - 1])
     ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
     assert np.array_equal(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref)
+
+
+@pytest.mark.parametrize("s_w", [16, 48, 56, 88, 112, 120])   # groups of less than a stage and the last stages of deeper ones: 16, 48, 64, 32, 48, 64 rows
+@pytest.mark.parametrize("r_w", [40, 168, 232])               # one, three and four 64-column boxes in a stage
+@pytest.mark.parametrize("q,rows", [(6, 40), (34, 136)])      # several types per tile; two m-tiles per type
+def test_big_stage_sizes(s_w, r_w, q, rows):
+    wl = _workload(q, q * rows, s_w, r_w, "interval", seed=s_w + r_w)
+    Y, _ = _forward(wl, "interval", torch.float32)
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(Y), ref)
