@@ -109,11 +109,15 @@ struct MoreMaps<true> {
   CUtensorMap A, B;
 };
 
-template <int TILE_N, int S, bool WHOLE>
+// ROWS: rows of A one behind the other and the canonical bank, known at compile time (as OPS = 1 in proj_tc.cu).
+template <int TILE_N, int S, bool WHOLE, bool ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a,
                   const __grid_constant__ MoreMaps<WHOLE> more) {
   using C = CfgS<TILE_N, S>;
+  const bool a_mn = WHOLE ? true : ROWS ? false : a.a_mn != 0;
+  const bool w_kmajor = WHOLE || ROWS ? false : a.w_kmajor != 0;
+  const bool b_3d = ROWS ? true : a.b_3d != 0, a_cyclic = ROWS ? false : a.a_cyclic_rows != 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   // partial sums arrive over the stages: nobody sends before every CTA of the cluster has used its operands up (the bytes
@@ -220,7 +224,7 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           const int k0 = k_begin + (i << 6);
           if (elect_one()) {
             mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
-            if (a.a_mn) {   // weight gradient: rows of X and G as they lie, features / columns contiguous
+            if (a_mn) {   // weight gradient: rows of X and G as they lie, features / columns contiguous
               const int pos0 = a.seg_rows ? i << 6 : k0, seg = a.seg_rows ? k : 0;
               const CUtensorMap *map_a = &tmA, *map_b = &tmB;
               if constexpr (WHOLE) {
@@ -231,11 +235,11 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 #pragma unroll
               for (int c = 0; c < TILE_N / 64; ++c) tma_load_3d(sa + kABytes + c * kBChunkBytes, map_b, bar, n0 + c * 64, seg, pos0);
             } else {
-              if (a.a_cyclic_rows) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
+              if (a_cyclic) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
               else tma_load_2d(sa, &tmA, bar, k0, a_row);
-              if (a.w_kmajor) {
+              if (w_kmajor) {
                 tma_load_2d(sa + kABytes, &tmB, bar, k0, n0);
-              } else if (a.b_3d) {
+              } else if (b_3d) {
                 tma_load_3d(sa + kABytes, &tmB, bar, 0, k0, n0 >> 6);
               } else {
 #pragma unroll
@@ -251,11 +255,11 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     } else if (warp == 1) {
       // ---------------- MMA issuer (operand layouts as in proj_tc.cu) ----------------
       const uint32_t full0 = smem_u32(&ctl->full[0]), empty0 = smem_u32(&ctl->empty[0]);
-      const uint64_t da0 = a.a_mn ? make_smem_desc(smem_u32(smem), 64 * 64 * 2, 1024) : make_smem_desc(smem_u32(smem), 16, 1024);
-      const uint64_t da_step = a.a_mn ? 128 : 2;
-      const uint64_t db0 = a.w_kmajor ? make_smem_desc(smem_u32(smem) + kABytes, 16, 1024) : make_smem_desc(smem_u32(smem) + kABytes, kBChunkBytes, 1024);
-      const uint64_t db_step = a.w_kmajor ? 2 : 128;
-      const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.a_mn ? (1u << 15) : 0u);
+      const uint64_t da0 = a_mn ? make_smem_desc(smem_u32(smem), 64 * 64 * 2, 1024) : make_smem_desc(smem_u32(smem), 16, 1024);
+      const uint64_t da_step = a_mn ? 128 : 2;
+      const uint64_t db0 = w_kmajor ? make_smem_desc(smem_u32(smem) + kABytes, 16, 1024) : make_smem_desc(smem_u32(smem) + kABytes, kBChunkBytes, 1024);
+      const uint64_t db_step = w_kmajor ? 2 : 128;
+      const uint32_t idesc = (w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a_mn ? (1u << 15) : 0u);
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -407,16 +411,19 @@ proj_split_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   }
 }
 
-template <int TILE_N, int S, bool WHOLE>
+template <int TILE_N, int S, bool WHOLE, bool ROWS>
 cudaError_t launch_w(const ProjArgs &a, int tiles, cudaStream_t st) {
   using C = CfgS<TILE_N, S>;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
-  cudaError_t e = cudaFuncSetAttribute(proj_split_kernel<TILE_N, S, WHOLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+  cudaError_t e = cudaFuncSetAttribute(proj_split_kernel<TILE_N, S, WHOLE, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   if (e != cudaSuccess) return e;
   CUtensorMap tmA, tmB;
   ProjArgs b = a;
   e = make_tc_maps(&tmA, &tmB, &b, TILE_N, 128, false, 64);
   if (e != cudaSuccess) return e;
+  if constexpr (ROWS) {
+    if (!b.b_3d) return launch_w<TILE_N, S, WHOLE, false>(a, tiles, st);
+  }
   MoreMaps<WHOLE> more;
   if constexpr (WHOLE) {
     e = make_grad_maps(&more.A, &more.B, a.whole_x, a.whole_ldx, a.M, a.whole_g, a.whole_ldg, a.N, 1, a.whole_rows);
@@ -435,11 +442,12 @@ cudaError_t launch_w(const ProjArgs &a, int tiles, cudaStream_t st) {
   cfg.attrs = at;
   cfg.numAttrs = 2;
   count_launch(1);
-  return cudaLaunchKernelEx(&cfg, proj_split_kernel<TILE_N, S, WHOLE>, tmA, tmB, b, more);
+  return cudaLaunchKernelEx(&cfg, proj_split_kernel<TILE_N, S, WHOLE, ROWS>, tmA, tmB, b, more);
 }
 template <int TILE_N, int S>
 cudaError_t launch_s(const ProjArgs &a, int tiles, cudaStream_t st) {
-  return a.whole_rows ? launch_w<TILE_N, S, true>(a, tiles, st) : launch_w<TILE_N, S, false>(a, tiles, st);
+  if (a.whole_rows) return launch_w<TILE_N, S, true, false>(a, tiles, st);
+  return a.a_mn || a.w_kmajor || a.a_cyclic_rows ? launch_w<TILE_N, S, false, false>(a, tiles, st) : launch_w<TILE_N, S, false, true>(a, tiles, st);
 }
 
 }  // namespace

@@ -127,11 +127,21 @@ template <>
 struct MoreMaps<3> {
   CUtensorMap A, B;
 };
-template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE>
+// OPS: the common operands, known at compile time.  1: rows of A one behind the other, B the canonical bank; 2: the same
+// with type-strided rows (cyclic schedule); 3: rows, bank used transposed; 0: any (asked at run time).  With the
+// tests in the loops of the producers and of the MMA warp, and a branch for empty tiles in the epilogue, us, asked / compiled
+// in: FFN 768 -> 3072 at q = 2, M = 1777 33.8 / 32.8; 1024 -> 4096 at q = 4, M = 3000 42.1 / 41.1, q = 8, M = 500 24.0 / 23.6;
+// gated 768 -> 1536 interval, M = 12288 59.1 / 56.9; forward and gradients of 768 -> 3072, M = 8003 151.8 / 150.0; even where
+// whole tiles fill the GPU (cyclic, M = 8192).
+template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE, int OPS>
 __global__ void __launch_bounds__(AMODE == 2 ? kThreads + 32 * kGatherWarps : kThreads, 1)
 proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const ProjArgs a,
                const __grid_constant__ MoreMaps<AMODE> more) {
   using C = Cfg<TILE_N, TILE_M, BK>;
+  const bool a_mn = AMODE == 3 ? true : OPS ? false : a.a_mn != 0;
+  const bool w_kmajor = OPS == 3 ? true : OPS || AMODE == 3 ? false : a.w_kmajor != 0;
+  const bool b_3d = OPS == 1 || OPS == 2 ? true : a.b_3d != 0;
+  const bool a_cyclic = OPS == 2 ? true : OPS ? false : a.a_cyclic_rows != 0;
   static_assert(!GATED || (TILE_N == 256 && TILE_M == 128), "the gated kernel pairs two 128-column halves");
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -292,7 +302,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               } else if (GATED) {
                 tma_load_3d(sa + C::kABytes, &tmB, bar, 0, k0, n0 >> 6);
                 tma_load_3d(sa + C::kABytes + 2 * C::kBChunkBytes, &tmB, bar, 0, k0, (a.gated_f + n0) >> 6);
-              } else if (a.b_3d) {
+              } else if (b_3d) {
                 tma_load_3d(sa + C::kABytes, &tmB, bar, 0, k0, n0 >> 6);
               } else {
 #pragma unroll
@@ -309,7 +319,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             g_rows[h][2], g_rows[h][3]);
             }
           } else if (elect_one()) {
-            if (a.a_mn) {
+            if (a_mn) {
               // weight gradient: 64 rows of X (A, features contiguous) and of G (B), in boxes of 64 features / 64 output
               // columns.  Cyclic schedule: rows k, k + q, ... from position k0 - so[k] on; else padded rows from k0 on
               const int pos0 = a.seg_rows ? k0 - k_begin : k0, seg = a.seg_rows ? k : 0;
@@ -336,16 +346,16 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               }
             } else if (loads_a) {
               mbar_expect_tx(bar, (uint32_t)C::kStageBytes);
-              if (a.a_cyclic_rows) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
+              if (a_cyclic) tma_load_3d(sa, &tmA, bar, k0, type_i, a_row);
               else tma_load_2d(sa, &tmA, bar, k0, a_row);
-            } else if (a.w_kmajor) {
+            } else if (w_kmajor) {
               // W used transposed: TILE_N rows of W (the output columns) x 64 of its columns (the reduction)
               tma_load_2d(sa + C::kABytes, &tmB, bar, k0, n0);
             } else if (GATED) {
               // two boxes of two 64-column chunks: the tile's gate columns, then its up columns
               tma_load_3d(sa + C::kABytes, &tmB, bar, 0, k0, n0 >> 6);
               tma_load_3d(sa + C::kABytes + 2 * C::kBChunkBytes, &tmB, bar, 0, k0, (a.gated_f + n0) >> 6);
-            } else if (a.b_3d) {
+            } else if (b_3d) {
               tma_load_3d(sa + C::kABytes, &tmB, bar, 0, k0, n0 >> 6);  // all 64-column chunks in one box
             } else {
 #pragma unroll
@@ -369,15 +379,15 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const uint32_t tfull0 = smem_u32(&ctl->tmem_full[0]), tempty0 = smem_u32(&ctl->tmem_empty[0]);
     // A: K-major rows of 128 (64) bytes; in the in-place weight-gradient pass the block lies MN-major like B
     // (64-feature chunks one box apart, 16 reduction rows = 128 descriptor units per K step)
-    const uint64_t da0 = a.a_mn ? make_smem_desc(smem_u32(smem), 64 * BK * 2, 1024)
+    const uint64_t da0 = a_mn ? make_smem_desc(smem_u32(smem), 64 * BK * 2, 1024)
                                     : make_smem_desc(smem_u32(smem), 16, C::kSboK, C::kSwzK);
-    const uint64_t da_step = a.a_mn ? 128 : 2;
+    const uint64_t da_step = a_mn ? 128 : 2;
     // B: the canonical bank lands MN-major (64-column chunks one box apart, 16 k-rows = two 8-row groups
     // = 128 descriptor units per K step); used transposed it lands K-major like A (32 bytes per K step)
-    const uint64_t db0 = a.w_kmajor ? make_smem_desc(smem_u32(smem) + C::kABytes, 16, C::kSboK, C::kSwzK)
+    const uint64_t db0 = w_kmajor ? make_smem_desc(smem_u32(smem) + C::kABytes, 16, C::kSboK, C::kSwzK)
                                     : make_smem_desc(smem_u32(smem) + C::kABytes, C::kBChunkBytes, 1024);
-    const uint32_t idesc = (a.w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a.a_mn ? (1u << 15) : 0u);
-    const uint64_t db_step = a.w_kmajor ? 2 : 128;
+    const uint32_t idesc = (w_kmajor ? (C::kIdesc & ~(1u << 16)) : C::kIdesc) | (a_mn ? (1u << 15) : 0u);
+    const uint64_t db_step = w_kmajor ? 2 : 128;
     TileRec rec = tile_seq_get(recs, tm, a.geom, 0, blockIdx.x, gridDim.x, ctl->nkb);
     while (ok && __shfl_sync(0xffffffffu, rec.row0, 0) >= 0) {
       ++round;
@@ -434,7 +444,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int tile_rows = rec.rows & 0xFFFF;
       // a tile without any K block (weight-gradient pass, row type absent from the batch): nothing was
       // accumulated, its result is zero
-      const bool empty_tile = ((uint32_t)rec.rows >> 16) == 0u;
+      const bool empty_tile = OPS == 0 && ((uint32_t)rec.rows >> 16) == 0u;
       if (r < tile_rows) {
         if (AMODE == 1 && a.out_cyclic_rows) {
           const int i = (rec.pair & 0xFFFF) / q;
@@ -562,11 +572,11 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
-template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE = 0>
+template <int TILE_N, int TILE_M, bool GATED, int BK, int AMODE = 0, int OPS = 0>
 cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   using C = Cfg<TILE_N, TILE_M, BK>;
   static OncePerDevice limit;
-  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
+  cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE, OPS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); });
   if (e != cudaSuccess) return e;
   int smem_bytes = C::kFixedSmemBytes + (int)tile_map_bytes(a.n_classes);
   if (smem_bytes > 227 * 1024) return cudaErrorInvalidConfiguration;
@@ -574,6 +584,9 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   ProjArgs b = a;
   e = make_tc_maps(&tmA, &tmB, &b, TILE_N, TILE_M, GATED, BK);
   if (e != cudaSuccess) return e;
+  if constexpr (OPS == 1 || OPS == 2) {
+    if (!b.b_3d) return launch_bk<TILE_N, TILE_M, GATED, BK, AMODE, 0>(a, num_sms, st);
+  }
   MoreMaps<AMODE> more;
   if constexpr (AMODE == 3) {
     e = make_grad_maps(&more.A, &more.B, a.whole_x, a.whole_ldx, a.M, a.whole_g, a.whole_ldg, a.N, 1, a.whole_rows);
@@ -593,7 +606,7 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE>, tmA, tmB, b, more);
+  e = cudaLaunchKernelEx(&cfg, proj_tc_kernel<TILE_N, TILE_M, GATED, BK, AMODE, OPS>, tmA, tmB, b, more);
   count_launch(1);
   return e;
 }
@@ -601,7 +614,8 @@ cudaError_t launch_bk(const ProjArgs &a, int num_sms, cudaStream_t st) {
 template <int TILE_N, int TILE_M, bool GATED = false>
 cudaError_t launch_t(const ProjArgs &a, int num_sms, cudaStream_t st) {
   // the in-place view of an interval schedule (runs of a type) is a kernel variant of its own, 64-deep stages only
-  if (a.run_rows) return a.block_k == 64 ? launch_bk<TILE_N, TILE_M, GATED, 64, 1>(a, num_sms, st) : cudaErrorInvalidValue;
+  if (a.run_rows && a.block_k != 64) return cudaErrorInvalidValue;
+  if (a.run_rows) return a.w_kmajor ? launch_bk<TILE_N, TILE_M, GATED, 64, 1, 0>(a, num_sms, st) : launch_bk<TILE_N, TILE_M, GATED, 64, 1, 1>(a, num_sms, st);
   // so are the rows of explicit types fetched through the permutation by the A producer
   if (a.in_perm) return a.block_k == 64 && !a.w_kmajor && !a.seg_rows ? launch_bk<TILE_N, TILE_M, GATED, 64, 2>(a, num_sms, st) : cudaErrorInvalidValue;
   if constexpr (TILE_M == 128 && !GATED) {
@@ -609,7 +623,13 @@ cudaError_t launch_t(const ProjArgs &a, int num_sms, cudaStream_t st) {
   }
   if (a.whole_rows) return cudaErrorInvalidValue;
   if (a.block_k == 32) return launch_bk<TILE_N, TILE_M, GATED, 32>(a, num_sms, st);
-  if (a.block_k == 64) return launch_bk<TILE_N, TILE_M, GATED, 64>(a, num_sms, st);
+  if (a.block_k == 64) {
+    if constexpr (!GATED) {
+      if (a.w_kmajor && !a.a_mn && !a.a_cyclic_rows) return launch_bk<TILE_N, TILE_M, GATED, 64, 0, 3>(a, num_sms, st);
+    }
+    if (a.w_kmajor || a.a_mn) return launch_bk<TILE_N, TILE_M, GATED, 64>(a, num_sms, st);
+    return a.a_cyclic_rows ? launch_bk<TILE_N, TILE_M, GATED, 64, 0, 2>(a, num_sms, st) : launch_bk<TILE_N, TILE_M, GATED, 64, 0, 1>(a, num_sms, st);
+  }
   return cudaErrorInvalidValue;
 }
 
