@@ -375,6 +375,7 @@ struct RowDecodeArgs {
   uint8_t *exch;            // FFN modes: hidden rows between the phases (exchange.cuh), buffers of exch_bytes
   int exch_bytes;
   int in_place;             // Y lies over X: no CTA stores Y before every CTA has used its X (FFN modes)
+  int warm2;                // one row: W2 is asked into L2 ahead of phase 2               (set by the launcher)
   int *status;
   long long wait_limit;
   int test_withhold;        // test hook: CTA 0 keeps its hidden values to itself, so that the waits for them run out

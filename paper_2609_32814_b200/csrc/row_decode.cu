@@ -107,6 +107,20 @@ __device__ __forceinline__ void load_chunk(uint4 (&w)[kLoads<GATED, RC>], const 
   }
 }
 
+// Asks L2 for the weights of this warp's first unit of a phase (a 16- or 8-column piece of a row is one sector).  Sent
+// before the launch's dependency resolves, so that W_down, which is loaded when phase 1 is over, comes from L2 and not from
+// HBM.  (A wrong type costs nothing but the hint.)
+__device__ __forceinline__ void prefetch_unit(const Phase &p, int n_units, int type) {
+  const int unit = unit_of(0, p.ks);
+  const Lane l = lane_of(p, unit);
+  if (unit >= n_units || !l.on || type < 0 || l.sub != 0) return;
+  for (int sg = 0; sg < (type == l.j ? 1 : 2); ++sg) {
+    const __nv_bfloat16 *base = p.W + (int64_t)(sg == 0 ? l.j : type) * p.s * p.ldw + l.col;
+    for (int kk = l.part * l.rl + l.lr; kk < p.s; kk += p.ks * l.rl)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(base + (int64_t)kk * p.ldw));
+  }
+}
+
 // Bound of the waits for hidden values.
 struct Wait {
   long long t0, limit;
@@ -318,6 +332,7 @@ __global__ void __launch_bounds__(kThreads, RC <= 4 ? 2 : 1) row_decode_kernel(c
     if (unit >= a.units1 || t_early < 0) l.on = false;
     load_chunk<GATED, RC>(w, p1, l, max(t_early, 0), 0);
   }
+  if (FFN && a.warm2) prefetch_unit(p2, a.units2, t_early);
   if (threadIdx.x == 0) ALG_TRACE(0, 2);
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (threadIdx.x == 0) ALG_TRACE(0, 3);
@@ -597,6 +612,11 @@ cudaError_t launch_row_decode(const RowDecodeArgs &in, int num_sms, cudaStream_t
   a.units2 = a.M * pieces2 * a.ks2;
   // every CTA of an FFN must be resident for the wait between the phases: one CTA per SM at most
   const int grid = std::min(num_sms, std::max(a.units1 / a.ks1, a.units2 / a.ks2));   // at most one piece group per CTA and slot
+  // W2's share of a row (two segments).  12 layers in a graph, without / with the hint, us: gated 2048 -> 6144 at q = 32 (1.6 MB)
+  // 73.3 / 72.3; 10 layers, gated 7168 -> 2048 (1.8 MB) 66.0 / 64.8, 2048 -> 8192 at q = 16 (4.2 MB) 86.8 / 85.5, gated 2560 ->
+  // 9728 (3.1 MB) 103.7 / 104.2; gated 4096 -> 12288 (6.3 MB) 133.1 / 134.8: there the hints stand in the way of the previous
+  // layer's loads.  Several rows, 2560 -> 9728, three of them: 209.9 / 217.9.
+  a.warm2 = a.mode != 2 && 4.0 * a.D * (double)a.F / a.q <= 5e6;
   if (a.mode == 0) return launch_mode<0>(a, grid, st);
   if (a.mode == 1) return launch_mode<1>(a, grid, st);
   return launch_mode<2>(a, grid, st);
