@@ -105,13 +105,17 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, Ctl *ctl
   return wait_slow(bar, parity, ctl, status);
 }
 
-template <int TILE_N, int BK>
+// KR = rows of W a stage holds: BK, or 32 where the groups of X are no wider (kNarrow); the stages are smaller then, and six of
+// them fit where four did.  What a CTA's operand fill hangs on is the bytes in flight: 5120 -> 25600 at q = 256 (groups of 24),
+// M = 2048 151.3 -> 136.3 us, M = 4096 200.0 -> 189.2.  Five stages of 48 rows (groups of 40, q = 128) were even or slower.
+template <int TILE_N, int BK, int KR>
 struct Cfg {
   static constexpr int kABytes = 128 * BK * 2;
-  static constexpr int kBChunkBytes = BK * 64 * 2;              // one BK(k) x 64(n) box
+  static constexpr int kBChunkBytes = KR * 64 * 2;              // one KR(k) x 64(n) box
   static constexpr int kChunks = TILE_N / 64;
   static constexpr int kStageBytes = kABytes + kBChunkBytes * kChunks;
-  static constexpr int kStages = (192 * 1024) / kStageBytes > 12 ? 12 : (192 * 1024) / kStageBytes;
+  static constexpr int kStageSmem = (KR == BK ? 192 : 204) * 1024;
+  static constexpr int kStages = kStageSmem / kStageBytes > 12 ? 12 : kStageSmem / kStageBytes;
   static constexpr int kTmemCols = 2 * TILE_N;
   static constexpr uint32_t kSwzK = BK == 64 ? 2 : 4;
   static constexpr uint32_t kSboK = 8 * BK * 2;
@@ -131,6 +135,11 @@ constexpr int kGroups = 2;   // several output groups per tile
 constexpr int kGated = 4;    // gated up projection (never with kGroups)
 constexpr int kTail = 8;     // segments that end inside a stage: of their last stage only the rows of W that the group has
                              // are fetched and multiplied, in multiples of 16
+
+constexpr int kNarrow = 16;  // groups of X of at most 32 columns
+constexpr int kAny = 32;     // types and groups per tile asked at run time.  Kept for several types and one group per tile without
+                             // kTail or kNarrow: 5120 -> 25600 at q = 128, M = 5888, bound by its stores, takes 156.7 us here and 170.3
+                             // as kPacked, M = 2048 the same in either
 
 struct Tile {
   int row0, rows;   // bucketed rows [row0, row0 + rows), all of type i; row0 < 0: no more tiles
@@ -154,7 +163,7 @@ __device__ __forceinline__ int fast_div(int t, int d, float inv_d) {
 // the column tile, then the output group.
 template <int MODE>
 __device__ __forceinline__ Tile decode_tile(const BigArgs &a, const Ctl *ctl, int t) {
-  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups;
+  const bool PACKED = MODE & kAny ? a.pack > 1 : (MODE & kPacked) != 0, GROUPS = MODE & kAny ? a.gpack > 1 : (MODE & kGroups) != 0;
   Tile o;
   o.row0 = -1, o.rows = 0, o.i = 0, o.j = 0, o.n0 = 0, o.cols = 0, o.n0_w = 0, o.np = 1, o.ng = 1;
   if (t >= ctl->total) return o;
@@ -277,8 +286,10 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2,
                 const __grid_constant__ CUtensorMap tmBt, const __grid_constant__ CUtensorMap tmB2t,
                 const __grid_constant__ BigArgs a) {
-  using C = Cfg<TILE_N, BK>;
-  constexpr bool PACKED = MODE & kPacked, GROUPS = MODE & kGroups, GATED = MODE & kGated, TAIL = MODE & kTail;
+  constexpr int KR = MODE & kNarrow ? 32 : BK;
+  using C = Cfg<TILE_N, BK, KR>;
+  constexpr bool GATED = MODE & kGated, TAIL = MODE & kTail;
+  const bool PACKED = MODE & kAny ? a.pack > 1 : (MODE & kPacked) != 0, GROUPS = MODE & kAny ? a.gpack > 1 : (MODE & kGroups) != 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t *store_buf = smem + C::kStages * C::kStageBytes;
@@ -317,8 +328,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
   // data or fill).  The rows below them are zeroed here and never written again -- X is zero there, but zero times what
   // the memory held may be NaN.  5120 -> 25600, q = 128 (groups of 40): M = 2048 92.0 -> 88.5 us, 8192 224 -> 214; q = 256
   // 161.8 -> 158.
-  if (a.b_box_rows < BK) {
-    const int pieces = (BK - a.b_box_rows) * 8;   // 16-byte pieces of a 64-column box
+  if (a.b_box_rows < KR) {
+    const int pieces = (KR - a.b_box_rows) * 8;   // 16-byte pieces of a 64-column box
     for (int e = threadIdx.x; e < C::kStages * C::kChunks * pieces; e += kThreads) {
       const int box = e / pieces, st = box / C::kChunks, c = box - st * C::kChunks;
       *(uint4 *)(smem + st * C::kStageBytes + C::kABytes + c * C::kBChunkBytes + a.b_box_rows * 128 + (e - box * pieces) * 16) = make_uint4(0, 0, 0, 0);
@@ -529,11 +540,11 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           d_seg += (uint32_t)(c_lo * 64);
           idesc_seg = (idesc & ~(0x3Fu << 17)) | ((uint32_t)(((c_hi - c_lo + 1) * 64) >> 3) << 17);
         }
-        const int steps = TAIL && left == 1 ? last_steps : BK / 16;
+        const int steps = TAIL && left == 1 ? last_steps : KR / 16;
         if (TAIL && --left == 0) left = nkb_seg;
         if (elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < BK / 16; ++kk)
+          for (int kk = 0; kk < KR / 16; ++kk)
             if (!TAIL || kk < steps) tc_mma_bf16(d_seg, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 128), idesc_seg, (kb | kk) ? 1u : 0u);
           tc_commit(empty0 + 8u * (uint32_t)stage);
         }
@@ -786,7 +797,7 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 
 template <int TILE_N, int BK, int MODE>
 cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
-  using C = Cfg<TILE_N, BK>;
+  using C = Cfg<TILE_N, BK, MODE & kNarrow ? 32 : BK>;
   static OncePerDevice limit;
   cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
   if (e != cudaSuccess) return e;
@@ -872,22 +883,23 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   return e;
 }
 
-template <int TILE_N, int BK, int TAIL>
+template <int TILE_N, int BK, int DEPTH>
 cudaError_t launch_s(const BigArgs &a, int num_sms, cudaStream_t st) {
   if (a.gated_f) {
     if constexpr (TILE_N == 256)
-      return a.pack > 1 ? launch_m<TILE_N, BK, kGated | kPacked | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, kGated | TAIL>(a, num_sms, st);
+      return a.pack > 1 ? launch_m<TILE_N, BK, kGated | kPacked | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, kGated | DEPTH>(a, num_sms, st);
     else
       return cudaErrorInvalidValue;
   }
   if (a.pack > 1)
-    return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, kPacked | TAIL>(a, num_sms, st);
-  return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups | TAIL>(a, num_sms, st) : launch_m<TILE_N, BK, TAIL>(a, num_sms, st);
+    return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, DEPTH ? kPacked | DEPTH : kAny>(a, num_sms, st);
+  return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, DEPTH>(a, num_sms, st);
 }
 template <int TILE_N, int BK>
 cudaError_t launch_t(const BigArgs &a, int num_sms, cudaStream_t st) {
   if constexpr (BK == 64) {
     if (a.b_tail_rows < a.b_box_rows) return launch_s<TILE_N, BK, kTail>(a, num_sms, st);
+    if (a.s <= 32) return launch_s<TILE_N, BK, kNarrow>(a, num_sms, st);
   }
   return launch_s<TILE_N, BK, 0>(a, num_sms, st);
 }
