@@ -128,7 +128,9 @@ struct MoreMaps<3> {
   CUtensorMap A, B;
 };
 // OPS: the common operands, known at compile time.  1: rows of A one behind the other, B the canonical bank; 2: the same
-// with type-strided rows (cyclic schedule); 3: rows, bank used transposed; 0: any (asked at run time).  With the
+// with type-strided rows (cyclic schedule); 3: rows, bank used transposed; 0: any (asked at run time).  Forms 1 to 3 take
+// segments of the handle's own widths: no tile of theirs is without a product.  Segments of the batch's rows (dyn_so,
+// seg_rows: the weight gradient) may all be empty, and only form 0 writes the zeros such a tile stands for.  With the
 // tests in the loops of the producers and of the MMA warp, and a branch for empty tiles in the epilogue, us, asked / compiled
 // in: FFN 768 -> 3072 at q = 2, M = 1777 33.8 / 32.8; 1024 -> 4096 at q = 4, M = 3000 42.1 / 41.1, q = 8, M = 500 24.0 / 23.6;
 // gated 768 -> 1536 interval, M = 12288 59.1 / 56.9; forward and gradients of 768 -> 3072, M = 8003 151.8 / 150.0; even where
@@ -627,7 +629,7 @@ cudaError_t launch_t(const ProjArgs &a, int num_sms, cudaStream_t st) {
     if constexpr (!GATED) {
       if (a.w_kmajor && !a.a_mn && !a.a_cyclic_rows) return launch_bk<TILE_N, TILE_M, GATED, 64, 0, 3>(a, num_sms, st);
     }
-    if (a.w_kmajor || a.a_mn) return launch_bk<TILE_N, TILE_M, GATED, 64>(a, num_sms, st);
+    if (a.w_kmajor || a.a_mn || a.dyn_so) return launch_bk<TILE_N, TILE_M, GATED, 64>(a, num_sms, st);
     return a.a_cyclic_rows ? launch_bk<TILE_N, TILE_M, GATED, 64, 0, 2>(a, num_sms, st) : launch_bk<TILE_N, TILE_M, GATED, 64, 0, 1>(a, num_sms, st);
   }
   return cudaErrorInvalidValue;

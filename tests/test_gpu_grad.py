@@ -164,3 +164,26 @@ def test_weight_gradient_blocks_that_take_every_row(q, M, s, r, schedule, bad):
     dW = grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), None if schedule == "cyclic" else H.dev_types(types), workspace=ws)
     assert grad.last_status() == (5 if bad else 0)
     assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X[good], G[good], types[good], s, r))
+
+
+@pytest.mark.parametrize("M,s,r", [
+    (60, [20, 44, 64], [128] * 3),       # one CTA per tile
+    (2000, [20, 44, 64], [128] * 3),     # clusters of CTAs per tile
+    (70, [1028, 1020], [4096] * 2),      # more tiles than CTAs: an accumulator holds the sums of the tile before
+    (70, [1024, 1024], [4096] * 2),      # the same with feature groups on 16 bytes: X as it is
+])
+@pytest.mark.parametrize("rows_of", [[0], [1], []])
+def test_weight_gradient_blocks_without_rows(M, s, r, rows_of):
+    """Blocks that no row of the batch belongs to are zero, whatever tensor memory held before: all rows of one type, and
+    no row of any."""
+    q = len(s)
+    wide = binding.ProjGrad([1024, 1024], [4096] * 2)   # leaves sums in the tensor memory of every SM
+    ones = torch.ones((64, 8192), dtype=torch.bfloat16, device="cuda")
+    wide.grad_weight(ones[:, :2048].contiguous(), ones, torch.zeros(64, dtype=torch.int32, device="cuda"))
+    types = np.full(M, rows_of[0] if rows_of else q, np.int32)
+    X, G = synth.small_ints(1, (M, sum(s)), -1, 1), synth.small_ints(2, (M, sum(r)), -1, 1)
+    grad = binding.ProjGrad(s, r)
+    dW = H.to_np(grad.grad_weight(H.to_dev(X, "bf16"), H.to_dev(G, "bf16"), H.dev_types(types)))
+    assert grad.last_status() == (0 if rows_of else 5)
+    ref = oracle.proj_vjp_w(X, G, types, s, r) if rows_of else np.zeros(dW.shape)
+    assert np.array_equal(dW, ref)
