@@ -189,6 +189,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // they were in its way where it has nothing to wait for: cyclic 2048 -> 4096 at q = 16, M = 4096 24.6 -> 21.0 us,
     // 512 -> 2048 at q = 8, M = 2048 8.65 -> 7.89; explicit types, FFN 2048 -> 4096 at q = 16, M = 8000 89.9 -> 83.3
     if (a.dyn_so) asm volatile("griddepcontrol.wait;" ::: "memory");
+    const bool whole = AMODE == 3 && __ldcg(a.whole_valid) == a.whole_rows;
     for (int e = lane; e < q * q; e += 32) {
       const uint32_t mask = a.st.valid ? a.st.keep[e] : tab->keep[e];
       int n = 0;
@@ -199,7 +200,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 : a.st.valid ? a.st.so[k + 1] - a.st.so[k]
                              : tab->so[k + 1] - tab->so[k]) /
                BK;
-      if (AMODE == 3 && e % (q + 1) == 0 && __ldcg(a.whole_valid) == a.whole_rows) n = (a.whole_rows + BK - 1) / BK;   // pair (k, k)
+      if (whole && e % (q + 1) == 0) n = (a.whole_rows + BK - 1) / BK;   // pair (k, k)
       ctl->nkb[e] = (uint16_t)n;
     }
     asm volatile("bar.arrive 1, 64;" ::: "memory");
