@@ -516,6 +516,7 @@ struct CopyArgs {
   int64_t ld_src[2];    // bytes
   int row_bytes[2];     // 0: no second matrix
   int pieces[2], piece[2];   // pieces per row, bytes of a piece (the last one may be shorter)
+  int whole_pieces[2], whole_piece[2];   // the same where `part` is asked for and whole rows are copied after all
   int slot, agents;     // bytes of a slot, slots of a CTA
   int rows;             // rows of dst
   const int *perm;
@@ -550,15 +551,17 @@ __global__ void __launch_bounds__(kMaxAgents) copy_rows_kernel(const CopyArgs a)
   if (tid >= a.agents) return;
   const uint32_t slot = base + (uint32_t)(tid * a.slot), zeros = base + (uint32_t)(a.agents * a.slot);
   const bool part = a.part && s_off[a.q] == a.part;
-  const int pieces0 = a.part && !part ? (int)((a.ld_dst[0] + a.piece[0] - 1) / a.piece[0]) : a.pieces[0];
-  const int pieces1 = a.part && !part ? (int)((a.ld_dst[1] + a.piece[1] - 1) / a.piece[1]) : a.pieces[1];
+  const bool all = a.part && !part;
+  const int pieces0 = all ? a.whole_pieces[0] : a.pieces[0], pieces1 = all ? a.whole_pieces[1] : a.pieces[1];
+  const int piece0 = all ? a.whole_piece[0] : a.piece[0], piece1 = all ? a.whole_piece[1] : a.piece[1];
   const int per_row = pieces0 + pieces1;
   const int64_t units = (int64_t)a.rows * per_row;
   uint32_t parity = 0;
   for (int64_t u = blockIdx.x + (int64_t)gridDim.x * tid; u < units; u += (int64_t)gridDim.x * a.agents) {
     const int row = (int)(u / per_row), c = (int)(u - (int64_t)row * per_row);
     const int m = c >= pieces0;
-    int at = (m ? c - pieces0 : c) * a.piece[m], length = a.part && !part ? (int)a.ld_dst[m] : a.row_bytes[m], gap_at = 1 << 30, gap = 0;
+    const int piece = m ? piece1 : piece0, at = (m ? c - pieces0 : c) * piece;
+    int length = all ? (int)a.ld_dst[m] : a.row_bytes[m], gap_at = 1 << 30, gap = 0;
     int src_row;
     if (a.hdr) {
       int t = 0;
@@ -574,7 +577,7 @@ __global__ void __launch_bounds__(kMaxAgents) copy_rows_kernel(const CopyArgs a)
       src_row = __ldg(a.perm + row);
     }
     if (at >= length) continue;
-    const uint32_t bytes = (uint32_t)min(a.piece[m], length - at);
+    const uint32_t bytes = (uint32_t)min(piece, length - at);
     // bytes [at, at + bytes) of what is taken of the row: `first` of them before the gap, the rest behind it
     const uint32_t first = (uint32_t)min(max(gap_at - at, 0), (int)bytes);
     uint8_t *dst = a.dst[m] + (int64_t)row * a.ld_dst[m] + at;
@@ -744,7 +747,18 @@ cudaError_t launch_copy_rows(CopyArgs a, cudaStream_t st) {
     a.piece[m] = a.pieces[m] ? (ceil_div(a.row_bytes[m], a.pieces[m]) + 15) / 16 * 16 : 0;
     slot = std::max(slot, a.piece[m]);
   }
+  // Whole rows have pieces of their own (in those of the parts, X of 32 groups went in 32 pieces of 128 bytes: 2048 x 8192
+  // over 16384 rows, one of them without a type, 863 us, 340 in whole pieces).  They take the slots as they are, or wider ones
+  // where that costs the parts at most a ninth of their slots.
+  int whole_slot = 0;
+  for (int m = 0; m < 2; ++m)
+    if (a.row_bytes[m]) whole_slot = std::max(whole_slot, (ceil_div((int)a.ld_dst[m], ceil_div((int)a.ld_dst[m], kMaxPiece)) + 15) / 16 * 16);
+  if (whole_slot * 8 <= slot * 9) slot = std::max(slot, whole_slot);
   a.slot = (slot + 127) / 128 * 128;
+  for (int m = 0; m < 2; ++m) {
+    a.whole_pieces[m] = a.row_bytes[m] ? ceil_div((int)a.ld_dst[m], a.slot) : 0;
+    a.whole_piece[m] = a.whole_pieces[m] ? (ceil_div((int)a.ld_dst[m], a.whole_pieces[m]) + 15) / 16 * 16 : 0;
+  }
   a.agents = std::min(kMaxAgents, kSlotBytes / a.slot - (a.hdr ? 1 : 0));
   static OncePerDevice limit;
   const cudaError_t e = limit([] { return cudaFuncSetAttribute(copy_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSlotBytes + 1024); });
