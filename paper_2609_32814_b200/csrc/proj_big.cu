@@ -280,12 +280,19 @@ __device__ __forceinline__ void decode_tiles(const BigArgs &a, Ctl *ctl) {   // 
   }
 }
 
+// kTail: the bank with the boxes of a segment's last stage.
+template <bool TAIL>
+struct TailMaps {};
+template <>
+struct TailMaps<true> {
+  CUtensorMap B, B2;
+};
+
 template <int TILE_N, int BK, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
 proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                 const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmB2,
-                const __grid_constant__ CUtensorMap tmBt, const __grid_constant__ CUtensorMap tmB2t,
-                const __grid_constant__ BigArgs a) {
+                const __grid_constant__ BigArgs a, const __grid_constant__ TailMaps<(MODE & kTail) != 0> tail) {
   constexpr int KR = MODE & kNarrow ? 32 : BK;
   using C = Cfg<TILE_N, BK, KR>;
   constexpr bool GATED = MODE & kGated, TAIL = MODE & kTail;
@@ -449,7 +456,10 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
           const uint32_t sa = smem0 + (uint32_t)stage * (uint32_t)C::kStageBytes;
           const bool last = TAIL && kb == nkb_seg - 1;
           const int box_bytes = (last ? a.b_tail_rows : a.b_box_rows) * 128;   // of a 64-column box
-          const CUtensorMap *map_b = last ? &tmBt : &tmB, *map_b2 = last ? &tmB2t : &tmB2;
+          const CUtensorMap *map_b = &tmB, *map_b2 = &tmB2;
+          if constexpr (TAIL) {
+            if (last) map_b = &tail.B, map_b2 = &tail.B2;
+          }
           if (elect_one()) {
             if (loads_a && packed) {
               if (diag_seg) {   // all rows of the tile: np types x rows_per_type rows, type-major
@@ -802,7 +812,9 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   cudaError_t e = limit([] { return cudaFuncSetAttribute(proj_big_kernel<TILE_N, BK, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes); });
   if (e != cudaSuccess) return e;
   static_assert(C::kSmemBytes <= 227 * 1024, "shared memory budget");
-  CUtensorMap tmA, tmA2, tmB, tmBt, tmB2t;
+  constexpr bool TAIL = MODE & kTail;
+  CUtensorMap tmA, tmA2, tmB;
+  TailMaps<TAIL> tail;
   const BigArgs &b = a;
   if (b.pack > 1) {
     // X as {k in group, group, row in type, type}: interval rows of a type are consecutive, cyclic ones q apart
@@ -843,7 +855,9 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
     const uint64_t str[3] = {(uint64_t)a.r * 2, (uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
     const uint32_t box[4] = {64, 1, (uint32_t)a.b_box_rows, 1}, box_t[4] = {64, 1, (uint32_t)a.b_tail_rows, 1};
     e = make_map_nd(&tmB2, a.W, 4, dims, str, box, 128);
-    if (e == cudaSuccess) e = make_map_nd(&tmB2t, a.W, 4, dims, str, box_t, 128);
+    if constexpr (TAIL) {
+      if (e == cudaSuccess) e = make_map_nd(&tail.B2, a.W, 4, dims, str, box_t, 128);
+    }
     if (e != cudaSuccess) return e;
   }
   {
@@ -852,7 +866,9 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
     const uint64_t str[2] = {(uint64_t)a.ldw * 2, (uint64_t)a.ldw * 2 * (uint64_t)a.s};
     const uint32_t box[3] = {64, (uint32_t)a.b_box_rows, 1}, box_t[3] = {64, (uint32_t)a.b_tail_rows, 1};
     e = make_map_nd(&tmB, a.W, 3, dims, str, box, 128);
-    if (e == cudaSuccess) e = make_map_nd(&tmBt, a.W, 3, dims, str, box_t, 128);
+    if constexpr (TAIL) {
+      if (e == cudaSuccess) e = make_map_nd(&tail.B, a.W, 3, dims, str, box_t, 128);
+    }
   }
   if (e != cudaSuccess) return e;
   long long tiles;
@@ -877,8 +893,11 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  if (b.gpack <= 1) tmB2 = tmB, tmB2t = tmBt;
-  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK, MODE>, tmA, tmA2, tmB, tmB2, tmBt, tmB2t, b);
+  if (b.gpack <= 1) {
+    tmB2 = tmB;
+    if constexpr (TAIL) tail.B2 = tail.B;
+  }
+  e = cudaLaunchKernelEx(&cfg, proj_big_kernel<TILE_N, BK, MODE>, tmA, tmA2, tmB, tmB2, b, tail);
   count_launch(1);
   return e;
 }
