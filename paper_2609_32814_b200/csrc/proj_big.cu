@@ -137,9 +137,7 @@ constexpr int kTail = 8;     // segments that end inside a stage: of their last 
                              // are fetched and multiplied, in multiples of 16
 
 constexpr int kNarrow = 16;  // groups of X of at most 32 columns
-constexpr int kAny = 32;     // types and groups per tile asked at run time.  Kept for several types and one group per tile without
-                             // kTail or kNarrow: 5120 -> 25600 at q = 128, M = 5888, bound by its stores, takes 156.7 us here and 170.3
-                             // as kPacked, M = 2048 the same in either
+constexpr int kAny = 32;     // the form of the tiles, gated or not too, asked at run time: see shares_lines
 
 struct Tile {
   int row0, rows;   // bucketed rows [row0, row0 + rows), all of type i; row0 < 0: no more tiles
@@ -295,7 +293,8 @@ proj_big_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const __grid_constant__ BigArgs a, const __grid_constant__ TailMaps<(MODE & kTail) != 0> tail) {
   constexpr int KR = MODE & kNarrow ? 32 : BK;
   using C = Cfg<TILE_N, BK, KR>;
-  constexpr bool GATED = MODE & kGated, TAIL = MODE & kTail;
+  constexpr bool TAIL = MODE & kTail;
+  const bool GATED = MODE & kAny ? a.gated_f != 0 : (MODE & kGated) != 0;
   const bool PACKED = MODE & kAny ? a.pack > 1 : (MODE & kPacked) != 0, GROUPS = MODE & kAny ? a.gpack > 1 : (MODE & kGroups) != 0;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -902,6 +901,17 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
   return e;
 }
 
+// Tiles of several types and one group: asked at run time (kAny) where neighbouring groups of Y share 128-byte lines and Y is
+// more than half of L2.  Such a launch is bound by its stores to the shared lines, and the compiled form only gets its CTAs
+// to them sooner; everywhere else that form is the faster one.  Asked / compiled in, us: q = 128, groups of 40 -> 200, M = 7168
+// 201.9 / 215.4, M = 5888 156 / 180, M = 2048 (105 MB) 104.9 / 110.0, M = 1536 93.1 / 96.6, M = 1024 (52 MB) 75.5 / 74.1; 40 -> 120, M = 7168 (220 MB)
+// 120.6 / 128.6, M = 1024 (31 MB) 60.2 / 48.5; whole lines: 40 -> 320, M = 6144 289 / 272, 40 -> 192, M = 2048 84 / 77; FFN at q = 32, cyclic,
+// M = 2048: 2048 -> 6144 45.6 / 37.2, 7168 -> 2048 (groups of 224) 45.4 / 40.3.
+bool shares_lines(const BigArgs &a) {
+  const int e = a.y_bf16 ? 2 : 4;
+  return a.r_out * e % 128 != 0 && (double)a.M * a.q * a.r_out * e > 64e6;
+}
+
 template <int TILE_N, int BK, int DEPTH>
 cudaError_t launch_s(const BigArgs &a, int num_sms, cudaStream_t st) {
   if (a.gated_f) {
@@ -910,8 +920,8 @@ cudaError_t launch_s(const BigArgs &a, int num_sms, cudaStream_t st) {
     else
       return cudaErrorInvalidValue;
   }
-  if (a.pack > 1)
-    return a.gpack > 1 ? launch_m<TILE_N, BK, kPacked | kGroups | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, DEPTH ? kPacked | DEPTH : kAny>(a, num_sms, st);
+  if (a.pack > 1 && a.gpack > 1) return launch_m<TILE_N, BK, kPacked | kGroups | DEPTH>(a, num_sms, st);
+  if (a.pack > 1) return DEPTH || !shares_lines(a) ? launch_m<TILE_N, BK, kPacked | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, kAny>(a, num_sms, st);
   return a.gpack > 1 ? launch_m<TILE_N, BK, kGroups | DEPTH>(a, num_sms, st) : launch_m<TILE_N, BK, DEPTH>(a, num_sms, st);
 }
 template <int TILE_N, int BK>
