@@ -612,11 +612,16 @@ cudaError_t launch_row_decode(const RowDecodeArgs &in, int num_sms, cudaStream_t
   a.units2 = a.M * pieces2 * a.ks2;
   // every CTA of an FFN must be resident for the wait between the phases: one CTA per SM at most
   const int grid = std::min(num_sms, std::max(a.units1 / a.ks1, a.units2 / a.ks2));   // at most one piece group per CTA and slot
-  // W2's share of a row (two segments).  12 layers in a graph, without / with the hint, us: gated 2048 -> 6144 at q = 32 (1.6 MB)
-  // 73.3 / 72.3; 10 layers, gated 7168 -> 2048 (1.8 MB) 66.0 / 64.8, 2048 -> 8192 at q = 16 (4.2 MB) 86.8 / 85.5, gated 2560 ->
-  // 9728 (3.1 MB) 103.7 / 104.2; gated 4096 -> 12288 (6.3 MB) 133.1 / 134.8: there the hints stand in the way of the previous
-  // layer's loads.  Several rows, 2560 -> 9728, three of them: 209.9 / 217.9.
-  a.warm2 = a.mode != 2 && 4.0 * a.D * (double)a.F / a.q <= 5e6;
+  // The hint pays where phase 2 has a piece for every CTA to itself (ks2 = all warps) up to 5 MB of W2 (a row's share, two
+  // segments), elsewhere up to 2.5 MB: with more, the hints stand in the way of the previous layer's loads.  Without / with,
+  // 10 layers in a graph, gated unless said, us.  ks2 = 8: 2048 -> 6144 at q = 32 (1.6 MB) 61.5 / 61.3, 12 layers 74.5 / 73.6; q = 16, plain:
+  // 2048 -> 6144 (3.1) 80.6 / 79.2, 2048 -> 8192 (4.2) 88.2 / 86.4; 1024 -> 4096 at q = 8 (2.1) 80.7 / 78.7; 768 -> 3072 at q = 2 (4.7)
+  // 157.6 / 153.6; 512 -> 2048 at q = 4 (1.0) 72.5 / 71.8, but 512 -> 1024 at q = 2 (1.0) 67.7 / 68.0; 2048 -> 8192 at q = 8 (8.4) 148.2 / 149.5.
+  // ks2 < 8: 7168 -> 2048 at q = 32 (1.8) 65.8 / 64.3; 4096 -> 4096, plain (2.1) 63.3 / 62.0; 3072 -> 3072 at q = 16 (2.4) 81.4 / 80.5; 2560 ->
+  // 9728 (3.1) 103.3 / 103.6; 5120 -> 5120 (3.3) even; 4096 -> 8192 (4.2) 95.1 / 95.5; 4096 -> 12288 (6.3) 133.4 / 135.2.  Not for next to
+  // nothing: 2048 -> 768 (0.2) 47.1 / 47.3.  Several rows, 2560 -> 9728, three of them: 209.9 / 217.9.
+  const double share = 4.0 * a.D * (double)a.F / a.q;
+  a.warm2 = a.mode != 2 && share >= 0.5e6 && share <= (a.ks2 == kWarps ? 5e6 : 2.5e6);
   if (a.mode == 0) return launch_mode<0>(a, grid, st);
   if (a.mode == 1) return launch_mode<1>(a, grid, st);
   return launch_mode<2>(a, grid, st);
