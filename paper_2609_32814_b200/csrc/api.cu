@@ -635,7 +635,7 @@ const PlanSlot *prepare_cyclic_plan(alg_proj_s &p, const TcChoice &tc, int64_t M
         const ClassRec &r = tab.cls[c];
         const int loc = (int)(idx - prefix[c]), ntl = (int)r.n_tiles, mt = loc / ntl, nt = loc - mt * ntl;
         rec.row0 = (int)r.i * bucket + mt * tile_m;
-        rec.rows = std::min(tile_m, bucket - mt * tile_m) | (nkb[(int)r.i * q + (int)r.j] << 16);
+        rec.rows = std::min(tile_m, bucket - mt * tile_m) | (int)((uint32_t)std::min(nkb[(int)r.i * q + (int)r.j], 0xFFFF) << 16);   // (kNkbMany)
         rec.pair = ((int)r.i * q + (int)r.j) | ((int)r.cols << 16);
         rec.n0 = r.col0 + nt * (int)r.cols;
       }

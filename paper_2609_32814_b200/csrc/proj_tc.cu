@@ -45,7 +45,7 @@ struct Ctl {
   int whole;                // the blocks (k, k) of a weight gradient take X and G as they lie
   int so[kMaxQ + 1];
   uint32_t keep[kMaxPairs];
-  uint16_t nkb[kMaxPairs];  // K blocks per tile of a pair
+  uint16_t nkb[kMaxPairs];  // K blocks per tile of a pair, at most kNkbMany
 };
 
 // Bounded wait. Returns false when the CTA is aborting.
@@ -201,7 +201,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                              : tab->so[k + 1] - tab->so[k]) /
                BK;
       if (whole && e % (q + 1) == 0) n = (a.whole_rows + BK - 1) / BK;   // pair (k, k)
-      ctl->nkb[e] = (uint16_t)n;
+      ctl->nkb[e] = (uint16_t)min(n, kNkbMany);
     }
     asm volatile("bar.arrive 1, 64;" ::: "memory");
   }
@@ -397,7 +397,12 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (lane == 0) ALG_TRACE(1, 1);
       // All kept products of the block run back to back into one accumulator, so this warp only
       // needs their total number of K blocks (upper half of rec.rows).
-      const int n_kb = __shfl_sync(0xffffffffu, (int)((uint32_t)rec.rows >> 16), 0);
+      int n_kb = __shfl_sync(0xffffffffu, (int)((uint32_t)rec.rows >> 16), 0);
+      if (n_kb == kNkbMany) {
+        const int pair = __shfl_sync(0xffffffffu, rec.pair & 0xFFFF, 0);
+        n_kb = AMODE == 3 && ctl->whole && pair % (q + 1) == 0 ? (a.whole_rows + BK - 1) / BK : blocks_of_pair<BK>(ctl->keep[pair], ctl->so, q);
+        n_kb = __shfl_sync(0xffffffffu, n_kb, 0);
+      }
       ok = __all_sync(0xffffffffu, wait_bar(tempty0 + 8u * (uint32_t)acc, acc_phase ^ 1u, ctl, a.status));
       if (!ok) break;
       if (lane == 0) ALG_TRACE(1, 2);

@@ -52,7 +52,7 @@ struct Ctl2 {
   volatile int abort_flag;
   long long wait_limit;     // bound of every wait, in clock64 cycles
   int so[kMaxQ + 1];
-  uint32_t keep[1];  // q*q entries follow, then q*q uint16 K-block counts (the request is sized for them)
+  uint32_t keep[1];  // q*q entries follow, then q*q uint16 K-block counts of at most kNkbMany (the request is sized for them)
 };
 constexpr int kMaxSmem = 227 * 1024;
 inline int smem_bytes(int n_stages, int q, int n_classes) {
@@ -170,7 +170,7 @@ proj_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     int n = 0;
     for (int k = 0; k < q; ++k)
       if ((mask >> k) & 1u) n += (a.st.valid ? a.st.so[k + 1] - a.st.so[k] : tab->so[k + 1] - tab->so[k]) / kTcBlockK;
-    nkb[e] = (uint16_t)n;
+    nkb[e] = (uint16_t)min(n, kNkbMany);
   }
   tile_map_classes(tm, tab, a.st, q, a.n_classes, threadIdx.x, kThreads);
   if (warp == 1) {  // both CTAs of the pair allocate together, same shared-memory slot
@@ -257,7 +257,11 @@ proj_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
       while (ok && __shfl_sync(0xffffffffu, rec.row0, 0) >= 0) {
         ++round;
         if (lane == 0) ALG_TRACE(1, 1);
-        const int n_kb = __shfl_sync(0xffffffffu, (int)((uint32_t)rec.rows >> 16), 0);
+        int n_kb = __shfl_sync(0xffffffffu, (int)((uint32_t)rec.rows >> 16), 0);
+        if (n_kb == kNkbMany) {
+          const int pair = __shfl_sync(0xffffffffu, rec.pair & 0xFFFF, 0);
+          n_kb = __shfl_sync(0xffffffffu, blocks_of_pair<kTcBlockK>(ctl->keep[pair], ctl->so, q), 0);
+        }
         const int cols = __shfl_sync(0xffffffffu, rec.pair >> 16, 0);
         ok = __all_sync(0xffffffffu, wait_bar2(tempty0 + 8u * (uint32_t)acc, acc_phase ^ 1u, ctl, a.status));
         if (!ok) break;

@@ -114,7 +114,17 @@ __device__ __forceinline__ int snake_index(int round, int worker, int n_workers)
   return round * n_workers + ((round & 1) ? (n_workers - 1 - worker) : worker);
 }
 // `nkb_of_pair` (optional, shared memory): number of K blocks of the tiles of a pair; it is packed
-// into the upper half of TileRec::rows so that the MMA thread needs nothing but the record.
+// into the upper half of TileRec::rows so that the MMA thread needs nothing but the record.  Reductions of kNkbMany
+// blocks and more (4.2 million rows of a weight gradient, or features) stand there as kNkbMany; the MMA warp
+// counts theirs when it comes to the tile (blocks_of_pair).
+constexpr int kNkbMany = 0xFFFF;
+template <int BK>
+__device__ __noinline__ int blocks_of_pair(uint32_t mask, const int *so, int q) {
+  int n = 0;
+  for (int k = 0; k < q; ++k)
+    if ((mask >> k) & 1u) n += (so[k + 1] - so[k]) / BK;
+  return n;
+}
 __device__ __forceinline__ TileRec tile_seq_decode(TileMap *tm, const TileGeom &g, int pos, int worker, int n_workers,
                                                    const uint16_t *nkb_of_pair) {
   const int n = tm->seq_valid;

@@ -629,3 +629,28 @@ def test_options_of_the_one_cta_kernel_hold_for_batches_that_fill_pairs():
     rows = np.arange(0, M, 41)
     ref = oracle.proj(wl.X[rows], wl.types[rows], wl.W_up, wl.d_widths, wl.f_widths)
     assert np.array_equal(H.to_np(want[torch.from_numpy(rows).cuda()]), ref)
+
+
+@pytest.mark.parametrize("kernel,stage,blocks", [
+    (1, 32, 65534), (1, 64, 65535), (1, 32, 65536),   # the last count a tile record holds, and those the MMA warp counts
+    (1, 64, 65539),
+    (2, 64, 65536),                                   # CTA pairs
+])
+@pytest.mark.parametrize("schedule", ["cyclic", "explicit"])   # tiles planned on the host and by the kernel
+def test_reductions_of_more_blocks_than_a_record_holds(kernel, stage, blocks, schedule):
+    K, N, M = blocks * stage, 128, 16
+    gen = torch.Generator(device="cuda").manual_seed(blocks)
+    X = torch.randint(-1, 2, (M, K), generator=gen, device="cuda", dtype=torch.int8).bfloat16()
+    W = torch.randint(-1, 2, (K, N), generator=gen, device="cuda", dtype=torch.int8).bfloat16()
+    proj = binding.Proj([K], [N], schedule=schedule)
+    proj.set_option("small_m_kernel", 0)
+    proj.set_option("gemm_kernel", kernel)
+    if stage == 32:
+        proj.set_option("stage_k", 32)
+    types = torch.zeros(M, dtype=torch.int32, device="cuda") if schedule == "explicit" else None
+    Y = proj.forward(X, types, W, out_dtype=torch.float32)
+    assert proj.last_status() == 0
+    want = torch.zeros((M, N), dtype=torch.float64, device="cuda")
+    for k in range(0, K, 1 << 18):   # whole numbers below 2^24: exact in either order
+        want += (X[:, k:k + (1 << 18)].double() @ W[k:k + (1 << 18)].double())
+    assert torch.equal(Y.double(), want)
