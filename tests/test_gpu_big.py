@@ -288,7 +288,9 @@ def test_more_tiles_than_records(q, M, s_w, r_w, schedule):
     assert np.array_equal(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref)
 
 
-@pytest.mark.parametrize("s_w", [16, 48, 56, 88, 112, 120])   # groups of less than a stage and the last stages of deeper ones: 16, 48, 64, 32, 48, 64 rows
+# groups of at most 32 columns (stages of 32 rows of W), of less than 64 (the stage's other rows zeroed once), and deeper ones
+# whose last stage has 32, 48 and 64 rows of W (the last is a whole stage again)
+@pytest.mark.parametrize("s_w", [16, 48, 56, 88, 112, 120])
 @pytest.mark.parametrize("r_w", [40, 168, 232])               # one, three and four 64-column boxes in a stage
 @pytest.mark.parametrize("q,rows", [(6, 40), (34, 136)])      # several types per tile; two m-tiles per type
 def test_big_stage_sizes(s_w, r_w, q, rows):
@@ -296,3 +298,28 @@ def test_big_stage_sizes(s_w, r_w, q, rows):
     Y, _ = _forward(wl, "interval", torch.float32)
     ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths)
     assert np.array_equal(H.to_np(Y), ref)
+
+
+@pytest.mark.parametrize("s_w", [16, 56, 88])                 # stages of 32 rows, whole stages, a partial last one
+@pytest.mark.parametrize("r_w", [40, 168, 256])               # one and three boxes; whole 128-byte lines
+@pytest.mark.parametrize("q,rows", [(6, 40), (34, 136), (40, 90)])   # (40, 90), 40 columns: several groups per tile
+@pytest.mark.parametrize("schedule", ["cyclic", "explicit"])
+def test_big_stage_sizes_of_other_schedules(s_w, r_w, q, rows, schedule):
+    wl = _workload(q, q * rows, s_w, r_w, schedule, seed=s_w + r_w + 1)
+    Y, _ = _forward(wl, schedule, torch.bfloat16)
+    ref = oracle.proj(wl.X, wl.types, wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(Y), H.bf16_rne(ref))
+
+
+@pytest.mark.parametrize("r_w,rows", [
+    (200, 12), (200, 13),   # 128 groups that share lines: Y of 63 and of 68 MB, either side of where tiles are asked at run time
+    (192, 13),              # whole lines
+    (120, 22),              # one box of the narrower tile, 86 MB
+])
+def test_big_packed_tiles_by_the_size_of_the_result(r_w, rows):
+    q, s_w = 128, 40
+    wl = _workload(q, q * rows, s_w, r_w, "interval", seed=rows)
+    Y, _ = _forward(wl, "interval", torch.bfloat16)
+    at = np.unique(np.r_[np.arange(0, q * rows, 5), q * rows - 1])
+    ref = oracle.proj(wl.X[at], wl.types[at], wl.W_up, wl.d_widths, wl.f_widths)
+    assert np.array_equal(H.to_np(Y[torch.from_numpy(at).cuda()]), H.bf16_rne(ref))

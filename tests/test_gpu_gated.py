@@ -160,6 +160,23 @@ def test_gated_ffn_groups_off_the_tile_grid(q, M, dw, fw, schedule):
     H.assert_bf16_close(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref, True, f"gated off-grid q={q} M={M}")
 
 
+@pytest.mark.parametrize("q,M,dw,fw,schedule", [
+    (32, 333, 24, 64, "explicit"),       # input groups of at most 32 columns: stages of 32 rows of W
+    (32, 32 * 40, 24, 64, "cyclic"),     # the same with several types per tile
+    (32, 32 * 40, 80, 304, "cyclic"),    # several types per tile, last stages of 16 rows, three column tiles
+    (20, 20 * 24, 112, 72, "cyclic"),    # last stages of 48 rows, five types per tile
+    (20, 20 * 24, 64, 200, "cyclic"),    # whole stages
+])
+def test_gated_ffn_forms_of_tiles_and_stages(q, M, dw, fw, schedule):
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(700 + q + M, M, q)
+    wl, Wg = synth.gated_ffn("gated-forms", q, M, q * dw, q * fw, types, variant=q + dw + fw)
+    wl.W_up, Wg, wl.W_down = (synth.bf16_round(w * 2.0) for w in (wl.W_up, Wg, wl.W_down))
+    Y, ffn = _run(wl, Wg, schedule=schedule, out_dtype=torch.bfloat16)
+    rows = np.unique(np.concatenate([_sample_rows(wl, 6, seed=3), np.arange(8)]))
+    ref = oracle.ffn_swiglu(wl.X[rows], wl.types[rows], Wg, wl.W_up, wl.W_down, wl.d_widths, wl.f_widths)
+    H.assert_bf16_close(H.to_np(Y[torch.from_numpy(rows).cuda()]), ref, True, f"gated forms q={q} M={M}")
+
+
 @pytest.mark.parametrize("q,dw,fw", [
     (32, 64, 192),       # 2048 -> 6144
     (32, 80, 304),       # 2560 -> 9728

@@ -140,22 +140,26 @@ def test_weight_gradient_row_copies(q, M, s, r, schedule):
     assert np.array_equal(H.to_np(dW), oracle.proj_vjp_w(X, G, types, s, r))
 
 
-@pytest.mark.parametrize("q,M,s,r,schedule", [
-    (3, 130, [64, 136, 8], [2560, 256, 2048], "explicit"),   # parts of a G row in several pieces, one of them around the gap
-    (2, 65, [128, 384], [1536, 1536], "explicit"),           # one row past whole blocks, clusters of CTAs per tile
-    (2, 1, [128, 128], [256, 256], "explicit"),              # a single row
-    (2, 2050, [1024, 1024], [4096, 4096], "explicit"),       # more tiles than CTAs: the persistent kernel
-    (4, 3 * 100, [64, 72, 80, 200], [128] * 4, "cyclic"),    # 75 rows per type: not read in place
+@pytest.mark.parametrize("q,M,s,r,schedule,bad", [
+    (3, 130, [64, 136, 8], [2560, 256, 2048], "explicit", False),   # parts of a G row in several pieces, one of them around the gap
+    (3, 130, [64, 136, 8], [2560, 256, 2048], "explicit", True),
+    (2, 65, [128, 384], [1536, 1536], "explicit", False),           # one row past whole blocks, clusters of CTAs per tile
+    (2, 65, [128, 384], [1536, 1536], "explicit", True),
+    (2, 1, [128, 128], [256, 256], "explicit", False),              # a single row
+    (2, 1, [128, 128], [256, 256], "explicit", True),
+    (2, 2050, [1024, 1024], [4096, 4096], "explicit", False),       # more tiles than CTAs: the persistent kernel
+    (2, 2050, [1024, 1024], [4096, 4096], "explicit", True),
+    (4, 3 * 100, [64, 72, 80, 200], [128] * 4, "cyclic", False),    # 75 rows per type: not read in place
+    (32, 700, [128] * 32, [128] * 32, "explicit", False),           # slots that whole rows may widen: X and G rows of one piece
+    (32, 700, [128] * 32, [128] * 32, "explicit", True),
+    (16, 300, [8] * 16, [640] * 16, "explicit", True),              # whole rows in more pieces than their parts
 ])
-@pytest.mark.parametrize("bad", [False, True])
 def test_weight_gradient_blocks_that_take_every_row(q, M, s, r, schedule, bad):
     """dW_kk is reduced over X and G as they lie, the other blocks over the parts of the rows that were copied; a batch with
     a type out of range takes everything from whole copies."""
     types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
     good = np.ones(M, bool)
     if bad:
-        if schedule == "cyclic":
-            pytest.skip("the schedule's own types are never out of range")
         types = types.copy()
         types[M // 2], good[M // 2] = q, False
     X, G = synth.small_ints(1, (M, sum(s)), -1, 1), synth.small_ints(2, (M, sum(r)), -1, 1)
@@ -187,3 +191,30 @@ def test_weight_gradient_blocks_without_rows(M, s, r, rows_of):
     assert grad.last_status() == (0 if rows_of else 5)
     ref = oracle.proj_vjp_w(X, G, types, s, r) if rows_of else np.zeros(dW.shape)
     assert np.array_equal(dW, ref)
+
+
+@pytest.mark.parametrize("q,M,s,r,schedule", [
+    (2, 300, [128, 128], [256, 256], "explicit"),        # clusters of CTAs per tile
+    (2, 70, [1024, 1024], [4096, 4096], "explicit"),     # one CTA per tile
+    (3, 515, [20, 44, 64], [128] * 3, "explicit"),       # X transposed
+    (2, 512, [128, 256], [128, 384], "cyclic"),          # X and G in place
+])
+def test_weight_gradient_of_strided_operands(q, M, s, r, schedule):
+    """X, G and a bf16 dW inside wider allocations; of explicit types also with one out of range."""
+    all_types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    K, N = sum(s), sum(r)
+    X, G = synth.small_ints(1, (M, K), -1, 1), synth.small_ints(2, (M, N), -1, 1)
+    Xp = torch.full((M, K + 24), float("nan"), dtype=torch.bfloat16, device="cuda")
+    Gp = torch.full((M, N + 8), float("nan"), dtype=torch.bfloat16, device="cuda")
+    Xp[:, :K], Gp[:, :N] = H.to_dev(X, "bf16"), H.to_dev(G, "bf16")
+    grad = binding.ProjGrad(s, r, schedule=schedule)
+    for bad in [False, True] if schedule == "explicit" else [False]:
+        types, good = all_types.copy(), np.ones(M, bool)
+        if bad:
+            types[M // 3], good[M // 3] = q, False
+        out = torch.full((K, N + 16), 7.0, dtype=torch.bfloat16, device="cuda")
+        grad.grad_weight(Xp[:, :K], Gp[:, :N], None if schedule == "cyclic" else H.dev_types(types), out=out[:, :N])
+        assert grad.last_status() == (5 if bad else 0)
+        ref = H.bf16_rne(oracle.proj_vjp_w(X[good], G[good], types[good], s, r))
+        assert np.array_equal(H.to_np(out[:, :N].contiguous()), ref)
+        assert torch.all(out[:, N:] == 7.0)
