@@ -339,10 +339,12 @@ alg_status_t alg_ffn_gated_forward(alg_ffn_t h, const void *X, const int32_t *ty
  * SIMT kernel.  A custom table must give every weight block at least one row type that uses it.
  *   grad_input : W is the forward bank (K x N, ldw >= N), used transposed in place.
  *   grad_weight: dW (K x N, lddw >= N) is overwritten, never accumulated into; blocks whose row
- *                types are absent from the batch come out zero.  Internally the rows are bucketed
- *                by type, X and G are copied into buckets padded to a multiple of 64 rows with zeros
- *                (X transposed where an input group is no multiple of 8 features), and one grouped
- *                GEMM reduces over the buckets.
+ *                types are absent from the batch come out zero.  dW may lie over X or G.  Internally
+ *                the rows are bucketed by type, X and G are copied into buckets padded to a multiple
+ *                of 64 rows with zeros (X transposed where an input group is no multiple of 8
+ *                features), and one grouped GEMM reduces over the buckets.  What every row takes part
+ *                in (the blocks dW[S_k, R_k] of the complete-graph law; all of it for whole 64-row
+ *                blocks of a cyclic schedule) is read from X and G as they lie, where dW is not there.
  * Workspace: alg_proj_grad_workspace_bytes(h, M), 256-byte aligned, no initialisation needed. */
 alg_status_t alg_proj_grad_create(alg_proj_grad_t *out, int q, const int32_t *in_widths,
                                   const int32_t *out_widths, alg_table_t table,

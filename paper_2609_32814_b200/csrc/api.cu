@@ -653,6 +653,9 @@ const PlanSlot *prepare_cyclic_plan(alg_proj_s &p, const TcChoice &tc, int64_t M
 }
 
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
+bool overlap(const void *a, size_t a_bytes, const void *b, size_t b_bytes) {
+  return (uintptr_t)a < (uintptr_t)b + b_bytes && (uintptr_t)b < (uintptr_t)a + a_bytes;
+}
 
 // Counted buckets (explicit types, or cyclic with q not dividing M) on the large-algebra kernel: always when the
 // handle has no other tensor-core kernel or asks for it; by the library's choice when the buckets are small
@@ -1450,7 +1453,10 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   // (tiled copies of feature columns start on 16 bytes: groups of a multiple of 8 features)
   bool mn = true;
   for (int e = 0; e < h->q; ++e) mn = mn && h->dx.r[e] % 8 == 0;
-  const bool in_place = mn && h->sched == ALG_SCHED_CYCLIC && M > 0 && M % (64 * (int64_t)h->q) == 0 && block_k_of(p) == 64;
+  // (a result over X or G is stored while other tiles still reduce: everything is copied then)
+  const size_t dw_bytes = ((size_t)(h->K - 1) * lddw + h->N) * elem_bytes(w_dtype), mm = (size_t)std::max<int64_t>(M, 1) - 1;
+  const bool apart = !overlap(dW, dw_bytes, X, (mm * ldx + h->K) * 2) && !overlap(dW, dw_bytes, G, (mm * ldg + h->N) * 2);
+  const bool in_place = mn && apart && h->sched == ALG_SCHED_CYCLIC && M > 0 && M % (64 * (int64_t)h->q) == 0 && block_k_of(p) == 64;
   // 1. row buckets of this batch (also for the cyclic schedule: the copies below need the permutation)
   BucketArgs b;
   b.types = h->sched == ALG_SCHED_CYCLIC ? nullptr : types;
@@ -1473,7 +1479,7 @@ alg_status_t alg_proj_grad_weight(alg_proj_grad_t h, const void *X, int64_t ldx,
   // Under the complete-graph law dW_kk is x_k^T g_k over ALL rows, whatever their types: those blocks read X and G as they
   // lie, and the buckets only need the columns that a row's type has to itself -- S_t of X and all but R_t of G, at q = 2
   // half of the bytes (768 x 3072 over 8003 rows, forward and both gradients: 158.3 -> 150.2 us; 512 x 2048 at q = 4, 7765 rows, 102.9 -> 100.4).
-  const bool whole = h->whole && mn && !in_place && block_k_of(p) == 64;
+  const bool whole = h->whole && mn && apart && !in_place && block_k_of(p) == 64;
   // 2. padded, bucketed copies of X (as it is, or transposed) and G; pad rows are zero
   if (!in_place) {
     if (!mn && launch_gather_transpose_padded(X, ldx, hdr, b.perm, h->q, mp, h->K, ws + L.xp, st) != cudaSuccess) return ALG_ERR_CUDA;

@@ -218,3 +218,23 @@ def test_weight_gradient_of_strided_operands(q, M, s, r, schedule):
         ref = H.bf16_rne(oracle.proj_vjp_w(X[good], G[good], types[good], s, r))
         assert np.array_equal(H.to_np(out[:, :N].contiguous()), ref)
         assert torch.all(out[:, N:] == 7.0)
+
+
+@pytest.mark.parametrize("schedule", ["explicit", "cyclic"])
+@pytest.mark.parametrize("over", ["X", "G"])
+def test_weight_gradient_over_an_operand(schedule, over):
+    """dW in the memory of X or G: more tiles than CTAs, so that tiles reduce after others have been stored."""
+    q, M, s, r = 2, 512, [512, 512], [5120, 5120]
+    K, N = sum(s), sum(r)
+    types = synth.cyclic_types(M, q) if schedule == "cyclic" else synth.uniform_types(M, M, q)
+    X, G = synth.small_ints(1, (M, K), -1, 1), synth.small_ints(2, (M, N), -1, 1)
+    room = torch.empty(max(M, K) * N, dtype=torch.bfloat16, device="cuda")
+    Xd, Gd = H.to_dev(X, "bf16"), H.to_dev(G, "bf16")
+    if over == "X":
+        Xd = room[:M * K].view(M, K).copy_(Xd)
+    else:
+        Gd = room[:M * N].view(M, N).copy_(Gd)
+    grad = binding.ProjGrad(s, r, schedule=schedule)
+    dW = grad.grad_weight(Xd, Gd, None if schedule == "cyclic" else H.dev_types(types), out=room[:K * N].view(K, N))
+    assert grad.last_status() == 0
+    assert np.array_equal(H.to_np(dW), H.bf16_rne(oracle.proj_vjp_w(X, G, types, s, r)))
