@@ -902,11 +902,13 @@ cudaError_t launch_m(const BigArgs &a, int num_sms, cudaStream_t st) {
 }
 
 // Tiles of several types and one group: asked at run time (kAny) where neighbouring groups of Y share 128-byte lines and Y is
-// more than half of L2.  Such a launch is bound by its stores to the shared lines, and the compiled form only gets its CTAs
-// to them sooner; everywhere else that form is the faster one.  Asked / compiled in, us: q = 128, groups of 40 -> 200, M = 7168
-// 201.9 / 215.4, M = 5888 156 / 180, M = 2048 (105 MB) 104.9 / 110.0, M = 1536 93.1 / 96.6, M = 1024 (52 MB) 75.5 / 74.1; 40 -> 120, M = 7168 (220 MB)
-// 120.6 / 128.6, M = 1024 (31 MB) 60.2 / 48.5; whole lines: 40 -> 320, M = 6144 289 / 272, 40 -> 192, M = 2048 84 / 77; FFN at q = 32, cyclic,
-// M = 2048: 2048 -> 6144 45.6 / 37.2, 7168 -> 2048 (groups of 224) 45.4 / 40.3.
+// more than half of L2.  A line that two tiles write then leaves L2 half written and is read back for the other half, the
+// more of them the further apart the CTAs run: 40 -> 200 at q = 128, M = 7168 reads 488 MB of DRAM compiled in and 410 asked, X and W
+// are 335; groups of 192 columns, whole lines, read X and W once (326 MB) in either form.  Everywhere else the compiled form is
+// the faster one.  Asked / compiled in, us: q = 128, 40 -> 200, M = 7168 201.9 / 215.4, M = 5888 156 / 180, M = 2048 (105 MB) 104.9 / 110.0,
+// M = 1536 93.1 / 96.6, M = 1024 (52 MB) 75.5 / 74.1; 40 -> 120, M = 7168 (220 MB) 120.6 / 128.6, M = 1024 (31 MB) 60.2 / 48.5; whole lines:
+// 40 -> 320, M = 6144 289 / 272, 40 -> 192, M = 2048 84 / 77; FFN at q = 32, cyclic, M = 2048: 2048 -> 6144 45.6 / 37.2, 7168 -> 2048 (groups
+// of 224) 45.4 / 40.3.
 bool shares_lines(const BigArgs &a) {
   const int e = a.y_bf16 ? 2 : 4;
   return a.r_out * e % 128 != 0 && (double)a.M * a.q * a.r_out * e > 64e6;
